@@ -273,7 +273,10 @@ qap_status qap_search_async(qap_ctx* ctx, const qap_search_params* params,
 /* Launch shape a search would use.  Errors: as qap_search_async. */
 typedef struct {
   int32_t threads_per_walk;
-  int32_t pairs_per_thread;  /* register slots per thread                 */
+  int32_t pairs_per_thread;  /* register slots per thread of the plan's row
+                                layout; int8 flows under QAP_TABU_PAIR without
+                                a penalty run a layout of the same threads in
+                                which fewer of them hold more pairs          */
   int32_t smem_bytes;        /* dynamic shared memory per CTA             */
   int32_t grid;              /* CTAs of the persistent launch             */
   int32_t ctas_per_sm;

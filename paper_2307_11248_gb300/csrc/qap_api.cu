@@ -46,8 +46,17 @@ struct qap_ctx {
 // Instances of a batch that share one launch plan (a size class).
 struct BatchClass {
   Plan plan;
-  const void* fn = nullptr;
-  int smem = 0, grid = 0, ctas_per_sm = 0;
+  // the launch of the plan, and of its row layout (the same unless the plan
+  // is in the rotation layout): both made with the class, so that a search
+  // whose tenures need the rows finds them ready
+  struct Shape {
+    const void* fn = nullptr;
+    int smem = 0, grid = 0, ctas_per_sm = 0, notr = 0;
+  } own, rows;
+  int nmax = 0;
+  const Shape& shape(const qap_search_params* p) const {
+    return plan.rot && !rot_holds_tenures(plan, p, nmax) ? rows : own;
+  }
   std::vector<int> members;  // instance indices, largest n first
   int item_off = 0, items = 0;
   size_t ws_off = 0, ws_stride = 0;
@@ -105,9 +114,10 @@ qap_status occupancy(Launch* L, int sms, int work) {
 
 qap_status plan_ctx(qap_ctx* ctx, const qap_search_params* p, Launch* L) {
   const bool many = p->starts >= 2 * ctx->sms;
-  if (!choose_plan_fit(ctx->di.n, p->threads_per_walk, many, &ctx->di, 1, ctx->fbytes,
-                       ctx->dbytes, ctx->smem_optin, 0, p->phase_x, &L->plan))
+  if (!search_plan(ctx->di.n, many, &ctx->di, 1, ctx->fbytes, ctx->dbytes, ctx->smem_optin, 0, p,
+                   &L->plan))
     return QAP_EUNSUPPORTED;
+  if (!rot_holds_tenures(L->plan, p, ctx->di.n)) L->plan = L->plan.rows();
   L->fn = reinterpret_cast<const void*>(pick_walk_kernel(ctx->dbytes, ctx->fbytes, L->plan));
   if (!L->fn) return QAP_EUNSUPPORTED;
   L->smem = plan_smem(L->plan, &ctx->di, 1, ctx->fbytes, ctx->dbytes);
@@ -118,9 +128,10 @@ qap_status plan_ctx(qap_ctx* ctx, const qap_search_params* p, Launch* L) {
 qap_status plan_batch(qap_batch* b, const qap_search_params* p, Launch* L) {
   // the batch kernel also holds one static int
   const bool many = (int64_t)b->count * p->starts >= 2 * (int64_t)b->sms;
-  if (!choose_plan_fit(b->nmax, p->threads_per_walk, many, b->di.data(), b->count, b->fbytes,
-                       b->dbytes, b->smem_optin, 16, p->phase_x, &L->plan))
+  if (!search_plan(b->nmax, many, b->di.data(), b->count, b->fbytes, b->dbytes, b->smem_optin, 16,
+                   p, &L->plan))
     return QAP_EUNSUPPORTED;
+  if (!rot_holds_tenures(L->plan, p, b->nmax)) L->plan = L->plan.rows();
   L->fn = reinterpret_cast<const void*>(pick_batch_kernel(b->dbytes, b->fbytes, L->plan));
   if (!L->fn) return QAP_EUNSUPPORTED;
   L->smem = plan_smem(L->plan, b->di.data(), b->count, b->fbytes, b->dbytes);
@@ -151,16 +162,24 @@ qap_status class_shape(qap_batch* b, BatchClass& c, int W, const qap_search_para
     dm.push_back(b->di[i]);
     nmax = std::max(nmax, b->di[i].n);
   }
-  c.smem = plan_smem(c.plan, dm.data(), (int)dm.size(), b->fbytes, b->dbytes);
-  c.fn = reinterpret_cast<const void*>(pick_batch_kernel(b->dbytes, b->fbytes, c.plan));
-  if (!c.fn) return QAP_EUNSUPPORTED;
-  QAP_TRY(prepare_kernel(c.fn, c.smem));
-  int occ = 0;
-  QAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, c.fn, c.plan.nt, c.smem));
-  if (occ < 1) return QAP_EUNSUPPORTED;
+  c.nmax = nmax;
   c.items = (int)c.members.size() * W;
-  c.ctas_per_sm = occ;
-  c.grid = std::min(c.items, occ * b->sms);
+  auto shape_of = [&](const Plan& plan, BatchClass::Shape* o) -> qap_status {
+    o->smem = plan_smem(plan, dm.data(), (int)dm.size(), b->fbytes, b->dbytes);
+    o->fn = reinterpret_cast<const void*>(pick_batch_kernel(b->dbytes, b->fbytes, plan));
+    if (!o->fn) return QAP_EUNSUPPORTED;
+    QAP_TRY(prepare_kernel(o->fn, o->smem));
+    int occ = 0;
+    QAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, o->fn, plan.nt, o->smem));
+    if (occ < 1) return QAP_EUNSUPPORTED;
+    o->ctas_per_sm = occ;
+    o->grid = std::min(c.items, occ * b->sms);
+    o->notr = (plan.store & qapk::kNoTransposed) != 0;
+    return QAP_OK;
+  };
+  QAP_TRY(shape_of(c.plan, &c.own));
+  c.rows = c.own;
+  if (c.plan.rot) QAP_TRY(shape_of(c.plan.rows(), &c.rows));
   const WsLayout wl = ws_layout(c.plan, b->dbytes, b->fbytes, nmax, p);
   c.ws_stride = wl.stride;
   c.p_off = wl.p_off;
@@ -197,14 +216,15 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
   for (int i = 0; i < b->count; ++i) {
     if (p->threads_per_walk == 0 && !b->tuned.empty() && b->tuned[i].nt != 0) {
       plan_of[i] = b->tuned[i];
+      if (p->phase_x == QAP_PHASE_X_DOTS || rules) plan_of[i] = plan_of[i].rows();
       if (p->phase_x == QAP_PHASE_X_DOTS) plan_of[i].store &= ~qapk::kProductM;
       continue;
     }
     // the batch kernel also holds one static int
     // the classes run together: walks of the whole batch fill the SMs
     const bool many = (int64_t)b->count * W >= 2 * (int64_t)b->sms;
-    if (!choose_plan_fit(b->di[i].n, p->threads_per_walk, many, &b->di[i], 1, b->fbytes,
-                         b->dbytes, b->smem_optin, 16, p->phase_x, &plan_of[i]))
+    if (!search_plan(b->di[i].n, many, &b->di[i], 1, b->fbytes, b->dbytes, b->smem_optin, 16, p,
+                     &plan_of[i]))
       return QAP_EUNSUPPORTED;
   }
   std::vector<int> order(b->count);
@@ -214,13 +234,10 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
   // keep the old classes' streams and events for reuse
   std::vector<BatchClass> old;
   old.swap(b->classes);
-  auto same = [](const Plan& x, const Plan& y) {
-    return x.nt == y.nt && x.maxpt == y.maxpt && x.store == y.store;
-  };
   for (int i : order) {  // classes appear in order of their largest n
     BatchClass* c = nullptr;
     for (BatchClass& k : b->classes)
-      if (same(k.plan, plan_of[i])) c = &k;
+      if (k.plan == plan_of[i]) c = &k;
     if (!c) {
       b->classes.emplace_back();
       c = &b->classes.back();
@@ -247,7 +264,7 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
     c.item_off = item_off;
     item_off += c.items;
     c.ws_off = ws_off;
-    ws_off += (c.ws_stride * c.grid + 255) / 256 * 256;
+    ws_off += (c.ws_stride * c.own.grid + 255) / 256 * 256;
     if (b->classes.size() > 1) {
       if (!c.side) QAP_CUDA(cudaStreamCreateWithFlags(&c.side, cudaStreamNonBlocking));
       if (!c.done) QAP_CUDA(cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming));
@@ -398,6 +415,7 @@ qap_status qap_search_async(qap_ctx* ctx, const qap_search_params* params,
   qapk::WalkArgs a{};
   a.inst = inst_args(ctx->di, ctx->dF, ctx->dFt, ctx->dD, L.plan.nt, ctx->fbytes);
   a.s = make_search_args(params, out, ctx->di.n);
+  a.notr = (L.plan.store & qapk::kNoTransposed) != 0;
   a.starts = d_starts;
   a.walks = params->starts;
   a.walk_offset = 0;
@@ -639,9 +657,10 @@ qap_status qap_batch_plan(qap_batch* b, const qap_search_params* params, qap_pla
   const BatchClass& c = b->classes.front();  // the class of the largest n
   out->threads_per_walk = c.plan.nt;
   out->pairs_per_thread = c.plan.maxpt;
-  out->smem_bytes = c.smem;
-  out->grid = c.grid;
-  out->ctas_per_sm = c.ctas_per_sm;
+  const BatchClass::Shape& sh = c.shape(params);
+  out->smem_bytes = sh.smem;
+  out->grid = sh.grid;
+  out->ctas_per_sm = sh.ctas_per_sm;
   out->sms = b->sms;
   out->classes = (int32_t)b->classes.size();
   out->products = products_form(c.plan);
@@ -682,9 +701,10 @@ qap_status qap_batch_classes(qap_batch* b, const qap_search_params* params,
     o.pairs_per_thread = c.plan.maxpt;
     o.products = products_form(c.plan);
     o.workspace = (c.plan.store & qapk::kGlobalDelta) != 0;
-    o.grid = c.grid;
-    o.ctas_per_sm = c.ctas_per_sm;
-    o.smem_bytes = c.smem;
+    const BatchClass::Shape& sh = c.shape(params);
+    o.grid = sh.grid;
+    o.ctas_per_sm = sh.ctas_per_sm;
+    o.smem_bytes = sh.smem;
     o.delta_bytes = b->dbytes;
     o.flow_bytes = b->fbytes;
     o.dist_bytes = pbytes_of(b->fbytes);
@@ -765,7 +785,9 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
                               b->smem_optin, 16))) {
         cands.push_back(p);
         const Plan m = with_products(p, b->fbytes, tp.phase_x, fits);
-        if (m.store != p.store) cands.push_back(m);
+        if (m.store != p.store)
+          cands.push_back(with_rotation(m, dm.data(), (int)dm.size(), b->fbytes,
+                                        uses_rule_tables(&tp), fits));
       }
     }
     if (qapk::row_segments(nmax, kLargePlan.maxpt) <= kLargePlan.nt) {
@@ -796,7 +818,8 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       c.plan = cand;
       c.members = rc.members;
       if ((st = class_shape(b, c, W, &tp)) != QAP_OK) return fail(st);
-      if ((st = grow(&b->ws, &b->ws_bytes, c.ws_stride * c.grid)) != QAP_OK) return fail(st);
+      const BatchClass::Shape& sh = c.shape(&tp);
+      if ((st = grow(&b->ws, &b->ws_bytes, c.ws_stride * sh.grid)) != QAP_OK) return fail(st);
       qapk::BatchArgs a{};
       a.insts = b->d_insts + (size_t)nt_index(c.plan.nt) * b->count;
       a.item_inst = d_items;
@@ -804,26 +827,25 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       a.row_base = d_items + 2 * items;
       a.items = c.items;
       a.counter = counter;
+      a.notr = sh.notr;
       a.s = make_search_args(&tp, &dout, b->nmax);
       a.s.rws_off = c.rws_off;
       a.s.p_off = c.p_off;
       a.ws_stride = c.ws_stride;
       a.ws = c.ws_stride ? static_cast<unsigned char*>(b->ws) : nullptr;
-      const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(c.fn));
+      const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(sh.fn));
       float ms = 0.f;
       for (int rep = 0; rep < 2; ++rep) {  // a warm-up run, then the timed one
         cudaMemsetAsync(counter, 0, sizeof(int), b->stream);
         if (rep) cudaEventRecord(t0, b->stream);
-        fn<<<c.grid, c.plan.nt, c.smem, b->stream>>>(a);
+        fn<<<sh.grid, c.plan.nt, sh.smem, b->stream>>>(a);
         if (rep) cudaEventRecord(t1, b->stream);
       }
       // a trial that did not launch would time as the fastest
       if ((st = chk(cudaGetLastError(), "autotune launch")) != QAP_OK) return fail(st);
       if ((st = chk(cudaEventSynchronize(t1), "autotune trial")) != QAP_OK) return fail(st);
       cudaEventElapsedTime(&ms, t0, t1);
-      const bool is_rule = cand.nt == rc.plan.nt && cand.maxpt == rc.plan.maxpt &&
-                           cand.store == rc.plan.store;
-      if (is_rule) rule_ms = ms;
+      if (cand == rc.plan) rule_ms = ms;
       if (best_ms < 0.f || ms < best_ms) {
         best_ms = ms;
         best = cand;
@@ -878,15 +900,17 @@ qap_status qap_batch_search_async(qap_batch* b, const qap_search_params* params,
     a.row_base = b->d_class_items + 2 * total;
     a.items = c.items;
     a.counter = b->d_counter + k * kCounterStride;
+    const BatchClass::Shape& sh = c.shape(params);
+    a.notr = sh.notr;
     a.s = make_search_args(params, out, p_stride);
     a.s.rws_off = c.rws_off;
     a.s.p_off = c.p_off;
     a.ws_stride = c.ws_stride;
     a.ws = c.ws_stride ? static_cast<unsigned char*>(b->ws) + c.ws_off : nullptr;
     QAP_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(int), cs));
-    const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(c.fn));
+    const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(sh.fn));
     if (b->timing) QAP_CUDA(cudaEventRecord(c.t0, cs));
-    fn<<<c.grid, c.plan.nt, c.smem, cs>>>(a);
+    fn<<<sh.grid, c.plan.nt, sh.smem, cs>>>(a);
     QAP_CUDA(cudaGetLastError());
     if (b->timing) QAP_CUDA(cudaEventRecord(c.t1, cs));
     c.timed = b->timing != 0;
@@ -1056,6 +1080,7 @@ extern "C" qap_status qap_batch_search_noalloc(qap_batch* b, const qap_search_pa
   a.row_base = d_items + 2 * items;
   a.items = (int)items;
   a.counter = d_counter;
+  a.notr = (L.plan.store & qapk::kNoTransposed) != 0;
   a.s = make_search_args(params, out, p_stride);
   const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(L.fn));
   fn<<<L.grid, L.plan.nt, L.smem, s>>>(a);

@@ -13,6 +13,7 @@
 
 #include "../../include/qap.h"
 #include "qap_kernels.cuh"
+#include "qap_rotation.cuh"
 
 namespace qapk {
 WalkKernelFn walk_kernel_i32_f8(int nt, int maxpt, int store);
@@ -25,6 +26,8 @@ BatchKernelFn batch_kernel_i32_f8m(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i32_f16(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i64_f16(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i64_f64(int nt, int maxpt, int store);
+WalkKernelFn rot_walk_kernel_f8(int nt, int c);
+BatchKernelFn rot_batch_kernel_f8(int nt, int c);
 }  // namespace qapk
 
 namespace qaph {
@@ -56,6 +59,13 @@ struct Plan {
   int nt;
   int maxpt;
   int store;  // qapk::kGlobalDelta, kGlobalFlow, kProductM, kGlobalP bits (0: all on chip)
+  int rot = 0;  // rotation layout (qap_rotation.cuh): partner blocks per thread, 0 for rows
+  int row = 0;  // with rot: `store` of the row layout, for the searches that need it
+
+  bool operator==(const Plan& o) const {
+    return nt == o.nt && maxpt == o.maxpt && store == o.store && rot == o.rot && row == o.row;
+  }
+  Plan rows() const { return rot ? Plan{nt, maxpt, row} : *this; }
 };
 
 // The large-n plan: 1024 threads, up to 40 slots each in a global workspace
@@ -122,6 +132,9 @@ struct DevInstance {
   int bytevec = 0;  // every difference of two F entries, and of two D entries, fits int8
   int diff16 = 0;   // every difference of two F entries fits int16, of two D entries int8
   int wide = 0;     // outside the narrow paths: int64 elements and arithmetic
+  // narrow paths: the largest difference of two F entries and of two D
+  // entries, and the range of a product of an F and a D entry
+  int64_t rangeF = 0, rangeD = 0, loFD = 0, hiFD = 0;
 };
 
 // Largest bound of the int64 path.  With B = (n^2 + 8n + 32) max|F| max|D|
@@ -184,6 +197,13 @@ inline qap_status inspect_instance(const int64_t* F, const int64_t* D, int n, De
   // overflow here: on this branch the ranges fit int16 and int8)
   di->bytevec = !di->wide && mF <= 127 && hiF - loF <= 127 && hiD - loD <= 127;
   di->diff16 = !di->wide && hiF - loF <= 32767 && hiD - loD <= 127;
+  if (!di->wide) {
+    di->rangeF = hiF - loF;
+    di->rangeD = hiD - loD;
+    const auto fd = std::minmax({loF * loD, loF * hiD, hiF * loD, hiF * hiD});
+    di->loFD = fd.first;
+    di->hiFD = fd.second;
+  }
   return QAP_OK;
 }
 
@@ -225,6 +245,7 @@ inline qap_status device_attrs(int* device, int* sms, int* smem_optin) {
 }
 
 inline qapk::WalkKernelFn pick_walk_kernel(int dbytes, int fbytes, const Plan& p) {
+  if (p.rot) return qapk::rot_walk_kernel_f8(p.nt, p.rot);
   if (fbytes == 8) return qapk::walk_kernel_i64_f64(p.nt, p.maxpt, p.store);
   if (dbytes == 8) return qapk::walk_kernel_i64_f16(p.nt, p.maxpt, p.store);
   if (fbytes == 1) return qapk::walk_kernel_i32_f8(p.nt, p.maxpt, p.store);
@@ -232,6 +253,7 @@ inline qapk::WalkKernelFn pick_walk_kernel(int dbytes, int fbytes, const Plan& p
 }
 
 inline qapk::BatchKernelFn pick_batch_kernel(int dbytes, int fbytes, const Plan& p) {
+  if (p.rot) return qapk::rot_batch_kernel_f8(p.nt, p.rot);
   if (fbytes == 8) return qapk::batch_kernel_i64_f64(p.nt, p.maxpt, p.store);
   if (dbytes == 8) return qapk::batch_kernel_i64_f16(p.nt, p.maxpt, p.store);
   if (fbytes == 1) return qapk::batch_kernel_i32_f8(p.nt, p.maxpt, p.store);
@@ -241,6 +263,14 @@ inline qapk::BatchKernelFn pick_batch_kernel(int dbytes, int fbytes, const Plan&
 // Shared memory of a plan for the instance shapes `d` (the largest over them).
 inline int plan_smem(const Plan& p, const DevInstance* d, int count, int fbytes, int dbytes) {
   int smem = 0;
+  if (p.rot) {
+    for (int i = 0; i < count; ++i)
+      smem = std::max(smem, qapk::rot_layout(d[i].n, d[i].ldF, d[i].ldP, d[i].symF, d[i].symD,
+                                             p.store & qapk::kNoTransposed,
+                                             qapk::rot_fixed_bytes(p.nt))
+                                .bytes);
+    return smem;
+  }
   for (int i = 0; i < count; ++i)
     smem = std::max(smem, qapk::smem_layout(d[i].n, d[i].ldF, fbytes, d[i].ldP, d[i].symF,
                                             d[i].symD, dbytes, p.nt * p.maxpt, p.store)
@@ -293,6 +323,49 @@ inline Plan with_products(Plan p, int fbytes, int form, Fits fits) {
   if (!has_notrans_form(p, fbytes)) return p;
   m.store |= qapk::kNoTransposed;
   return fits(m) ? m : p;
+}
+
+// Whether every scan candidate of an instance, (delta + g - g0) 2^S plus its
+// low bits, stays within 2^30 of zero: a delta is at most 2 (n - 1) products of
+// an F and a D difference, g the sum of 2n products of an F and a D entry, g0
+// its mid-range.
+inline bool rot_fits_keys(const DevInstance& d, int nt) {
+  const int64_t x = 2 * (d.n - 1) * d.rangeF * d.rangeD + d.n * (d.hiFD - d.loFD) + 1;
+  return x << qapk::rot_key_bits(nt) < (int64_t)1 << 30;
+}
+
+// The rotation layout in place of the row layout's products form: int8
+// flows, the paper's own criterion without a penalty, and the fewest partner
+// blocks per thread that hold every instance `d`; without the transposed
+// copies of F and P where it fits only so.  `fits` says whether a plan fits.
+template <typename Fits>
+inline Plan with_rotation(Plan p, const DevInstance* d, int count, int fbytes, bool rules,
+                          Fits fits) {
+  if (rules || fbytes != 1 || !(p.store & qapk::kProductM)) return p;
+  for (int i = 0; i < count; ++i)
+    if (!rot_fits_keys(d[i], p.nt)) return p;
+  for (int c = 1; c <= qapk::kRotMaxC; ++c) {
+    bool holds = qapk::rot_compiled(p.nt, c);
+    for (int i = 0; i < count; ++i) holds &= qapk::rot_chunks(d[i].n, p.nt, c) > 0;
+    if (!holds) continue;
+    Plan q = p;
+    q.rot = c;
+    q.row = p.store;
+    if (fits(q)) return q;
+    q.store |= qapk::kNoTransposed;
+    return fits(q) ? q : p;
+  }
+  return p;
+}
+
+// Whether a plan's rotation layout holds a search's tenures on instances of
+// up to nmax indices (see kernel's ring); else its row layout runs.
+inline bool rot_holds_tenures(const Plan& p, const qap_search_params* sp, int nmax) {
+  if (sp->iters == 0) return true;
+  int tmax = sp->tenure.tmax;
+  if (sp->tenure_per_n)
+    tmax = std::max(std::max(1, sp->tenure.tmin * nmax / 100), (tmax * nmax + 99) / 100);
+  return qapk::rot_ring_holds(p.nt, tmax);
 }
 
 // The int64 element path reads F and F^T from global memory (L1-cached,
@@ -366,6 +439,25 @@ inline size_t p_workspace(const Plan& p, int fbytes, int nmax) {
 
 inline bool uses_rule_tables(const qap_search_params* sp) {
   return sp->iters > 0 && (sp->criterion != QAP_TABU_PAIR || sp->freq_penalty != 0);
+}
+
+// The plan a search takes: choose_plan_fit's, in the rotation layout where
+// that applies and still lets two CTAs share an SM where the row layout does.
+// (Its tenures are another condition: rot_holds_tenures.)
+inline bool search_plan(int nmax, bool many, const DevInstance* d, int count, int fbytes,
+                        int dbytes, int smem_optin, int reserve, const qap_search_params* sp,
+                        Plan* out) {
+  if (!choose_plan_fit(nmax, sp->threads_per_walk, many, d, count, fbytes, dbytes, smem_optin,
+                       reserve, sp->phase_x, out))
+    return false;
+  auto ctas = [&](const Plan& x) {  // by shared memory (1 KB reserved for each), 2 at most
+    const int smem = plan_smem(x, d, count, fbytes, dbytes) + reserve;
+    return smem > smem_optin ? 0 : 2 * (smem + 1024) <= smem_optin + 1024 ? 2 : 1;
+  };
+  const int want = out->nt <= 256 ? ctas(*out) : 1;  // (above, registers hold one)
+  *out = with_rotation(*out, d, count, fbytes, uses_rule_tables(sp),
+                       [&](const Plan& x) { return ctas(x) >= want; });
+  return true;
 }
 
 struct WsLayout {
@@ -591,6 +683,7 @@ inline qapk::InstArgs inst_args(const DevInstance& d, const void* F, const void*
   I.symD = d.symD;
   I.group = group_for(d.n, nt, fbytes);
   I.diff16 = d.diff16;
+  I.g0 = (int)(d.n * (d.loFD + d.hiFD));
   I.F = F;
   I.Ft = d.symF ? F : Ft;
   I.D = D;

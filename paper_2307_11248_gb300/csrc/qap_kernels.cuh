@@ -62,6 +62,7 @@ struct InstArgs {
   int symF, symD;
   int group;          // lanes per phase-X task (1, 2, 4 or 8)
   int diff16;         // differences of two F entries fit int16, of two D entries int8
+  int g0;             // rotation layout: mid-range of g
   const void* F;      // n x ldF (int8, int16 or int64), row-major, zero padded
   const void* Ft;     // transpose of F (== F when symF)
   const void* D;      // n x n, row-major (int8, or int64 with int64 flows)
@@ -97,6 +98,7 @@ struct WalkArgs {
   SearchArgs s;
   unsigned char* ws;      // large-n plans: per-CTA workspace (deltas, tabu stamps)
   size_t ws_stride;       // bytes per CTA
+  int notr;               // rotation layout: no transposed copies of F and P
   int walks;              // walks processed by this launch
   int walk_offset;        // index of this launch's first walk among the instance's walks
   const int32_t* starts;  // (walk_offset + walks) x n, or null
@@ -112,6 +114,7 @@ struct BatchArgs {
   const int32_t* row_base;
   int items;
   int* counter;           // zeroed before the launch
+  int notr;               // rotation layout: no transposed copies of F and P
   SearchArgs s;
   unsigned char* ws;      // large-n plans: per-CTA workspace (deltas, tabu stamps)
   size_t ws_stride;       // bytes per CTA

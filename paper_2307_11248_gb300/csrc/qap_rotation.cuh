@@ -1,0 +1,1100 @@
+// Rotation layout of the walk kernels (sm_103a): int8 flows, the paper's own
+// tabu criterion, phase X from the maintained products M.
+//
+// Same search and same two barriers per iteration as qap_kernels.cuh; what
+// differs is how a walk's pairs lie in the registers, what a pair costs, and
+// that warps have roles.
+//
+// Layout.  The n indices form n2 = ceil(n / 2) blocks of two (a phantom index
+// fills an odd n).  Thread (m, j) holds block m against the C partner blocks
+// m + 1 + jC + i (mod n2), i < C: 4 pairs each, and the pair inside block m.
+// Going round, every unordered pair of blocks lies within n2 / 2 steps of one
+// of its members, so J threads per block with J C >= n2 / 2 hold every pair;
+// steps past n2 / 2 hold pairs a second time, which changes nothing (equal
+// values, equal keys).  No slot is ever invalid, so the loops carry no bounds
+// checks; consecutive threads read consecutive 16-byte words (two partners'
+// operands, 4 pairs), free of bank conflicts; and a thread's own operands
+// stay in registers for all its slots.
+//
+// What a pair costs.  The table holds d(u, v) = delta(u, v) + g[u] + g[v]
+// (with g less its mid-range), whose O(1) update is one dp4a accumulating into
+// it: the w terms of the plain delta's update are exactly the changes of g.
+// The scan's candidate is e = d 2^S + psi[u], one multiply-add: delta + g[v]
+// in the high bits, an index of the partner in the low S, so that a running
+// minimum carries its argument (the lowest partner is also the lowest pair of
+// a fixed v).  A tabu pair's d carries 2^(31 - S) on top, the sign bit of e:
+// with psi lowered by 2^30 the others are negative and tabu pairs are not, the
+// signed minimum of e is the best pair that is not tabu and the unsigned one
+// the best that is.  The 2 C pairs with r or s as partner, and the rows of r
+// and s, take phase X's values before the scan; those bring their tabu bits
+// along (phase X reads the pairs' end times), so marking the applied pair
+// costs nothing, and the end of a tabu time is an event: the pairs that end at
+// an iteration hang on that iteration's word of a ring.
+//
+// Roles.  The first warps hold the pairs, then come phase X's (one thread per
+// index), the rest help to bring M up to date; an iteration is phase X, a
+// barrier, then table and scan beside M's update, a barrier.
+//
+// M's update is put off: the byte operands of up to 2 moves (4 on symmetric
+// instances, whose two products are equal) collect in one word per index, one
+// dp4a per entry of M then applies them together, and phase X corrects the
+// four entries per index that it reads by one dp4a each.
+//
+// Bound: the fixed latencies of one iteration's chain (arg-min, phase X,
+// table, scan, two barriers) with one or two walks on an SM, integer issue
+// with more.  Measured against the row layout's products form (one GB300, same
+// box): n = 100 grid, 1024 walks x (2opt + 10^4) 150.0 -> 50.5 ms; n = 50
+// asymmetric, 256 walks x 5000 7.85 -> 4.66 ms; n = 139 asymmetric, 150 walks
+// x 2000 8.73 -> 3.18 ms; n = 23, 100 walks x 1000 in one blocking call 1.21 ->
+// 0.83 ms; 2opt from 32 starts at n = 12 16.4 -> 12.3 us.  Warp instructions per
+// walk-iteration: n = 100 grid 10360 -> 3370, n = 50 asymmetric 3606 -> 1920.
+// Tried and slower: every warp holding pairs and phase X on some of them
+// (n = 100 2.33 against 1.44 us per iteration of two walks per SM); tabu times
+// checked by each thread through its earliest (0.3 us per iteration on the
+// critical path); M updated by 4 moves at once every fourth move (the burst
+// outlasts the scan beside it).
+#pragma once
+#include "qap_kernels.cuh"
+
+namespace qapk {
+
+// Threads that may hold pairs: the same number of warps on each of an SM's
+// four schedulers (from 256 threads).
+__host__ __device__ constexpr int rot_owners(int nt) { return nt == 1024 ? 768 : nt / 2; }
+
+// Indices, with a phantom, that a thread count holds at most.
+__host__ __device__ constexpr int rot_max_n(int nt) { return nt == 128 ? 64 : nt == 256 ? 128 : 192; }
+
+// Threads per block of two (J) at c partner blocks each: the fewest that hold
+// every pair; 0 when nt threads do not hold n (its pairs, or its indices).
+__host__ __device__ inline int rot_chunks(int n, int nt, int c) {
+  const int n2 = (n + 1) / 2, j = (n2 / 2 + c - 1) / c;
+  return n >= 3 && n <= rot_max_n(nt) && j * n2 <= rot_owners(nt) &&
+                 (n + 31) / 32 * 32 <= nt - rot_owners(nt) && j * c <= n2 - 1
+             ? j
+             : 0;
+}
+
+// Low bits S of a scan candidate.  Up to 256 threads (n <= 128) they are the
+// partner itself; beyond, its rank in the thread's window (at most 31), with
+// 32 on top before the circle's wrap, half an addition more per pair.
+__host__ __device__ constexpr bool rot_rank(int nt) { return nt >= 512; }
+__host__ __device__ constexpr int rot_key_bits(int nt) { return rot_rank(nt) ? 6 : 7; }
+
+// Ends of tabu times that lie ahead are kept in a ring of this many
+// iterations; searches with longer tenures take the row layout.
+__host__ __device__ constexpr int rot_ring(int nt) { return nt <= 256 ? 256 : 512; }
+__host__ __device__ inline bool rot_ring_holds(int nt, int tmax) {
+  return tmax <= rot_ring(nt) - 2;
+}
+
+// Barrier of the CTA; the warps of each role reach it from their own code.
+__device__ __forceinline__ void rot_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
+
+// What a walk is, for the functions of its roles: in shared memory, so that
+// no register holds it through the iterations.
+struct RotWalkArgs {
+  InstArgs I;
+  SearchArgs s;
+  int64_t cost;    // of the start permutation
+  const int32_t* start;
+  int row, notr;
+  uint32_t wid;
+};
+constexpr int kRotArgsBytes = (sizeof(RotWalkArgs) + 15) / 16 * 16;
+
+// Shared memory: arrays of a fixed size per thread count first, so that their
+// addresses are constants, then the instance's own.
+template <int NT>
+struct RotFixed {
+  static constexpr int NE = rot_max_n(NT);
+  // per position (the indices, then the indices again): dp4a word, scan
+  // addend, and d of the pairs {r, k} and {s, k} after the move (int2)
+  static constexpr int X = 0;
+  static constexpr int psi = X + 8 * NE;
+  static constexpr int R = psi + 8 * NE;
+  // per index: the negated, permuted dp4a word; label (row of P0); start
+  // permutation
+  static constexpr int own = R + 16 * NE;
+  static constexpr int sigma = own + 4 * NE;
+  static constexpr int p0 = sigma + 4 * NE;
+  // pending operands of M's update (two buffers, by the move's parity): rows
+  // by index, columns by label
+  static constexpr int NW = NE + 4;  // ld_m(n) at most
+  static constexpr int vw = p0 + 4 * NE;
+  static constexpr int vwu = vw + 8 * NW;
+  // ring: the pairs whose tabu time ends at iteration i, at i mod its length:
+  // key of the first in the low half, node of the rest in the high half;
+  // nodes: such words moved aside, at the iteration that moved them
+  static constexpr int ring = vwu + 8 * NW;
+  static constexpr int node = ring + 4 * rot_ring(NT);
+  // tenures of the iterations, at (it - 1) mod 64
+  static constexpr int ten = node + 4 * rot_ring(NT);
+  // arg-min candidates of the warps (int2) and, at 32, whether the walk is
+  // over; block sums
+  static constexpr int red = ten + 4 * 64;
+  static constexpr int sum = red + 8 * 34;
+  // what the walk is (RotWalkArgs)
+  static constexpr int args = sum + 8 * 32;
+  static constexpr int bytes = args + kRotArgsBytes;
+};
+
+struct RotLayout {
+  int F, Ft, P, Pt, M, mark, bytes;
+};
+
+// notr: no transposed copies of F and P (kNoTransposed plans)
+__host__ __device__ inline RotLayout rot_layout(int n, int ldF, int ldP, int symF, int symD,
+                                                int notr, int fixed) {
+  RotLayout L;
+  int o = fixed;
+  L.F = o;    o = align16(o + n * ldF);
+  L.Ft = o;   o = (symF || notr) ? o : align16(o + n * ldF);
+  L.P = o;    o = align16(o + n * ldP);
+  L.Pt = o;   o = (symD || notr) ? o : align16(o + n * ldP);
+  L.M = o;    o = align16(o + n * ld_m(n) * 4);
+  // one word more: the thread of k = r reads past the triangle's end at
+  // r = n - 1 (and drops it)
+  L.mark = o; o = align16(o + (n * (n - 1) / 2 + 1) * 4);
+  L.bytes = o;
+  return L;
+}
+
+__host__ __device__ inline int rot_fixed_bytes(int nt) {
+  return nt == 128   ? RotFixed<128>::bytes
+         : nt == 256 ? RotFixed<256>::bytes
+         : nt == 512 ? RotFixed<512>::bytes
+                     : RotFixed<1024>::bytes;
+}
+
+extern __shared__ __align__(16) unsigned char rot_smem[];
+
+template <typename T>
+__device__ __forceinline__ T* rot_at(int off) {
+  return reinterpret_cast<T*>(rot_smem + off);
+}
+
+// Views of the shared memory.
+template <int NT>
+struct RotSmem {
+  using X_ = RotFixed<NT>;
+  RotLayout L;
+  int ft, pt;          // offsets that F^T and P0^T are read from:
+  int fr, fk, pr, pk;  // entry [r][k] at r fr + k fk
+  __device__ __forceinline__ RotSmem(const InstArgs& I, int n, bool notr) {
+    L = rot_layout(n, I.ldF, I.ldP, I.symF, I.symD, notr, X_::bytes);
+    ft = I.symF || notr ? L.F : L.Ft;
+    pt = I.symD || notr ? L.P : L.Pt;
+    // without copies F^T is read from F's columns
+    const bool fc = !I.symF && notr, pc = !I.symD && notr;
+    fr = fc ? 1 : I.ldF;
+    fk = fc ? I.ldF : 1;
+    pr = pc ? 1 : I.ldP;
+    pk = pc ? I.ldP : 1;
+  }
+  __device__ __forceinline__ int8_t* F() const { return rot_at<int8_t>(L.F); }
+  __device__ __forceinline__ int8_t* Ft() const { return rot_at<int8_t>(ft); }
+  __device__ __forceinline__ int8_t* P() const { return rot_at<int8_t>(L.P); }  // P0 = D[p0][p0]
+  __device__ __forceinline__ int8_t* Pt() const { return rot_at<int8_t>(pt); }
+  // M[x][label], halved on symmetric instances
+  __device__ __forceinline__ int32_t* M() const { return rot_at<int32_t>(L.M); }
+  // tabu_until of pair u < v at v (v - 1) / 2 + u
+  __device__ __forceinline__ int32_t* mark() const { return rot_at<int32_t>(L.mark); }
+  __device__ __forceinline__ static int32_t* X() { return rot_at<int32_t>(X_::X); }
+  __device__ __forceinline__ static int32_t* psi() { return rot_at<int32_t>(X_::psi); }
+  __device__ __forceinline__ static int2* R() { return rot_at<int2>(X_::R); }
+  __device__ __forceinline__ static int32_t* own() { return rot_at<int32_t>(X_::own); }
+  __device__ __forceinline__ static int32_t* sigma() { return rot_at<int32_t>(X_::sigma); }
+  __device__ __forceinline__ static int32_t* p0() { return rot_at<int32_t>(X_::p0); }
+  __device__ __forceinline__ static int32_t* vw() { return rot_at<int32_t>(X_::vw); }
+  __device__ __forceinline__ static int32_t* vwu() { return rot_at<int32_t>(X_::vwu); }
+  __device__ __forceinline__ static uint32_t* ring() { return rot_at<uint32_t>(X_::ring); }
+  __device__ __forceinline__ static uint32_t* node() { return rot_at<uint32_t>(X_::node); }
+  __device__ __forceinline__ static int32_t* ten() { return rot_at<int32_t>(X_::ten); }
+  __device__ __forceinline__ static int2* red() { return rot_at<int2>(X_::red); }
+  __device__ __forceinline__ static int64_t* sum() { return rot_at<int64_t>(X_::sum); }
+  __device__ __forceinline__ static RotWalkArgs& args() { return *rot_at<RotWalkArgs>(X_::args); }
+};
+
+// The course of a walk, as the pairs' warps and phase X's follow it.
+struct RotCourse {
+  int cur, best, it, dmoves, iters, cap, ow;
+  int bd, r, s;          // the move
+  bool tabu_phase, stalled;
+
+  __device__ __forceinline__ RotCourse(const RotWalkArgs& w, int warps)
+      : cur((int)w.cost), best(cur), it(0), dmoves(0), iters(w.s.iters),
+        cap(w.s.max_descent >= 0 ? w.s.max_descent : kDescentCap), ow(warps), bd(0), r(0), s(1),
+        tabu_phase(!w.s.descend), stalled(false) {}
+
+  // The arg-min over the warps' candidates, after the barrier that ends a
+  // scan; false when the walk is over.
+  __device__ __forceinline__ bool next(int2* red) {
+    const int lane = threadIdx.x & 31;
+    rot_barrier();
+    const int2 c = lane < ow ? red[lane] : make_int2(INT_MAX, (int)kNoMove);
+    bd = __reduce_min_sync(kFull, c.x);
+    const uint32_t bk = __reduce_min_sync(kFull, c.x == bd ? (uint32_t)c.y : kNoMove);
+    stalled = bk == kNoMove;
+    if (__builtin_expect(!tabu_phase, 0)) {
+      if (stalled || bd >= 0 || dmoves == cap) {
+        // the descent ends; its last arg-min is also that of tabu iteration
+        // 1, where no pair is tabu
+        tabu_phase = true;
+        best = cur;
+      } else {
+        ++dmoves;
+      }
+    }
+    if (tabu_phase) {
+      if (__builtin_expect(it == iters || stalled, 0)) {
+        if (lane == 0) red[32].x = 1;  // for the helpers
+        rot_barrier();
+        return false;
+      }
+      ++it;
+    }
+    r = (int)(bk >> 8);
+    s = (int)(bk & 0xffu);
+    cur += bd;
+    return true;
+  }
+};
+
+// What an instance fixes for a thread.
+struct RotThread {
+  int n, n2, nE;    // indices; blocks of two and their indices (a phantom when n is odd)
+  int J;            // threads per block
+  int role;         // of the thread's warp: 0 holds pairs, 1 phase X, 2 helps with M
+  int m;            // role 0: block of two that the thread holds
+  int pb, pbm;      // role 0: first partner block, as position and mod n2
+  int k;            // role 1: index (past the last: a repeat of n - 1 that stores nothing)
+  bool live;        // role 1: the index is the thread's own
+  int ow;           // warps with role 0
+  int ug, ux, urows;  // roles 1, 2: column group and first row of M, rows at once
+};
+
+template <int NT, int C>
+__device__ __forceinline__ RotThread rot_thread(int n) {
+  RotThread t;
+  const int tid = threadIdx.x;
+  t.n = n;
+  t.n2 = (n + 1) / 2;
+  t.nE = 2 * t.n2;
+  const int J = t.J = rot_chunks(n, NT, C);
+  const int jt = tid / t.n2;
+  t.m = tid - jt * t.n2;
+  const int j = jt < J ? jt : 0;  // threads past the last repeat the first chunk's pairs
+  t.pb = t.m + 1 + j * C;
+  t.pbm = t.pb < t.n2 ? t.pb : t.pb - t.n2;
+  t.ow = (J * t.n2 + 31) / 32;
+  const int k = tid - rot_owners(NT);
+  t.live = k >= 0 && k < n;
+  t.k = k < n ? k : n - 1;
+  t.role = tid < 32 * t.ow ? 0 : k >= 0 && k < (n + 31) / 32 * 32 ? 1 : 2;
+  const int gpr = ld_m(n) / 4, f = tid - 32 * t.ow;
+  t.ug = f % gpr;
+  t.ux = f / gpr;
+  t.urows = (NT - 32 * t.ow) / gpr;
+  return t;
+}
+
+// Shared-memory loads and stores by 32-bit address.
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ int lds32(uint32_t at) {
+  int v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+__device__ __forceinline__ int lds8(uint32_t at) {
+  int v;
+  asm volatile("ld.shared.s8 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+__device__ __forceinline__ int4 lds128(uint32_t at) {
+  int4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(at)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts32(uint32_t at, int v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t at, int x, int y) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t at, int4 v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v.x), "r"(v.y),
+               "r"(v.z), "r"(v.w)
+               : "memory");
+}
+
+__device__ __forceinline__ uint32_t pack4(int b0, int b1, int b2, int b3) {
+  return __byte_perm(__byte_perm((uint32_t)b0, (uint32_t)b1, 0x0040u),
+                     __byte_perm((uint32_t)b2, (uint32_t)b3, 0x0040u), 0x5410u);
+}
+
+// M at the start of a walk, from F and P0: one dot product per entry over
+// rows, a second over columns when F or D is asymmetric.  A warp takes four
+// rows of F at once (each 16-byte chunk of a row of P0 serves four dot
+// products), its lanes the columns.  Symmetric instances keep half of M.
+template <int NT>
+__device__ __forceinline__ void rot_compute_m(const RotSmem<NT>& S, int n, int ldF, int ldP, bool sym,
+                                              bool notr) {
+  using C = Chunk<int8_t>;
+  const int nc = (n + 15) / 16, ldm = ld_m(n);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int x0 = 4 * warp; x0 < n; x0 += NT / 8) {
+    const int xm = n - 1;
+    const int x1 = min(x0 + 1, xm), x2 = min(x0 + 2, xm), x3 = min(x0 + 3, xm);
+    for (int k = lane; k < n; k += 32) {
+      int a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+      auto rows = [&](const int8_t* F, const int8_t* P) {
+        const int4* q = reinterpret_cast<const int4*>(P + k * ldP);
+        const int4* f0 = reinterpret_cast<const int4*>(F + x0 * ldF);
+        const int4* f1 = reinterpret_cast<const int4*>(F + x1 * ldF);
+        const int4* f2 = reinterpret_cast<const int4*>(F + x2 * ldF);
+        const int4* f3 = reinterpret_cast<const int4*>(F + x3 * ldF);
+#pragma unroll 1
+        for (int c = 0; c < nc; ++c) {
+          const int4 v = q[c];
+          a0 = C::dot(f0[c], v, a0);
+          a1 = C::dot(f1[c], v, a1);
+          a2 = C::dot(f2[c], v, a2);
+          a3 = C::dot(f3[c], v, a3);
+        }
+      };
+      rows(S.F(), S.P());
+      if (!sym && !notr) rows(S.Ft(), S.Pt());
+      if (!sym && notr) {
+        // columns x0..x0+3 of F (x0 a multiple of 4) and column k of P0
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) {
+          const char4 f = *reinterpret_cast<const char4*>(S.F() + j * ldF + x0);
+          const int p = S.P()[j * ldP + k];
+          a0 += f.x * p;
+          a1 += f.y * p;
+          a2 += f.z * p;
+          a3 += f.w * p;
+        }
+      }
+      S.M()[x0 * ldm + k] = a0;
+      if (x0 + 1 < n) S.M()[x1 * ldm + k] = a1;
+      if (x0 + 2 < n) S.M()[x2 * ldm + k] = a2;
+      if (x0 + 3 < n) S.M()[x3 * ldm + k] = a3;
+    }
+  }
+}
+
+// The marks, after the pairs' warps have taken the table from their place;
+// by the other warps.
+template <int NT>
+__device__ __forceinline__ void rot_clear_marks(int32_t* mark, int n, int ow) {
+  rot_barrier();
+  for (int x = (int)threadIdx.x - 32 * ow; x < n * (n - 1) / 2; x += NT - 32 * ow) mark[x] = 0;
+}
+
+// Tenure of iteration it (from 1).
+struct RotTenure {
+  int tmin, tmax, period;
+  __device__ __forceinline__ RotTenure(const SearchArgs& a, int n)
+      : tmin(a.tmin), tmax(a.tmax), period(a.period) {
+    if (a.tenure_per_n) {
+      tmin = max(1, a.tmin * n / 100);
+      tmax = max(tmin, (a.tmax * n + 99) / 100);
+      period = a.period * n / 100;
+    }
+  }
+  __device__ __forceinline__ int of(uint64_t seed, uint32_t wid, int it) const {
+    const uint32_t i = (uint32_t)(it - 1);
+    const uint32_t x = walk_draw(seed, wid, 1u, period > 0 ? i / (uint32_t)period : i);
+    return tmin + (int)below(x, (uint32_t)(tmax - tmin + 1));
+  }
+};
+
+// M[x][.] after a move, for the rows x = slot mod Q: one dp4a per entry with
+// the pending words, a group of 4 columns of every urows-th such row per
+// thread, 4 rows in flight.
+template <int Q>
+__device__ __forceinline__ void rot_update_m(const RotThread& T, uint32_t aM, uint32_t aVw,
+                                             uint32_t aVwu, int n, int ldm, int slot) {
+  if (T.ux >= T.urows) return;
+  const int4 w = lds128(aVwu + 16 * T.ug);
+  const int step = Q * T.urows;
+  auto upd = [&](int u, int4 v) {
+    v.x = __dp4a(u, w.x, v.x);
+    v.y = __dp4a(u, w.y, v.y);
+    v.z = __dp4a(u, w.z, v.z);
+    v.w = __dp4a(u, w.w, v.w);
+    return v;
+  };
+  uint32_t am = aM + 16 * T.ug + 4 * ldm * (slot + Q * T.ux);
+  uint32_t av = aVw + 4 * (slot + Q * T.ux);
+  const uint32_t sm = 4 * ldm * step, sv = 4 * step;
+#pragma unroll 1
+  for (int x = slot + Q * T.ux; x < n; x += 4 * step) {
+    // rows past the last repeat the first: the same entry, loaded before it
+    // is stored, takes the same value again
+    const uint32_t m1 = x + step < n ? sm : 0, m2 = x + 2 * step < n ? 2 * sm : 0;
+    const uint32_t m3 = x + 3 * step < n ? 3 * sm : 0;
+    const uint32_t v1 = x + step < n ? sv : 0, v2 = x + 2 * step < n ? 2 * sv : 0;
+    const uint32_t v3 = x + 3 * step < n ? 3 * sv : 0;
+    const int4 a0 = lds128(am), a1 = lds128(am + m1), a2 = lds128(am + m2), a3 = lds128(am + m3);
+    const int b0 = lds32(av), b1 = lds32(av + v1), b2 = lds32(av + v2), b3 = lds32(av + v3);
+    sts128(am, upd(b0, a0));
+    sts128(am + m1, upd(b1, a1));
+    sts128(am + m2, upd(b2, a2));
+    sts128(am + m3, upd(b3, a3));
+    am += 4 * sm;
+    av += 4 * sv;
+  }
+}
+
+// d[q] less `big`, q the same in every lane: a branch tree.
+template <int LO, int HI, int NS>
+__device__ __forceinline__ void clear_tabu(int (&d)[NS], int q, int big) {
+  if constexpr (HI - LO > 3) {
+    constexpr int MID = (LO + HI) / 2;
+    if (q < MID) clear_tabu<LO, MID>(d, q, big);
+    else clear_tabu<MID, HI>(d, q, big);
+  } else {
+#pragma unroll
+    for (int i = LO; i < HI; ++i) d[i] -= q == i ? big : 0;
+  }
+}
+
+// The warps that hold pairs: the table, its update after each move, and the
+// scan for the next iteration.
+template <int NT, int C>
+__device__ __forceinline__ void rot_owner() {
+  using S = RotSmem<NT>;
+  const RotWalkArgs& W = S::args();
+  const InstArgs& I = W.I;
+  const int aspiration = W.s.aspiration;
+  const RotThread T = rot_thread<NT, C>(I.n);
+  const int n = T.n, n2 = T.n2, nE = T.nE, m = T.m;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int v0 = 2 * m, v1 = v0 + 1;
+  const bool half = v1 >= n;  // the block's second index is the phantom of an odd n
+  constexpr bool RANK = rot_rank(NT);
+  constexpr int SB = rot_key_bits(NT);
+  constexpr uint32_t MUL = 1u << SB;
+  constexpr int BIG = 1 << (31 - SB);  // on top of a tabu pair's d
+  constexpr int NS = 4 * C + 1;        // slots; the last holds the pair inside the block
+
+  // the table, from where rot_start left it
+  int32_t* const mark = S(I, n, W.notr != 0).mark();
+  int d[NS];
+  auto d_init = [&](int u, int v) -> int {
+    const int hi = max(u, v);
+    return hi < n ? mark[hi * (hi - 1) / 2 + min(u, v)] : 0;
+  };
+#pragma unroll
+  for (int i = 0; i < C; ++i) {
+    const int b = T.pb + i < n2 ? T.pb + i : T.pb + i - n2;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) d[4 * i + q] = d_init(v0 + (q >> 1), 2 * b + (q & 1));
+  }
+  d[4 * C] = d_init(v0, v1);
+  rot_barrier();  // the others now clear the marks
+
+  const int2* const X = reinterpret_cast<const int2*>(S::X());
+  const int2* const psi = reinterpret_cast<const int2*>(S::psi());
+  const int2* const own = reinterpret_cast<const int2*>(S::own());
+  const int4* const R = reinterpret_cast<const int4*>(S::R());
+
+  // Scan of the table: the warp's candidate into red.  A tabu pair aspires
+  // when its delta is below `lim` (at most 0).
+  auto scan = [&](int lim) {
+    int m0 = INT_MAX, m1 = INT_MAX;
+    uint32_t t0 = 0xffffffffu, t1 = 0xffffffffu;
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+      const int2 y = psi[T.pb + i];
+      const uint32_t y0 = (uint32_t)y.x + (RANK ? 2 * i + 1 : 0);
+      const uint32_t y1 = (uint32_t)y.y + (RANK ? 2 * i + 2 : 0);
+      const uint32_t e00 = (uint32_t)d[4 * i] * MUL + y0;
+      const uint32_t e01 = (uint32_t)d[4 * i + 1] * MUL + y1;
+      const uint32_t e10 = (uint32_t)d[4 * i + 2] * MUL + y0;
+      const uint32_t e11 = (uint32_t)d[4 * i + 3] * MUL + y1;
+      m0 = min(m0, min((int)e00, (int)e01));
+      m1 = min(m1, min((int)e10, (int)e11));
+      t0 = min(t0, min(e00, e01));
+      t1 = min(t1, min(e10, e11));
+    }
+    const int2 o = psi[m];
+    {
+      const uint32_t e = (uint32_t)d[4 * C] * MUL + (uint32_t)o.y;
+      m0 = min(m0, (int)e);
+      t0 = min(t0, e);
+    }
+    // delta 2^S + index of each row's best, by the own index's psi: q is
+    // 2^30 less g[v]
+    const uint32_t q0 = (uint32_t)o.x - (RANK ? 32 : v0) + 0x80000000u;
+    const uint32_t q1 = (uint32_t)o.y - (RANK ? 32 : v1) + 0x80000000u;
+    const int ls = (int)((uint32_t)max(lim, -(INT_MAX >> SB)) * MUL);
+    int c0 = m0 < 0 ? (int)((uint32_t)m0 + q0) : INT_MAX;
+    int c1 = m1 < 0 ? (int)((uint32_t)m1 + q1) : INT_MAX;
+    const int x0 = (int)(t0 + q0 + 0x80000000u), x1 = (int)(t1 + q1 + 0x80000000u);
+    if ((int)t0 >= 0 && x0 < ls) c0 = min(c0, x0);
+    if ((int)t1 >= 0 && x1 < ls) c1 = min(c1, x1);
+    if (half) c1 = INT_MAX;  // the phantom's row
+    // the lower pair of the two rows
+    const int d0 = c0 >> SB, d1 = c1 >> SB;
+    int u0 = c0 & (int)(MUL - 1), u1 = c1 & (int)(MUL - 1);
+    if (RANK) {
+      u0 = (u0 & 31) + 2 * T.pb - 1;
+      u0 = u0 >= nE ? u0 - nE : u0;
+      u0 = (c0 & 31) == 0 ? v1 : u0;
+      u1 = (u1 & 31) + 2 * T.pb - 1;
+      u1 = u1 >= nE ? u1 - nE : u1;
+    }
+    const uint32_t k0 = (uint32_t)(min(u0, v0) << 8 | max(u0, v0));
+    const uint32_t k1 = (uint32_t)(min(u1, v1) << 8 | max(u1, v1));
+    const bool second = d1 < d0 || (d1 == d0 && k1 < k0);
+    const int dd = second ? d1 : d0;
+    const uint32_t kk = second ? k1 : k0;
+    const int wd = __reduce_min_sync(kFull, dd);
+    const uint32_t wk = __reduce_min_sync(kFull, dd == wd ? kk : kNoMove);
+    const bool none = wd == INT_MAX >> SB;
+    if (lane == 0) S::red()[warp] = make_int2(none ? INT_MAX : wd, (int)(none ? kNoMove : wk));
+  };
+
+  scan(INT_MIN);
+
+  RotCourse c(W, T.ow);
+  while (c.next(S::red())) {
+    const int r = c.r, s = c.s, it = c.it;
+    c.best = c.tabu_phase ? min(c.best, c.cur) : c.cur;
+    const int lim = aspiration ? c.best - c.cur : INT_MIN;
+    // pairs whose tabu time ends with the next iteration (in the shadow of
+    // phase X)
+    uint32_t w = S::ring()[(it + 1) & (rot_ring(NT) - 1)];
+    while (__builtin_expect(w != 0xffffffffu, 1)) {
+      const int u = (int)(w >> 8 & 0xffu), v = (int)(w & 0xffu);
+      const int bu = u >> 1, bv = v >> 1;
+      const bool own_u = m == bu;
+      int kx = (own_u ? bv : bu) - T.pbm;  // slot group of the other one
+      kx = kx < 0 ? kx + n2 : kx;
+      int q = 4 * kx + (own_u ? 2 * (u & 1) + (v & 1) : 2 * (v & 1) + (u & 1));
+      q = bu == bv ? 4 * C : q;
+      // (applied again since: its end is another)
+      const bool ends = mark[v * (v - 1) / 2 + u] == it + 1;
+      const bool hold = ends && (own_u || m == bv) && (kx < C || bu == bv);
+      for (unsigned b = __ballot_sync(kFull, hold); b; b &= b - 1) {
+        const int src = __ffs(b) - 1;
+        clear_tabu<0, NS>(d, __shfl_sync(kFull, q, src), lane == src ? BIG : 0);
+      }
+      w = w >> 16 == 0xffffu ? 0xffffffffu : S::node()[w >> 16];
+    }
+    const int br = r >> 1, bs = s >> 1;
+    int kr = br - T.pbm, ks = bs - T.pbm;  // slot groups of r and s as partners, if below C
+    kr = kr < 0 ? kr + n2 : kr;
+    ks = ks < 0 ? ks + n2 : ks;
+    const bool row0 = v0 == r || v0 == s, row1 = v1 == r || v1 == s;
+    rot_barrier();
+
+    // the new table
+    const int2 A = own[m];
+    const int4 Rm = R[m];  // the pairs (v0, r), (v0, s), (v1, r), (v1, s)
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+      const int2 x = X[T.pb + i];
+      d[4 * i] = __dp4a(A.x, x.x, d[4 * i]);
+      d[4 * i + 1] = __dp4a(A.x, x.y, d[4 * i + 1]);
+      d[4 * i + 2] = __dp4a(A.y, x.x, d[4 * i + 2]);
+      d[4 * i + 3] = __dp4a(A.y, x.y, d[4 * i + 3]);
+    }
+    d[4 * C] = __dp4a(A.x, X[m].y, d[4 * C]);
+    // partners r and s
+    auto partner = [&](int kk, bool odd, int w0, int w1) {
+      if (odd) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          d[4 * i + 1] = kk == i ? w0 : d[4 * i + 1];
+          d[4 * i + 3] = kk == i ? w1 : d[4 * i + 3];
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          d[4 * i] = kk == i ? w0 : d[4 * i];
+          d[4 * i + 2] = kk == i ? w1 : d[4 * i + 2];
+        }
+      }
+    };
+    partner(kr, r & 1, Rm.x, Rm.z);
+    partner(ks, s & 1, Rm.y, Rm.w);
+    // the rows of r and s
+    if (row0 || row1) {
+      const int* const x0 = reinterpret_cast<const int*>(R) + (v0 == r ? 0 : 1);
+      const int* const x1 = reinterpret_cast<const int*>(R) + (v1 == r ? 0 : 1);
+      if (row0) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          d[4 * i] = x0[4 * (T.pb + i)];
+          d[4 * i + 1] = x0[4 * (T.pb + i) + 2];
+        }
+        d[4 * C] = x0[4 * m + 2];
+      }
+      if (row1) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          d[4 * i + 2] = x1[4 * (T.pb + i)];
+          d[4 * i + 3] = x1[4 * (T.pb + i) + 2];
+        }
+        d[4 * C] = x1[4 * m];
+      }
+    }
+    scan(lim);
+  }
+}
+
+// The phase X warps: one thread per index k computes what move (r, s) changes
+// (see phase_m_prep for the algebra), and keeps the labels, the pending words,
+// the tabu times and the walk's results.
+//
+// M's rows are brought up to date in turn, those with x mod Q = t mod Q after
+// move t, by the last Q moves at once: byte (pair) t mod Q of the pending
+// words belongs to move t.  A row's word is cleared when the row is done, so
+// its entries' correction is one dp4a whatever the row's place in the turn.
+template <int NT, int C, bool SYM>
+__device__ __forceinline__ void rot_phase_x() {
+  constexpr int Q = SYM ? 4 : 2;
+  constexpr int SB = rot_key_bits(NT);
+  constexpr int BIG = 1 << (31 - SB);
+  using X_ = RotFixed<NT>;
+  const RotWalkArgs& W = RotSmem<NT>::args();
+  const InstArgs& I = W.I;
+  const RotThread T = rot_thread<NT, C>(I.n);
+  const RotSmem<NT> S(I, T.n, W.notr != 0);
+  const int n = T.n, ldF = I.ldF, ldP = I.ldP, ldm = ld_m(n), nE = T.nE;
+  const int g0 = I.g0, g2 = 2 * g0;
+  const uint32_t wid = W.wid;
+  const uint64_t seed = W.s.seed;
+  int32_t* const fq = W.s.freq ? W.s.freq + (size_t)W.row * W.s.p_stride * W.s.p_stride : nullptr;
+  const int k = T.k;
+  const int lane = threadIdx.x & 31;
+  const bool live = T.live, first = k < 32;  // first: the first warp, that keeps the tabu times
+  // addresses
+  const uint32_t base = smem_addr(rot_smem);
+  const uint32_t aF = base + S.L.F, aP = base + S.L.P, aM = base + S.L.M;
+  const uint32_t aFt = base + S.ft, aPt = base + S.pt, aMark = base + S.L.mark;
+  const uint32_t aVw = base + X_::vw, aVwu = base + X_::vwu, aSig = base + X_::sigma;
+  const uint32_t aX = base + X_::X, aPsi = base + X_::psi, aOwn = base + X_::own;
+  const uint32_t aR = base + X_::R, aTen = base + X_::ten;
+  const uint32_t oMk = aM + 4 * ldm * k;
+  const int ktri = k * (k - 1) / 2;
+  int uk = k, wk = 0, best_uk = k, best_iter = 0, mv = 0;
+  const int Fkk = S.F()[k * ldF + k];
+  int Qkk = S.P()[k * ldP + k];
+  int gk = (S.M()[k * ldm + k] << (SYM ? 1 : 0)) - g0;
+  const RotTenure tenure(W.s, n);
+  const uint64_t h0 = 14695981039346656037ull;
+  uint64_t h = h0, dh = h0;
+  rot_clear_marks<NT>(S.mark(), n, T.ow);
+  RotCourse course(W, T.ow);
+  bool was_tabu = course.tabu_phase;
+
+  while (course.next(S.red())) {
+    const int r = course.r, s = course.s, it = course.it;
+    const bool tabu_phase = course.tabu_phase;
+    const uint32_t oFr = aF + r * ldF, oFs = aF + s * ldF;
+    const uint32_t oMr = aM + 4 * r * ldm, oMs = aM + 4 * s * ldm;
+    const int ur = lds32(aSig + 4 * r), us = lds32(aSig + 4 * s);
+    // the moves that the rows r, s and k of M do not hold yet
+    const int rd = (mv & 1) * 4 * ldm, wt = 4 * ldm - rd;  // this move's buffers
+    const int done = (mv - 1) & (Q - 1);                   // rows finished after the last move
+    int wr = lds32(aVw + rd + 4 * r), ws = lds32(aVw + rd + 4 * s);
+    wr = (r & (Q - 1)) == done ? 0 : wr;
+    ws = (s & (Q - 1)) == done ? 0 : ws;
+    const int fRR = lds8(oFr + r), fRS = lds8(oFr + s), fSS = lds8(oFs + s);
+    const int fSR = SYM ? fRS : lds8(oFs + r);
+    const int Frk = lds8(oFr + k), Fsk = lds8(oFs + k);
+    const int Fkr = SYM ? Frk : lds8(aFt + r * S.fr + k * S.fk);
+    const int Fks = SYM ? Fsk : lds8(aFt + s * S.fr + k * S.fk);
+    // ends of the tabu times of the pairs {r, k} and {s, k}
+    const int rtri = r * (r - 1) / 2, stri = s * (s - 1) / 2;
+    const int end_r = lds32(aMark + 4 * (k < r ? rtri + k : ktri + r));
+    const int end_s = lds32(aMark + 4 * (k < s ? stri + k : ktri + s));
+    const int ten = lds32(aTen + 4 * ((it - 1) & 63));
+    const uint32_t u4 = 4 * (uint32_t)uk;
+    const int wuk = lds32(aVwu + rd + u4);
+    int Ar = lds32(oMr + u4), As = lds32(oMs + u4);
+    const uint32_t oQr = aP + ur * ldP, oQs = aP + us * ldP;
+    const int wur = lds32(aVwu + rd + 4 * ur), wus = lds32(aVwu + rd + 4 * us);
+    const int qRR = lds8(oQr + ur), qRS = lds8(oQr + us), qSS = lds8(oQs + us);
+    const int qSR = SYM ? qRS : lds8(oQs + ur);
+    const int Qrk = lds8(oQr + uk), Qsk = lds8(oQs + uk);
+    const int Qkr = SYM ? Qrk : lds8(aPt + ur * S.pr + uk * S.pk);
+    const int Qks = SYM ? Qsk : lds8(aPt + us * S.pr + uk * S.pk);
+    int Bs = lds32(oMk + 4 * us), Br = lds32(oMk + 4 * ur);
+    int mrs = lds32(oMr + 4 * us), msr = lds32(oMs + 4 * ur);
+    // the byte (pair) of the pending words that this move takes
+    const int slot = mv & (Q - 1);
+    const uint32_t sel = SYM ? (0x3210u & ~(0xfu << (4 * slot))) | 4u << (4 * slot)
+                             : slot ? 0x5410u : 0x3254u;
+    const int wkj = (k & (Q - 1)) == done ? 0 : wk;
+    Ar = __dp4a(wr, wuk, Ar);
+    As = __dp4a(ws, wuk, As);
+    Bs = __dp4a(wkj, wus, Bs);
+    Br = __dp4a(wkj, wur, Br);
+    mrs = __dp4a(wr, wus, mrs);
+    msr = __dp4a(ws, wur, msr);
+    const int av = Frk - Fsk, b = Qrk - Qsk;
+    const int c = Fkr - Fks, e = Qkr - Qks;
+    uint32_t own, word;
+    int gr, gs, gn, Rr, Rs;
+    if (SYM) {
+      gr = 2 * (mrs - (fRR - fRS) * (qRS - qSS)) - g0;
+      gs = 2 * (msr - (fRS - fSS) * (qRR - qRS)) - g0;
+      own = __byte_perm((uint32_t)-av, (uint32_t)-b, 0x4400u);
+      word = __byte_perm((uint32_t)b, (uint32_t)av, 0x4400u);
+      gn = gk - 2 * av * b;
+      Rr = 2 * (Ar + Bs + (qSS - qRS) * av - (fRR - fRS) * b) - g2 +
+           (fRR + Fkk - 2 * Frk) * (qSS + Qkk - 2 * Qsk);
+      Rs = 2 * (As + Br + (qRS - qRR) * av - (fRS - fSS) * b) - g2 +
+           (fSS + Fkk - 2 * Fsk) * (qRR + Qkk - 2 * Qrk);
+    } else {
+      gr = mrs - (fRR - fRS) * (qSR - qSS) - (fRR - fSR) * (qRS - qSS) - g0;
+      gs = msr - (fSR - fSS) * (qRR - qRS) - (fRS - fSS) * (qRR - qSR) - g0;
+      own = pack4(-av, -c, -b, -e);
+      word = pack4(b, e, av, c);
+      gn = gk - av * b - c * e;
+      Rr = Ar + Bs - g2 + (fRR - Frk - Fkr + Fkk) * (qSS - Qsk - Qks + Qkk) - (fRR - fRS) * e -
+           (fRR - fSR) * b + (qSS - qSR) * c + (qSS - qRS) * av;
+      Rs = As + Br - g2 + (fSS - Fsk - Fks + Fkk) * (qRR - Qrk - Qkr + Qkk) - (fSR - fSS) * e -
+           (fRS - fSS) * b + (qRS - qRR) * c + (qSR - qRR) * av;
+    }
+    Rr += end_r > it + 1 ? BIG : 0;
+    Rs += end_s > it + 1 ? BIG : 0;
+    // M's operands of this move: bytes (-a, -c) by index, (b, e) by label
+    // (symmetric: -a and b)
+    wk = (int)__byte_perm((uint32_t)wkj, own, sel);
+    const int wun = (int)__byte_perm((uint32_t)wuk, word, sel);
+    const bool isr = k == r, iss = k == s;
+    // the pair (r, s) itself only changes sign, and turns tabu
+    const int drs = gr + gs - course.bd + (tabu_phase && ten > 1 ? BIG : 0);
+    gn = isr ? gr : iss ? gs : gn;
+    Rr = isr || iss ? drs : Rr;
+    Rs = isr || iss ? drs : Rs;
+    gk = gn;
+    if (live) {
+      const int psi = (int)(0u - ((uint32_t)gn << SB) - (1u << 30)) + (rot_rank(NT) ? 32 : k);
+      sts32(aX + 4 * k, (int)word);
+      sts32(aX + 4 * nE + 4 * k, (int)word);
+      sts32(aPsi + 4 * k, psi);
+      sts32(aPsi + 4 * nE + 4 * k, rot_rank(NT) ? psi - 32 : psi);
+      sts32(aOwn + 4 * k, (int)own);
+      sts64(aR + 8 * k, Rr, Rs);
+      sts64(aR + 8 * nE + 8 * k, Rr, Rs);
+      sts32(aVw + wt + 4 * k, wk);
+      sts32(aVwu + wt + u4, wun);
+    }
+    rot_barrier();
+    // while the other warps bring the table up to date: M, the labels, the
+    // best solution, the tabu times and the hash
+    rot_update_m<Q>(T, aM, aVw + wt, aVwu + wt, n, ldm, slot);
+    ++mv;
+    uk = isr ? us : iss ? ur : uk;
+    Qkk = isr ? qSS : iss ? qRR : Qkk;
+    if (live && (isr || iss)) sts32(aSig + 4 * k, uk);
+    const bool better = !tabu_phase || course.cur < course.best;
+    best_uk = better ? uk : best_uk;
+    course.best = better ? course.cur : course.best;
+    best_iter = better ? it : best_iter;  // 0 in the descent
+    if (first) {
+      if (tabu_phase && !was_tabu) {  // this was the first tabu move
+        was_tabu = true;
+        dh = h;
+        h = h0;
+      }
+      h = fnv_step(h, r, s);
+      if (tabu_phase) {
+        if ((it & 31) == 0)  // the tenures of iterations it + 33 .. it + 64
+          S.ten()[(it + 32 + lane) & 63] = tenure.of(seed, wid, it + 33 + lane);
+        if (k == 0) {
+          const int end = it + ten;
+          // the ring word of the iteration just served is free again
+          S.ring()[(it + 1) & (rot_ring(NT) - 1)] = 0xffffffffu;
+          S.mark()[stri + r] = end;
+          if (end > it + 1 && end <= course.iters) {
+            uint32_t* const at = S.ring() + (end & (rot_ring(NT) - 1));
+            const uint32_t old = *at, key = (uint32_t)(r << 8 | s);
+            const uint32_t nd = (uint32_t)it & (rot_ring(NT) - 1);
+            // (there already when the pair, applied while tabu, ends when it
+            // once did: the owners would clear its bit twice)
+            bool there = false;
+            for (uint32_t w = old; w != 0xffffffffu;
+                 w = w >> 16 == 0xffffu ? 0xffffffffu : S.node()[w >> 16])
+              there |= (w & 0xffffu) == key;
+            if (!there) {
+              if (old != 0xffffffffu) S.node()[nd] = old;
+              *at = key | (old != 0xffffffffu ? nd : 0xffffu) << 16;
+            }
+          }
+          if (fq) atomicAdd(fq + s * W.s.p_stride + r, 1);
+        }
+      }
+    }
+  }
+
+  // ---- outputs
+  const SearchArgs& a = W.s;
+  const int row = W.row;
+  if (a.best_p && live) a.best_p[(size_t)row * a.p_stride + k] = S.p0()[best_uk];
+  if (live && k == 0) {
+    if (!was_tabu) {
+      dh = h;
+      h = h0;
+    }
+    a.best_cost[row] = (int64_t)course.best;
+    if (a.final_cost) a.final_cost[row] = (int64_t)course.cur;
+    if (a.best_iter) a.best_iter[row] = best_iter;
+    if (a.iters_done) a.iters_done[row] = course.it;
+    if (a.status) a.status[row] = course.stalled && course.it < course.iters ? 1 : 0;
+    if (a.descent_moves) a.descent_moves[row] = course.dmoves;
+    if (a.hash) a.hash[row] = h;
+    if (a.descent_hash) a.descent_hash[row] = dh;
+  }
+}
+
+// The other warps: M's update, until the flag beside the candidates is set.
+template <int NT, int C, int Q>
+__device__ __forceinline__ void rot_helper() {
+  using X_ = RotFixed<NT>;
+  const RotWalkArgs& W = RotSmem<NT>::args();
+  const RotThread T = rot_thread<NT, C>(W.I.n);
+  const RotSmem<NT> S(W.I, T.n, W.notr != 0);
+  const int n = T.n, ldm = ld_m(n);
+  const uint32_t base = smem_addr(rot_smem);
+  rot_clear_marks<NT>(S.mark(), n, T.ow);
+  for (int mv = 0;; ++mv) {
+    rot_barrier();
+    rot_barrier();
+    if (lds32(base + X_::red + 8 * 32)) break;
+    const uint32_t wt = mv & 1 ? 0 : 4 * ldm;
+    rot_update_m<Q>(T, base + S.L.M, base + X_::vw + wt, base + X_::vwu + wt, n, ldm,
+                    mv & (Q - 1));
+  }
+}
+
+// The start of a walk: permutation, P0, M, the scan addends and the cost.
+// Starts and ends with every thread of the CTA together.
+template <int NT>
+__device__ __forceinline__ void rot_start() {
+  RotWalkArgs& W = RotSmem<NT>::args();
+  const InstArgs& I = W.I;
+  const SearchArgs& a = W.s;
+  const bool notr = W.notr != 0;
+  const int32_t* const start = W.start;
+  const uint32_t wid = W.wid;
+  const int n = I.n, ldF = I.ldF, ldP = I.ldP, tid = threadIdx.x;
+  const RotSmem<NT> S(I, n, notr);
+  const int lane = tid & 31, warp = tid >> 5;
+  const bool sym = I.symF && I.symD;
+  const int ldm = ld_m(n), nE = (n + 1) / 2 * 2, g0 = I.g0;
+  const int hsh = sym ? 1 : 0;  // M is stored halved
+  constexpr int SB = rot_key_bits(NT);
+
+  // ---- start permutation: given, or Fisher-Yates on stream 0 (the draws by
+  // all threads, the exchanges by one)
+  if (start) {
+    for (int x = tid; x < n; x += NT) S.p0()[x] = start[x];
+  } else {
+    for (int i = tid; i < n; i += NT) {
+      S.p0()[i] = i;
+      if (i >= 1) S.vw()[i] = (int)below(walk_draw(a.seed, wid, 0u, (uint32_t)(n - 1 - i)),
+                                         (uint32_t)(i + 1));
+    }
+    __syncthreads();
+    if (tid == 0)
+      for (int i = n - 1; i >= 1; --i) {
+        const int j = S.vw()[i];
+        const int32_t t = S.p0()[i];
+        S.p0()[i] = S.p0()[j];
+        S.p0()[j] = t;
+      }
+  }
+  __syncthreads();
+
+  // ---- P0 = D[p0][p0] gathered from global memory, and the walk's state
+  {
+    const int8_t* Dg = static_cast<const int8_t*>(I.D);
+    const bool tr = !I.symD && !notr;
+    int8_t* Pt = S.Pt();
+    for (int i = warp; i < n; i += NT / 32) {
+      const int8_t* Di = Dg + (size_t)S.p0()[i] * n;
+      for (int j = lane; j < n; j += 32) {
+        const int8_t v = Di[S.p0()[j]];
+        S.P()[i * ldP + j] = v;
+        if (tr) Pt[j * ldP + i] = v;
+      }
+    }
+    for (int x = tid; x < n; x += NT) S.sigma()[x] = x;
+    // phantom indices: never candidates, never updated
+    for (int x = n + tid; x < nE; x += NT) {
+      S.X()[x] = S.X()[x + nE] = 0;
+      S.psi()[x] = S.psi()[x + nE] = INT_MAX - 64;
+      S.R()[x] = S.R()[x + nE] = make_int2(0, 0);
+      S.own()[x] = 0;
+    }
+    // no pending moves; M's padding columns take updates from these words only
+    for (int x = tid; x < 2 * ldm; x += NT) S.vw()[x] = S.vwu()[x] = 0;
+    for (int x = tid; x < rot_ring(NT); x += NT) S.ring()[x] = 0xffffffffu;
+    if (a.iters > 0) {
+      const RotTenure tenure(a, n);
+      for (int x = tid; x < 64; x += NT) S.ten()[x] = tenure.of(a.seed, wid, x + 1);
+    }
+    if (tid == 0) S.red()[32] = make_int2(0, 0);
+  }
+  __syncthreads();
+  rot_compute_m<NT>(S, n, ldF, ldP, sym, notr);
+  __syncthreads();
+
+  // ---- the pairs' table, in the marks' place: d = M[u][v] + M[v][u] + the
+  // 2x2 term of Eq. 2
+  {
+    const int8_t* F = S.F();
+    const int8_t* P = S.P();
+    const int32_t* M = S.M();
+    for (int v = 1 + warp; v < n; v += NT / 32) {
+      const int fv = F[v * ldF + v], pv = P[v * ldP + v];
+      for (int u = lane; u < v; u += 32) {
+        const int f = fv + F[u * ldF + u] - F[u * ldF + v] - F[v * ldF + u];
+        const int p = pv + P[u * ldP + u] - P[u * ldP + v] - P[v * ldP + u];
+        S.mark()[v * (v - 1) / 2 + u] =
+            ((M[u * ldm + v] + M[v * ldm + u]) << hsh) + f * p - 2 * g0;
+      }
+    }
+  }
+
+  // ---- scan addends of every index; the walk's cost (Eq. 1): M's diagonal
+  // sums to twice the cost
+  int64_t c0 = 0;
+  for (int x = tid; x < n; x += NT) {
+    const int mxx = S.M()[x * ldm + x];
+    c0 += mxx;
+    const uint32_t psi = 0u - ((uint32_t)((mxx << hsh) - g0) << SB) - (1u << 30);
+    S.psi()[x] = (int)(psi + (rot_rank(NT) ? 32 : x));
+    S.psi()[x + nE] = (int)(psi + (rot_rank(NT) ? 0 : x));
+  }
+  c0 = block_sum<NT>(c0, S.sum());
+  if (tid == 0) W.cost = sym ? c0 : c0 >> 1;
+  if (a.freq) {
+    int32_t* fq = a.freq + (size_t)W.row * a.p_stride * a.p_stride;
+    for (int c = tid; c < a.p_stride * a.p_stride; c += NT) fq[c] = 0;
+  }
+  __syncthreads();
+}
+
+// One whole walk of the instance in shared memory (see RotWalkArgs).  Starts
+// and ends with every thread of the CTA together.
+template <int NT, int C>
+__device__ __forceinline__ void rot_walk() {
+  rot_start<NT>();
+  const RotWalkArgs& W = RotSmem<NT>::args();
+  const int role = rot_thread<NT, C>(W.I.n).role;
+  const bool sym = W.I.symF && W.I.symD;
+  if (role == 0) rot_owner<NT, C>();
+  else if (role == 1 && sym) rot_phase_x<NT, C, true>();
+  else if (role == 1) rot_phase_x<NT, C, false>();
+  else if (sym) rot_helper<NT, C, 4>();
+  else rot_helper<NT, C, 2>();
+  __syncthreads();
+}
+
+// The instance into shared memory: F (and F^T); P (and P^T) zeroed so that
+// their padding columns stay zero.  Ends with a barrier.
+template <int NT>
+__device__ __forceinline__ void rot_load(const InstArgs& I, bool notr) {
+  const RotLayout L =
+      rot_layout(I.n, I.ldF, I.ldP, I.symF, I.symD, notr, RotFixed<NT>::bytes);
+  const bool ft = !I.symF && !notr, pt = !I.symD && !notr;
+  const int tid = threadIdx.x;
+  const int fvec = I.n * I.ldF / 16, pvec = I.n * I.ldP / 16;
+  const int4* gF = static_cast<const int4*>(I.F);
+  const int4* gFt = static_cast<const int4*>(I.Ft);
+#pragma unroll 2
+  for (int i = tid; i < fvec; i += NT) {
+    rot_at<int4>(L.F)[i] = gF[i];
+    if (ft) rot_at<int4>(L.Ft)[i] = gFt[i];
+  }
+  const int4 zero = make_int4(0, 0, 0, 0);
+#pragma unroll 2
+  for (int i = tid; i < pvec; i += NT) {
+    rot_at<int4>(L.P)[i] = zero;
+    if (pt) rot_at<int4>(L.Pt)[i] = zero;
+  }
+  __syncthreads();
+}
+
+// The partner blocks per thread (C) compiled for a thread count: at most 15,
+// for ranks below 32.
+constexpr int kRotMaxC = 13;
+__host__ __device__ constexpr bool rot_compiled(int nt, int c) {
+  return nt == 128   ? c == 1 || c == 2 || c == 4 || c == 7
+         : nt == 256 ? c <= 4 || c == 6 || c == 7 || c == 11 || c == 13
+         : nt == 512 ? c <= 3 || c == 5 || c == 7 || c == 8 || c == 11 || c == 13
+                     : c == 2 || c == 4 || c == 5 || c == 6;
+}
+
+// CTAs per SM to compile for.
+constexpr int rot_min_blocks(int nt) {
+  return nt == 128 ? 4 : nt == 256 ? 2 : 1;
+}
+
+template <int NT, int C>
+__global__ void __launch_bounds__(NT, rot_min_blocks(NT)) rot_walk_kernel(const WalkArgs a) {
+  RotWalkArgs& W = RotSmem<NT>::args();
+  if (threadIdx.x == 0) {
+    W.I = a.inst;
+    W.s = a.s;
+    W.notr = a.notr;
+  }
+  rot_load<NT>(a.inst, a.notr != 0);
+  for (int w = blockIdx.x; w < a.walks; w += gridDim.x) {
+    if (threadIdx.x == 0) {
+      const int wi = a.walk_offset + w;
+      W.row = wi;
+      W.wid = a.s.walk_base + (uint32_t)wi;
+      W.start = a.starts ? a.starts + (size_t)wi * a.inst.n : nullptr;
+    }
+    __syncthreads();
+    rot_walk<NT, C>();
+  }
+}
+
+template <int NT, int C>
+__global__ void __launch_bounds__(NT, rot_min_blocks(NT)) rot_batch_kernel(const BatchArgs b) {
+  __shared__ int item_s;
+  RotWalkArgs& W = RotSmem<NT>::args();
+  int cur_inst = -1;
+  for (;;) {
+    if (threadIdx.x == 0) item_s = atomicAdd(b.counter, 1);
+    __syncthreads();
+    const int item = item_s;
+    if (item >= b.items) break;
+    const int inst = b.item_inst[item];
+    if (inst != cur_inst) rot_load<NT>(b.insts[inst], b.notr != 0);
+    if (threadIdx.x == 0) {
+      const int w = b.item_walk[item];
+      if (inst != cur_inst) {
+        W.I = b.insts[inst];
+        W.s = b.s;
+        W.notr = b.notr;
+        W.start = nullptr;
+      }
+      W.row = b.row_base[inst] + w;
+      W.wid = b.s.walk_base + (uint32_t)w;
+    }
+    cur_inst = inst;
+    __syncthreads();
+    rot_walk<NT, C>();
+  }
+}
+
+}  // namespace qapk

@@ -157,9 +157,10 @@ qap_status place(qap_server* sv, Request* r) {
   const int W = r->params.starts, n = r->di.n;
   // a request's own walks decide (several requests share the GPU)
   const bool many = W >= 2 * sv->sms;
-  if (!choose_plan_fit(n, r->params.threads_per_walk, many, &r->di, 1, r->fbytes, r->dbytes,
-                       sv->smem_optin, 0, r->params.phase_x, &r->plan))
+  if (!search_plan(n, many, &r->di, 1, r->fbytes, r->dbytes, sv->smem_optin, 0, &r->params,
+                   &r->plan))
     return QAP_EUNSUPPORTED;
+  if (!rot_holds_tenures(r->plan, &r->params, n)) r->plan = r->plan.rows();
   r->fn = reinterpret_cast<const void*>(pick_walk_kernel(r->dbytes, r->fbytes, r->plan));
   if (!r->fn) return QAP_EUNSUPPORTED;
   r->smem = plan_smem(r->plan, &r->di, 1, r->fbytes, r->dbytes);
@@ -238,6 +239,7 @@ qap_status launch(qap_server* sv, Request* r) {
                      dev + r->offD, r->plan.nt, r->fbytes);
   const qap_walk_outputs d = carve_outputs(reinterpret_cast<char*>(dev + r->offOut), OL, W);
   a.s = make_search_args(&r->params, &d, n);
+  a.notr = (r->plan.store & qapk::kNoTransposed) != 0;
   a.s.rws_off = r->rws_off;
   a.s.p_off = r->p_off;
   a.walks = W;

@@ -1,0 +1,92 @@
+// Host-only checks of the rotation layout's geometry and admission
+// (qap_rotation.cuh, qap_host.cuh): no GPU, no CUDA calls.  For every n, thread
+// count and compiled number of partner blocks that rot_chunks admits: every
+// pair has a slot, no slot pairs an index with itself, window positions stay on
+// the doubled circle, phase X has a thread per index, ranks fit their bits, and
+// the fixed arrays hold n.  Built and run by tests/test_host_rotation.py.
+#include <cstdio>
+#include <vector>
+
+#include "../paper_2307_11248_gb300/csrc/qap_host.cuh"
+
+namespace {
+int fails = 0;
+void fail(const char* what, int n, int nt, int c) {
+  if (fails++ < 10) std::printf("FAIL %s: n=%d threads=%d c=%d\n", what, n, nt, c);
+}
+
+void check(int n, int nt, int c) {
+  const int J = qapk::rot_chunks(n, nt, c);
+  if (J == 0) return;
+  const int n2 = (n + 1) / 2, nE = 2 * n2;
+  if (n > qapk::rot_max_n(nt)) fail("fixed arrays too small", n, nt, c);
+  if (qapk::ld_m(n) > qapk::rot_max_n(nt) + 4) fail("pending words too small", n, nt, c);
+  if (J * n2 > qapk::rot_owners(nt)) fail("too many pair threads", n, nt, c);
+  if ((n + 31) / 32 * 32 > nt - qapk::rot_owners(nt)) fail("no thread per index", n, nt, c);
+  if (qapk::rot_rank(nt) ? 2 * c > 31 - 1 : nE > 1 << qapk::rot_key_bits(nt))
+    fail("partner does not fit the key bits", n, nt, c);
+  std::vector<char> held((size_t)nE * nE, 0);
+  for (int tid = 0; tid < J * n2; ++tid) {
+    const int j = tid / n2, m = tid - j * n2, pb = m + 1 + j * c;
+    held[(size_t)2 * m * nE + 2 * m + 1] = 1;
+    if (pb + c - 1 >= 2 * n2) fail("window beyond the doubled circle", n, nt, c);
+    for (int i = 0; i < c; ++i) {
+      const int b = (pb + i) % n2;
+      if (b == m) fail("a block against itself", n, nt, c);
+      for (int q = 0; q < 4; ++q) {
+        const int v = 2 * m + (q >> 1), u = 2 * b + (q & 1);
+        held[(size_t)std::min(u, v) * nE + std::max(u, v)] = 1;
+      }
+    }
+  }
+  for (int u = 0; u < n; ++u)
+    for (int v = u + 1; v < n; ++v)
+      if (!held[(size_t)u * nE + v]) return fail("a pair without a slot", n, nt, c);
+}
+}  // namespace
+
+int main() {
+  for (int n = 2; n <= 256; ++n)
+    for (int nt : {128, 256, 512, 1024})
+      for (int c = 1; c <= qapk::kRotMaxC; ++c)
+        if (qapk::rot_compiled(nt, c)) check(n, nt, c);
+  // every size that the automatic int8 products plans take has a layout
+  for (int n = 3; n <= 150; ++n)
+    for (int many = 0; many < 2; ++many) {
+      qaph::Plan p;
+      if (!qaph::choose_plan(n, 0, many != 0, &p)) continue;
+      bool any = false;
+      for (int c = 1; c <= qapk::kRotMaxC; ++c)
+        any |= qapk::rot_compiled(p.nt, c) && qapk::rot_chunks(n, p.nt, c) > 0;
+      if (!any && p.nt < 1024) fail("no layout", n, p.nt, many);
+    }
+  // the scan candidates' bound, at its edge: n = 100 at 256 threads (7 low
+  // bits) admits |values| up to 2 * 99 * rF * rD + 100 * rFD + 1 < 2^23
+  qaph::DevInstance d;
+  d.n = 100;
+  d.rangeF = 127;
+  d.rangeD = 127;
+  d.loFD = 0;
+  d.hiFD = 127 * 127;
+  if (!qaph::rot_fits_keys(d, 256)) fail("int8 extremes at n = 100", 100, 256, 0);
+  d.rangeF = 300;
+  if (qaph::rot_fits_keys(d, 256) != ((int64_t)(198 * 300 * 127 + 100 * 127 * 127 + 1) < 1 << 23))
+    fail("key bound", 100, 256, 0);
+  // tenures: up to the ring's length less 2
+  qap_search_params sp{};
+  sp.iters = 10;
+  for (int nt : {128, 256, 512, 1024}) {
+    qaph::Plan p{nt, 8, qapk::kProductM, 1, qapk::kProductM};
+    sp.tenure = {1, qapk::rot_ring(nt) - 2, 0};
+    if (!qaph::rot_holds_tenures(p, &sp, 50)) fail("longest tenure", 50, nt, 0);
+    ++sp.tenure.tmax;
+    if (qaph::rot_holds_tenures(p, &sp, 50)) fail("tenure beyond the ring", 50, nt, 0);
+    sp.tenure_per_n = 1;
+    sp.tenure = {90, 110, 200};
+    if (!qaph::rot_holds_tenures(p, &sp, 181)) fail("tenure per n", 181, nt, 0);
+    sp.tenure_per_n = 0;
+  }
+  if (fails) return 1;
+  std::printf("ok\n");
+  return 0;
+}

@@ -1,0 +1,87 @@
+"""GPU parity of the rotation layout (int8 flows, phase X from the maintained
+products): sizes at the edges of its circle, its warps and its arrays, tenures
+at the edges of its ring, and pairs applied while tabu whose new end equals
+an old one.  Every walk equals the oracle's bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2307_11248_gb300 as q
+from paper_2307_11248_gb300 import instances
+
+pytestmark = pytest.mark.gpu
+
+FIELDS = ["best_p", "best_cost", "final_cost", "best_iter", "iters_done", "status",
+          "descent_moves", "hash", "descent_hash"]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.fail("GPU test selected but no CUDA device is available")
+    oracle.build()
+    q.lib()
+    return torch
+
+
+def check(F, D, W, threads=0, **kw):
+    with q.Instance(F, D) as inst:
+        assert inst.info["flow_bytes"] == 1
+        g = inst.search(q.make_params(W, threads_per_walk=threads, **kw))
+    o = oracle.run_walks(F, D, W, **kw)
+    for k in FIELDS:
+        assert np.array_equal(g[k].astype(np.int64), o[k].astype(np.int64)), k
+
+
+# the smallest circles, even and odd n, a block count that C divides and not,
+# the last n of a warp of phase X, of the fixed arrays, and of a plan; n = 40:
+# the triangle of marks ends on a 16-byte boundary
+@pytest.mark.parametrize("sym", [False, True])
+@pytest.mark.parametrize("n", [3, 4, 5, 6, 7, 9, 16, 31, 32, 33, 40, 49, 63, 64, 65, 99, 104, 127,
+                               128, 129, 138, 149, 151, 160])
+def test_sizes(n, sym):
+    F, D = instances.uniform_instance(n, 2000 + n, symmetric=sym)
+    np.fill_diagonal(F, np.arange(n) % 7)  # diagonal terms count too
+    np.fill_diagonal(D, np.arange(n) % 5)
+    check(F, D, 3, seed=5, iters=150, tenure=instances.periodic_tenure(n), descend=True)
+
+
+@pytest.mark.parametrize("threads", [128, 256, 512, 1024])
+@pytest.mark.parametrize("n", [12, 37, 60])
+def test_thread_counts(n, threads):
+    F, D = instances.uniform_instance(n, 2100 + n, symmetric=n % 2 == 0)
+    if threads == 128 and n > 52:
+        pytest.skip("128 threads hold n up to 52")
+    check(F, D, 3, threads=threads, seed=6, iters=200, tenure=instances.paper_tenure(n))
+
+
+# many ties (small values), short random tenures with aspiration: pairs are
+# applied again while tabu, ends coincide
+@pytest.mark.parametrize("n,hi", [(14, 3), (30, 99), (50, 9), (100, 99), (100, 2), (130, 99)])
+def test_short_random_tenures(n, hi):
+    F, D = instances.uniform_instance(n, 2200 + n, symmetric=hi < 10, hi=hi)
+    check(F, D, 4, seed=13, iters=600, tenure=(1, 9, 0))
+
+
+# the longest tenure of the ring (254 and 510 iterations) and one more, which
+# the row layout takes; a walk whose every pair turns tabu
+@pytest.mark.parametrize("n,tmax,iters", [(30, 254, 700), (30, 255, 700), (110, 510, 1100),
+                                          (110, 511, 1100), (12, 200, 400)])
+def test_long_tenures(n, tmax, iters):
+    F, D = instances.uniform_instance(n, 2300 + n, symmetric=True)
+    check(F, D, 2, seed=14, iters=iters, tenure=(tmax - 3, tmax, 0))
+
+
+def test_batch_changes_layout_with_the_tenure(gpu):
+    """One batch, searched with tenures the ring holds and then longer ones."""
+    ns = [20, 33, 50, 77, 104]
+    pairs = [instances.uniform_instance(n, 2400 + n, symmetric=n % 2 == 0) for n in ns]
+    with q.Batch([F for F, _ in pairs], [D for _, D in pairs]) as b:
+        for tn in ((5, 30, 0), (250, 300, 0), (500, 600, 0), (5, 30, 0)):
+            g = b.search(q.make_params(3, seed=15, iters=120, tenure=tn, descend=True))
+            for i, (F, D) in enumerate(pairs):
+                o = oracle.run_walks(F, D, 3, seed=15, iters=120, tenure=tn, descend=True)
+                for k in FIELDS[1:]:
+                    assert np.array_equal(g[k][3 * i:3 * i + 3].astype(np.int64),
+                                          o[k].astype(np.int64)), (i, k)
