@@ -40,7 +40,8 @@
  * Arithmetic is exact integer arithmetic for any int64 F and D whose bound
  * B = (n^2 + 8n + 32) * max|F| * max|D| is below 2^62 (else QAP_EOVERFLOW).
  * Deltas are int32 when B is at most 2^31 - 2 and the instance is on a
- * narrow element path, else int64 (also when QAP_FORCE_INT64 is given).
+ * narrow element path, else int64 (also when QAP_FORCE_INT64 is given; without
+ * it deltas whose own bound allows may be held in 32 bits beside 64-bit costs).
  * Element paths, chosen per instance (per batch: the widest any instance
  * needs):
  *   int8 F, int8 D    every difference of two F entries and of two D
@@ -274,9 +275,10 @@ qap_status qap_search_async(qap_ctx* ctx, const qap_search_params* params,
 typedef struct {
   int32_t threads_per_walk;
   int32_t pairs_per_thread;  /* register slots per thread of the plan's row
-                                layout; int8 flows under QAP_TABU_PAIR without
-                                a penalty run a layout of the same threads in
-                                which fewer of them hold more pairs          */
+                                layout; int8 and int16 flows under
+                                QAP_TABU_PAIR without a penalty run a layout
+                                of the same threads in which fewer of them
+                                hold more pairs                              */
   int32_t smem_bytes;        /* dynamic shared memory per CTA             */
   int32_t grid;              /* CTAs of the persistent launch             */
   int32_t ctas_per_sm;

@@ -31,6 +31,7 @@ struct qap_ctx {
   DevInstance di;
   int dbytes = 4;  // delta width
   int fbytes = 2;  // flow element width in device memory (1: int8, 2: int16)
+  bool force64 = false;  // QAP_FORCE_INT64
   void* dF = nullptr;
   void* dFt = nullptr;
   void* dD = nullptr;
@@ -71,6 +72,7 @@ struct qap_batch {
   int device = 0, sms = 0, smem_optin = 0;
   int count = 0, nmax = 0;
   int dbytes = 4, fbytes = 2;
+  bool force64 = false;  // QAP_FORCE_INT64
   std::vector<DevInstance> di;
   std::vector<size_t> offF, offFt, offD;
   void* data = nullptr;  // every instance's F, F^T and D
@@ -114,11 +116,11 @@ qap_status occupancy(Launch* L, int sms, int work) {
 
 qap_status plan_ctx(qap_ctx* ctx, const qap_search_params* p, Launch* L) {
   const bool many = p->starts >= 2 * ctx->sms;
-  if (!search_plan(ctx->di.n, many, &ctx->di, 1, ctx->fbytes, ctx->dbytes, ctx->smem_optin, 0, p,
-                   &L->plan))
+  if (!search_plan(ctx->di.n, many, &ctx->di, 1, ctx->fbytes, ctx->dbytes, ctx->force64,
+                   ctx->smem_optin, 0, p, &L->plan))
     return QAP_EUNSUPPORTED;
   if (!rot_holds_tenures(L->plan, p, ctx->di.n)) L->plan = L->plan.rows();
-  L->fn = reinterpret_cast<const void*>(pick_walk_kernel(ctx->dbytes, ctx->fbytes, L->plan));
+  L->fn = pick_walk_kernel(ctx->dbytes, ctx->fbytes, L->plan);
   if (!L->fn) return QAP_EUNSUPPORTED;
   L->smem = plan_smem(L->plan, &ctx->di, 1, ctx->fbytes, ctx->dbytes);
   QAP_TRY(prepare_kernel(L->fn, L->smem));
@@ -128,11 +130,11 @@ qap_status plan_ctx(qap_ctx* ctx, const qap_search_params* p, Launch* L) {
 qap_status plan_batch(qap_batch* b, const qap_search_params* p, Launch* L) {
   // the batch kernel also holds one static int
   const bool many = (int64_t)b->count * p->starts >= 2 * (int64_t)b->sms;
-  if (!search_plan(b->nmax, many, b->di.data(), b->count, b->fbytes, b->dbytes, b->smem_optin, 16,
-                   p, &L->plan))
+  if (!search_plan(b->nmax, many, b->di.data(), b->count, b->fbytes, b->dbytes, b->force64,
+                   b->smem_optin, 16, p, &L->plan))
     return QAP_EUNSUPPORTED;
   if (!rot_holds_tenures(L->plan, p, b->nmax)) L->plan = L->plan.rows();
-  L->fn = reinterpret_cast<const void*>(pick_batch_kernel(b->dbytes, b->fbytes, L->plan));
+  L->fn = pick_batch_kernel(b->dbytes, b->fbytes, L->plan);
   if (!L->fn) return QAP_EUNSUPPORTED;
   L->smem = plan_smem(L->plan, b->di.data(), b->count, b->fbytes, b->dbytes);
   QAP_TRY(prepare_kernel(L->fn, L->smem));
@@ -166,7 +168,7 @@ qap_status class_shape(qap_batch* b, BatchClass& c, int W, const qap_search_para
   c.items = (int)c.members.size() * W;
   auto shape_of = [&](const Plan& plan, BatchClass::Shape* o) -> qap_status {
     o->smem = plan_smem(plan, dm.data(), (int)dm.size(), b->fbytes, b->dbytes);
-    o->fn = reinterpret_cast<const void*>(pick_batch_kernel(b->dbytes, b->fbytes, plan));
+    o->fn = pick_batch_kernel(b->dbytes, b->fbytes, plan);
     if (!o->fn) return QAP_EUNSUPPORTED;
     QAP_TRY(prepare_kernel(o->fn, o->smem));
     int occ = 0;
@@ -223,8 +225,8 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
     // the batch kernel also holds one static int
     // the classes run together: walks of the whole batch fill the SMs
     const bool many = (int64_t)b->count * W >= 2 * (int64_t)b->sms;
-    if (!search_plan(b->di[i].n, many, &b->di[i], 1, b->fbytes, b->dbytes, b->smem_optin, 16, p,
-                     &plan_of[i]))
+    if (!search_plan(b->di[i].n, many, &b->di[i], 1, b->fbytes, b->dbytes, b->force64,
+                     b->smem_optin, 16, p, &plan_of[i]))
       return QAP_EUNSUPPORTED;
   }
   std::vector<int> order(b->count);
@@ -335,6 +337,7 @@ qap_status qap_create(const int64_t* F, const int64_t* D, int32_t n, uint32_t fl
     return s;
   };
   c->dbytes = ((flags & QAP_FORCE_INT64) || di.wide || di.bound > (int64_t)INT_MAX - 1) ? 8 : 4;
+  c->force64 = (flags & QAP_FORCE_INT64) != 0;
   c->fbytes = flow_bytes(di, c->dbytes);
   di.ldF = pad_ldF(n, c->fbytes);
   di.ldP = pad_ldP(n, pbytes_of(c->fbytes));
@@ -415,7 +418,6 @@ qap_status qap_search_async(qap_ctx* ctx, const qap_search_params* params,
   qapk::WalkArgs a{};
   a.inst = inst_args(ctx->di, ctx->dF, ctx->dFt, ctx->dD, L.plan.nt, ctx->fbytes);
   a.s = make_search_args(params, out, ctx->di.n);
-  a.notr = (L.plan.store & qapk::kNoTransposed) != 0;
   a.starts = d_starts;
   a.walks = params->starts;
   a.walk_offset = 0;
@@ -429,15 +431,14 @@ qap_status qap_search_async(qap_ctx* ctx, const qap_search_params* params,
     QAP_TRY(grow(&ctx->ws, &ctx->ws_bytes, a.ws_stride * ctas));
     a.ws = static_cast<unsigned char*>(ctx->ws);
   }
-  const auto fn = reinterpret_cast<qapk::WalkKernelFn>(const_cast<void*>(L.fn));
   if (params->launch == QAP_LAUNCH_PLAIN) {
     a.walks = 1;
     for (int w = 0; w < params->starts; ++w) {
       a.walk_offset = w;
-      fn<<<1, L.plan.nt, L.smem, s>>>(a);
+      launch_walks(L.fn, L.plan, 1, L.smem, s, a);
     }
   } else {
-    fn<<<L.grid, L.plan.nt, L.smem, s>>>(a);
+    launch_walks(L.fn, L.plan, L.grid, L.smem, s, a);
   }
   QAP_CUDA(cudaGetLastError());
   return QAP_OK;
@@ -586,6 +587,7 @@ qap_status qap_batch_create(int32_t count, const int64_t* const* F, const int64_
   }
   // one delta width and one element width for the whole batch
   b->dbytes = ((flags & QAP_FORCE_INT64) || wide || maxB > (int64_t)INT_MAX - 1) ? 8 : 4;
+  b->force64 = (flags & QAP_FORCE_INT64) != 0;
   DevInstance all;
   all.bytevec = bytevec;
   all.wide = wide;
@@ -786,8 +788,8 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
         cands.push_back(p);
         const Plan m = with_products(p, b->fbytes, tp.phase_x, fits);
         if (m.store != p.store)
-          cands.push_back(with_rotation(m, dm.data(), (int)dm.size(), b->fbytes,
-                                        uses_rule_tables(&tp), fits));
+          cands.push_back(with_rotation(m, dm.data(), (int)dm.size(),
+                                        b->force64 || uses_rule_tables(&tp), fits));
       }
     }
     if (qapk::row_segments(nmax, kLargePlan.maxpt) <= kLargePlan.nt) {

@@ -26,8 +26,7 @@ BatchKernelFn batch_kernel_i32_f8m(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i32_f16(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i64_f16(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i64_f64(int nt, int maxpt, int store);
-WalkKernelFn rot_walk_kernel_f8(int nt, int c);
-BatchKernelFn rot_batch_kernel_f8(int nt, int c);
+BatchKernelFn rot_kernel_of(int fbytes, int nt, int c);
 }  // namespace qapk
 
 namespace qaph {
@@ -132,10 +131,44 @@ struct DevInstance {
   int bytevec = 0;  // every difference of two F entries, and of two D entries, fits int8
   int diff16 = 0;   // every difference of two F entries fits int16, of two D entries int8
   int wide = 0;     // outside the narrow paths: int64 elements and arithmetic
-  // narrow paths: the largest difference of two F entries and of two D
-  // entries, and the range of a product of an F and a D entry
-  int64_t rangeF = 0, rangeD = 0, loFD = 0, hiFD = 0;
+  // narrow paths, for the rotation layout: the mid-range of g[u] = sum_j
+  // F[u][j] P[u][j] + F[j][u] P[j][u] over all u and P, and a bound on |delta|
+  // plus g's half range (see rot_bounds)
+  int64_t g0 = 0, rotX = 0;
 };
+
+// Bounds of the rotation layout's values.  A delta is a sum of products of a
+// difference of two F entries of one column (or row) and one of two D
+// entries: at most (max D - min D) (A_r + A_s), with A_u the sum of |F[u][j]| +
+// |F[j][u]| over j.  g[u] lies between the sums of the products' lowest and
+// highest values.
+inline void rot_bounds(const int64_t* F, int n, int64_t loD, int64_t hiD, DevInstance* di) {
+  std::vector<int64_t> A(n, 0), pos(n, 0);  // sums of |F| and of F above 0
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < n; ++j) {
+      const int64_t f = F[(size_t)i * n + j], m = f < 0 ? -f : f;
+      A[i] += m;
+      A[j] += m;
+      if (f > 0) {
+        pos[i] += f;
+        pos[j] += f;
+      }
+    }
+  int64_t a1 = 0, a2 = 0, lo = INT64_MAX, hi = INT64_MIN;
+  for (int u = 0; u < n; ++u) {
+    if (A[u] > a1) {
+      a2 = a1;
+      a1 = A[u];
+    } else {
+      a2 = std::max(a2, A[u]);
+    }
+    const int64_t neg = A[u] - pos[u];
+    lo = std::min(lo, pos[u] * loD - neg * hiD);
+    hi = std::max(hi, pos[u] * hiD - neg * loD);
+  }
+  di->g0 = lo + (hi - lo) / 2;
+  di->rotX = (hiD - loD) * (a1 + a2) + (hi - lo + 1) / 2 + 1;
+}
 
 // Largest bound of the int64 path.  With B = (n^2 + 8n + 32) max|F| max|D|
 // below 2^62, every cost (at most n^2 max|F| max|D|), delta, dot-product sum
@@ -197,13 +230,7 @@ inline qap_status inspect_instance(const int64_t* F, const int64_t* D, int n, De
   // overflow here: on this branch the ranges fit int16 and int8)
   di->bytevec = !di->wide && mF <= 127 && hiF - loF <= 127 && hiD - loD <= 127;
   di->diff16 = !di->wide && hiF - loF <= 32767 && hiD - loD <= 127;
-  if (!di->wide) {
-    di->rangeF = hiF - loF;
-    di->rangeD = hiD - loD;
-    const auto fd = std::minmax({loF * loD, loF * hiD, hiF * loD, hiF * hiD});
-    di->loFD = fd.first;
-    di->hiFD = fd.second;
-  }
+  if (di->diff16) rot_bounds(F, n, loD, hiD, di);
   return QAP_OK;
 }
 
@@ -244,20 +271,43 @@ inline qap_status device_attrs(int* device, int* sms, int* smem_optin) {
   return QAP_OK;
 }
 
-inline qapk::WalkKernelFn pick_walk_kernel(int dbytes, int fbytes, const Plan& p) {
-  if (p.rot) return qapk::rot_walk_kernel_f8(p.nt, p.rot);
-  if (fbytes == 8) return qapk::walk_kernel_i64_f64(p.nt, p.maxpt, p.store);
-  if (dbytes == 8) return qapk::walk_kernel_i64_f16(p.nt, p.maxpt, p.store);
-  if (fbytes == 1) return qapk::walk_kernel_i32_f8(p.nt, p.maxpt, p.store);
-  return qapk::walk_kernel_i32_f16(p.nt, p.maxpt, p.store);
+inline const void* pick_walk_kernel(int dbytes, int fbytes, const Plan& p) {
+  auto row = [&]() -> qapk::WalkKernelFn {
+    if (fbytes == 8) return qapk::walk_kernel_i64_f64(p.nt, p.maxpt, p.store);
+    if (dbytes == 8) return qapk::walk_kernel_i64_f16(p.nt, p.maxpt, p.store);
+    if (fbytes == 1) return qapk::walk_kernel_i32_f8(p.nt, p.maxpt, p.store);
+    return qapk::walk_kernel_i32_f16(p.nt, p.maxpt, p.store);
+  };
+  return p.rot ? reinterpret_cast<const void*>(qapk::rot_kernel_of(fbytes, p.nt, p.rot))
+               : reinterpret_cast<const void*>(row());
 }
 
-inline qapk::BatchKernelFn pick_batch_kernel(int dbytes, int fbytes, const Plan& p) {
-  if (p.rot) return qapk::rot_batch_kernel_f8(p.nt, p.rot);
-  if (fbytes == 8) return qapk::batch_kernel_i64_f64(p.nt, p.maxpt, p.store);
-  if (dbytes == 8) return qapk::batch_kernel_i64_f16(p.nt, p.maxpt, p.store);
-  if (fbytes == 1) return qapk::batch_kernel_i32_f8(p.nt, p.maxpt, p.store);
-  return qapk::batch_kernel_i32_f16(p.nt, p.maxpt, p.store);
+inline const void* pick_batch_kernel(int dbytes, int fbytes, const Plan& p) {
+  auto row = [&]() -> qapk::BatchKernelFn {
+    if (fbytes == 8) return qapk::batch_kernel_i64_f64(p.nt, p.maxpt, p.store);
+    if (dbytes == 8) return qapk::batch_kernel_i64_f16(p.nt, p.maxpt, p.store);
+    if (fbytes == 1) return qapk::batch_kernel_i32_f8(p.nt, p.maxpt, p.store);
+    return qapk::batch_kernel_i32_f16(p.nt, p.maxpt, p.store);
+  };
+  return reinterpret_cast<const void*>(p.rot ? qapk::rot_kernel_of(fbytes, p.nt, p.rot) : row());
+}
+
+// A launch of walks of one instance by the kernel of pick_walk_kernel.
+inline void launch_walks(const void* fn, const Plan& p, int grid, int smem, cudaStream_t stream,
+                         const qapk::WalkArgs& a) {
+  if (!p.rot) {
+    reinterpret_cast<qapk::WalkKernelFn>(const_cast<void*>(fn))<<<grid, p.nt, smem, stream>>>(a);
+    return;
+  }
+  qapk::BatchArgs b{};
+  b.items = a.walks;
+  b.notr = (p.store & qapk::kNoTransposed) != 0;
+  b.s = a.s;
+  b.single = 1;
+  b.walk_offset = a.walk_offset;
+  b.starts = a.starts;
+  b.inst = a.inst;
+  reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(fn))<<<grid, p.nt, smem, stream>>>(b);
 }
 
 // Shared memory of a plan for the instance shapes `d` (the largest over them).
@@ -265,9 +315,9 @@ inline int plan_smem(const Plan& p, const DevInstance* d, int count, int fbytes,
   int smem = 0;
   if (p.rot) {
     for (int i = 0; i < count; ++i)
-      smem = std::max(smem, qapk::rot_layout(d[i].n, d[i].ldF, d[i].ldP, d[i].symF, d[i].symD,
-                                             p.store & qapk::kNoTransposed,
-                                             qapk::rot_fixed_bytes(p.nt))
+      smem = std::max(smem, qapk::rot_layout(d[i].n, d[i].ldF, fbytes, d[i].ldP, d[i].symF,
+                                             d[i].symD, p.store & qapk::kNoTransposed,
+                                             qapk::rot_fixed_bytes(p.nt, fbytes))
                                 .bytes);
     return smem;
   }
@@ -326,24 +376,23 @@ inline Plan with_products(Plan p, int fbytes, int form, Fits fits) {
 }
 
 // Whether every scan candidate of an instance, (delta + g - g0) 2^S plus its
-// low bits, stays within 2^30 of zero: a delta is at most 2 (n - 1) products of
-// an F and a D difference, g the sum of 2n products of an F and a D entry, g0
-// its mid-range.
+// low bits, stays within 2^30 of zero.
 inline bool rot_fits_keys(const DevInstance& d, int nt) {
-  const int64_t x = 2 * (d.n - 1) * d.rangeF * d.rangeD + d.n * (d.hiFD - d.loFD) + 1;
-  return x << qapk::rot_key_bits(nt) < (int64_t)1 << 30;
+  return d.rotX < (int64_t)1 << (30 - qapk::rot_key_bits(nt));
 }
 
-// The rotation layout in place of the row layout's products form: int8
-// flows, the paper's own criterion without a penalty, and the fewest partner
-// blocks per thread that hold every instance `d`; without the transposed
-// copies of F and P where it fits only so.  `fits` says whether a plan fits.
+// The rotation layout in place of the row layout's products form: int8 or
+// int16 flows (whose differences fit), the paper's own criterion without a
+// penalty, and the fewest partner blocks per thread that hold every instance
+// `d`; without the transposed copies of F and P where it fits only so.  Its
+// table holds 32-bit deltas, exact by rot_fits_keys also where the cost needs
+// 64 bits; `rows`: the search must keep the row layout (other criteria, or
+// deltas asked for in 64 bits).  `fits` says whether a plan fits.
 template <typename Fits>
-inline Plan with_rotation(Plan p, const DevInstance* d, int count, int fbytes, bool rules,
-                          Fits fits) {
-  if (rules || fbytes != 1 || !(p.store & qapk::kProductM)) return p;
+inline Plan with_rotation(Plan p, const DevInstance* d, int count, bool rows, Fits fits) {
+  if (rows || !(p.store & qapk::kProductM)) return p;
   for (int i = 0; i < count; ++i)
-    if (!rot_fits_keys(d[i], p.nt)) return p;
+    if (!d[i].diff16 || !rot_fits_keys(d[i], p.nt)) return p;
   for (int c = 1; c <= qapk::kRotMaxC; ++c) {
     bool holds = qapk::rot_compiled(p.nt, c);
     for (int i = 0; i < count; ++i) holds &= qapk::rot_chunks(d[i].n, p.nt, c) > 0;
@@ -445,8 +494,8 @@ inline bool uses_rule_tables(const qap_search_params* sp) {
 // that applies and still lets two CTAs share an SM where the row layout does.
 // (Its tenures are another condition: rot_holds_tenures.)
 inline bool search_plan(int nmax, bool many, const DevInstance* d, int count, int fbytes,
-                        int dbytes, int smem_optin, int reserve, const qap_search_params* sp,
-                        Plan* out) {
+                        int dbytes, bool force64, int smem_optin, int reserve,
+                        const qap_search_params* sp, Plan* out) {
   if (!choose_plan_fit(nmax, sp->threads_per_walk, many, d, count, fbytes, dbytes, smem_optin,
                        reserve, sp->phase_x, out))
     return false;
@@ -455,7 +504,7 @@ inline bool search_plan(int nmax, bool many, const DevInstance* d, int count, in
     return smem > smem_optin ? 0 : 2 * (smem + 1024) <= smem_optin + 1024 ? 2 : 1;
   };
   const int want = out->nt <= 256 ? ctas(*out) : 1;  // (above, registers hold one)
-  *out = with_rotation(*out, d, count, fbytes, uses_rule_tables(sp),
+  *out = with_rotation(*out, d, count, force64 || uses_rule_tables(sp),
                        [&](const Plan& x) { return ctas(x) >= want; });
   return true;
 }
@@ -683,7 +732,7 @@ inline qapk::InstArgs inst_args(const DevInstance& d, const void* F, const void*
   I.symD = d.symD;
   I.group = group_for(d.n, nt, fbytes);
   I.diff16 = d.diff16;
-  I.g0 = (int)(d.n * (d.loFD + d.hiFD));
+  I.g0 = (int)d.g0;
   I.F = F;
   I.Ft = d.symF ? F : Ft;
   I.D = D;

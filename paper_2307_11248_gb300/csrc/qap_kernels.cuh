@@ -98,7 +98,6 @@ struct WalkArgs {
   SearchArgs s;
   unsigned char* ws;      // large-n plans: per-CTA workspace (deltas, tabu stamps)
   size_t ws_stride;       // bytes per CTA
-  int notr;               // rotation layout: no transposed copies of F and P
   int walks;              // walks processed by this launch
   int walk_offset;        // index of this launch's first walk among the instance's walks
   const int32_t* starts;  // (walk_offset + walks) x n, or null
@@ -118,6 +117,10 @@ struct BatchArgs {
   SearchArgs s;
   unsigned char* ws;      // large-n plans: per-CTA workspace (deltas, tabu stamps)
   size_t ws_stride;       // bytes per CTA
+  // rotation layout, walks of one instance (as WalkArgs; items are its walks)
+  int single, walk_offset;
+  const int32_t* starts;
+  InstArgs inst;
 };
 
 // Where a plan keeps its state.  Register plans hold each thread's deltas in

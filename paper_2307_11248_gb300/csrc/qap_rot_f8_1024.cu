@@ -1,0 +1,16 @@
+// Rotation-layout kernels, int8 flows, 1024 threads per walk.
+#include "qap_rotation.cuh"
+
+namespace qapk {
+
+BatchKernelFn rot_f8_1024(int c) {
+  switch (c) {
+    case 2: return rot_kernel<1024, 2, int8_t>;
+    case 4: return rot_kernel<1024, 4, int8_t>;
+    case 5: return rot_kernel<1024, 5, int8_t>;
+    case 6: return rot_kernel<1024, 6, int8_t>;
+    default: return nullptr;
+  }
+}
+
+}  // namespace qapk

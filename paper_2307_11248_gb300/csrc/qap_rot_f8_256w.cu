@@ -1,0 +1,16 @@
+// Rotation-layout kernels, int8 flows, 256 threads per walk.
+#include "qap_rotation.cuh"
+
+namespace qapk {
+
+BatchKernelFn rot_f8_256w(int c) {
+  switch (c) {
+    case 6: return rot_kernel<256, 6, int8_t>;
+    case 7: return rot_kernel<256, 7, int8_t>;
+    case 11: return rot_kernel<256, 11, int8_t>;
+    case 13: return rot_kernel<256, 13, int8_t>;
+    default: return nullptr;
+  }
+}
+
+}  // namespace qapk

@@ -1,5 +1,5 @@
-// Rotation layout of the walk kernels (sm_103a): int8 flows, the paper's own
-// tabu criterion, phase X from the maintained products M.
+// Rotation layout of the walk kernels (sm_103a): int8 or int16 flows, the
+// paper's own tabu criterion, phase X from the maintained products M.
 //
 // Same search and same two barriers per iteration as qap_kernels.cuh; what
 // differs is how a walk's pairs lie in the registers, what a pair costs, and
@@ -48,6 +48,10 @@
 // x 2000 8.73 -> 3.18 ms; n = 23, 100 walks x 1000 in one blocking call 1.21 ->
 // 0.83 ms; 2opt from 32 starts at n = 12 16.4 -> 12.3 us.  Warp instructions per
 // walk-iteration: n = 100 grid 10360 -> 3370, n = 50 asymmetric 3606 -> 1920.
+// int16 flows (two dp2a per pair): 96 lognormal instances of n = 20-150, 64
+// walks x 1000 each, 103.4 -> 38.6 ms; their costs need 64 bits, their deltas
+// do not: the rows' sums of |F| bound them (rot_bounds), where the row layout
+// holds every delta as wide as the cost.
 // Tried and slower: every warp holding pairs and phase X on some of them
 // (n = 100 2.33 against 1.44 us per iteration of two walks per SM); tabu times
 // checked by each thread through its earliest (0.3 us per iteration on the
@@ -103,26 +107,33 @@ struct RotWalkArgs {
 };
 constexpr int kRotArgsBytes = (sizeof(RotWalkArgs) + 15) / 16 * 16;
 
+// Words of an index in the pairs' update: one (int8 flows: bytes b, e, a, c,
+// one dp4a) or two (int16: halves a, c, and bytes b, e, one dp2a each way).
+template <typename FE>
+constexpr int kRotWords = sizeof(FE) == 1 ? 1 : 2;
+
 // Shared memory: arrays of a fixed size per thread count first, so that their
 // addresses are constants, then the instance's own.
-template <int NT>
+template <int NT, typename FE>
 struct RotFixed {
   static constexpr int NE = rot_max_n(NT);
-  // per position (the indices, then the indices again): dp4a word, scan
+  static constexpr int W = kRotWords<FE>;
+  // per position (the indices, then the indices again): update word(s), scan
   // addend, and d of the pairs {r, k} and {s, k} after the move (int2)
   static constexpr int X = 0;
-  static constexpr int psi = X + 8 * NE;
+  static constexpr int X2 = X + 8 * NE;
+  static constexpr int psi = X + 8 * W * NE;
   static constexpr int R = psi + 8 * NE;
-  // per index: the negated, permuted dp4a word; label (row of P0); start
-  // permutation
+  // per index: the negated words that meet a partner's (W); label (row of
+  // P0); start permutation
   static constexpr int own = R + 16 * NE;
-  static constexpr int sigma = own + 4 * NE;
+  static constexpr int sigma = own + 4 * W * NE;
   static constexpr int p0 = sigma + 4 * NE;
   // pending operands of M's update (two buffers, by the move's parity): rows
-  // by index, columns by label
+  // by index (W words), columns by label
   static constexpr int NW = NE + 4;  // ld_m(n) at most
   static constexpr int vw = p0 + 4 * NE;
-  static constexpr int vwu = vw + 8 * NW;
+  static constexpr int vwu = vw + 8 * W * NW;
   // ring: the pairs whose tabu time ends at iteration i, at i mod its length:
   // key of the first in the low half, node of the rest in the high half;
   // nodes: such words moved aside, at the iteration that moved them
@@ -144,12 +155,12 @@ struct RotLayout {
 };
 
 // notr: no transposed copies of F and P (kNoTransposed plans)
-__host__ __device__ inline RotLayout rot_layout(int n, int ldF, int ldP, int symF, int symD,
-                                                int notr, int fixed) {
+__host__ __device__ inline RotLayout rot_layout(int n, int ldF, int fbytes, int ldP, int symF,
+                                                int symD, int notr, int fixed) {
   RotLayout L;
   int o = fixed;
-  L.F = o;    o = align16(o + n * ldF);
-  L.Ft = o;   o = (symF || notr) ? o : align16(o + n * ldF);
+  L.F = o;    o = align16(o + n * ldF * fbytes);
+  L.Ft = o;   o = (symF || notr) ? o : align16(o + n * ldF * fbytes);
   L.P = o;    o = align16(o + n * ldP);
   L.Pt = o;   o = (symD || notr) ? o : align16(o + n * ldP);
   L.M = o;    o = align16(o + n * ld_m(n) * 4);
@@ -160,11 +171,15 @@ __host__ __device__ inline RotLayout rot_layout(int n, int ldF, int ldP, int sym
   return L;
 }
 
-__host__ __device__ inline int rot_fixed_bytes(int nt) {
-  return nt == 128   ? RotFixed<128>::bytes
-         : nt == 256 ? RotFixed<256>::bytes
-         : nt == 512 ? RotFixed<512>::bytes
-                     : RotFixed<1024>::bytes;
+template <typename FE>
+__host__ __device__ inline int rot_fixed_of(int nt) {
+  return nt == 128   ? RotFixed<128, FE>::bytes
+         : nt == 256 ? RotFixed<256, FE>::bytes
+         : nt == 512 ? RotFixed<512, FE>::bytes
+                     : RotFixed<1024, FE>::bytes;
+}
+__host__ __device__ inline int rot_fixed_bytes(int nt, int fbytes) {
+  return fbytes == 1 ? rot_fixed_of<int8_t>(nt) : rot_fixed_of<int16_t>(nt);
 }
 
 extern __shared__ __align__(16) unsigned char rot_smem[];
@@ -175,14 +190,14 @@ __device__ __forceinline__ T* rot_at(int off) {
 }
 
 // Views of the shared memory.
-template <int NT>
+template <int NT, typename FE>
 struct RotSmem {
-  using X_ = RotFixed<NT>;
+  using X_ = RotFixed<NT, FE>;
   RotLayout L;
   int ft, pt;          // offsets that F^T and P0^T are read from:
   int fr, fk, pr, pk;  // entry [r][k] at r fr + k fk
   __device__ __forceinline__ RotSmem(const InstArgs& I, int n, bool notr) {
-    L = rot_layout(n, I.ldF, I.ldP, I.symF, I.symD, notr, X_::bytes);
+    L = rot_layout(n, I.ldF, sizeof(FE), I.ldP, I.symF, I.symD, notr, X_::bytes);
     ft = I.symF || notr ? L.F : L.Ft;
     pt = I.symD || notr ? L.P : L.Pt;
     // without copies F^T is read from F's columns
@@ -192,8 +207,8 @@ struct RotSmem {
     pr = pc ? 1 : I.ldP;
     pk = pc ? I.ldP : 1;
   }
-  __device__ __forceinline__ int8_t* F() const { return rot_at<int8_t>(L.F); }
-  __device__ __forceinline__ int8_t* Ft() const { return rot_at<int8_t>(ft); }
+  __device__ __forceinline__ FE* F() const { return rot_at<FE>(L.F); }
+  __device__ __forceinline__ FE* Ft() const { return rot_at<FE>(ft); }
   __device__ __forceinline__ int8_t* P() const { return rot_at<int8_t>(L.P); }  // P0 = D[p0][p0]
   __device__ __forceinline__ int8_t* Pt() const { return rot_at<int8_t>(pt); }
   // M[x][label], halved on symmetric instances
@@ -201,6 +216,7 @@ struct RotSmem {
   // tabu_until of pair u < v at v (v - 1) / 2 + u
   __device__ __forceinline__ int32_t* mark() const { return rot_at<int32_t>(L.mark); }
   __device__ __forceinline__ static int32_t* X() { return rot_at<int32_t>(X_::X); }
+  __device__ __forceinline__ static int32_t* X2() { return rot_at<int32_t>(X_::X2); }
   __device__ __forceinline__ static int32_t* psi() { return rot_at<int32_t>(X_::psi); }
   __device__ __forceinline__ static int2* R() { return rot_at<int2>(X_::R); }
   __device__ __forceinline__ static int32_t* own() { return rot_at<int32_t>(X_::own); }
@@ -217,13 +233,17 @@ struct RotSmem {
 };
 
 // The course of a walk, as the pairs' warps and phase X's follow it.
+template <typename FE>
 struct RotCourse {
-  int cur, best, it, dmoves, iters, cap, ow;
+  // costs: int8 flows have int32 deltas by the bound on the cost
+  using Cost = std::conditional_t<sizeof(FE) == 1, int, int64_t>;
+  Cost cur, best;
+  int it, dmoves, iters, cap, ow;
   int bd, r, s;          // the move
   bool tabu_phase, stalled;
 
   __device__ __forceinline__ RotCourse(const RotWalkArgs& w, int warps)
-      : cur((int)w.cost), best(cur), it(0), dmoves(0), iters(w.s.iters),
+      : cur((Cost)w.cost), best(cur), it(0), dmoves(0), iters(w.s.iters),
         cap(w.s.max_descent >= 0 ? w.s.max_descent : kDescentCap), ow(warps), bd(0), r(0), s(1),
         tabu_phase(!w.s.descend), stalled(false) {}
 
@@ -313,6 +333,24 @@ __device__ __forceinline__ int lds8(uint32_t at) {
   asm volatile("ld.shared.s8 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
   return v;
 }
+__device__ __forceinline__ int lds16(uint32_t at) {
+  int v;
+  asm volatile("{.reg .b16 t; ld.shared.s16 t, [%1]; cvt.s32.s16 %0, t;}"
+               : "=r"(v)
+               : "r"(at)
+               : "memory");
+  return v;
+}
+// an element of F
+template <typename FE>
+__device__ __forceinline__ int ldsf(uint32_t at) {
+  return sizeof(FE) == 1 ? lds8(at) : lds16(at);
+}
+__device__ __forceinline__ int2 lds64(uint32_t at) {
+  int2 v;
+  asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(at) : "memory");
+  return v;
+}
 __device__ __forceinline__ int4 lds128(uint32_t at) {
   int4 v;
   asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
@@ -333,6 +371,9 @@ __device__ __forceinline__ void sts128(uint32_t at, int4 v) {
                : "memory");
 }
 
+__device__ __forceinline__ uint32_t pack2(int h0, int h1) {
+  return __byte_perm((uint32_t)h0, (uint32_t)h1, 0x5410u);
+}
 __device__ __forceinline__ uint32_t pack4(int b0, int b1, int b2, int b3) {
   return __byte_perm(__byte_perm((uint32_t)b0, (uint32_t)b1, 0x0040u),
                      __byte_perm((uint32_t)b2, (uint32_t)b3, 0x0040u), 0x5410u);
@@ -342,26 +383,28 @@ __device__ __forceinline__ uint32_t pack4(int b0, int b1, int b2, int b3) {
 // rows, a second over columns when F or D is asymmetric.  A warp takes four
 // rows of F at once (each 16-byte chunk of a row of P0 serves four dot
 // products), its lanes the columns.  Symmetric instances keep half of M.
-template <int NT>
-__device__ __forceinline__ void rot_compute_m(const RotSmem<NT>& S, int n, int ldF, int ldP, bool sym,
-                                              bool notr) {
-  using C = Chunk<int8_t>;
-  const int nc = (n + 15) / 16, ldm = ld_m(n);
+template <int NT, typename FE>
+__device__ __forceinline__ void rot_compute_m(const RotSmem<NT, FE>& S, int n, int ldF, int ldP,
+                                              bool sym, bool notr) {
+  using C = Chunk<FE>;
+  using FV = typename C::FV;
+  using QV = typename C::QV;
+  const int nc = (n + C::W - 1) / C::W, ldm = ld_m(n);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int x0 = 4 * warp; x0 < n; x0 += NT / 8) {
     const int xm = n - 1;
     const int x1 = min(x0 + 1, xm), x2 = min(x0 + 2, xm), x3 = min(x0 + 3, xm);
     for (int k = lane; k < n; k += 32) {
       int a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-      auto rows = [&](const int8_t* F, const int8_t* P) {
-        const int4* q = reinterpret_cast<const int4*>(P + k * ldP);
-        const int4* f0 = reinterpret_cast<const int4*>(F + x0 * ldF);
-        const int4* f1 = reinterpret_cast<const int4*>(F + x1 * ldF);
-        const int4* f2 = reinterpret_cast<const int4*>(F + x2 * ldF);
-        const int4* f3 = reinterpret_cast<const int4*>(F + x3 * ldF);
+      auto rows = [&](const FE* F, const int8_t* P) {
+        const QV* q = reinterpret_cast<const QV*>(P + k * ldP);
+        const FV* f0 = reinterpret_cast<const FV*>(F + x0 * ldF);
+        const FV* f1 = reinterpret_cast<const FV*>(F + x1 * ldF);
+        const FV* f2 = reinterpret_cast<const FV*>(F + x2 * ldF);
+        const FV* f3 = reinterpret_cast<const FV*>(F + x3 * ldF);
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {
-          const int4 v = q[c];
+          const QV v = q[c];
           a0 = C::dot(f0[c], v, a0);
           a1 = C::dot(f1[c], v, a1);
           a2 = C::dot(f2[c], v, a2);
@@ -374,7 +417,8 @@ __device__ __forceinline__ void rot_compute_m(const RotSmem<NT>& S, int n, int l
         // columns x0..x0+3 of F (x0 a multiple of 4) and column k of P0
 #pragma unroll 4
         for (int j = 0; j < n; ++j) {
-          const char4 f = *reinterpret_cast<const char4*>(S.F() + j * ldF + x0);
+          using F4 = std::conditional_t<sizeof(FE) == 1, char4, short4>;
+          const F4 f = *reinterpret_cast<const F4*>(S.F() + j * ldF + x0);
           const int p = S.P()[j * ldP + k];
           a0 += f.x * p;
           a1 += f.y * p;
@@ -416,25 +460,36 @@ struct RotTenure {
   }
 };
 
-// M[x][.] after a move, for the rows x = slot mod Q: one dp4a per entry with
-// the pending words, a group of 4 columns of every urows-th such row per
-// thread, 4 rows in flight.
-template <int Q>
+// M[x][.] after a move, for the rows x = slot mod Q: one dp4a per entry (int16
+// flows: two dp2a) with the pending words, a group of 4 columns of every
+// urows-th such row per thread, 4 rows in flight.
+template <int Q, int W>
 __device__ __forceinline__ void rot_update_m(const RotThread& T, uint32_t aM, uint32_t aVw,
                                              uint32_t aVwu, int n, int ldm, int slot) {
   if (T.ux >= T.urows) return;
   const int4 w = lds128(aVwu + 16 * T.ug);
   const int step = Q * T.urows;
-  auto upd = [&](int u, int4 v) {
-    v.x = __dp4a(u, w.x, v.x);
-    v.y = __dp4a(u, w.y, v.y);
-    v.z = __dp4a(u, w.z, v.z);
-    v.w = __dp4a(u, w.w, v.w);
+  auto upd = [&](int2 u, int4 v) {
+    if constexpr (W == 1) {
+      v.x = __dp4a(u.x, w.x, v.x);
+      v.y = __dp4a(u.x, w.y, v.y);
+      v.z = __dp4a(u.x, w.z, v.z);
+      v.w = __dp4a(u.x, w.w, v.w);
+    } else {
+      v.x = __dp2a_hi(u.y, w.x, __dp2a_lo(u.x, w.x, v.x));
+      v.y = __dp2a_hi(u.y, w.y, __dp2a_lo(u.x, w.y, v.y));
+      v.z = __dp2a_hi(u.y, w.z, __dp2a_lo(u.x, w.z, v.z));
+      v.w = __dp2a_hi(u.y, w.w, __dp2a_lo(u.x, w.w, v.w));
+    }
     return v;
   };
+  auto word = [&](uint32_t at) {
+    if constexpr (W == 1) return make_int2(lds32(at), 0);
+    else return lds64(at);
+  };
   uint32_t am = aM + 16 * T.ug + 4 * ldm * (slot + Q * T.ux);
-  uint32_t av = aVw + 4 * (slot + Q * T.ux);
-  const uint32_t sm = 4 * ldm * step, sv = 4 * step;
+  uint32_t av = aVw + 4 * W * (slot + Q * T.ux);
+  const uint32_t sm = 4 * ldm * step, sv = 4 * W * step;
 #pragma unroll 1
   for (int x = slot + Q * T.ux; x < n; x += 4 * step) {
     // rows past the last repeat the first: the same entry, loaded before it
@@ -444,7 +499,7 @@ __device__ __forceinline__ void rot_update_m(const RotThread& T, uint32_t aM, ui
     const uint32_t v1 = x + step < n ? sv : 0, v2 = x + 2 * step < n ? 2 * sv : 0;
     const uint32_t v3 = x + 3 * step < n ? 3 * sv : 0;
     const int4 a0 = lds128(am), a1 = lds128(am + m1), a2 = lds128(am + m2), a3 = lds128(am + m3);
-    const int b0 = lds32(av), b1 = lds32(av + v1), b2 = lds32(av + v2), b3 = lds32(av + v3);
+    const int2 b0 = word(av), b1 = word(av + v1), b2 = word(av + v2), b3 = word(av + v3);
     sts128(am, upd(b0, a0));
     sts128(am + m1, upd(b1, a1));
     sts128(am + m2, upd(b2, a2));
@@ -469,9 +524,9 @@ __device__ __forceinline__ void clear_tabu(int (&d)[NS], int q, int big) {
 
 // The warps that hold pairs: the table, its update after each move, and the
 // scan for the next iteration.
-template <int NT, int C>
+template <int NT, int C, typename FE>
 __device__ __forceinline__ void rot_owner() {
-  using S = RotSmem<NT>;
+  using S = RotSmem<NT, FE>;
   const RotWalkArgs& W = S::args();
   const InstArgs& I = W.I;
   const int aspiration = W.s.aspiration;
@@ -504,11 +559,12 @@ __device__ __forceinline__ void rot_owner() {
 
   const int2* const X = reinterpret_cast<const int2*>(S::X());
   const int2* const psi = reinterpret_cast<const int2*>(S::psi());
-  const int2* const own = reinterpret_cast<const int2*>(S::own());
+  const int2* const X2 = reinterpret_cast<const int2*>(S::X2());  // int16 flows
   const int4* const R = reinterpret_cast<const int4*>(S::R());
 
   // Scan of the table: the warp's candidate into red.  A tabu pair aspires
-  // when its delta is below `lim` (at most 0).
+  // when its delta is below `lim` (at most 0, at least NOLIM).
+  constexpr int NOLIM = -(INT_MAX >> SB);
   auto scan = [&](int lim) {
     int m0 = INT_MAX, m1 = INT_MAX;
     uint32_t t0 = 0xffffffffu, t1 = 0xffffffffu;
@@ -536,7 +592,7 @@ __device__ __forceinline__ void rot_owner() {
     // 2^30 less g[v]
     const uint32_t q0 = (uint32_t)o.x - (RANK ? 32 : v0) + 0x80000000u;
     const uint32_t q1 = (uint32_t)o.y - (RANK ? 32 : v1) + 0x80000000u;
-    const int ls = (int)((uint32_t)max(lim, -(INT_MAX >> SB)) * MUL);
+    const int ls = (int)((uint32_t)lim * MUL);
     int c0 = m0 < 0 ? (int)((uint32_t)m0 + q0) : INT_MAX;
     int c1 = m1 < 0 ? (int)((uint32_t)m1 + q1) : INT_MAX;
     const int x0 = (int)(t0 + q0 + 0x80000000u), x1 = (int)(t1 + q1 + 0x80000000u);
@@ -564,13 +620,14 @@ __device__ __forceinline__ void rot_owner() {
     if (lane == 0) S::red()[warp] = make_int2(none ? INT_MAX : wd, (int)(none ? kNoMove : wk));
   };
 
-  scan(INT_MIN);
+  scan(NOLIM);
 
-  RotCourse c(W, T.ow);
+  RotCourse<FE> c(W, T.ow);
   while (c.next(S::red())) {
     const int r = c.r, s = c.s, it = c.it;
     c.best = c.tabu_phase ? min(c.best, c.cur) : c.cur;
-    const int lim = aspiration ? c.best - c.cur : INT_MIN;
+    using Cost = typename RotCourse<FE>::Cost;
+    const int lim = aspiration ? (int)max(c.best - c.cur, (Cost)NOLIM) : NOLIM;
     // pairs whose tabu time ends with the next iteration (in the shadow of
     // phase X)
     uint32_t w = S::ring()[(it + 1) & (rot_ring(NT) - 1)];
@@ -599,17 +656,34 @@ __device__ __forceinline__ void rot_owner() {
     rot_barrier();
 
     // the new table
-    const int2 A = own[m];
     const int4 Rm = R[m];  // the pairs (v0, r), (v0, s), (v1, r), (v1, s)
+    if constexpr (sizeof(FE) == 1) {
+      const int2 A = reinterpret_cast<const int2*>(S::own())[m];
 #pragma unroll
-    for (int i = 0; i < C; ++i) {
-      const int2 x = X[T.pb + i];
-      d[4 * i] = __dp4a(A.x, x.x, d[4 * i]);
-      d[4 * i + 1] = __dp4a(A.x, x.y, d[4 * i + 1]);
-      d[4 * i + 2] = __dp4a(A.y, x.x, d[4 * i + 2]);
-      d[4 * i + 3] = __dp4a(A.y, x.y, d[4 * i + 3]);
+      for (int i = 0; i < C; ++i) {
+        const int2 x = X[T.pb + i];
+        d[4 * i] = __dp4a(A.x, x.x, d[4 * i]);
+        d[4 * i + 1] = __dp4a(A.x, x.y, d[4 * i + 1]);
+        d[4 * i + 2] = __dp4a(A.y, x.x, d[4 * i + 2]);
+        d[4 * i + 3] = __dp4a(A.y, x.y, d[4 * i + 3]);
+      }
+      d[4 * C] = __dp4a(A.x, X[m].y, d[4 * C]);
+    } else {
+      // (-a, -c) of a row with the partner's (b, e), its (-b, -e) with (a, c)
+      const int4 A = reinterpret_cast<const int4*>(S::own())[m];
+      auto upd = [](int ac, int be, int x, int x2, int t) {
+        return __dp2a_lo(x, be, __dp2a_lo(ac, x2, t));
+      };
+#pragma unroll
+      for (int i = 0; i < C; ++i) {
+        const int2 x = X[T.pb + i], x2 = X2[T.pb + i];
+        d[4 * i] = upd(A.x, A.y, x.x, x2.x, d[4 * i]);
+        d[4 * i + 1] = upd(A.x, A.y, x.y, x2.y, d[4 * i + 1]);
+        d[4 * i + 2] = upd(A.z, A.w, x.x, x2.x, d[4 * i + 2]);
+        d[4 * i + 3] = upd(A.z, A.w, x.y, x2.y, d[4 * i + 3]);
+      }
+      d[4 * C] = upd(A.x, A.y, X[m].y, X2[m].y, d[4 * C]);
     }
-    d[4 * C] = __dp4a(A.x, X[m].y, d[4 * C]);
     // partners r and s
     auto partner = [&](int kk, bool odd, int w0, int w1) {
       if (odd) {
@@ -661,16 +735,17 @@ __device__ __forceinline__ void rot_owner() {
 // move t, by the last Q moves at once: byte (pair) t mod Q of the pending
 // words belongs to move t.  A row's word is cleared when the row is done, so
 // its entries' correction is one dp4a whatever the row's place in the turn.
-template <int NT, int C, bool SYM>
+template <int NT, int C, bool SYM, typename FE>
 __device__ __forceinline__ void rot_phase_x() {
+  constexpr int FB = sizeof(FE), PW = kRotWords<FE>;
   constexpr int Q = SYM ? 4 : 2;
   constexpr int SB = rot_key_bits(NT);
   constexpr int BIG = 1 << (31 - SB);
-  using X_ = RotFixed<NT>;
-  const RotWalkArgs& W = RotSmem<NT>::args();
+  using X_ = RotFixed<NT, FE>;
+  const RotWalkArgs& W = RotSmem<NT, FE>::args();
   const InstArgs& I = W.I;
   const RotThread T = rot_thread<NT, C>(I.n);
-  const RotSmem<NT> S(I, T.n, W.notr != 0);
+  const RotSmem<NT, FE> S(I, T.n, W.notr != 0);
   const int n = T.n, ldF = I.ldF, ldP = I.ldP, ldm = ld_m(n), nE = T.nE;
   const int g0 = I.g0, g2 = 2 * g0;
   const uint32_t wid = W.wid;
@@ -688,7 +763,8 @@ __device__ __forceinline__ void rot_phase_x() {
   const uint32_t aR = base + X_::R, aTen = base + X_::ten;
   const uint32_t oMk = aM + 4 * ldm * k;
   const int ktri = k * (k - 1) / 2;
-  int uk = k, wk = 0, best_uk = k, best_iter = 0, mv = 0;
+  int uk = k, best_uk = k, best_iter = 0, mv = 0;
+  int2 wk = make_int2(0, 0);  // the pending word(s) of row k
   const int Fkk = S.F()[k * ldF + k];
   int Qkk = S.P()[k * ldP + k];
   int gk = (S.M()[k * ldm + k] << (SYM ? 1 : 0)) - g0;
@@ -696,26 +772,34 @@ __device__ __forceinline__ void rot_phase_x() {
   const uint64_t h0 = 14695981039346656037ull;
   uint64_t h = h0, dh = h0;
   rot_clear_marks<NT>(S.mark(), n, T.ow);
-  RotCourse course(W, T.ow);
+  RotCourse<FE> course(W, T.ow);
   bool was_tabu = course.tabu_phase;
 
   while (course.next(S.red())) {
     const int r = course.r, s = course.s, it = course.it;
     const bool tabu_phase = course.tabu_phase;
-    const uint32_t oFr = aF + r * ldF, oFs = aF + s * ldF;
+    const uint32_t oFr = aF + r * ldF * FB, oFs = aF + s * ldF * FB;
     const uint32_t oMr = aM + 4 * r * ldm, oMs = aM + 4 * s * ldm;
     const int ur = lds32(aSig + 4 * r), us = lds32(aSig + 4 * s);
     // the moves that the rows r, s and k of M do not hold yet
     const int rd = (mv & 1) * 4 * ldm, wt = 4 * ldm - rd;  // this move's buffers
     const int done = (mv - 1) & (Q - 1);                   // rows finished after the last move
-    int wr = lds32(aVw + rd + 4 * r), ws = lds32(aVw + rd + 4 * s);
-    wr = (r & (Q - 1)) == done ? 0 : wr;
-    ws = (s & (Q - 1)) == done ? 0 : ws;
-    const int fRR = lds8(oFr + r), fRS = lds8(oFr + s), fSS = lds8(oFs + s);
-    const int fSR = SYM ? fRS : lds8(oFs + r);
-    const int Frk = lds8(oFr + k), Fsk = lds8(oFs + k);
-    const int Fkr = SYM ? Frk : lds8(aFt + r * S.fr + k * S.fk);
-    const int Fks = SYM ? Fsk : lds8(aFt + s * S.fr + k * S.fk);
+    auto pending = [&](int x) {
+      int2 w = make_int2(lds32(aVw + PW * rd + 4 * PW * x), 0);
+      if constexpr (PW == 2) w.y = lds32(aVw + PW * rd + 4 * PW * x + 4);
+      return (x & (Q - 1)) == done ? make_int2(0, 0) : w;
+    };
+    // an entry of M less what is pending: row word(s), label word
+    auto entry = [&](int2 w, int u, int m) {
+      if constexpr (PW == 1) return __dp4a(w.x, u, m);
+      else return __dp2a_hi(w.y, u, __dp2a_lo(w.x, u, m));
+    };
+    const int2 wr = pending(r), ws = pending(s);
+    const int fRR = ldsf<FE>(oFr + FB * r), fRS = ldsf<FE>(oFr + FB * s);
+    const int fSS = ldsf<FE>(oFs + FB * s), fSR = SYM ? fRS : ldsf<FE>(oFs + FB * r);
+    const int Frk = ldsf<FE>(oFr + FB * k), Fsk = ldsf<FE>(oFs + FB * k);
+    const int Fkr = SYM ? Frk : ldsf<FE>(aFt + FB * (r * S.fr + k * S.fk));
+    const int Fks = SYM ? Fsk : ldsf<FE>(aFt + FB * (s * S.fr + k * S.fk));
     // ends of the tabu times of the pairs {r, k} and {s, k}
     const int rtri = r * (r - 1) / 2, stri = s * (s - 1) / 2;
     const int end_r = lds32(aMark + 4 * (k < r ? rtri + k : ktri + r));
@@ -737,22 +821,33 @@ __device__ __forceinline__ void rot_phase_x() {
     const int slot = mv & (Q - 1);
     const uint32_t sel = SYM ? (0x3210u & ~(0xfu << (4 * slot))) | 4u << (4 * slot)
                              : slot ? 0x5410u : 0x3254u;
-    const int wkj = (k & (Q - 1)) == done ? 0 : wk;
-    Ar = __dp4a(wr, wuk, Ar);
-    As = __dp4a(ws, wuk, As);
-    Bs = __dp4a(wkj, wus, Bs);
-    Br = __dp4a(wkj, wur, Br);
-    mrs = __dp4a(wr, wus, mrs);
-    msr = __dp4a(ws, wur, msr);
+    const int2 wkj = (k & (Q - 1)) == done ? make_int2(0, 0) : wk;
+    Ar = entry(wr, wuk, Ar);
+    As = entry(ws, wuk, As);
+    Bs = entry(wkj, wus, Bs);
+    Br = entry(wkj, wur, Br);
+    mrs = entry(wr, wus, mrs);
+    msr = entry(ws, wur, msr);
     const int av = Frk - Fsk, b = Qrk - Qsk;
     const int c = Fkr - Fks, e = Qkr - Qks;
-    uint32_t own, word;
+    // the words of k in the pairs' update (int16 flows: (a, c), then (b, e))
+    uint32_t own, word, own2 = 0, word2 = 0;
     int gr, gs, gn, Rr, Rs;
+    if constexpr (PW == 2) {
+      own = pack2(-av, -c);
+      word = pack2(av, c);
+      own2 = __byte_perm((uint32_t)-b, (uint32_t)-e, 0x0040u);
+      word2 = __byte_perm((uint32_t)b, (uint32_t)e, 0x0040u);
+    } else if constexpr (SYM) {
+      own = __byte_perm((uint32_t)-av, (uint32_t)-b, 0x4400u);
+      word = __byte_perm((uint32_t)b, (uint32_t)av, 0x4400u);
+    } else {
+      own = pack4(-av, -c, -b, -e);
+      word = pack4(b, e, av, c);
+    }
     if (SYM) {
       gr = 2 * (mrs - (fRR - fRS) * (qRS - qSS)) - g0;
       gs = 2 * (msr - (fRS - fSS) * (qRR - qRS)) - g0;
-      own = __byte_perm((uint32_t)-av, (uint32_t)-b, 0x4400u);
-      word = __byte_perm((uint32_t)b, (uint32_t)av, 0x4400u);
       gn = gk - 2 * av * b;
       Rr = 2 * (Ar + Bs + (qSS - qRS) * av - (fRR - fRS) * b) - g2 +
            (fRR + Fkk - 2 * Frk) * (qSS + Qkk - 2 * Qsk);
@@ -761,8 +856,6 @@ __device__ __forceinline__ void rot_phase_x() {
     } else {
       gr = mrs - (fRR - fRS) * (qSR - qSS) - (fRR - fSR) * (qRS - qSS) - g0;
       gs = msr - (fSR - fSS) * (qRR - qRS) - (fRS - fSS) * (qRR - qSR) - g0;
-      own = pack4(-av, -c, -b, -e);
-      word = pack4(b, e, av, c);
       gn = gk - av * b - c * e;
       Rr = Ar + Bs - g2 + (fRR - Frk - Fkr + Fkk) * (qSS - Qsk - Qks + Qkk) - (fRR - fRS) * e -
            (fRR - fSR) * b + (qSS - qSR) * c + (qSS - qRS) * av;
@@ -771,10 +864,21 @@ __device__ __forceinline__ void rot_phase_x() {
     }
     Rr += end_r > it + 1 ? BIG : 0;
     Rs += end_s > it + 1 ? BIG : 0;
-    // M's operands of this move: bytes (-a, -c) by index, (b, e) by label
+    // M's operands of this move: (-a, -c) by index, bytes (b, e) by label
     // (symmetric: -a and b)
-    wk = (int)__byte_perm((uint32_t)wkj, own, sel);
-    const int wun = (int)__byte_perm((uint32_t)wuk, word, sel);
+    wk = wkj;
+    if constexpr (PW == 1) {
+      wk.x = (int)__byte_perm((uint32_t)wkj.x, own, sel);
+    } else if constexpr (SYM) {
+      const uint32_t hs = slot & 1 ? 0x5410u : 0x3254u;  // half slot mod 2 of word slot / 2
+      const int h = (int)__byte_perm((uint32_t)(slot & 2 ? wkj.y : wkj.x), own, hs);
+      wk.x = slot & 2 ? wk.x : h;
+      wk.y = slot & 2 ? h : wk.y;
+    } else {
+      wk.x = slot ? wk.x : (int)own;
+      wk.y = slot ? (int)own : wk.y;
+    }
+    const int wun = (int)__byte_perm((uint32_t)wuk, PW == 1 ? word : word2, sel);
     const bool isr = k == r, iss = k == s;
     // the pair (r, s) itself only changes sign, and turns tabu
     const int drs = gr + gs - course.bd + (tabu_phase && ten > 1 ? BIG : 0);
@@ -786,18 +890,24 @@ __device__ __forceinline__ void rot_phase_x() {
       const int psi = (int)(0u - ((uint32_t)gn << SB) - (1u << 30)) + (rot_rank(NT) ? 32 : k);
       sts32(aX + 4 * k, (int)word);
       sts32(aX + 4 * nE + 4 * k, (int)word);
+      if constexpr (PW == 2) {
+        sts32(base + X_::X2 + 4 * k, (int)word2);
+        sts32(base + X_::X2 + 4 * nE + 4 * k, (int)word2);
+      }
       sts32(aPsi + 4 * k, psi);
       sts32(aPsi + 4 * nE + 4 * k, rot_rank(NT) ? psi - 32 : psi);
-      sts32(aOwn + 4 * k, (int)own);
+      if constexpr (PW == 1) sts32(aOwn + 4 * k, (int)own);
+      else sts64(aOwn + 8 * k, (int)own, (int)own2);
       sts64(aR + 8 * k, Rr, Rs);
       sts64(aR + 8 * nE + 8 * k, Rr, Rs);
-      sts32(aVw + wt + 4 * k, wk);
+      if constexpr (PW == 1) sts32(aVw + wt + 4 * k, wk.x);
+      else sts64(aVw + 2 * wt + 8 * k, wk.x, wk.y);
       sts32(aVwu + wt + u4, wun);
     }
     rot_barrier();
     // while the other warps bring the table up to date: M, the labels, the
     // best solution, the tabu times and the hash
-    rot_update_m<Q>(T, aM, aVw + wt, aVwu + wt, n, ldm, slot);
+    rot_update_m<Q, PW>(T, aM, aVw + PW * wt, aVwu + wt, n, ldm, slot);
     ++mv;
     uk = isr ? us : iss ? ur : uk;
     Qkk = isr ? qSS : iss ? qRR : Qkk;
@@ -863,12 +973,13 @@ __device__ __forceinline__ void rot_phase_x() {
 }
 
 // The other warps: M's update, until the flag beside the candidates is set.
-template <int NT, int C, int Q>
+template <int NT, int C, int Q, typename FE>
 __device__ __forceinline__ void rot_helper() {
-  using X_ = RotFixed<NT>;
-  const RotWalkArgs& W = RotSmem<NT>::args();
+  constexpr int PW = kRotWords<FE>;
+  using X_ = RotFixed<NT, FE>;
+  const RotWalkArgs& W = RotSmem<NT, FE>::args();
   const RotThread T = rot_thread<NT, C>(W.I.n);
-  const RotSmem<NT> S(W.I, T.n, W.notr != 0);
+  const RotSmem<NT, FE> S(W.I, T.n, W.notr != 0);
   const int n = T.n, ldm = ld_m(n);
   const uint32_t base = smem_addr(rot_smem);
   rot_clear_marks<NT>(S.mark(), n, T.ow);
@@ -877,23 +988,23 @@ __device__ __forceinline__ void rot_helper() {
     rot_barrier();
     if (lds32(base + X_::red + 8 * 32)) break;
     const uint32_t wt = mv & 1 ? 0 : 4 * ldm;
-    rot_update_m<Q>(T, base + S.L.M, base + X_::vw + wt, base + X_::vwu + wt, n, ldm,
-                    mv & (Q - 1));
+    rot_update_m<Q, PW>(T, base + S.L.M, base + X_::vw + PW * wt, base + X_::vwu + wt, n, ldm,
+                        mv & (Q - 1));
   }
 }
 
 // The start of a walk: permutation, P0, M, the scan addends and the cost.
 // Starts and ends with every thread of the CTA together.
-template <int NT>
+template <int NT, typename FE>
 __device__ __forceinline__ void rot_start() {
-  RotWalkArgs& W = RotSmem<NT>::args();
+  RotWalkArgs& W = RotSmem<NT, FE>::args();
   const InstArgs& I = W.I;
   const SearchArgs& a = W.s;
   const bool notr = W.notr != 0;
   const int32_t* const start = W.start;
   const uint32_t wid = W.wid;
   const int n = I.n, ldF = I.ldF, ldP = I.ldP, tid = threadIdx.x;
-  const RotSmem<NT> S(I, n, notr);
+  const RotSmem<NT, FE> S(I, n, notr);
   const int lane = tid & 31, warp = tid >> 5;
   const bool sym = I.symF && I.symD;
   const int ldm = ld_m(n), nE = (n + 1) / 2 * 2, g0 = I.g0;
@@ -940,10 +1051,12 @@ __device__ __forceinline__ void rot_start() {
       S.X()[x] = S.X()[x + nE] = 0;
       S.psi()[x] = S.psi()[x + nE] = INT_MAX - 64;
       S.R()[x] = S.R()[x + nE] = make_int2(0, 0);
-      S.own()[x] = 0;
+      for (int w = 0; w < kRotWords<FE>; ++w) S.own()[kRotWords<FE> * x + w] = 0;
+      if (kRotWords<FE> == 2) S.X2()[x] = S.X2()[x + nE] = 0;
     }
     // no pending moves; M's padding columns take updates from these words only
-    for (int x = tid; x < 2 * ldm; x += NT) S.vw()[x] = S.vwu()[x] = 0;
+    for (int x = tid; x < 2 * ldm; x += NT) S.vwu()[x] = 0;
+    for (int x = tid; x < 2 * kRotWords<FE> * ldm; x += NT) S.vw()[x] = 0;
     for (int x = tid; x < rot_ring(NT); x += NT) S.ring()[x] = 0xffffffffu;
     if (a.iters > 0) {
       const RotTenure tenure(a, n);
@@ -952,13 +1065,13 @@ __device__ __forceinline__ void rot_start() {
     if (tid == 0) S.red()[32] = make_int2(0, 0);
   }
   __syncthreads();
-  rot_compute_m<NT>(S, n, ldF, ldP, sym, notr);
+  rot_compute_m<NT, FE>(S, n, ldF, ldP, sym, notr);
   __syncthreads();
 
   // ---- the pairs' table, in the marks' place: d = M[u][v] + M[v][u] + the
   // 2x2 term of Eq. 2
   {
-    const int8_t* F = S.F();
+    const FE* F = S.F();
     const int8_t* P = S.P();
     const int32_t* M = S.M();
     for (int v = 1 + warp; v < n; v += NT / 32) {
@@ -993,29 +1106,29 @@ __device__ __forceinline__ void rot_start() {
 
 // One whole walk of the instance in shared memory (see RotWalkArgs).  Starts
 // and ends with every thread of the CTA together.
-template <int NT, int C>
+template <int NT, int C, typename FE>
 __device__ __forceinline__ void rot_walk() {
-  rot_start<NT>();
-  const RotWalkArgs& W = RotSmem<NT>::args();
+  rot_start<NT, FE>();
+  const RotWalkArgs& W = RotSmem<NT, FE>::args();
   const int role = rot_thread<NT, C>(W.I.n).role;
   const bool sym = W.I.symF && W.I.symD;
-  if (role == 0) rot_owner<NT, C>();
-  else if (role == 1 && sym) rot_phase_x<NT, C, true>();
-  else if (role == 1) rot_phase_x<NT, C, false>();
-  else if (sym) rot_helper<NT, C, 4>();
-  else rot_helper<NT, C, 2>();
+  if (role == 0) rot_owner<NT, C, FE>();
+  else if (role == 1 && sym) rot_phase_x<NT, C, true, FE>();
+  else if (role == 1) rot_phase_x<NT, C, false, FE>();
+  else if (sym) rot_helper<NT, C, 4, FE>();
+  else rot_helper<NT, C, 2, FE>();
   __syncthreads();
 }
 
 // The instance into shared memory: F (and F^T); P (and P^T) zeroed so that
 // their padding columns stay zero.  Ends with a barrier.
-template <int NT>
+template <int NT, typename FE>
 __device__ __forceinline__ void rot_load(const InstArgs& I, bool notr) {
-  const RotLayout L =
-      rot_layout(I.n, I.ldF, I.ldP, I.symF, I.symD, notr, RotFixed<NT>::bytes);
+  const RotLayout L = rot_layout(I.n, I.ldF, sizeof(FE), I.ldP, I.symF, I.symD, notr,
+                                 RotFixed<NT, FE>::bytes);
   const bool ft = !I.symF && !notr, pt = !I.symD && !notr;
   const int tid = threadIdx.x;
-  const int fvec = I.n * I.ldF / 16, pvec = I.n * I.ldP / 16;
+  const int fvec = I.n * I.ldF * (int)sizeof(FE) / 16, pvec = I.n * I.ldP / 16;
   const int4* gF = static_cast<const int4*>(I.F);
   const int4* gFt = static_cast<const int4*>(I.Ft);
 #pragma unroll 2
@@ -1047,53 +1160,37 @@ constexpr int rot_min_blocks(int nt) {
   return nt == 128 ? 4 : nt == 256 ? 2 : 1;
 }
 
-template <int NT, int C>
-__global__ void __launch_bounds__(NT, rot_min_blocks(NT)) rot_walk_kernel(const WalkArgs a) {
-  RotWalkArgs& W = RotSmem<NT>::args();
-  if (threadIdx.x == 0) {
-    W.I = a.inst;
-    W.s = a.s;
-    W.notr = a.notr;
-  }
-  rot_load<NT>(a.inst, a.notr != 0);
-  for (int w = blockIdx.x; w < a.walks; w += gridDim.x) {
-    if (threadIdx.x == 0) {
-      const int wi = a.walk_offset + w;
-      W.row = wi;
-      W.wid = a.s.walk_base + (uint32_t)wi;
-      W.start = a.starts ? a.starts + (size_t)wi * a.inst.n : nullptr;
-    }
-    __syncthreads();
-    rot_walk<NT, C>();
-  }
-}
-
-template <int NT, int C>
-__global__ void __launch_bounds__(NT, rot_min_blocks(NT)) rot_batch_kernel(const BatchArgs b) {
+// Walks of one instance (b.single: CTAs step over its walks) or of many (CTAs
+// take items from the counter and reload the instance when it changes).
+template <int NT, int C, typename FE>
+__global__ void __launch_bounds__(NT, rot_min_blocks(NT)) rot_kernel(const BatchArgs b) {
   __shared__ int item_s;
-  RotWalkArgs& W = RotSmem<NT>::args();
-  int cur_inst = -1;
-  for (;;) {
-    if (threadIdx.x == 0) item_s = atomicAdd(b.counter, 1);
-    __syncthreads();
-    const int item = item_s;
+  RotWalkArgs& W = RotSmem<NT, FE>::args();
+  int cur_inst = -1, item = blockIdx.x;
+  for (;; item += gridDim.x) {
+    if (!b.single) {
+      if (threadIdx.x == 0) item_s = atomicAdd(b.counter, 1);
+      __syncthreads();
+      item = item_s;
+    }
     if (item >= b.items) break;
-    const int inst = b.item_inst[item];
-    if (inst != cur_inst) rot_load<NT>(b.insts[inst], b.notr != 0);
+    const int inst = b.single ? 0 : b.item_inst[item];
+    const InstArgs* const I = b.single ? &b.inst : b.insts + inst;
+    if (inst != cur_inst) rot_load<NT, FE>(*I, b.notr != 0);
     if (threadIdx.x == 0) {
-      const int w = b.item_walk[item];
       if (inst != cur_inst) {
-        W.I = b.insts[inst];
+        W.I = *I;
         W.s = b.s;
         W.notr = b.notr;
-        W.start = nullptr;
       }
-      W.row = b.row_base[inst] + w;
+      const int w = b.single ? b.walk_offset + item : b.item_walk[item];
+      W.row = b.single ? w : b.row_base[inst] + w;
       W.wid = b.s.walk_base + (uint32_t)w;
+      W.start = b.starts ? b.starts + (size_t)w * I->n : nullptr;
     }
     cur_inst = inst;
     __syncthreads();
-    rot_walk<NT, C>();
+    rot_walk<NT, C, FE>();
   }
 }
 

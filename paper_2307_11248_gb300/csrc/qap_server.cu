@@ -86,6 +86,7 @@ struct Request {
   uint64_t ticket = 0;
   DevInstance di;
   int dbytes = 4, fbytes = 2;
+  bool force64 = false;  // QAP_FORCE_INT64
   std::vector<unsigned char> iF, iFt, iD;  // upload images (while not in the pinned slab)
   size_t szF = 0, szFt = 0, szD = 0;       // image sizes
   size_t host_off = 0, host_bytes = 0;     // range of the images in the pinned slab (bytes 0: none)
@@ -157,11 +158,11 @@ qap_status place(qap_server* sv, Request* r) {
   const int W = r->params.starts, n = r->di.n;
   // a request's own walks decide (several requests share the GPU)
   const bool many = W >= 2 * sv->sms;
-  if (!search_plan(n, many, &r->di, 1, r->fbytes, r->dbytes, sv->smem_optin, 0, &r->params,
-                   &r->plan))
+  if (!search_plan(n, many, &r->di, 1, r->fbytes, r->dbytes, r->force64, sv->smem_optin, 0,
+                   &r->params, &r->plan))
     return QAP_EUNSUPPORTED;
   if (!rot_holds_tenures(r->plan, &r->params, n)) r->plan = r->plan.rows();
-  r->fn = reinterpret_cast<const void*>(pick_walk_kernel(r->dbytes, r->fbytes, r->plan));
+  r->fn = pick_walk_kernel(r->dbytes, r->fbytes, r->plan);
   if (!r->fn) return QAP_EUNSUPPORTED;
   r->smem = plan_smem(r->plan, &r->di, 1, r->fbytes, r->dbytes);
   QAP_TRY(prepare_kernel(r->fn, r->smem));
@@ -239,7 +240,6 @@ qap_status launch(qap_server* sv, Request* r) {
                      dev + r->offD, r->plan.nt, r->fbytes);
   const qap_walk_outputs d = carve_outputs(reinterpret_cast<char*>(dev + r->offOut), OL, W);
   a.s = make_search_args(&r->params, &d, n);
-  a.notr = (r->plan.store & qapk::kNoTransposed) != 0;
   a.s.rws_off = r->rws_off;
   a.s.p_off = r->p_off;
   a.walks = W;
@@ -247,9 +247,8 @@ qap_status launch(qap_server* sv, Request* r) {
   a.starts = nullptr;
   a.ws_stride = r->ws_stride;
   a.ws = r->ws_stride ? dev + r->offWs : nullptr;
-  const auto fn = reinterpret_cast<qapk::WalkKernelFn>(const_cast<void*>(r->fn));
   QAP_CUDA(cudaEventRecord(sl.k0, sl.stream));
-  fn<<<r->grid, r->plan.nt, r->smem, sl.stream>>>(a);
+  launch_walks(r->fn, r->plan, r->grid, r->smem, sl.stream, a);
   QAP_CUDA(cudaGetLastError());
   QAP_CUDA(cudaEventRecord(sl.k1, sl.stream));
   QAP_CUDA(cudaMemcpyAsync(sl.pinned, dev + r->offOut, OL.total, cudaMemcpyDeviceToHost,
@@ -399,6 +398,7 @@ qap_status qap_server_submit(qap_server* sv, const int64_t* F, const int64_t* D,
   if (!r) return QAP_ENOMEM;
   QAP_TRY(inspect_instance(F, D, n, &r->di));
   // int64 deltas when B, or B plus the largest frequency penalty, needs them
+  r->force64 = (flags & QAP_FORCE_INT64) != 0;
   r->dbytes = ((flags & QAP_FORCE_INT64) || r->di.wide || r->di.bound > (int64_t)INT_MAX - 1 ||
                check_penalty(params, 4, r->di.bound) != QAP_OK) ? 8 : 4;
   r->fbytes = flow_bytes(r->di, r->dbytes);

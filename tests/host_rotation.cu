@@ -4,7 +4,10 @@
 // pair has a slot, no slot pairs an index with itself, window positions stay on
 // the doubled circle, phase X has a thread per index, ranks fit their bits, and
 // the fixed arrays hold n.  Built and run by tests/test_host_rotation.py.
+#include <algorithm>
 #include <cstdio>
+#include <cstdlib>
+#include <random>
 #include <vector>
 
 #include "../paper_2307_11248_gb300/csrc/qap_host.cuh"
@@ -60,18 +63,49 @@ int main() {
         any |= qapk::rot_compiled(p.nt, c) && qapk::rot_chunks(n, p.nt, c) > 0;
       if (!any && p.nt < 1024) fail("no layout", n, p.nt, many);
     }
-  // the scan candidates' bound, at its edge: n = 100 at 256 threads (7 low
-  // bits) admits |values| up to 2 * 99 * rF * rD + 100 * rFD + 1 < 2^23
+  // the scan candidates' bound: by brute force over permutations and pairs it
+  // holds every delta and g; F of any sign, skewed or dense
+  std::mt19937 rng(3);
+  for (int kind = 0; kind < 6; ++kind) {
+    const int n = 9 + kind;
+    std::vector<int64_t> F(n * n), D(n * n);
+    for (auto& f : F) f = kind % 3 == 0 ? rng() % 100 : kind % 3 == 1 ? rng() % 9000 * (rng() % 4 == 0)
+                                                                 : (int)(rng() % 2001) - 1000;
+    for (auto& d : D) d = kind < 3 ? rng() % 100 : (int)(rng() % 120) - 60;
+    qaph::DevInstance d;
+    if (qaph::inspect_instance(F.data(), D.data(), n, &d) != QAP_OK || !d.diff16)
+      fail("inspect", n, 0, kind);
+    std::vector<int> p(n);
+    for (int i = 0; i < n; ++i) p[i] = i;
+    auto cost = [&]() {
+      int64_t c = 0;
+      for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) c += F[i * n + j] * D[p[i] * n + p[j]];
+      return c;
+    };
+    for (int rep = 0; rep < 40; ++rep) {
+      std::shuffle(p.begin(), p.end(), rng);
+      const int64_t c0 = cost();
+      int64_t g1 = 0, dmax = 0;
+      for (int u = 0; u < n; ++u) {
+        int64_t g = -d.g0;
+        for (int j = 0; j < n; ++j)
+          g += F[u * n + j] * D[p[u] * n + p[j]] + F[j * n + u] * D[p[j] * n + p[u]];
+        g1 = std::max(g1, std::abs(g));
+        for (int v = u + 1; v < n; ++v) {
+          std::swap(p[u], p[v]);
+          dmax = std::max(dmax, std::abs(cost() - c0));
+          std::swap(p[u], p[v]);
+        }
+      }
+      if (g1 + dmax >= d.rotX) fail("values beyond the bound", n, 0, kind);
+    }
+  }
   qaph::DevInstance d;
-  d.n = 100;
-  d.rangeF = 127;
-  d.rangeD = 127;
-  d.loFD = 0;
-  d.hiFD = 127 * 127;
-  if (!qaph::rot_fits_keys(d, 256)) fail("int8 extremes at n = 100", 100, 256, 0);
-  d.rangeF = 300;
-  if (qaph::rot_fits_keys(d, 256) != ((int64_t)(198 * 300 * 127 + 100 * 127 * 127 + 1) < 1 << 23))
-    fail("key bound", 100, 256, 0);
+  d.rotX = ((int64_t)1 << 23) - 1;
+  if (!qaph::rot_fits_keys(d, 256)) fail("largest value at 7 low bits", 0, 256, 0);
+  ++d.rotX;
+  if (qaph::rot_fits_keys(d, 256) || !qaph::rot_fits_keys(d, 512)) fail("key bound", 0, 256, 0);
   // tenures: up to the ring's length less 2
   qap_search_params sp{};
   sp.iters = 10;

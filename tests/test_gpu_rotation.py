@@ -25,9 +25,9 @@ def gpu():
     return torch
 
 
-def check(F, D, W, threads=0, **kw):
+def check(F, D, W, threads=0, flow_bytes=1, **kw):
     with q.Instance(F, D) as inst:
-        assert inst.info["flow_bytes"] == 1
+        assert inst.info["flow_bytes"] == flow_bytes
         g = inst.search(q.make_params(W, threads_per_walk=threads, **kw))
     o = oracle.run_walks(F, D, W, **kw)
     for k in FIELDS:
@@ -45,6 +45,32 @@ def test_sizes(n, sym):
     np.fill_diagonal(F, np.arange(n) % 7)  # diagonal terms count too
     np.fill_diagonal(D, np.arange(n) % 5)
     check(F, D, 3, seed=5, iters=150, tenure=instances.periodic_tenure(n), descend=True)
+
+
+# int16 flows: skewed values (costs in 64 bits from n of about 50 on), and
+# flows a few times a byte's range on a dense instance with a diagonal
+@pytest.mark.parametrize("sym", [False, True])
+@pytest.mark.parametrize("n", [5, 16, 31, 33, 40, 64, 65, 90, 99, 100, 104, 127, 129, 140, 150,
+                               151])
+def test_int16_flows(n, sym):
+    F, D = instances.lognormal_instance(n, 2600 + n, sym)
+    F[0, n - 1] = F[n - 1, 0] = 700  # beyond a byte whatever the draw
+    check(F, D, 3, flow_bytes=2, seed=5, iters=150, tenure=instances.periodic_tenure(n),
+          descend=True)
+    if n <= 65:
+        F, D = instances.uniform_instance(n, 2700 + n, symmetric=sym, lo=-150, hi=150)
+        _, D = instances.uniform_instance(n, 2800 + n, symmetric=sym, lo=-20, hi=60)
+        np.fill_diagonal(F, np.arange(n) - 7)
+        np.fill_diagonal(D, np.arange(n) % 9)
+        check(F, D, 3, flow_bytes=2, seed=6, iters=200, tenure=instances.paper_tenure(n))
+
+
+def test_int16_flows_at_the_key_bound():
+    """Flows scaled up to the largest values that the scan's candidates hold
+    and past them: the walks do not change their kind of answer."""
+    F, D = instances.uniform_instance(26, 2900, symmetric=False, lo=1)
+    for scale in (2, 9, 14, 15, 16, 17, 20, 40):
+        check(F * scale, D, 3, flow_bytes=2, seed=7, iters=200, tenure=(3, 9, 0), descend=True)
 
 
 @pytest.mark.parametrize("threads", [128, 256, 512, 1024])
