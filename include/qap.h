@@ -146,8 +146,10 @@ typedef struct {
  *          the caller may free them when the call returns.  The element path
  *          and the delta width follow from the values (see above).
  *   n      2 <= n <= 256.  Up to n = 181 a walk keeps its deltas in
- *          registers; beyond, in a workspace in device memory (allocated by
- *          the library on first use), with F in shared or global memory.
+ *          registers; beyond, a workspace in device memory (allocated by the
+ *          library on first use) holds its products M (int8 flows; batches and
+ *          the serving loop use it from n = 152 on) or its deltas and marks,
+ *          with F in shared or global memory.
  *   flags  0 or QAP_FORCE_INT64.
  *   out    receives the context (NULL on error).
  * Uses the CUDA device current at the call for all later calls.
@@ -191,7 +193,9 @@ typedef struct {
                               with at most 8 pairs per thread, or 512 with
                               any; with starts >= 2 x SMs also 256 with any
                               (two walks per SM).  Else 128, 256, 512 or
-                              1024 (n > 181 always uses 1024)                */
+                              1024 (n > 181 uses 512 where the workspace
+                              holds the products, when the count is automatic,
+                              else 1024)                                     */
   int32_t tenure_per_n;    /* 1: tenure.tmin, tmax, period are hundredths of
                               each instance's n:
                               tmin' = max(1, floor(tmin n / 100)),
@@ -291,7 +295,9 @@ typedef struct {
                                 transposed copies of F and P, whose entries
                                 are then read from columns (where M fits
                                 only so)                                    */
-  int32_t workspace;         /* 1: deltas and marks in the device workspace */
+  int32_t workspace;         /* 1: a device workspace holds the products (in
+                                place of dot products; products is 0 then) or
+                                the deltas and marks                         */
 } qap_plan_info;
 qap_status qap_plan(qap_ctx* ctx, const qap_search_params* params, qap_plan_info* out);
 

@@ -52,7 +52,8 @@ struct BatchClass {
   // whose tenures need the rows finds them ready
   struct Shape {
     const void* fn = nullptr;
-    int smem = 0, grid = 0, ctas_per_sm = 0, notr = 0;
+    int nt = 0, smem = 0, grid = 0, ctas_per_sm = 0, notr = 0;
+    size_t ws_stride = 0, p_off = 0, rws_off = 0;  // workspace: bytes per CTA, offsets in them
   } own, rows;
   int nmax = 0;
   const Shape& shape(const qap_search_params* p) const {
@@ -60,8 +61,10 @@ struct BatchClass {
   }
   std::vector<int> members;  // instance indices, largest n first
   int item_off = 0, items = 0;
-  size_t ws_off = 0, ws_stride = 0;
-  size_t p_off = 0, rws_off = 0;  // offsets inside a CTA's workspace slice
+  size_t ws_off = 0;
+  size_t workspace() const {
+    return std::max(own.ws_stride * own.grid, rows.ws_stride * rows.grid);
+  }
   cudaStream_t side = nullptr;
   cudaEvent_t done = nullptr;
   cudaEvent_t t0 = nullptr, t1 = nullptr;  // timing events (qap_batch_set_timing)
@@ -117,7 +120,7 @@ qap_status occupancy(Launch* L, int sms, int work) {
 qap_status plan_ctx(qap_ctx* ctx, const qap_search_params* p, Launch* L) {
   const bool many = p->starts >= 2 * ctx->sms;
   if (!search_plan(ctx->di.n, many, &ctx->di, 1, ctx->fbytes, ctx->dbytes, ctx->force64,
-                   ctx->smem_optin, 0, p, &L->plan))
+                   ctx->smem_optin, 0, ctx->di.n > 181, p, &L->plan))
     return QAP_EUNSUPPORTED;
   if (!rot_holds_tenures(L->plan, p, ctx->di.n)) L->plan = L->plan.rows();
   L->fn = pick_walk_kernel(ctx->dbytes, ctx->fbytes, L->plan);
@@ -131,7 +134,7 @@ qap_status plan_batch(qap_batch* b, const qap_search_params* p, Launch* L) {
   // the batch kernel also holds one static int
   const bool many = (int64_t)b->count * p->starts >= 2 * (int64_t)b->sms;
   if (!search_plan(b->nmax, many, b->di.data(), b->count, b->fbytes, b->dbytes, b->force64,
-                   b->smem_optin, 16, p, &L->plan))
+                   b->smem_optin, 16, b->nmax > 181, p, &L->plan))
     return QAP_EUNSUPPORTED;
   if (!rot_holds_tenures(L->plan, p, b->nmax)) L->plan = L->plan.rows();
   L->fn = pick_batch_kernel(b->dbytes, b->fbytes, L->plan);
@@ -177,26 +180,28 @@ qap_status class_shape(qap_batch* b, BatchClass& c, int W, const qap_search_para
     o->ctas_per_sm = occ;
     o->grid = std::min(c.items, occ * b->sms);
     o->notr = (plan.store & qapk::kNoTransposed) != 0;
+    o->nt = plan.nt;
+    const WsLayout wl = ws_layout(plan, b->dbytes, b->fbytes, nmax, p);
+    o->ws_stride = wl.stride;
+    o->p_off = wl.p_off;
+    o->rws_off = wl.rws_off;
+    // the instance table for this thread count
+    const int t = nt_index(plan.nt);
+    if (!(b->insts_written & (1 << t))) {
+      std::vector<qapk::InstArgs> h(b->count);
+      char* base = static_cast<char*>(b->data);
+      for (int i = 0; i < b->count; ++i)
+        h[i] = inst_args(b->di[i], base + b->offF[i], base + b->offFt[i], base + b->offD[i],
+                         plan.nt, b->fbytes);
+      QAP_CUDA(cudaMemcpy(b->d_insts + (size_t)t * b->count, h.data(),
+                          sizeof(qapk::InstArgs) * b->count, cudaMemcpyHostToDevice));
+      b->insts_written |= 1 << t;
+    }
     return QAP_OK;
   };
   QAP_TRY(shape_of(c.plan, &c.own));
   c.rows = c.own;
   if (c.plan.rot) QAP_TRY(shape_of(c.plan.rows(), &c.rows));
-  const WsLayout wl = ws_layout(c.plan, b->dbytes, b->fbytes, nmax, p);
-  c.ws_stride = wl.stride;
-  c.p_off = wl.p_off;
-  c.rws_off = wl.rws_off;
-  const int t = nt_index(c.plan.nt);
-  if (!(b->insts_written & (1 << t))) {
-    std::vector<qapk::InstArgs> h(b->count);
-    char* base = static_cast<char*>(b->data);
-    for (int i = 0; i < b->count; ++i)
-      h[i] = inst_args(b->di[i], base + b->offF[i], base + b->offFt[i],
-                       base + b->offD[i], c.plan.nt, b->fbytes);
-    QAP_CUDA(cudaMemcpy(b->d_insts + (size_t)t * b->count, h.data(),
-                        sizeof(qapk::InstArgs) * b->count, cudaMemcpyHostToDevice));
-    b->insts_written |= 1 << t;
-  }
   return QAP_OK;
 }
 
@@ -226,7 +231,7 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
     // the classes run together: walks of the whole batch fill the SMs
     const bool many = (int64_t)b->count * W >= 2 * (int64_t)b->sms;
     if (!search_plan(b->di[i].n, many, &b->di[i], 1, b->fbytes, b->dbytes, b->force64,
-                     b->smem_optin, 16, p, &plan_of[i]))
+                     b->smem_optin, 16, true, p, &plan_of[i]))
       return QAP_EUNSUPPORTED;
   }
   std::vector<int> order(b->count);
@@ -266,7 +271,7 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
     c.item_off = item_off;
     item_off += c.items;
     c.ws_off = ws_off;
-    ws_off += (c.ws_stride * c.own.grid + 255) / 256 * 256;
+    ws_off += (c.workspace() + 255) / 256 * 256;
     if (b->classes.size() > 1) {
       if (!c.side) QAP_CUDA(cudaStreamCreateWithFlags(&c.side, cudaStreamNonBlocking));
       if (!c.done) QAP_CUDA(cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming));
@@ -399,7 +404,7 @@ qap_status qap_plan(qap_ctx* ctx, const qap_search_params* params, qap_plan_info
   out->sms = ctx->sms;
   out->classes = 1;
   out->products = products_form(L.plan);
-  out->workspace = (L.plan.store & qapk::kGlobalDelta) != 0;
+  out->workspace = (L.plan.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
   return QAP_OK;
 }
 
@@ -657,16 +662,16 @@ qap_status qap_batch_plan(qap_batch* b, const qap_search_params* params, qap_pla
   QAP_TRY(dg.set(b->device));
   QAP_TRY(plan_classes(b, params));
   const BatchClass& c = b->classes.front();  // the class of the largest n
-  out->threads_per_walk = c.plan.nt;
   out->pairs_per_thread = c.plan.maxpt;
   const BatchClass::Shape& sh = c.shape(params);
+  out->threads_per_walk = sh.nt;
   out->smem_bytes = sh.smem;
   out->grid = sh.grid;
   out->ctas_per_sm = sh.ctas_per_sm;
   out->sms = b->sms;
   out->classes = (int32_t)b->classes.size();
   out->products = products_form(c.plan);
-  out->workspace = (c.plan.store & qapk::kGlobalDelta) != 0;
+  out->workspace = (c.plan.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
   return QAP_OK;
 }
 
@@ -699,11 +704,11 @@ qap_status qap_batch_classes(qap_batch* b, const qap_search_params* params,
     }
     o.instances = (int32_t)c.members.size();
     o.walks = c.items;
-    o.threads_per_walk = c.plan.nt;
     o.pairs_per_thread = c.plan.maxpt;
     o.products = products_form(c.plan);
-    o.workspace = (c.plan.store & qapk::kGlobalDelta) != 0;
     const BatchClass::Shape& sh = c.shape(params);
+    o.threads_per_walk = sh.nt;
+    o.workspace = (c.plan.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
     o.grid = sh.grid;
     o.ctas_per_sm = sh.ctas_per_sm;
     o.smem_bytes = sh.smem;
@@ -798,7 +803,13 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
         p = wide_store(p, dm.data(), (int)dm.size(), b->fbytes, b->dbytes, b->smem_optin, 16);
       else if (!fits(p))
         p.store |= qapk::kGlobalFlow;
-      if (fits(p)) cands.push_back(p);
+      if (fits(p)) {
+        cands.push_back(p);
+        const bool rows = b->force64 || uses_rule_tables(&tp) || tp.phase_x == QAP_PHASE_X_DOTS;
+        const Plan big =
+            rows ? p : with_big_rotation(p, dm.data(), (int)dm.size(), b->fbytes, fits);
+        if (big.rot) cands.push_back(big);
+      }
     }
     // items of this class, longest instances first; row bases for all
     const size_t items = rc.members.size() * (size_t)W;
@@ -821,9 +832,9 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       c.members = rc.members;
       if ((st = class_shape(b, c, W, &tp)) != QAP_OK) return fail(st);
       const BatchClass::Shape& sh = c.shape(&tp);
-      if ((st = grow(&b->ws, &b->ws_bytes, c.ws_stride * sh.grid)) != QAP_OK) return fail(st);
+      if ((st = grow(&b->ws, &b->ws_bytes, c.workspace())) != QAP_OK) return fail(st);
       qapk::BatchArgs a{};
-      a.insts = b->d_insts + (size_t)nt_index(c.plan.nt) * b->count;
+      a.insts = b->d_insts + (size_t)nt_index(sh.nt) * b->count;
       a.item_inst = d_items;
       a.item_walk = d_items + items;
       a.row_base = d_items + 2 * items;
@@ -831,16 +842,16 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       a.counter = counter;
       a.notr = sh.notr;
       a.s = make_search_args(&tp, &dout, b->nmax);
-      a.s.rws_off = c.rws_off;
-      a.s.p_off = c.p_off;
-      a.ws_stride = c.ws_stride;
-      a.ws = c.ws_stride ? static_cast<unsigned char*>(b->ws) : nullptr;
+      a.s.rws_off = sh.rws_off;
+      a.s.p_off = sh.p_off;
+      a.ws_stride = sh.ws_stride;
+      a.ws = sh.ws_stride ? static_cast<unsigned char*>(b->ws) : nullptr;
       const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(sh.fn));
       float ms = 0.f;
       for (int rep = 0; rep < 2; ++rep) {  // a warm-up run, then the timed one
         cudaMemsetAsync(counter, 0, sizeof(int), b->stream);
         if (rep) cudaEventRecord(t0, b->stream);
-        fn<<<sh.grid, c.plan.nt, sh.smem, b->stream>>>(a);
+        fn<<<sh.grid, sh.nt, sh.smem, b->stream>>>(a);
         if (rep) cudaEventRecord(t1, b->stream);
       }
       // a trial that did not launch would time as the fastest
@@ -862,7 +873,7 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       r.candidates = (int32_t)cands.size();
       r.threads_per_walk = best.nt;
       r.pairs_per_thread = best.maxpt;
-      r.workspace = (best.store & qapk::kGlobalDelta) != 0;
+      r.workspace = (best.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
       r.products = products_form(best);
       r.trial_ms = best_ms;
       r.rule_ms = rule_ms;
@@ -895,24 +906,24 @@ qap_status qap_batch_search_async(qap_batch* b, const qap_search_params* params,
     if (b->timing && !c.t0) QAP_CUDA(cudaEventCreate(&c.t0));
     if (b->timing && !c.t1) QAP_CUDA(cudaEventCreate(&c.t1));
     if (fork) QAP_CUDA(cudaStreamWaitEvent(cs, b->fork, 0));
+    const BatchClass::Shape& sh = c.shape(params);
     qapk::BatchArgs a{};
-    a.insts = b->d_insts + (size_t)nt_index(c.plan.nt) * b->count;
+    a.insts = b->d_insts + (size_t)nt_index(sh.nt) * b->count;
     a.item_inst = b->d_class_items + c.item_off;
     a.item_walk = b->d_class_items + total + c.item_off;
     a.row_base = b->d_class_items + 2 * total;
     a.items = c.items;
     a.counter = b->d_counter + k * kCounterStride;
-    const BatchClass::Shape& sh = c.shape(params);
     a.notr = sh.notr;
     a.s = make_search_args(params, out, p_stride);
-    a.s.rws_off = c.rws_off;
-    a.s.p_off = c.p_off;
-    a.ws_stride = c.ws_stride;
-    a.ws = c.ws_stride ? static_cast<unsigned char*>(b->ws) + c.ws_off : nullptr;
+    a.s.rws_off = sh.rws_off;
+    a.s.p_off = sh.p_off;
+    a.ws_stride = sh.ws_stride;
+    a.ws = sh.ws_stride ? static_cast<unsigned char*>(b->ws) + c.ws_off : nullptr;
     QAP_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(int), cs));
     const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(sh.fn));
     if (b->timing) QAP_CUDA(cudaEventRecord(c.t0, cs));
-    fn<<<sh.grid, c.plan.nt, sh.smem, cs>>>(a);
+    fn<<<sh.grid, sh.nt, sh.smem, cs>>>(a);
     QAP_CUDA(cudaGetLastError());
     if (b->timing) QAP_CUDA(cudaEventRecord(c.t1, cs));
     c.timed = b->timing != 0;

@@ -59,12 +59,15 @@ struct Plan {
   int maxpt;
   int store;  // qapk::kGlobalDelta, kGlobalFlow, kProductM, kGlobalP bits (0: all on chip)
   int rot = 0;  // rotation layout (qap_rotation.cuh): partner blocks per thread, 0 for rows
-  int row = 0;  // with rot: `store` of the row layout, for the searches that need it
+  int row = 0;  // with rot: `store` and threads of the row layout, for the
+  int row_nt = 0;  // searches that need it
 
   bool operator==(const Plan& o) const {
-    return nt == o.nt && maxpt == o.maxpt && store == o.store && rot == o.rot && row == o.row;
+    return nt == o.nt && maxpt == o.maxpt && store == o.store && rot == o.rot && row == o.row &&
+           row_nt == o.row_nt;
   }
-  Plan rows() const { return rot ? Plan{nt, maxpt, row} : *this; }
+  Plan rows() const { return rot ? Plan{row_nt, maxpt, row} : *this; }
+  int shape() const { return store & qapk::kGlobalM ? qapk::kRotBig : nt; }
 };
 
 // The large-n plan: 1024 threads, up to 40 slots each in a global workspace
@@ -142,18 +145,30 @@ struct DevInstance {
 // entries: at most (max D - min D) (A_r + A_s), with A_u the sum of |F[u][j]| +
 // |F[j][u]| over j.  g[u] lies between the sums of the products' lowest and
 // highest values.
-inline void rot_bounds(const int64_t* F, int n, int64_t loD, int64_t hiD, DevInstance* di) {
-  std::vector<int64_t> A(n, 0), pos(n, 0);  // sums of |F| and of F above 0
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) {
-      const int64_t f = F[(size_t)i * n + j], m = f < 0 ? -f : f;
-      A[i] += m;
-      A[j] += m;
-      if (f > 0) {
-        pos[i] += f;
-        pos[j] += f;
+inline void rot_bounds(const int64_t* F, int n, int64_t loF, int64_t loD, int64_t hiD,
+                       DevInstance* di) {
+  int64_t A[kMaxN] = {}, pos[kMaxN] = {};  // sums of |F| and of F above 0
+  for (int i = 0; i < n; ++i) {
+    const int64_t* Fi = F + (size_t)i * n;
+    int64_t row = 0, above = 0;
+    if (loF >= 0) {
+      for (int j = 0; j < n; ++j) {
+        row += Fi[j];
+        A[j] += Fi[j];
       }
+    } else {
+      for (int j = 0; j < n; ++j) {
+        const int64_t m = Fi[j] < 0 ? -Fi[j] : Fi[j], p = Fi[j] > 0 ? Fi[j] : 0;
+        row += m;
+        above += p;
+        A[j] += m;
+        pos[j] += p;
+      }
+      pos[i] += above;
     }
+    A[i] += row;
+  }
+  if (loF >= 0) std::copy(A, A + n, pos);
   int64_t a1 = 0, a2 = 0, lo = INT64_MAX, hi = INT64_MIN;
   for (int u = 0; u < n; ++u) {
     if (A[u] > a1) {
@@ -230,7 +245,7 @@ inline qap_status inspect_instance(const int64_t* F, const int64_t* D, int n, De
   // overflow here: on this branch the ranges fit int16 and int8)
   di->bytevec = !di->wide && mF <= 127 && hiF - loF <= 127 && hiD - loD <= 127;
   di->diff16 = !di->wide && hiF - loF <= 32767 && hiD - loD <= 127;
-  if (di->diff16) rot_bounds(F, n, loD, hiD, di);
+  if (di->diff16) rot_bounds(F, n, loF, loD, hiD, di);
   return QAP_OK;
 }
 
@@ -278,7 +293,7 @@ inline const void* pick_walk_kernel(int dbytes, int fbytes, const Plan& p) {
     if (fbytes == 1) return qapk::walk_kernel_i32_f8(p.nt, p.maxpt, p.store);
     return qapk::walk_kernel_i32_f16(p.nt, p.maxpt, p.store);
   };
-  return p.rot ? reinterpret_cast<const void*>(qapk::rot_kernel_of(fbytes, p.nt, p.rot))
+  return p.rot ? reinterpret_cast<const void*>(qapk::rot_kernel_of(fbytes, p.shape(), p.rot))
                : reinterpret_cast<const void*>(row());
 }
 
@@ -289,7 +304,7 @@ inline const void* pick_batch_kernel(int dbytes, int fbytes, const Plan& p) {
     if (fbytes == 1) return qapk::batch_kernel_i32_f8(p.nt, p.maxpt, p.store);
     return qapk::batch_kernel_i32_f16(p.nt, p.maxpt, p.store);
   };
-  return reinterpret_cast<const void*>(p.rot ? qapk::rot_kernel_of(fbytes, p.nt, p.rot) : row());
+  return reinterpret_cast<const void*>(p.rot ? qapk::rot_kernel_of(fbytes, p.shape(), p.rot) : row());
 }
 
 // A launch of walks of one instance by the kernel of pick_walk_kernel.
@@ -307,6 +322,8 @@ inline void launch_walks(const void* fn, const Plan& p, int grid, int smem, cuda
   b.walk_offset = a.walk_offset;
   b.starts = a.starts;
   b.inst = a.inst;
+  b.ws = a.ws;
+  b.ws_stride = a.ws_stride;
   reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(fn))<<<grid, p.nt, smem, stream>>>(b);
 }
 
@@ -317,7 +334,8 @@ inline int plan_smem(const Plan& p, const DevInstance* d, int count, int fbytes,
     for (int i = 0; i < count; ++i)
       smem = std::max(smem, qapk::rot_layout(d[i].n, d[i].ldF, fbytes, d[i].ldP, d[i].symF,
                                              d[i].symD, p.store & qapk::kNoTransposed,
-                                             qapk::rot_fixed_bytes(p.nt, fbytes))
+                                             p.store & qapk::kGlobalM,
+                                             qapk::rot_fixed_bytes(p.shape(), fbytes))
                                 .bytes);
     return smem;
   }
@@ -400,6 +418,32 @@ inline Plan with_rotation(Plan p, const DevInstance* d, int count, bool rows, Fi
     Plan q = p;
     q.rot = c;
     q.row = p.store;
+    q.row_nt = p.nt;
+    if (fits(q)) return q;
+    q.store |= qapk::kNoTransposed;
+    return fits(q) ? q : p;
+  }
+  return p;
+}
+
+// The rotation layout's large-n shape in place of the workspace plan, and of
+// the 1024-thread plans by dot products (int8 flows, 152 <= n <= 256): M in the
+// workspace, deltas in the registers of 512 threads.
+template <typename Fits>
+inline Plan with_big_rotation(Plan p, const DevInstance* d, int count, int fbytes, Fits fits) {
+  if (p.nt != 1024 || fbytes != 1 || (p.store & qapk::kProductM)) return p;
+  for (int i = 0; i < count; ++i)
+    if (!d[i].diff16 || !rot_fits_keys(d[i], qapk::kRotBig)) return p;
+  for (int c = 1; c <= qapk::kRotMaxC; ++c) {
+    bool holds = qapk::rot_compiled(qapk::kRotBig, c);
+    for (int i = 0; i < count; ++i) holds &= qapk::rot_chunks(d[i].n, qapk::kRotBig, c) > 0;
+    if (!holds) continue;
+    Plan q = p;
+    q.nt = 512;
+    q.store = qapk::kGlobalM;
+    q.rot = c;
+    q.row = p.store;
+    q.row_nt = p.nt;
     if (fits(q)) return q;
     q.store |= qapk::kNoTransposed;
     return fits(q) ? q : p;
@@ -414,7 +458,7 @@ inline bool rot_holds_tenures(const Plan& p, const qap_search_params* sp, int nm
   int tmax = sp->tenure.tmax;
   if (sp->tenure_per_n)
     tmax = std::max(std::max(1, sp->tenure.tmin * nmax / 100), (tmax * nmax + 99) / 100);
-  return qapk::rot_ring_holds(p.nt, tmax);
+  return qapk::rot_ring_holds(p.shape(), tmax);
 }
 
 // The int64 element path reads F and F^T from global memory (L1-cached,
@@ -492,9 +536,10 @@ inline bool uses_rule_tables(const qap_search_params* sp) {
 
 // The plan a search takes: choose_plan_fit's, in the rotation layout where
 // that applies and still lets two CTAs share an SM where the row layout does.
-// (Its tenures are another condition: rot_holds_tenures.)
+// (Its tenures are another condition: rot_holds_tenures.)  `workspace`: a plan
+// may use a workspace where the row layout has none.
 inline bool search_plan(int nmax, bool many, const DevInstance* d, int count, int fbytes,
-                        int dbytes, bool force64, int smem_optin, int reserve,
+                        int dbytes, bool force64, int smem_optin, int reserve, bool workspace,
                         const qap_search_params* sp, Plan* out) {
   if (!choose_plan_fit(nmax, sp->threads_per_walk, many, d, count, fbytes, dbytes, smem_optin,
                        reserve, sp->phase_x, out))
@@ -504,8 +549,11 @@ inline bool search_plan(int nmax, bool many, const DevInstance* d, int count, in
     return smem > smem_optin ? 0 : 2 * (smem + 1024) <= smem_optin + 1024 ? 2 : 1;
   };
   const int want = out->nt <= 256 ? ctas(*out) : 1;  // (above, registers hold one)
-  *out = with_rotation(*out, d, count, force64 || uses_rule_tables(sp),
-                       [&](const Plan& x) { return ctas(x) >= want; });
+  const bool rows = force64 || uses_rule_tables(sp);
+  auto fits = [&](const Plan& x) { return ctas(x) >= want; };
+  *out = with_rotation(*out, d, count, rows, fits);
+  if (workspace && !rows && sp->threads_per_walk == 0 && sp->phase_x == QAP_PHASE_X_AUTO)
+    *out = with_big_rotation(*out, d, count, fbytes, fits);
   return true;
 }
 
@@ -518,6 +566,8 @@ struct WsLayout {
 inline WsLayout ws_layout(const Plan& p, int dbytes, int fbytes, int nmax,
                           const qap_search_params* sp) {
   WsLayout w;
+  if (p.store & qapk::kGlobalM)
+    return WsLayout{0, 0, ((size_t)nmax * qapk::ld_m(nmax) * 4 + 255) / 256 * 256};
   w.p_off = delta_workspace(p, dbytes);
   w.rws_off = w.p_off + p_workspace(p, fbytes, nmax);
   w.stride = w.rws_off;

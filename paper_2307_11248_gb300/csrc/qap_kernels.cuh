@@ -145,6 +145,8 @@ constexpr int kGlobalP = 8;
 // in shared memory (room for M on large asymmetric instances): the few
 // transposed reads, at the start of a walk and in phase X, read columns.
 constexpr int kNoTransposed = 16;
+// The rotation layout's shape for large n: M in the CTA's workspace.
+constexpr int kGlobalM = 32;
 
 // row stride of M in int32 words: whole 16-byte groups, an odd number of
 // them (rows read side by side by consecutive threads spread over banks)

@@ -11,6 +11,7 @@ BatchKernelFn rot_f8_256w(int c);
 BatchKernelFn rot_f8_512(int c);
 BatchKernelFn rot_f8_512w(int c);
 BatchKernelFn rot_f8_1024(int c);
+BatchKernelFn rot_f8_big(int c);
 BatchKernelFn rot_f16_128(int c);
 BatchKernelFn rot_f16_256(int c);
 BatchKernelFn rot_f16_256w(int c);
@@ -20,6 +21,7 @@ BatchKernelFn rot_f16_1024(int c);
 
 BatchKernelFn rot_kernel_of(int fbytes, int nt, int c) {
   const bool w = c >= 5;
+  if (nt == kRotBig) return fbytes == 1 ? rot_f8_big(c) : nullptr;
   if (fbytes == 1)
     return nt == 128   ? rot_f8_128(c)
            : nt == 256 ? (w ? rot_f8_256w(c) : rot_f8_256(c))

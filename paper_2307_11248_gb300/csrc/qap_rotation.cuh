@@ -52,6 +52,10 @@
 // walks x 1000 each, 103.4 -> 38.6 ms; their costs need 64 bits, their deltas
 // do not: the rows' sums of |F| bound them (rot_bounds), where the row layout
 // holds every delta as wide as the cost.
+// Large n (M in the workspace, two dp4a words of pending moves): n = 256 grid,
+// 64 walks x (2opt + 1000) 21.7 -> 7.0 ms, n = 203 asymmetric, 48 walks x 1000
+// 15.7 -> 4.2 ms against the workspace plan, that keeps deltas and marks in L2
+// and recomputes dot products; 24 requests of n = 12-256 24.5 -> 6.8 ms.
 // Tried and slower: every warp holding pairs and phase X on some of them
 // (n = 100 2.33 against 1.44 us per iteration of two walks per SM); tabu times
 // checked by each thread through its earliest (0.3 us per iteration on the
@@ -62,28 +66,48 @@
 
 namespace qapk {
 
+// A shape: the threads of a CTA, or kRotBig, the one of 512 threads for large
+// n, where M does not fit shared memory and lies in the CTA's workspace (L2).
+constexpr int kRotBig = 513;
+__host__ __device__ constexpr bool rot_big(int nt) { return nt == kRotBig; }
+__host__ __device__ constexpr int rot_threads(int nt) { return rot_big(nt) ? 512 : nt; }
+
 // Threads that may hold pairs: the same number of warps on each of an SM's
 // four schedulers (from 256 threads).
-__host__ __device__ constexpr int rot_owners(int nt) { return nt == 1024 ? 768 : nt / 2; }
+__host__ __device__ constexpr int rot_owners(int nt) {
+  return rot_big(nt) ? 384 : nt == 1024 ? 768 : nt / 2;
+}
 
-// Indices, with a phantom, that a thread count holds at most.
-__host__ __device__ constexpr int rot_max_n(int nt) { return nt == 128 ? 64 : nt == 256 ? 128 : 192; }
+// Indices per phase X thread.
+__host__ __device__ constexpr int rot_kx(int nt) { return rot_big(nt) ? 2 : 1; }
+
+// Phase X threads: whole warps.
+__host__ __device__ constexpr int rot_px(int n, int nt) {
+  return (n + 32 * rot_kx(nt) - 1) / (32 * rot_kx(nt)) * 32;
+}
+
+// Indices, with a phantom, that a shape holds at most.
+__host__ __device__ constexpr int rot_max_n(int nt) {
+  return rot_big(nt) ? 256 : nt == 128 ? 64 : nt == 256 ? 128 : 192;
+}
 
 // Threads per block of two (J) at c partner blocks each: the fewest that hold
-// every pair; 0 when nt threads do not hold n (its pairs, or its indices).
+// every pair; 0 when the shape does not hold n (its pairs, or its indices).
 __host__ __device__ inline int rot_chunks(int n, int nt, int c) {
   const int n2 = (n + 1) / 2, j = (n2 / 2 + c - 1) / c;
   return n >= 3 && n <= rot_max_n(nt) && j * n2 <= rot_owners(nt) &&
-                 (n + 31) / 32 * 32 <= nt - rot_owners(nt) && j * c <= n2 - 1
+                 rot_px(n, nt) <= rot_threads(nt) - rot_owners(nt) && j * c <= n2 - 1
              ? j
              : 0;
 }
 
 // Low bits S of a scan candidate.  Up to 256 threads (n <= 128) they are the
-// partner itself; beyond, its rank in the thread's window (at most 31), with
-// 32 on top before the circle's wrap, half an addition more per pair.
+// partner itself; beyond, its rank in the thread's window, below the top bit,
+// that is set before the circle's wrap: half an addition more per pair.
 __host__ __device__ constexpr bool rot_rank(int nt) { return nt >= 512; }
-__host__ __device__ constexpr int rot_key_bits(int nt) { return rot_rank(nt) ? 6 : 7; }
+__host__ __device__ constexpr int rot_key_bits(int nt) {
+  return rot_rank(nt) && !rot_big(nt) ? 6 : 7;
+}
 
 // Ends of tabu times that lie ahead are kept in a ring of this many
 // iterations; searches with longer tenures take the row layout.
@@ -91,6 +115,18 @@ __host__ __device__ constexpr int rot_ring(int nt) { return nt <= 256 ? 256 : 51
 __host__ __device__ inline bool rot_ring_holds(int nt, int tmax) {
   return tmax <= rot_ring(nt) - 2;
 }
+
+// Pending moves of M: words of 32 bits per row and per column, and the moves
+// they hold (symmetric instances twice as many): one dp4a takes 2 asymmetric
+// moves of int8 flows, one dp2a 1 of int16 flows.  Large n keeps two dp4a
+// words: half the traffic with M.
+template <int NT, typename FE>
+struct RotPending {
+  static constexpr int RW = sizeof(FE) == 2 || rot_big(NT) ? 2 : 1;
+  static constexpr int LW = sizeof(FE) == 1 ? RW : 1;
+  template <bool SYM>
+  static constexpr int Q = (rot_big(NT) ? 4 : 2) * (SYM ? 2 : 1);
+};
 
 // Barrier of the CTA; the warps of each role reach it from their own code.
 __device__ __forceinline__ void rot_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
@@ -104,6 +140,7 @@ struct RotWalkArgs {
   const int32_t* start;
   int row, notr;
   uint32_t wid;
+  int32_t* M;      // large n: M in the workspace
 };
 constexpr int kRotArgsBytes = (sizeof(RotWalkArgs) + 15) / 16 * 16;
 
@@ -130,14 +167,15 @@ struct RotFixed {
   static constexpr int sigma = own + 4 * W * NE;
   static constexpr int p0 = sigma + 4 * NE;
   // pending operands of M's update (two buffers, by the move's parity): rows
-  // by index (W words), columns by label
+  // by index (RW words), columns by label (LW)
   static constexpr int NW = NE + 4;  // ld_m(n) at most
+  static constexpr int RW = RotPending<NT, FE>::RW, LW = RotPending<NT, FE>::LW;
   static constexpr int vw = p0 + 4 * NE;
-  static constexpr int vwu = vw + 8 * W * NW;
+  static constexpr int vwu = vw + 8 * RW * NW;
   // ring: the pairs whose tabu time ends at iteration i, at i mod its length:
   // key of the first in the low half, node of the rest in the high half;
   // nodes: such words moved aside, at the iteration that moved them
-  static constexpr int ring = vwu + 8 * NW;
+  static constexpr int ring = vwu + 8 * LW * NW;
   static constexpr int node = ring + 4 * rot_ring(NT);
   // tenures of the iterations, at (it - 1) mod 64
   static constexpr int ten = node + 4 * rot_ring(NT);
@@ -156,17 +194,17 @@ struct RotLayout {
 
 // notr: no transposed copies of F and P (kNoTransposed plans)
 __host__ __device__ inline RotLayout rot_layout(int n, int ldF, int fbytes, int ldP, int symF,
-                                                int symD, int notr, int fixed) {
+                                                int symD, int notr, int big, int fixed) {
   RotLayout L;
   int o = fixed;
   L.F = o;    o = align16(o + n * ldF * fbytes);
   L.Ft = o;   o = (symF || notr) ? o : align16(o + n * ldF * fbytes);
   L.P = o;    o = align16(o + n * ldP);
   L.Pt = o;   o = (symD || notr) ? o : align16(o + n * ldP);
-  L.M = o;    o = align16(o + n * ld_m(n) * 4);
-  // one word more: the thread of k = r reads past the triangle's end at
+  L.M = o;    o = big ? o : align16(o + n * ld_m(n) * 4);
+  // one entry more: the thread of k = r reads past the triangle's end at
   // r = n - 1 (and drops it)
-  L.mark = o; o = align16(o + (n * (n - 1) / 2 + 1) * 4);
+  L.mark = o; o = align16(o + (n * (n - 1) / 2 + 1) * (big ? 2 : 4));
   L.bytes = o;
   return L;
 }
@@ -176,6 +214,7 @@ __host__ __device__ inline int rot_fixed_of(int nt) {
   return nt == 128   ? RotFixed<128, FE>::bytes
          : nt == 256 ? RotFixed<256, FE>::bytes
          : nt == 512 ? RotFixed<512, FE>::bytes
+         : rot_big(nt) ? RotFixed<kRotBig, FE>::bytes
                      : RotFixed<1024, FE>::bytes;
 }
 __host__ __device__ inline int rot_fixed_bytes(int nt, int fbytes) {
@@ -197,7 +236,7 @@ struct RotSmem {
   int ft, pt;          // offsets that F^T and P0^T are read from:
   int fr, fk, pr, pk;  // entry [r][k] at r fr + k fk
   __device__ __forceinline__ RotSmem(const InstArgs& I, int n, bool notr) {
-    L = rot_layout(n, I.ldF, sizeof(FE), I.ldP, I.symF, I.symD, notr, X_::bytes);
+    L = rot_layout(n, I.ldF, sizeof(FE), I.ldP, I.symF, I.symD, notr, rot_big(NT), X_::bytes);
     ft = I.symF || notr ? L.F : L.Ft;
     pt = I.symD || notr ? L.P : L.Pt;
     // without copies F^T is read from F's columns
@@ -212,8 +251,10 @@ struct RotSmem {
   __device__ __forceinline__ int8_t* P() const { return rot_at<int8_t>(L.P); }  // P0 = D[p0][p0]
   __device__ __forceinline__ int8_t* Pt() const { return rot_at<int8_t>(pt); }
   // M[x][label], halved on symmetric instances
-  __device__ __forceinline__ int32_t* M() const { return rot_at<int32_t>(L.M); }
-  // tabu_until of pair u < v at v (v - 1) / 2 + u
+  __device__ __forceinline__ int32_t* M() const {
+    return rot_big(NT) ? args().M : rot_at<int32_t>(L.M);
+  }
+  // tabu_until of pair u < v at v (v - 1) / 2 + u (large n: see rot_mark16)
   __device__ __forceinline__ int32_t* mark() const { return rot_at<int32_t>(L.mark); }
   __device__ __forceinline__ static int32_t* X() { return rot_at<int32_t>(X_::X); }
   __device__ __forceinline__ static int32_t* X2() { return rot_at<int32_t>(X_::X2); }
@@ -288,8 +329,7 @@ struct RotThread {
   int role;         // of the thread's warp: 0 holds pairs, 1 phase X, 2 helps with M
   int m;            // role 0: block of two that the thread holds
   int pb, pbm;      // role 0: first partner block, as position and mod n2
-  int k;            // role 1: index (past the last: a repeat of n - 1 that stores nothing)
-  bool live;        // role 1: the index is the thread's own
+  int pt, pxt;      // role 1: the thread among phase X's, their number
   int ow;           // warps with role 0
   int ug, ux, urows;  // roles 1, 2: column group and first row of M, rows at once
 };
@@ -308,14 +348,13 @@ __device__ __forceinline__ RotThread rot_thread(int n) {
   t.pb = t.m + 1 + j * C;
   t.pbm = t.pb < t.n2 ? t.pb : t.pb - t.n2;
   t.ow = (J * t.n2 + 31) / 32;
-  const int k = tid - rot_owners(NT);
-  t.live = k >= 0 && k < n;
-  t.k = k < n ? k : n - 1;
-  t.role = tid < 32 * t.ow ? 0 : k >= 0 && k < (n + 31) / 32 * 32 ? 1 : 2;
+  t.pt = tid - rot_owners(NT);
+  t.pxt = rot_px(n, NT);
+  t.role = tid < 32 * t.ow ? 0 : t.pt >= 0 && t.pt < t.pxt ? 1 : 2;
   const int gpr = ld_m(n) / 4, f = tid - 32 * t.ow;
   t.ug = f % gpr;
   t.ux = f / gpr;
-  t.urows = (NT - 32 * t.ow) / gpr;
+  t.urows = (rot_threads(NT) - 32 * t.ow) / gpr;
   return t;
 }
 
@@ -371,6 +410,51 @@ __device__ __forceinline__ void sts128(uint32_t at, int4 v) {
                : "memory");
 }
 
+__device__ __forceinline__ int lds16u(uint32_t at) {
+  int v;
+  asm volatile("{.reg .b16 t; ld.shared.u16 t, [%1]; cvt.u32.u16 %0, t;}"
+               : "=r"(v)
+               : "r"(at)
+               : "memory");
+  return v;
+}
+// A tabu time's end in 16 bits: 0 for a pair that is not tabu.
+__device__ __forceinline__ int rot_mark16(int end) { return (end & 0x7fff) | 0x8000; }
+// Entries of M at byte offset `at`: in shared memory, or (large n) in the
+// workspace, past L1.
+template <int NT>
+__device__ __forceinline__ int ldm32(const char* g, uint32_t at) {
+  if constexpr (rot_big(NT)) {
+    int v;
+    asm volatile("ld.global.cg.b32 %0, [%1];" : "=r"(v) : "l"(g + at) : "memory");
+    return v;
+  } else {
+    return lds32(at);
+  }
+}
+template <int NT>
+__device__ __forceinline__ int4 ldm128(const char* g, uint32_t at) {
+  if constexpr (rot_big(NT)) {
+    int4 v;
+    asm volatile("ld.global.cg.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(g + at)
+                 : "memory");
+    return v;
+  } else {
+    return lds128(at);
+  }
+}
+template <int NT>
+__device__ __forceinline__ void stm128(char* g, uint32_t at, int4 v) {
+  if constexpr (rot_big(NT))
+    asm volatile("st.global.cg.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(g + at), "r"(v.x),
+                 "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+  else
+    sts128(at, v);
+}
+
 __device__ __forceinline__ uint32_t pack2(int h0, int h1) {
   return __byte_perm((uint32_t)h0, (uint32_t)h1, 0x5410u);
 }
@@ -391,7 +475,7 @@ __device__ __forceinline__ void rot_compute_m(const RotSmem<NT, FE>& S, int n, i
   using QV = typename C::QV;
   const int nc = (n + C::W - 1) / C::W, ldm = ld_m(n);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int x0 = 4 * warp; x0 < n; x0 += NT / 8) {
+  for (int x0 = 4 * warp; x0 < n; x0 += rot_threads(NT) / 8) {
     const int xm = n - 1;
     const int x1 = min(x0 + 1, xm), x2 = min(x0 + 2, xm), x3 = min(x0 + 3, xm);
     for (int k = lane; k < n; k += 32) {
@@ -434,12 +518,13 @@ __device__ __forceinline__ void rot_compute_m(const RotSmem<NT, FE>& S, int n, i
   }
 }
 
-// The marks, after the pairs' warps have taken the table from their place;
-// by the other warps.
+// The marks, after the pairs' warps have taken the table from their place (or
+// made it); by the other warps.
 template <int NT>
 __device__ __forceinline__ void rot_clear_marks(int32_t* mark, int n, int ow) {
   rot_barrier();
-  for (int x = (int)threadIdx.x - 32 * ow; x < n * (n - 1) / 2; x += NT - 32 * ow) mark[x] = 0;
+  const int words = rot_big(NT) ? (n * (n - 1) / 2 + 1) / 2 : n * (n - 1) / 2;
+  for (int x = (int)threadIdx.x - 32 * ow; x < words; x += rot_threads(NT) - 32 * ow) mark[x] = 0;
 }
 
 // Tenure of iteration it (from 1).
@@ -460,52 +545,64 @@ struct RotTenure {
   }
 };
 
-// M[x][.] after a move, for the rows x = slot mod Q: one dp4a per entry (int16
-// flows: two dp2a) with the pending words, a group of 4 columns of every
-// urows-th such row per thread, 4 rows in flight.
-template <int Q, int W>
-__device__ __forceinline__ void rot_update_m(const RotThread& T, uint32_t aM, uint32_t aVw,
-                                             uint32_t aVwu, int n, int ldm, int slot) {
+// An entry of M with its pending moves: row words, column words.
+template <int NT, typename FE>
+__device__ __forceinline__ int rot_entry(int2 w, int2 u, int m) {
+  using P = RotPending<NT, FE>;
+  if constexpr (P::RW == 1) return __dp4a(w.x, u.x, m);
+  else if constexpr (P::LW == 2) return __dp4a(w.y, u.y, __dp4a(w.x, u.x, m));
+  else return __dp2a_hi(w.y, u.x, __dp2a_lo(w.x, u.x, m));
+}
+
+// M[x][.] after a move, for the rows x = slot mod Q, with the pending words:
+// a group of 4 columns of every urows-th such row per thread, 4 rows (large n:
+// 8) in flight.
+template <int NT, int Q, typename FE>
+__device__ __forceinline__ void rot_update_m(const RotThread& T, char* gM, uint32_t aM,
+                                             uint32_t aVw, uint32_t aVwu, int n, int ldm,
+                                             int slot) {
+  using P = RotPending<NT, FE>;
+  constexpr int B = rot_big(NT) ? 8 : 4;
   if (T.ux >= T.urows) return;
-  const int4 w = lds128(aVwu + 16 * T.ug);
+  int4 w, w2 = make_int4(0, 0, 0, 0);
+  if constexpr (P::LW == 1) {
+    w = lds128(aVwu + 16 * T.ug);
+  } else {
+    const int4 a = lds128(aVwu + 32 * T.ug), b = lds128(aVwu + 32 * T.ug + 16);
+    w = make_int4(a.x, a.z, b.x, b.z);
+    w2 = make_int4(a.y, a.w, b.y, b.w);
+  }
   const int step = Q * T.urows;
   auto upd = [&](int2 u, int4 v) {
-    if constexpr (W == 1) {
-      v.x = __dp4a(u.x, w.x, v.x);
-      v.y = __dp4a(u.x, w.y, v.y);
-      v.z = __dp4a(u.x, w.z, v.z);
-      v.w = __dp4a(u.x, w.w, v.w);
-    } else {
-      v.x = __dp2a_hi(u.y, w.x, __dp2a_lo(u.x, w.x, v.x));
-      v.y = __dp2a_hi(u.y, w.y, __dp2a_lo(u.x, w.y, v.y));
-      v.z = __dp2a_hi(u.y, w.z, __dp2a_lo(u.x, w.z, v.z));
-      v.w = __dp2a_hi(u.y, w.w, __dp2a_lo(u.x, w.w, v.w));
-    }
+    v.x = rot_entry<NT, FE>(u, make_int2(w.x, w2.x), v.x);
+    v.y = rot_entry<NT, FE>(u, make_int2(w.y, w2.y), v.y);
+    v.z = rot_entry<NT, FE>(u, make_int2(w.z, w2.z), v.z);
+    v.w = rot_entry<NT, FE>(u, make_int2(w.w, w2.w), v.w);
     return v;
   };
-  auto word = [&](uint32_t at) {
-    if constexpr (W == 1) return make_int2(lds32(at), 0);
-    else return lds64(at);
-  };
   uint32_t am = aM + 16 * T.ug + 4 * ldm * (slot + Q * T.ux);
-  uint32_t av = aVw + 4 * W * (slot + Q * T.ux);
-  const uint32_t sm = 4 * ldm * step, sv = 4 * W * step;
+  uint32_t av = aVw + 4 * P::RW * (slot + Q * T.ux);
+  const uint32_t sm = 4 * ldm * step, sv = 4 * P::RW * step;
 #pragma unroll 1
-  for (int x = slot + Q * T.ux; x < n; x += 4 * step) {
+  for (int x = slot + Q * T.ux; x < n; x += B * step) {
     // rows past the last repeat the first: the same entry, loaded before it
     // is stored, takes the same value again
-    const uint32_t m1 = x + step < n ? sm : 0, m2 = x + 2 * step < n ? 2 * sm : 0;
-    const uint32_t m3 = x + 3 * step < n ? 3 * sm : 0;
-    const uint32_t v1 = x + step < n ? sv : 0, v2 = x + 2 * step < n ? 2 * sv : 0;
-    const uint32_t v3 = x + 3 * step < n ? 3 * sv : 0;
-    const int4 a0 = lds128(am), a1 = lds128(am + m1), a2 = lds128(am + m2), a3 = lds128(am + m3);
-    const int2 b0 = word(av), b1 = word(av + v1), b2 = word(av + v2), b3 = word(av + v3);
-    sts128(am, upd(b0, a0));
-    sts128(am + m1, upd(b1, a1));
-    sts128(am + m2, upd(b2, a2));
-    sts128(am + m3, upd(b3, a3));
-    am += 4 * sm;
-    av += 4 * sv;
+    int4 a[B];
+    int2 b[B];
+    uint32_t at[B];
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      const bool in = x + i * step < n;
+      at[i] = am + (in ? i * sm : 0);
+      a[i] = ldm128<NT>(gM, at[i]);
+      const uint32_t ab = av + (in ? i * sv : 0);
+      if constexpr (P::RW == 1) b[i] = make_int2(lds32(ab), 0);
+      else b[i] = lds64(ab);
+    }
+#pragma unroll
+    for (int i = 0; i < B; ++i) stm128<NT>(gM, at[i], upd(b[i], a[i]));
+    am += B * sm;
+    av += B * sv;
   }
 }
 
@@ -520,6 +617,19 @@ __device__ __forceinline__ void clear_tabu(int (&d)[NS], int q, int big) {
 #pragma unroll
     for (int i = LO; i < HI; ++i) d[i] -= q == i ? big : 0;
   }
+}
+
+// A pair's entry of the table at the start of a walk: M[u][v] + M[v][u] + the
+// 2x2 term of Eq. 2, less twice g's mid-range.
+template <int NT, typename FE>
+__device__ __forceinline__ int rot_pair(const RotSmem<NT, FE>& S, const InstArgs& I, int u, int v) {
+  const int ldF = I.ldF, ldP = I.ldP, ldm = ld_m(I.n);
+  const FE* F = S.F();
+  const int8_t* P = S.P();
+  const int32_t* M = S.M();
+  const int f = (int)F[u * ldF + u] - F[u * ldF + v] - F[v * ldF + u] + F[v * ldF + v];
+  const int p = (int)P[u * ldP + u] - P[u * ldP + v] - P[v * ldP + u] + P[v * ldP + v];
+  return ((M[u * ldm + v] + M[v * ldm + u]) << (I.symF && I.symD ? 1 : 0)) + f * p - 2 * I.g0;
 }
 
 // The warps that hold pairs: the table, its update after each move, and the
@@ -538,21 +648,30 @@ __device__ __forceinline__ void rot_owner() {
   constexpr bool RANK = rot_rank(NT);
   constexpr int SB = rot_key_bits(NT);
   constexpr uint32_t MUL = 1u << SB;
+  constexpr int TOP = (int)(MUL / 2);  // with RANK: on the partners before the wrap
+  static_assert(!RANK || 2 * C < TOP, "ranks fit below the top bit");
   constexpr int BIG = 1 << (31 - SB);  // on top of a tabu pair's d
   constexpr int NS = 4 * C + 1;        // slots; the last holds the pair inside the block
 
-  // the table, from where rot_start left it
+  // the table: from where rot_start left it, or (large n) by the pairs
   int32_t* const mark = S(I, n, W.notr != 0).mark();
   int d[NS];
   auto d_init = [&](int u, int v) -> int {
-    const int hi = max(u, v);
-    return hi < n ? mark[hi * (hi - 1) / 2 + min(u, v)] : 0;
+    const int hi = max(u, v), lo = min(u, v);
+    if (hi >= n) return 0;
+    if constexpr (rot_big(NT)) return rot_pair(S(I, n, W.notr != 0), I, lo, hi);
+    else return mark[hi * (hi - 1) / 2 + lo];
   };
 #pragma unroll
   for (int i = 0; i < C; ++i) {
     const int b = T.pb + i < n2 ? T.pb + i : T.pb + i - n2;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) d[4 * i + q] = d_init(v0 + (q >> 1), 2 * b + (q & 1));
+    for (int q = 0; q < 4; ++q) {
+      d[4 * i + q] = d_init(v0 + (q >> 1), 2 * b + (q & 1));
+      // large n: one after the other (together they take more registers
+      // than the iterations have)
+      if constexpr (rot_big(NT)) asm volatile("" : "+r"(d[4 * i + q])::"memory");
+    }
   }
   d[4 * C] = d_init(v0, v1);
   rot_barrier();  // the others now clear the marks
@@ -571,7 +690,7 @@ __device__ __forceinline__ void rot_owner() {
 #pragma unroll
     for (int i = 0; i < C; ++i) {
       const int2 y = psi[T.pb + i];
-      const uint32_t y0 = (uint32_t)y.x + (RANK ? 2 * i + 1 : 0);
+      const uint32_t y0 = (uint32_t)y.x + (RANK ? 2 * i + 1 : 0);  // (the pair inside: rank 0)
       const uint32_t y1 = (uint32_t)y.y + (RANK ? 2 * i + 2 : 0);
       const uint32_t e00 = (uint32_t)d[4 * i] * MUL + y0;
       const uint32_t e01 = (uint32_t)d[4 * i + 1] * MUL + y1;
@@ -590,8 +709,8 @@ __device__ __forceinline__ void rot_owner() {
     }
     // delta 2^S + index of each row's best, by the own index's psi: q is
     // 2^30 less g[v]
-    const uint32_t q0 = (uint32_t)o.x - (RANK ? 32 : v0) + 0x80000000u;
-    const uint32_t q1 = (uint32_t)o.y - (RANK ? 32 : v1) + 0x80000000u;
+    const uint32_t q0 = (uint32_t)o.x - (RANK ? TOP : v0) + 0x80000000u;
+    const uint32_t q1 = (uint32_t)o.y - (RANK ? TOP : v1) + 0x80000000u;
     const int ls = (int)((uint32_t)lim * MUL);
     int c0 = m0 < 0 ? (int)((uint32_t)m0 + q0) : INT_MAX;
     int c1 = m1 < 0 ? (int)((uint32_t)m1 + q1) : INT_MAX;
@@ -603,10 +722,10 @@ __device__ __forceinline__ void rot_owner() {
     const int d0 = c0 >> SB, d1 = c1 >> SB;
     int u0 = c0 & (int)(MUL - 1), u1 = c1 & (int)(MUL - 1);
     if (RANK) {
-      u0 = (u0 & 31) + 2 * T.pb - 1;
+      u0 = (u0 & (TOP - 1)) + 2 * T.pb - 1;
       u0 = u0 >= nE ? u0 - nE : u0;
-      u0 = (c0 & 31) == 0 ? v1 : u0;
-      u1 = (u1 & 31) + 2 * T.pb - 1;
+      u0 = (c0 & (TOP - 1)) == 0 ? v1 : u0;
+      u1 = (u1 & (TOP - 1)) + 2 * T.pb - 1;
       u1 = u1 >= nE ? u1 - nE : u1;
     }
     const uint32_t k0 = (uint32_t)(min(u0, v0) << 8 | max(u0, v0));
@@ -640,7 +759,10 @@ __device__ __forceinline__ void rot_owner() {
       int q = 4 * kx + (own_u ? 2 * (u & 1) + (v & 1) : 2 * (v & 1) + (u & 1));
       q = bu == bv ? 4 * C : q;
       // (applied again since: its end is another)
-      const bool ends = mark[v * (v - 1) / 2 + u] == it + 1;
+      const int at = v * (v - 1) / 2 + u;
+      const bool ends = rot_big(NT) ? reinterpret_cast<const uint16_t*>(mark)[at] ==
+                                          rot_mark16(it + 1)
+                                    : mark[at] == it + 1;
       const bool hold = ends && (own_u || m == bv) && (kx < C || bu == bv);
       for (unsigned b = __ballot_sync(kFull, hold); b; b &= b - 1) {
         const int src = __ffs(b) - 1;
@@ -727,8 +849,8 @@ __device__ __forceinline__ void rot_owner() {
   }
 }
 
-// The phase X warps: one thread per index k computes what move (r, s) changes
-// (see phase_m_prep for the algebra), and keeps the labels, the pending words,
+// The phase X warps: one thread per index k (large n: two indices) computes what
+// move (r, s) changes (see phase_m_prep for the algebra), and keeps the labels, the pending words,
 // the tabu times and the walk's results.
 //
 // M's rows are brought up to date in turn, those with x mod Q = t mod Q after
@@ -737,10 +859,14 @@ __device__ __forceinline__ void rot_owner() {
 // its entries' correction is one dp4a whatever the row's place in the turn.
 template <int NT, int C, bool SYM, typename FE>
 __device__ __forceinline__ void rot_phase_x() {
-  constexpr int FB = sizeof(FE), PW = kRotWords<FE>;
-  constexpr int Q = SYM ? 4 : 2;
+  constexpr int FB = sizeof(FE), KX = rot_kx(NT);
+  constexpr bool PW2 = kRotWords<FE> == 2;
+  using P = RotPending<NT, FE>;
+  constexpr int RW = P::RW, LW = P::LW, Q = P::template Q<SYM>;
+  constexpr bool M16 = rot_big(NT);
   constexpr int SB = rot_key_bits(NT);
   constexpr int BIG = 1 << (31 - SB);
+  constexpr int TOP = 1 << (SB - 1);
   using X_ = RotFixed<NT, FE>;
   const RotWalkArgs& W = RotSmem<NT, FE>::args();
   const InstArgs& I = W.I;
@@ -751,23 +877,33 @@ __device__ __forceinline__ void rot_phase_x() {
   const uint32_t wid = W.wid;
   const uint64_t seed = W.s.seed;
   int32_t* const fq = W.s.freq ? W.s.freq + (size_t)W.row * W.s.p_stride * W.s.p_stride : nullptr;
-  const int k = T.k;
   const int lane = threadIdx.x & 31;
-  const bool live = T.live, first = k < 32;  // first: the first warp, that keeps the tabu times
+  const bool first = T.pt < 32;  // the first warp, that keeps the tabu times
   // addresses
   const uint32_t base = smem_addr(rot_smem);
-  const uint32_t aF = base + S.L.F, aP = base + S.L.P, aM = base + S.L.M;
+  const uint32_t aF = base + S.L.F, aP = base + S.L.P, aM = rot_big(NT) ? 0 : base + S.L.M;
   const uint32_t aFt = base + S.ft, aPt = base + S.pt, aMark = base + S.L.mark;
   const uint32_t aVw = base + X_::vw, aVwu = base + X_::vwu, aSig = base + X_::sigma;
   const uint32_t aX = base + X_::X, aPsi = base + X_::psi, aOwn = base + X_::own;
   const uint32_t aR = base + X_::R, aTen = base + X_::ten;
-  const uint32_t oMk = aM + 4 * ldm * k;
-  const int ktri = k * (k - 1) / 2;
-  int uk = k, best_uk = k, best_iter = 0, mv = 0;
-  int2 wk = make_int2(0, 0);  // the pending word(s) of row k
-  const int Fkk = S.F()[k * ldF + k];
-  int Qkk = S.P()[k * ldP + k];
-  int gk = (S.M()[k * ldm + k] << (SYM ? 1 : 0)) - g0;
+  char* const gM = reinterpret_cast<char*>(W.M);
+  // per index of the thread (past the last: a repeat of n - 1 that stores
+  // nothing)
+  int k[KX], uk[KX], best_uk[KX], Fkk[KX], Qkk[KX], gk[KX];
+  int2 wk[KX];  // the pending word(s) of row k
+  bool live[KX];
+#pragma unroll
+  for (int j = 0; j < KX; ++j) {
+    const int kj = T.pt + j * T.pxt;
+    live[j] = kj < n;
+    k[j] = min(kj, n - 1);
+    uk[j] = best_uk[j] = k[j];
+    wk[j] = make_int2(0, 0);
+    Fkk[j] = S.F()[k[j] * ldF + k[j]];
+    Qkk[j] = S.P()[k[j] * ldP + k[j]];
+    gk[j] = (S.M()[k[j] * ldm + k[j]] << (SYM ? 1 : 0)) - g0;
+  }
+  int best_iter = 0, mv = 0;
   const RotTenure tenure(W.s, n);
   const uint64_t h0 = 14695981039346656037ull;
   uint64_t h = h0, dh = h0;
@@ -785,135 +921,174 @@ __device__ __forceinline__ void rot_phase_x() {
     const int rd = (mv & 1) * 4 * ldm, wt = 4 * ldm - rd;  // this move's buffers
     const int done = (mv - 1) & (Q - 1);                   // rows finished after the last move
     auto pending = [&](int x) {
-      int2 w = make_int2(lds32(aVw + PW * rd + 4 * PW * x), 0);
-      if constexpr (PW == 2) w.y = lds32(aVw + PW * rd + 4 * PW * x + 4);
+      int2 w = make_int2(lds32(aVw + RW * rd + 4 * RW * x), 0);
+      if constexpr (RW == 2) w.y = lds32(aVw + RW * rd + 4 * RW * x + 4);
       return (x & (Q - 1)) == done ? make_int2(0, 0) : w;
     };
-    // an entry of M less what is pending: row word(s), label word
-    auto entry = [&](int2 w, int u, int m) {
-      if constexpr (PW == 1) return __dp4a(w.x, u, m);
-      else return __dp2a_hi(w.y, u, __dp2a_lo(w.x, u, m));
+    auto column = [&](int u) {
+      int2 w = make_int2(lds32(aVwu + LW * rd + 4 * LW * u), 0);
+      if constexpr (LW == 2) w.y = lds32(aVwu + LW * rd + 4 * LW * u + 4);
+      return w;
     };
+    // M's entries first: with large n they come from L2
+    int Ar[KX], As[KX], Bs[KX], Br[KX];
+#pragma unroll
+    for (int j = 0; j < KX; ++j) {
+      const uint32_t oMk = aM + 4 * ldm * k[j], u4 = 4 * (uint32_t)uk[j];
+      Ar[j] = ldm32<NT>(gM, oMr + u4);
+      As[j] = ldm32<NT>(gM, oMs + u4);
+      Bs[j] = ldm32<NT>(gM, oMk + 4 * us);
+      Br[j] = ldm32<NT>(gM, oMk + 4 * ur);
+    }
+    int mrs = ldm32<NT>(gM, oMr + 4 * us), msr = ldm32<NT>(gM, oMs + 4 * ur);
     const int2 wr = pending(r), ws = pending(s);
     const int fRR = ldsf<FE>(oFr + FB * r), fRS = ldsf<FE>(oFr + FB * s);
     const int fSS = ldsf<FE>(oFs + FB * s), fSR = SYM ? fRS : ldsf<FE>(oFs + FB * r);
-    const int Frk = ldsf<FE>(oFr + FB * k), Fsk = ldsf<FE>(oFs + FB * k);
-    const int Fkr = SYM ? Frk : ldsf<FE>(aFt + FB * (r * S.fr + k * S.fk));
-    const int Fks = SYM ? Fsk : ldsf<FE>(aFt + FB * (s * S.fr + k * S.fk));
-    // ends of the tabu times of the pairs {r, k} and {s, k}
     const int rtri = r * (r - 1) / 2, stri = s * (s - 1) / 2;
-    const int end_r = lds32(aMark + 4 * (k < r ? rtri + k : ktri + r));
-    const int end_s = lds32(aMark + 4 * (k < s ? stri + k : ktri + s));
     const int ten = lds32(aTen + 4 * ((it - 1) & 63));
-    const uint32_t u4 = 4 * (uint32_t)uk;
-    const int wuk = lds32(aVwu + rd + u4);
-    int Ar = lds32(oMr + u4), As = lds32(oMs + u4);
     const uint32_t oQr = aP + ur * ldP, oQs = aP + us * ldP;
-    const int wur = lds32(aVwu + rd + 4 * ur), wus = lds32(aVwu + rd + 4 * us);
+    const int2 wur = column(ur), wus = column(us);
     const int qRR = lds8(oQr + ur), qRS = lds8(oQr + us), qSS = lds8(oQs + us);
     const int qSR = SYM ? qRS : lds8(oQs + ur);
-    const int Qrk = lds8(oQr + uk), Qsk = lds8(oQs + uk);
-    const int Qkr = SYM ? Qrk : lds8(aPt + ur * S.pr + uk * S.pk);
-    const int Qks = SYM ? Qsk : lds8(aPt + us * S.pr + uk * S.pk);
-    int Bs = lds32(oMk + 4 * us), Br = lds32(oMk + 4 * ur);
-    int mrs = lds32(oMr + 4 * us), msr = lds32(oMs + 4 * ur);
     // the byte (pair) of the pending words that this move takes
     const int slot = mv & (Q - 1);
-    const uint32_t sel = SYM ? (0x3210u & ~(0xfu << (4 * slot))) | 4u << (4 * slot)
-                             : slot ? 0x5410u : 0x3254u;
-    const int2 wkj = (k & (Q - 1)) == done ? make_int2(0, 0) : wk;
-    Ar = entry(wr, wuk, Ar);
-    As = entry(ws, wuk, As);
-    Bs = entry(wkj, wus, Bs);
-    Br = entry(wkj, wur, Br);
-    mrs = entry(wr, wus, mrs);
-    msr = entry(ws, wur, msr);
-    const int av = Frk - Fsk, b = Qrk - Qsk;
-    const int c = Fkr - Fks, e = Qkr - Qks;
-    // the words of k in the pairs' update (int16 flows: (a, c), then (b, e))
-    uint32_t own, word, own2 = 0, word2 = 0;
-    int gr, gs, gn, Rr, Rs;
-    if constexpr (PW == 2) {
-      own = pack2(-av, -c);
-      word = pack2(av, c);
-      own2 = __byte_perm((uint32_t)-b, (uint32_t)-e, 0x0040u);
-      word2 = __byte_perm((uint32_t)b, (uint32_t)e, 0x0040u);
-    } else if constexpr (SYM) {
-      own = __byte_perm((uint32_t)-av, (uint32_t)-b, 0x4400u);
-      word = __byte_perm((uint32_t)b, (uint32_t)av, 0x4400u);
-    } else {
-      own = pack4(-av, -c, -b, -e);
-      word = pack4(b, e, av, c);
-    }
+    const uint32_t selb = (0x3210u & ~(0xfu << (4 * (slot & 3)))) | 4u << (4 * (slot & 3));
+    const uint32_t selh = slot & 1 ? 0x5410u : 0x3254u;
+    const uint32_t sel = SYM ? selb : selh;
+    const bool high = (SYM ? slot >> 2 : slot >> 1) != 0;  // of two dp4a words
+    mrs = rot_entry<NT, FE>(wr, wus, mrs);
+    msr = rot_entry<NT, FE>(ws, wur, msr);
+    int gr, gs;
     if (SYM) {
       gr = 2 * (mrs - (fRR - fRS) * (qRS - qSS)) - g0;
       gs = 2 * (msr - (fRS - fSS) * (qRR - qRS)) - g0;
-      gn = gk - 2 * av * b;
-      Rr = 2 * (Ar + Bs + (qSS - qRS) * av - (fRR - fRS) * b) - g2 +
-           (fRR + Fkk - 2 * Frk) * (qSS + Qkk - 2 * Qsk);
-      Rs = 2 * (As + Br + (qRS - qRR) * av - (fRS - fSS) * b) - g2 +
-           (fSS + Fkk - 2 * Fsk) * (qRR + Qkk - 2 * Qrk);
     } else {
       gr = mrs - (fRR - fRS) * (qSR - qSS) - (fRR - fSR) * (qRS - qSS) - g0;
       gs = msr - (fSR - fSS) * (qRR - qRS) - (fRS - fSS) * (qRR - qSR) - g0;
-      gn = gk - av * b - c * e;
-      Rr = Ar + Bs - g2 + (fRR - Frk - Fkr + Fkk) * (qSS - Qsk - Qks + Qkk) - (fRR - fRS) * e -
-           (fRR - fSR) * b + (qSS - qSR) * c + (qSS - qRS) * av;
-      Rs = As + Br - g2 + (fSS - Fsk - Fks + Fkk) * (qRR - Qrk - Qkr + Qkk) - (fSR - fSS) * e -
-           (fRS - fSS) * b + (qRS - qRR) * c + (qSR - qRR) * av;
     }
-    Rr += end_r > it + 1 ? BIG : 0;
-    Rs += end_s > it + 1 ? BIG : 0;
-    // M's operands of this move: (-a, -c) by index, bytes (b, e) by label
-    // (symmetric: -a and b)
-    wk = wkj;
-    if constexpr (PW == 1) {
-      wk.x = (int)__byte_perm((uint32_t)wkj.x, own, sel);
-    } else if constexpr (SYM) {
-      const uint32_t hs = slot & 1 ? 0x5410u : 0x3254u;  // half slot mod 2 of word slot / 2
-      const int h = (int)__byte_perm((uint32_t)(slot & 2 ? wkj.y : wkj.x), own, hs);
-      wk.x = slot & 2 ? wk.x : h;
-      wk.y = slot & 2 ? h : wk.y;
-    } else {
-      wk.x = slot ? wk.x : (int)own;
-      wk.y = slot ? (int)own : wk.y;
-    }
-    const int wun = (int)__byte_perm((uint32_t)wuk, PW == 1 ? word : word2, sel);
-    const bool isr = k == r, iss = k == s;
     // the pair (r, s) itself only changes sign, and turns tabu
     const int drs = gr + gs - course.bd + (tabu_phase && ten > 1 ? BIG : 0);
-    gn = isr ? gr : iss ? gs : gn;
-    Rr = isr || iss ? drs : Rr;
-    Rs = isr || iss ? drs : Rs;
-    gk = gn;
-    if (live) {
-      const int psi = (int)(0u - ((uint32_t)gn << SB) - (1u << 30)) + (rot_rank(NT) ? 32 : k);
-      sts32(aX + 4 * k, (int)word);
-      sts32(aX + 4 * nE + 4 * k, (int)word);
-      if constexpr (PW == 2) {
-        sts32(base + X_::X2 + 4 * k, (int)word2);
-        sts32(base + X_::X2 + 4 * nE + 4 * k, (int)word2);
+#pragma unroll
+    for (int j = 0; j < KX; ++j) {
+      const int kj = k[j], uj = uk[j];
+      const int Frk = ldsf<FE>(oFr + FB * kj), Fsk = ldsf<FE>(oFs + FB * kj);
+      const int Fkr = SYM ? Frk : ldsf<FE>(aFt + FB * (r * S.fr + kj * S.fk));
+      const int Fks = SYM ? Fsk : ldsf<FE>(aFt + FB * (s * S.fr + kj * S.fk));
+      // whether the pairs {r, k} and {s, k} are tabu at the next iteration
+      const int ktri = kj * (kj - 1) / 2;
+      const int ar = kj < r ? rtri + kj : ktri + r, as = kj < s ? stri + kj : ktri + s;
+      bool tabu_r, tabu_s;
+      if constexpr (M16) {
+        const int er = lds16u(aMark + 2 * ar), es = lds16u(aMark + 2 * as);
+        tabu_r = er != 0 && er != rot_mark16(it + 1);
+        tabu_s = es != 0 && es != rot_mark16(it + 1);
+      } else {
+        tabu_r = lds32(aMark + 4 * ar) > it + 1;
+        tabu_s = lds32(aMark + 4 * as) > it + 1;
       }
-      sts32(aPsi + 4 * k, psi);
-      sts32(aPsi + 4 * nE + 4 * k, rot_rank(NT) ? psi - 32 : psi);
-      if constexpr (PW == 1) sts32(aOwn + 4 * k, (int)own);
-      else sts64(aOwn + 8 * k, (int)own, (int)own2);
-      sts64(aR + 8 * k, Rr, Rs);
-      sts64(aR + 8 * nE + 8 * k, Rr, Rs);
-      if constexpr (PW == 1) sts32(aVw + wt + 4 * k, wk.x);
-      else sts64(aVw + 2 * wt + 8 * k, wk.x, wk.y);
-      sts32(aVwu + wt + u4, wun);
+      int2 wuk = column(uj);
+      const int Qrk = lds8(oQr + uj), Qsk = lds8(oQs + uj);
+      const int Qkr = SYM ? Qrk : lds8(aPt + ur * S.pr + uj * S.pk);
+      const int Qks = SYM ? Qsk : lds8(aPt + us * S.pr + uj * S.pk);
+      const int2 wkj = (kj & (Q - 1)) == done ? make_int2(0, 0) : wk[j];
+      const int mAr = rot_entry<NT, FE>(wr, wuk, Ar[j]), mAs = rot_entry<NT, FE>(ws, wuk, As[j]);
+      const int mBs = rot_entry<NT, FE>(wkj, wus, Bs[j]), mBr = rot_entry<NT, FE>(wkj, wur, Br[j]);
+      const int av = Frk - Fsk, b = Qrk - Qsk;
+      const int c = Fkr - Fks, e = Qkr - Qks;
+      // the words of k in the pairs' update (int16 flows: (a, c), then (b, e))
+      uint32_t own, word, own2 = 0, word2 = 0;
+      if constexpr (PW2) {
+        own = pack2(-av, -c);
+        word = pack2(av, c);
+        own2 = __byte_perm((uint32_t)-b, (uint32_t)-e, 0x0040u);
+        word2 = __byte_perm((uint32_t)b, (uint32_t)e, 0x0040u);
+      } else if constexpr (SYM) {
+        own = __byte_perm((uint32_t)-av, (uint32_t)-b, 0x4400u);
+        word = __byte_perm((uint32_t)b, (uint32_t)av, 0x4400u);
+      } else {
+        own = pack4(-av, -c, -b, -e);
+        word = pack4(b, e, av, c);
+      }
+      int gn, Rr, Rs;
+      if (SYM) {
+        gn = gk[j] - 2 * av * b;
+        Rr = 2 * (mAr + mBs + (qSS - qRS) * av - (fRR - fRS) * b) - g2 +
+             (fRR + Fkk[j] - 2 * Frk) * (qSS + Qkk[j] - 2 * Qsk);
+        Rs = 2 * (mAs + mBr + (qRS - qRR) * av - (fRS - fSS) * b) - g2 +
+             (fSS + Fkk[j] - 2 * Fsk) * (qRR + Qkk[j] - 2 * Qrk);
+      } else {
+        gn = gk[j] - av * b - c * e;
+        Rr = mAr + mBs - g2 + (fRR - Frk - Fkr + Fkk[j]) * (qSS - Qsk - Qks + Qkk[j]) -
+             (fRR - fRS) * e - (fRR - fSR) * b + (qSS - qSR) * c + (qSS - qRS) * av;
+        Rs = mAs + mBr - g2 + (fSS - Fsk - Fks + Fkk[j]) * (qRR - Qrk - Qkr + Qkk[j]) -
+             (fSR - fSS) * e - (fRS - fSS) * b + (qRS - qRR) * c + (qSR - qRR) * av;
+      }
+      Rr += tabu_r ? BIG : 0;
+      Rs += tabu_s ? BIG : 0;
+      // M's operands of this move: (-a, -c) by index, bytes (b, e) by label
+      // (symmetric: -a and b)
+      int2 wn = wkj;
+      if constexpr (PW2) {
+        if constexpr (SYM) {
+          const int hw = (int)__byte_perm((uint32_t)(slot & 2 ? wkj.y : wkj.x), own, selh);
+          wn.x = slot & 2 ? wn.x : hw;
+          wn.y = slot & 2 ? hw : wn.y;
+        } else {
+          wn.x = slot ? wn.x : (int)own;
+          wn.y = slot ? (int)own : wn.y;
+        }
+        wuk.x = (int)__byte_perm((uint32_t)wuk.x, word2, sel);
+      } else if constexpr (RW == 1) {
+        wn.x = (int)__byte_perm((uint32_t)wkj.x, own, sel);
+        wuk.x = (int)__byte_perm((uint32_t)wuk.x, word, sel);
+      } else {
+        const int hr = (int)__byte_perm((uint32_t)(high ? wkj.y : wkj.x), own, sel);
+        const int hc = (int)__byte_perm((uint32_t)(high ? wuk.y : wuk.x), word, sel);
+        wn.x = high ? wn.x : hr;
+        wn.y = high ? hr : wn.y;
+        wuk.x = high ? wuk.x : hc;
+        wuk.y = high ? hc : wuk.y;
+      }
+      wk[j] = wn;
+      const bool isr = kj == r, iss = kj == s;
+      gn = isr ? gr : iss ? gs : gn;
+      Rr = isr || iss ? drs : Rr;
+      Rs = isr || iss ? drs : Rs;
+      gk[j] = gn;
+      if (live[j]) {
+        const int psi = (int)(0u - ((uint32_t)gn << SB) - (1u << 30)) + (rot_rank(NT) ? TOP : kj);
+        sts32(aX + 4 * kj, (int)word);
+        sts32(aX + 4 * nE + 4 * kj, (int)word);
+        if constexpr (PW2) {
+          sts32(base + X_::X2 + 4 * kj, (int)word2);
+          sts32(base + X_::X2 + 4 * nE + 4 * kj, (int)word2);
+        }
+        sts32(aPsi + 4 * kj, psi);
+        sts32(aPsi + 4 * nE + 4 * kj, rot_rank(NT) ? psi - TOP : psi);
+        if constexpr (!PW2) sts32(aOwn + 4 * kj, (int)own);
+        else sts64(aOwn + 8 * kj, (int)own, (int)own2);
+        sts64(aR + 8 * kj, Rr, Rs);
+        sts64(aR + 8 * nE + 8 * kj, Rr, Rs);
+        if constexpr (RW == 1) sts32(aVw + wt + 4 * kj, wn.x);
+        else sts64(aVw + 2 * wt + 8 * kj, wn.x, wn.y);
+        if constexpr (LW == 1) sts32(aVwu + wt + 4 * uj, wuk.x);
+        else sts64(aVwu + 2 * wt + 8 * uj, wuk.x, wuk.y);
+      }
     }
     rot_barrier();
     // while the other warps bring the table up to date: M, the labels, the
     // best solution, the tabu times and the hash
-    rot_update_m<Q, PW>(T, aM, aVw + PW * wt, aVwu + wt, n, ldm, slot);
+    rot_update_m<NT, Q, FE>(T, gM, aM, aVw + RW * wt, aVwu + LW * wt, n, ldm, slot);
     ++mv;
-    uk = isr ? us : iss ? ur : uk;
-    Qkk = isr ? qSS : iss ? qRR : Qkk;
-    if (live && (isr || iss)) sts32(aSig + 4 * k, uk);
     const bool better = !tabu_phase || course.cur < course.best;
-    best_uk = better ? uk : best_uk;
+#pragma unroll
+    for (int j = 0; j < KX; ++j) {
+      const bool isr = k[j] == r, iss = k[j] == s;
+      uk[j] = isr ? us : iss ? ur : uk[j];
+      Qkk[j] = isr ? qSS : iss ? qRR : Qkk[j];
+      if (live[j] && (isr || iss)) sts32(aSig + 4 * k[j], uk[j]);
+      best_uk[j] = better ? uk[j] : best_uk[j];
+    }
     course.best = better ? course.cur : course.best;
     best_iter = better ? it : best_iter;  // 0 in the descent
     if (first) {
@@ -926,11 +1101,24 @@ __device__ __forceinline__ void rot_phase_x() {
       if (tabu_phase) {
         if ((it & 31) == 0)  // the tenures of iterations it + 33 .. it + 64
           S.ten()[(it + 32 + lane) & 63] = tenure.of(seed, wid, it + 33 + lane);
-        if (k == 0) {
+        if (T.pt == 0) {
           const int end = it + ten;
+          uint32_t* const now = S.ring() + ((it + 1) & (rot_ring(NT) - 1));
+          if constexpr (M16) {
+            // the marks that end with the next iteration
+            uint16_t* const mark = reinterpret_cast<uint16_t*>(S.mark());
+            for (uint32_t w = *now; w != 0xffffffffu;
+                 w = w >> 16 == 0xffffu ? 0xffffffffu : S.node()[w >> 16]) {
+              const int u = (int)(w >> 8 & 0xffu), v = (int)(w & 0xffu);
+              uint16_t* const m = mark + v * (v - 1) / 2 + u;
+              if (*m == rot_mark16(it + 1)) *m = 0;
+            }
+            mark[stri + r] = end > it + 1 ? (uint16_t)rot_mark16(end) : 0;
+          } else {
+            S.mark()[stri + r] = end;
+          }
           // the ring word of the iteration just served is free again
-          S.ring()[(it + 1) & (rot_ring(NT) - 1)] = 0xffffffffu;
-          S.mark()[stri + r] = end;
+          *now = 0xffffffffu;
           if (end > it + 1 && end <= course.iters) {
             uint32_t* const at = S.ring() + (end & (rot_ring(NT) - 1));
             const uint32_t old = *at, key = (uint32_t)(r << 8 | s);
@@ -955,8 +1143,10 @@ __device__ __forceinline__ void rot_phase_x() {
   // ---- outputs
   const SearchArgs& a = W.s;
   const int row = W.row;
-  if (a.best_p && live) a.best_p[(size_t)row * a.p_stride + k] = S.p0()[best_uk];
-  if (live && k == 0) {
+#pragma unroll
+  for (int j = 0; j < KX; ++j)
+    if (a.best_p && live[j]) a.best_p[(size_t)row * a.p_stride + k[j]] = S.p0()[best_uk[j]];
+  if (T.pt == 0) {
     if (!was_tabu) {
       dh = h;
       h = h0;
@@ -973,9 +1163,10 @@ __device__ __forceinline__ void rot_phase_x() {
 }
 
 // The other warps: M's update, until the flag beside the candidates is set.
-template <int NT, int C, int Q, typename FE>
+template <int NT, int C, bool SYM, typename FE>
 __device__ __forceinline__ void rot_helper() {
-  constexpr int PW = kRotWords<FE>;
+  using P = RotPending<NT, FE>;
+  constexpr int Q = P::template Q<SYM>;
   using X_ = RotFixed<NT, FE>;
   const RotWalkArgs& W = RotSmem<NT, FE>::args();
   const RotThread T = rot_thread<NT, C>(W.I.n);
@@ -988,8 +1179,9 @@ __device__ __forceinline__ void rot_helper() {
     rot_barrier();
     if (lds32(base + X_::red + 8 * 32)) break;
     const uint32_t wt = mv & 1 ? 0 : 4 * ldm;
-    rot_update_m<Q, PW>(T, base + S.L.M, base + X_::vw + PW * wt, base + X_::vwu + wt, n, ldm,
-                        mv & (Q - 1));
+    rot_update_m<NT, Q, FE>(T, reinterpret_cast<char*>(W.M), rot_big(NT) ? 0 : base + S.L.M,
+                            base + X_::vw + P::RW * wt, base + X_::vwu + P::LW * wt, n, ldm,
+                            mv & (Q - 1));
   }
 }
 
@@ -997,6 +1189,7 @@ __device__ __forceinline__ void rot_helper() {
 // Starts and ends with every thread of the CTA together.
 template <int NT, typename FE>
 __device__ __forceinline__ void rot_start() {
+  constexpr int TH = rot_threads(NT);
   RotWalkArgs& W = RotSmem<NT, FE>::args();
   const InstArgs& I = W.I;
   const SearchArgs& a = W.s;
@@ -1014,9 +1207,9 @@ __device__ __forceinline__ void rot_start() {
   // ---- start permutation: given, or Fisher-Yates on stream 0 (the draws by
   // all threads, the exchanges by one)
   if (start) {
-    for (int x = tid; x < n; x += NT) S.p0()[x] = start[x];
+    for (int x = tid; x < n; x += TH) S.p0()[x] = start[x];
   } else {
-    for (int i = tid; i < n; i += NT) {
+    for (int i = tid; i < n; i += TH) {
       S.p0()[i] = i;
       if (i >= 1) S.vw()[i] = (int)below(walk_draw(a.seed, wid, 0u, (uint32_t)(n - 1 - i)),
                                          (uint32_t)(i + 1));
@@ -1037,7 +1230,7 @@ __device__ __forceinline__ void rot_start() {
     const int8_t* Dg = static_cast<const int8_t*>(I.D);
     const bool tr = !I.symD && !notr;
     int8_t* Pt = S.Pt();
-    for (int i = warp; i < n; i += NT / 32) {
+    for (int i = warp; i < n; i += TH / 32) {
       const int8_t* Di = Dg + (size_t)S.p0()[i] * n;
       for (int j = lane; j < n; j += 32) {
         const int8_t v = Di[S.p0()[j]];
@@ -1045,22 +1238,23 @@ __device__ __forceinline__ void rot_start() {
         if (tr) Pt[j * ldP + i] = v;
       }
     }
-    for (int x = tid; x < n; x += NT) S.sigma()[x] = x;
+    for (int x = tid; x < n; x += TH) S.sigma()[x] = x;
     // phantom indices: never candidates, never updated
-    for (int x = n + tid; x < nE; x += NT) {
+    for (int x = n + tid; x < nE; x += TH) {
       S.X()[x] = S.X()[x + nE] = 0;
-      S.psi()[x] = S.psi()[x + nE] = INT_MAX - 64;
+      S.psi()[x] = S.psi()[x + nE] = INT_MAX - 128;
       S.R()[x] = S.R()[x + nE] = make_int2(0, 0);
       for (int w = 0; w < kRotWords<FE>; ++w) S.own()[kRotWords<FE> * x + w] = 0;
       if (kRotWords<FE> == 2) S.X2()[x] = S.X2()[x + nE] = 0;
     }
     // no pending moves; M's padding columns take updates from these words only
-    for (int x = tid; x < 2 * ldm; x += NT) S.vwu()[x] = 0;
-    for (int x = tid; x < 2 * kRotWords<FE> * ldm; x += NT) S.vw()[x] = 0;
-    for (int x = tid; x < rot_ring(NT); x += NT) S.ring()[x] = 0xffffffffu;
+    using Pd = RotPending<NT, FE>;
+    for (int x = tid; x < 2 * Pd::LW * ldm; x += TH) S.vwu()[x] = 0;
+    for (int x = tid; x < 2 * Pd::RW * ldm; x += TH) S.vw()[x] = 0;
+    for (int x = tid; x < rot_ring(NT); x += TH) S.ring()[x] = 0xffffffffu;
     if (a.iters > 0) {
       const RotTenure tenure(a, n);
-      for (int x = tid; x < 64; x += NT) S.ten()[x] = tenure.of(a.seed, wid, x + 1);
+      for (int x = tid; x < 64; x += TH) S.ten()[x] = tenure.of(a.seed, wid, x + 1);
     }
     if (tid == 0) S.red()[32] = make_int2(0, 0);
   }
@@ -1068,38 +1262,26 @@ __device__ __forceinline__ void rot_start() {
   rot_compute_m<NT, FE>(S, n, ldF, ldP, sym, notr);
   __syncthreads();
 
-  // ---- the pairs' table, in the marks' place: d = M[u][v] + M[v][u] + the
-  // 2x2 term of Eq. 2
-  {
-    const FE* F = S.F();
-    const int8_t* P = S.P();
-    const int32_t* M = S.M();
-    for (int v = 1 + warp; v < n; v += NT / 32) {
-      const int fv = F[v * ldF + v], pv = P[v * ldP + v];
-      for (int u = lane; u < v; u += 32) {
-        const int f = fv + F[u * ldF + u] - F[u * ldF + v] - F[v * ldF + u];
-        const int p = pv + P[u * ldP + u] - P[u * ldP + v] - P[v * ldP + u];
-        S.mark()[v * (v - 1) / 2 + u] =
-            ((M[u * ldm + v] + M[v * ldm + u]) << hsh) + f * p - 2 * g0;
-      }
-    }
-  }
+  // ---- the pairs' table, in the marks' place (large n: they are too small)
+  if (!rot_big(NT))
+    for (int v = 1 + warp; v < n; v += rot_threads(NT) / 32)
+      for (int u = lane; u < v; u += 32) S.mark()[v * (v - 1) / 2 + u] = rot_pair(S, I, u, v);
 
   // ---- scan addends of every index; the walk's cost (Eq. 1): M's diagonal
   // sums to twice the cost
   int64_t c0 = 0;
-  for (int x = tid; x < n; x += NT) {
+  for (int x = tid; x < n; x += TH) {
     const int mxx = S.M()[x * ldm + x];
     c0 += mxx;
     const uint32_t psi = 0u - ((uint32_t)((mxx << hsh) - g0) << SB) - (1u << 30);
-    S.psi()[x] = (int)(psi + (rot_rank(NT) ? 32 : x));
+    S.psi()[x] = (int)(psi + (rot_rank(NT) ? 1 << (SB - 1) : x));
     S.psi()[x + nE] = (int)(psi + (rot_rank(NT) ? 0 : x));
   }
-  c0 = block_sum<NT>(c0, S.sum());
+  c0 = block_sum<TH>(c0, S.sum());
   if (tid == 0) W.cost = sym ? c0 : c0 >> 1;
   if (a.freq) {
     int32_t* fq = a.freq + (size_t)W.row * a.p_stride * a.p_stride;
-    for (int c = tid; c < a.p_stride * a.p_stride; c += NT) fq[c] = 0;
+    for (int c = tid; c < a.p_stride * a.p_stride; c += TH) fq[c] = 0;
   }
   __syncthreads();
 }
@@ -1115,8 +1297,8 @@ __device__ __forceinline__ void rot_walk() {
   if (role == 0) rot_owner<NT, C, FE>();
   else if (role == 1 && sym) rot_phase_x<NT, C, true, FE>();
   else if (role == 1) rot_phase_x<NT, C, false, FE>();
-  else if (sym) rot_helper<NT, C, 4, FE>();
-  else rot_helper<NT, C, 2, FE>();
+  else if (sym) rot_helper<NT, C, true, FE>();
+  else rot_helper<NT, C, false, FE>();
   __syncthreads();
 }
 
@@ -1125,45 +1307,44 @@ __device__ __forceinline__ void rot_walk() {
 template <int NT, typename FE>
 __device__ __forceinline__ void rot_load(const InstArgs& I, bool notr) {
   const RotLayout L = rot_layout(I.n, I.ldF, sizeof(FE), I.ldP, I.symF, I.symD, notr,
-                                 RotFixed<NT, FE>::bytes);
+                                 rot_big(NT), RotFixed<NT, FE>::bytes);
   const bool ft = !I.symF && !notr, pt = !I.symD && !notr;
   const int tid = threadIdx.x;
   const int fvec = I.n * I.ldF * (int)sizeof(FE) / 16, pvec = I.n * I.ldP / 16;
   const int4* gF = static_cast<const int4*>(I.F);
   const int4* gFt = static_cast<const int4*>(I.Ft);
 #pragma unroll 2
-  for (int i = tid; i < fvec; i += NT) {
+  for (int i = tid; i < fvec; i += rot_threads(NT)) {
     rot_at<int4>(L.F)[i] = gF[i];
     if (ft) rot_at<int4>(L.Ft)[i] = gFt[i];
   }
   const int4 zero = make_int4(0, 0, 0, 0);
 #pragma unroll 2
-  for (int i = tid; i < pvec; i += NT) {
+  for (int i = tid; i < pvec; i += rot_threads(NT)) {
     rot_at<int4>(L.P)[i] = zero;
     if (pt) rot_at<int4>(L.Pt)[i] = zero;
   }
   __syncthreads();
 }
 
-// The partner blocks per thread (C) compiled for a thread count: at most 15,
-// for ranks below 32.
-constexpr int kRotMaxC = 13;
+// The partner blocks per thread (C) compiled for a shape: below 16 (large n: 32)
+// for their ranks.
+constexpr int kRotMaxC = 22;
 __host__ __device__ constexpr bool rot_compiled(int nt, int c) {
-  return nt == 128   ? c == 1 || c == 2 || c == 4 || c == 7
-         : nt == 256 ? c <= 4 || c == 6 || c == 7 || c == 11 || c == 13
-         : nt == 512 ? c <= 3 || c == 5 || c == 7 || c == 8 || c == 11 || c == 13
-                     : c == 2 || c == 4 || c == 5 || c == 6;
+  return rot_big(nt)  ? c == 8 || c == 10 || c == 12 || c == 16 || c == 19 || c == 22
+         : nt == 128  ? c == 1 || c == 2 || c == 4 || c == 7
+         : nt == 256  ? c <= 4 || c == 6 || c == 7 || c == 11 || c == 13
+         : nt == 512  ? c <= 3 || c == 5 || c == 7 || c == 8 || c == 11 || c == 13
+                      : c == 2 || c == 4 || c == 5 || c == 6;
 }
 
 // CTAs per SM to compile for.
-constexpr int rot_min_blocks(int nt) {
-  return nt == 128 ? 4 : nt == 256 ? 2 : 1;
-}
+constexpr int rot_min_blocks(int nt) { return nt == 128 ? 4 : nt == 256 ? 2 : 1; }
 
 // Walks of one instance (b.single: CTAs step over its walks) or of many (CTAs
 // take items from the counter and reload the instance when it changes).
 template <int NT, int C, typename FE>
-__global__ void __launch_bounds__(NT, rot_min_blocks(NT)) rot_kernel(const BatchArgs b) {
+__global__ void __launch_bounds__(rot_threads(NT), rot_min_blocks(NT)) rot_kernel(const BatchArgs b) {
   __shared__ int item_s;
   RotWalkArgs& W = RotSmem<NT, FE>::args();
   int cur_inst = -1, item = blockIdx.x;
@@ -1182,6 +1363,7 @@ __global__ void __launch_bounds__(NT, rot_min_blocks(NT)) rot_kernel(const Batch
         W.I = *I;
         W.s = b.s;
         W.notr = b.notr;
+        W.M = reinterpret_cast<int32_t*>(b.ws ? b.ws + b.ws_stride * blockIdx.x : nullptr);
       }
       const int w = b.single ? b.walk_offset + item : b.item_walk[item];
       W.row = b.single ? w : b.row_base[inst] + w;

@@ -153,13 +153,14 @@ struct qap_server {
 
 namespace {
 
-// Plans the launch and sizes the device block of one request.
-qap_status place(qap_server* sv, Request* r) {
+// Plans the launch and sizes the device block of one request.  `workspace`:
+// whether it may take a workspace where the row layout has none.
+qap_status place(qap_server* sv, Request* r, bool workspace) {
   const int W = r->params.starts, n = r->di.n;
   // a request's own walks decide (several requests share the GPU)
   const bool many = W >= 2 * sv->sms;
   if (!search_plan(n, many, &r->di, 1, r->fbytes, r->dbytes, r->force64, sv->smem_optin, 0,
-                   &r->params, &r->plan))
+                   workspace, &r->params, &r->plan))
     return QAP_EUNSUPPORTED;
   if (!rot_holds_tenures(r->plan, &r->params, n)) r->plan = r->plan.rows();
   r->fn = pick_walk_kernel(r->dbytes, r->fbytes, r->plan);
@@ -409,7 +410,8 @@ qap_status qap_server_submit(qap_server* sv, const int64_t* F, const int64_t* D,
   if (r->di.symF) r->iFt.clear();
   DeviceGuard dg;
   QAP_TRY(dg.set(sv->device));
-  QAP_TRY(place(sv, r.get()));
+  QAP_TRY(place(sv, r.get(), true));
+  if (r->bytes > sv->arena.size()) QAP_TRY(place(sv, r.get(), false));
   if (r->bytes > sv->arena.size()) return QAP_ENOMEM;  // could never be admitted
   // the images into the pinned slab when it has room, so the worker only
   // enqueues their copies

@@ -25,8 +25,9 @@ void check(int n, int nt, int c) {
   if (n > qapk::rot_max_n(nt)) fail("fixed arrays too small", n, nt, c);
   if (qapk::ld_m(n) > qapk::rot_max_n(nt) + 4) fail("pending words too small", n, nt, c);
   if (J * n2 > qapk::rot_owners(nt)) fail("too many pair threads", n, nt, c);
-  if ((n + 31) / 32 * 32 > nt - qapk::rot_owners(nt)) fail("no thread per index", n, nt, c);
-  if (qapk::rot_rank(nt) ? 2 * c > 31 - 1 : nE > 1 << qapk::rot_key_bits(nt))
+  if (n > qapk::rot_kx(nt) * (qapk::rot_threads(nt) - qapk::rot_owners(nt))) fail("no thread per index", n, nt, c);
+  if (qapk::rot_rank(nt) ? 2 * c >= 1 << (qapk::rot_key_bits(nt) - 1)
+                         : nE > 1 << qapk::rot_key_bits(nt))
     fail("partner does not fit the key bits", n, nt, c);
   std::vector<char> held((size_t)nE * nE, 0);
   for (int tid = 0; tid < J * n2; ++tid) {
@@ -50,7 +51,7 @@ void check(int n, int nt, int c) {
 
 int main() {
   for (int n = 2; n <= 256; ++n)
-    for (int nt : {128, 256, 512, 1024})
+    for (int nt : {128, 256, 512, 1024, qapk::kRotBig})
       for (int c = 1; c <= qapk::kRotMaxC; ++c)
         if (qapk::rot_compiled(nt, c)) check(n, nt, c);
   // every size that the automatic int8 products plans take has a layout
@@ -63,6 +64,17 @@ int main() {
         any |= qapk::rot_compiled(p.nt, c) && qapk::rot_chunks(n, p.nt, c) > 0;
       if (!any && p.nt < 1024) fail("no layout", n, p.nt, many);
     }
+  // and every larger size the workspace shape
+  for (int n = 152; n <= 256; ++n) {
+    bool any = false;
+    for (int c = 1; c <= qapk::kRotMaxC; ++c)
+      any |= qapk::rot_compiled(qapk::kRotBig, c) && qapk::rot_chunks(n, qapk::kRotBig, c) > 0;
+    if (!any) fail("no large-n layout", n, 512, 0);
+    const int ld = qaph::pad_ldF(n, 1);
+    if (qapk::rot_layout(n, ld, 1, ld, 0, 0, 1, 1, qapk::rot_fixed_bytes(qapk::kRotBig, 1)).bytes +
+            16 > 232448)
+      fail("large n beyond shared memory", n, 512, 0);
+  }
   // the scan candidates' bound: by brute force over permutations and pairs it
   // holds every delta and g; F of any sign, skewed or dense
   std::mt19937 rng(3);
@@ -110,7 +122,7 @@ int main() {
   qap_search_params sp{};
   sp.iters = 10;
   for (int nt : {128, 256, 512, 1024}) {
-    qaph::Plan p{nt, 8, qapk::kProductM, 1, qapk::kProductM};
+    qaph::Plan p{nt, 8, qapk::kProductM, 1, qapk::kProductM, nt};
     sp.tenure = {1, qapk::rot_ring(nt) - 2, 0};
     if (!qaph::rot_holds_tenures(p, &sp, 50)) fail("longest tenure", 50, nt, 0);
     ++sp.tenure.tmax;

@@ -82,6 +82,55 @@ def test_thread_counts(n, threads):
     check(F, D, 3, threads=threads, seed=6, iters=200, tenure=instances.paper_tenure(n))
 
 
+# M in the workspace: the sizes at the edges of its plans, of its warps and of
+# its marks, with the frequency memory, both tenure rules, 2opt first
+@pytest.mark.parametrize("sym", [False, True])
+@pytest.mark.parametrize("n", [182, 183, 191, 192, 193, 200, 217, 255, 256])
+def test_large_n(n, sym):
+    F, D = instances.uniform_instance(n, 3000 + n, symmetric=sym)
+    np.fill_diagonal(F, np.arange(n) % 7)
+    np.fill_diagonal(D, np.arange(n) % 5)
+    kw = dict(seed=5, iters=120, tenure=instances.periodic_tenure(n), descend=n % 2 == 0,
+              max_descent=40)
+    check(F, D, 3, **kw)
+    check(F, D, 2, seed=6, iters=300, tenure=(1, 9, 0))
+    with q.Instance(F, D) as inst:
+        prm = q.make_params(2, **kw)
+        assert inst.plan(prm)["workspace"] == 1
+        g = inst.search(prm, freq=True)
+        assert (g["freq"].sum(axis=(1, 2)) == g["iters_done"]).all()
+
+
+@pytest.mark.parametrize("tmax", [300, 510, 511])
+def test_large_n_long_tenures(tmax):
+    F, D = instances.grid_instance(190, 3300)
+    check(F, D, 2, seed=14, iters=800, tenure=(tmax - 3, tmax, 0))
+
+
+def test_large_n_in_batches_and_from_several_walks(gpu):
+    """Batches take M's workspace from n = 152 on; more walks than CTAs."""
+    ns = [30, 152, 163, 181, 182, 220]
+    pairs = [instances.uniform_instance(n, 3400 + n, symmetric=n % 2 == 0) for n in ns]
+    with q.Batch([F for F, _ in pairs], [D for _, D in pairs]) as b:
+        for tn in ((5, 30, 0), (500, 600, 0), (90, 110, 200)):
+            per_n = tn[0] == 90
+            g = b.search(q.make_params(3, seed=15, iters=100, tenure=tn, tenure_per_n=per_n))
+            for i, (F, D) in enumerate(pairs):
+                t = instances.periodic_tenure(ns[i]) if per_n else tn
+                o = oracle.run_walks(F, D, 3, seed=15, iters=100, tenure=t)
+                for k in FIELDS[1:]:
+                    assert np.array_equal(g[k][3 * i:3 * i + 3].astype(np.int64),
+                                          o[k].astype(np.int64)), (i, k)
+    F, D = pairs[-1]
+    W = 2 * gpu.cuda.get_device_properties(0).multi_processor_count + 5
+    with q.Instance(F, D) as inst:
+        g = inst.search(q.make_params(W, seed=16, iters=60, tenure=(5, 30, 0)))
+    o = oracle.run_walks(F, D, 3, seed=16, iters=60, tenure=(5, 30, 0),
+                         walk_ids=np.array([0, W // 2, W - 1]))
+    for k in FIELDS:
+        assert np.array_equal(g[k][[0, W // 2, W - 1]].astype(np.int64), o[k].astype(np.int64)), k
+
+
 # many ties (small values), short random tenures with aspiration: pairs are
 # applied again while tabu, ends coincide
 @pytest.mark.parametrize("n,hi", [(14, 3), (30, 99), (50, 9), (100, 99), (100, 2), (130, 99)])
