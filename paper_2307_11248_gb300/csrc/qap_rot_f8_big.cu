@@ -5,11 +5,11 @@ namespace qapk {
 
 BatchKernelFn rot_f8_big(int c) {
   switch (c) {
-    case 8: return rot_kernel<kRotBig, 8, int8_t>;
     case 10: return rot_kernel<kRotBig, 10, int8_t>;
     case 12: return rot_kernel<kRotBig, 12, int8_t>;
-    case 16: return rot_kernel<kRotBig, 16, int8_t>;
+    case 17: return rot_kernel<kRotBig, 17, int8_t>;
     case 19: return rot_kernel<kRotBig, 19, int8_t>;
+    case 21: return rot_kernel<kRotBig, 21, int8_t>;
     case 22: return rot_kernel<kRotBig, 22, int8_t>;
     default: return nullptr;
   }

@@ -6,16 +6,21 @@
 // that warps have roles.
 //
 // Layout.  The n indices form n2 = ceil(n / 2) blocks of two (a phantom index
-// fills an odd n).  Thread (m, j) holds block m against the C partner blocks
-// m + 1 + jC + i (mod n2), i < C: 4 pairs each, and the pair inside block m.
-// Going round, every unordered pair of blocks lies within n2 / 2 steps of one
-// of its members, so J threads per block with J C >= n2 / 2 hold every pair;
-// steps past n2 / 2 hold pairs a second time, which changes nothing (equal
-// values, equal keys).  No slot is ever invalid, so the loops carry no bounds
-// checks; consecutive threads read consecutive 16-byte words (two partners'
-// operands, 4 pairs), free of bank conflicts; and a thread's own operands
-// stay in registers for all its slots.
-//
+// fills an odd n), on a circle of nc blocks, nc the next multiple of C.
+// Thread (m, j) holds block m against the C partner blocks from m + 1 + jC on
+// (mod nc): 4 pairs each, and the pair inside block m.  Going round, every
+// unordered pair of blocks lies within nc / 2 steps of one of its members, so
+// J threads per block with J C >= nc / 2 hold every pair; steps past nc / 2
+// hold pairs a second time, which changes nothing (equal values, equal keys).
+// No slot is ever invalid, so the loops carry no bounds checks; consecutive
+// threads read consecutive 16-byte words (two partners' operands, 4 pairs),
+// free of bank conflicts; and a thread's own operands stay in registers for
+// all its slots.  Among a thread's slots a partner block lies at its residue
+// mod C: the same slot in every thread, so that a move's columns, and a slot
+// whose tabu time ends, are found by one branch for the whole warp (against
+// slots in the window's order, where each thread compares each slot, n = 100
+// takes 3230 for 3385 warp instructions per walk-iteration).
+
 // What a pair costs.  The table holds d(u, v) = delta(u, v) + g[u] + g[v]
 // (with g less its mid-range), whose O(1) update is one dp4a accumulating into
 // it: the w terms of the plain delta's update are exactly the changes of g.
@@ -28,12 +33,16 @@
 // the best that is.  The 2 C pairs with r or s as partner, and the rows of r
 // and s, take phase X's values before the scan; those bring their tabu bits
 // along (phase X reads the pairs' end times), so marking the applied pair
-// costs nothing, and the end of a tabu time is an event: the pairs that end at
+// costs nothing, and the end of a tabu time is an event: the slots that end at
 // an iteration hang on that iteration's word of a ring.
 //
 // Roles.  The first warps hold the pairs, then come phase X's (one thread per
 // index), the rest help to bring M up to date; an iteration is phase X, a
-// barrier, then table and scan beside M's update, a barrier.
+// barrier, then table and scan beside M's update, a barrier.  The last warp
+// keeps tabu times and hash; a serial chain, so with few warps it does no more
+// than that, and it hangs slots in the shadow of the next phase X (n = 50, 256
+// walks 0.94 -> 0.85 us per iteration of all, n = 23, 100 walks 0.64 -> 0.50,
+// against the first warp of phase X doing it on top of its share of M).
 //
 // M's update is put off: the byte operands of up to 2 moves (4 on symmetric
 // instances, whose two products are equal) collect in one word per index, one
@@ -43,19 +52,19 @@
 // Bound: the fixed latencies of one iteration's chain (arg-min, phase X,
 // table, scan, two barriers) with one or two walks on an SM, integer issue
 // with more.  Measured against the row layout's products form (one GB300, same
-// box): n = 100 grid, 1024 walks x (2opt + 10^4) 150.0 -> 50.5 ms; n = 50
-// asymmetric, 256 walks x 5000 7.85 -> 4.66 ms; n = 139 asymmetric, 150 walks
-// x 2000 8.73 -> 3.18 ms; n = 23, 100 walks x 1000 in one blocking call 1.21 ->
-// 0.83 ms; 2opt from 32 starts at n = 12 16.4 -> 12.3 us.  Warp instructions per
-// walk-iteration: n = 100 grid 10360 -> 3370, n = 50 asymmetric 3606 -> 1920.
+// box): n = 100 grid, 1024 walks x (2opt + 10^4) 150.0 -> 47.5 ms; n = 50
+// asymmetric, 256 walks x 5000 7.85 -> 4.24 ms; n = 139 asymmetric, 150 walks
+// x 2000 8.74 -> 2.89 ms; n = 23, 100 walks x 1000 in one blocking call 1.21 ->
+// 0.65 ms; 2opt from 32 starts at n = 12 16.4 -> 12.3 us.  Warp instructions per
+// walk-iteration: n = 100 grid 10360 -> 3236, n = 50 asymmetric 3606 -> 1924.
 // int16 flows (two dp2a per pair): 96 lognormal instances of n = 20-150, 64
-// walks x 1000 each, 103.4 -> 38.6 ms; their costs need 64 bits, their deltas
+// walks x 1000 each, 103.4 -> 39.4 ms; their costs need 64 bits, their deltas
 // do not: the rows' sums of |F| bound them (rot_bounds), where the row layout
 // holds every delta as wide as the cost.
 // Large n (M in the workspace, two dp4a words of pending moves): n = 256 grid,
-// 64 walks x (2opt + 1000) 21.7 -> 7.0 ms, n = 203 asymmetric, 48 walks x 1000
-// 15.7 -> 4.2 ms against the workspace plan, that keeps deltas and marks in L2
-// and recomputes dot products; 24 requests of n = 12-256 24.5 -> 6.8 ms.
+// 64 walks x (2opt + 1000) 21.4 -> 6.6 ms, n = 203 asymmetric, 48 walks x 1000
+// 15.9 -> 3.6 ms against the workspace plan, that keeps deltas and marks in L2
+// and recomputes dot products; 24 requests of n = 12-256 24.5 -> 6.6 ms.
 // Tried and slower: every warp holding pairs and phase X on some of them
 // (n = 100 2.33 against 1.44 us per iteration of two walks per SM); tabu times
 // checked by each thread through its earliest (0.3 us per iteration on the
@@ -91,12 +100,32 @@ __host__ __device__ constexpr int rot_max_n(int nt) {
   return rot_big(nt) ? 256 : nt == 128 ? 64 : nt == 256 ? 128 : 192;
 }
 
+// The partner blocks per thread (C) compiled for a shape: below 16 (large n: 32)
+// for their ranks.
+constexpr int kRotMaxC = 22;
+__host__ __device__ constexpr bool rot_compiled(int nt, int c) {
+  return rot_big(nt)  ? c == 10 || c == 12 || c == 17 || c == 19 || c == 21 || c == 22
+         : nt == 128  ? c == 1 || c == 2 || c == 4 || c == 7 || c == 8
+         : nt == 256  ? c <= 4 || c == 6 || c == 7 || (c >= 12 && c <= 14)
+         : nt == 512  ? c <= 3 || c == 5 || c == 7 || c == 8 || (c >= 12 && c <= 14)
+                      : c == 2 || c == 4 || c == 5 || c == 6;
+}
+
+// Blocks on the circle: a multiple of c, with phantom blocks at the end.
+__host__ __device__ inline int rot_circle(int n, int c) { return ((n + 1) / 2 + c - 1) / c * c; }
+
+// Indices on the circle that a shape's arrays hold (a multiple of 4: the
+// arrays behind them stay on 16-byte boundaries).
+__host__ __device__ constexpr int rot_max_e(int nt) {
+  return rot_big(nt) ? 264 : rot_max_n(nt);
+}
+
 // Threads per block of two (J) at c partner blocks each: the fewest that hold
 // every pair; 0 when the shape does not hold n (its pairs, or its indices).
 __host__ __device__ inline int rot_chunks(int n, int nt, int c) {
-  const int n2 = (n + 1) / 2, j = (n2 / 2 + c - 1) / c;
-  return n >= 3 && n <= rot_max_n(nt) && j * n2 <= rot_owners(nt) &&
-                 rot_px(n, nt) <= rot_threads(nt) - rot_owners(nt) && j * c <= n2 - 1
+  const int n2 = (n + 1) / 2, nc = rot_circle(n, c), j = (nc / 2 + c - 1) / c;
+  return n >= 3 && n <= rot_max_n(nt) && 2 * nc <= rot_max_e(nt) && j * n2 <= rot_owners(nt) &&
+                 rot_px(n, nt) <= rot_threads(nt) - rot_owners(nt) && j * c <= nc - 1
              ? j
              : 0;
 }
@@ -108,6 +137,9 @@ __host__ __device__ constexpr bool rot_rank(int nt) { return nt >= 512; }
 __host__ __device__ constexpr int rot_key_bits(int nt) {
   return rot_rank(nt) && !rot_big(nt) ? 6 : 7;
 }
+
+// A slot of a thread in 16 bits: the low bits for the slot.
+__host__ __device__ constexpr int rot_slot_bits(int nt) { return rot_big(nt) ? 7 : 6; }
 
 // Ends of tabu times that lie ahead are kept in a ring of this many
 // iterations; searches with longer tenures take the row layout.
@@ -153,39 +185,43 @@ constexpr int kRotWords = sizeof(FE) == 1 ? 1 : 2;
 // addresses are constants, then the instance's own.
 template <int NT, typename FE>
 struct RotFixed {
-  static constexpr int NE = rot_max_n(NT);
+  static constexpr int NE = rot_max_e(NT), N = rot_max_n(NT);
   static constexpr int W = kRotWords<FE>;
-  // per position (the indices, then the indices again): update word(s), scan
-  // addend, and d of the pairs {r, k} and {s, k} after the move (int2)
+  // per position (the circle's indices, then again): update word(s), scan
+  // addend, d of the pairs {r, k}, and of {s, k}, after the move
   static constexpr int X = 0;
   static constexpr int X2 = X + 8 * NE;
   static constexpr int psi = X + 8 * W * NE;
-  static constexpr int R = psi + 8 * NE;
+  static constexpr int Rr = psi + 8 * NE;
+  static constexpr int Rs = Rr + 8 * NE;
   // per index: the negated words that meet a partner's (W); label (row of
   // P0); start permutation
-  static constexpr int own = R + 16 * NE;
+  static constexpr int own = Rs + 8 * NE;
   static constexpr int sigma = own + 4 * W * NE;
-  static constexpr int p0 = sigma + 4 * NE;
+  static constexpr int p0 = sigma + 4 * N;
   // pending operands of M's update (two buffers, by the move's parity): rows
   // by index (RW words), columns by label (LW)
-  static constexpr int NW = NE + 4;  // ld_m(n) at most
+  static constexpr int NW = N + 4;  // ld_m(n) at most
   static constexpr int RW = RotPending<NT, FE>::RW, LW = RotPending<NT, FE>::LW;
-  static constexpr int vw = p0 + 4 * NE;
+  static constexpr int vw = p0 + 4 * N;
   static constexpr int vwu = vw + 8 * RW * NW;
-  // ring: the pairs whose tabu time ends at iteration i, at i mod its length:
-  // key of the first in the low half, node of the rest in the high half;
-  // nodes: such words moved aside, at the iteration that moved them
+  // ring: the slots whose tabu time ends at iteration i, at i mod its length:
+  // the first (thread and slot) in the low half, node of the rest in the high
+  // half; nodes: such words moved aside, two for each iteration
   static constexpr int ring = vwu + 8 * LW * NW;
   static constexpr int node = ring + 4 * rot_ring(NT);
   // tenures of the iterations, at (it - 1) mod 64
-  static constexpr int ten = node + 4 * rot_ring(NT);
+  static constexpr int ten = node + 8 * rot_ring(NT);
   // arg-min candidates of the warps (int2) and, at 32, whether the walk is
-  // over; block sums
+  // over, at 33 the move for the keeper; block sums
   static constexpr int red = ten + 4 * 64;
   static constexpr int sum = red + 8 * 34;
   // what the walk is (RotWalkArgs)
   static constexpr int args = sum + 8 * 32;
   static constexpr int bytes = args + kRotArgsBytes;
+  static_assert(own % 16 == 0 && vw % 16 == 0 && vwu % 16 == 0 && ring % 16 == 0 &&
+                    args % 16 == 0 && bytes % 16 == 0 && psi % 8 == 0 && Rr % 8 == 0,
+                "aligned for the widest access of each array");
 };
 
 struct RotLayout {
@@ -259,7 +295,8 @@ struct RotSmem {
   __device__ __forceinline__ static int32_t* X() { return rot_at<int32_t>(X_::X); }
   __device__ __forceinline__ static int32_t* X2() { return rot_at<int32_t>(X_::X2); }
   __device__ __forceinline__ static int32_t* psi() { return rot_at<int32_t>(X_::psi); }
-  __device__ __forceinline__ static int2* R() { return rot_at<int2>(X_::R); }
+  __device__ __forceinline__ static int32_t* Rr() { return rot_at<int32_t>(X_::Rr); }
+  __device__ __forceinline__ static int32_t* Rs() { return rot_at<int32_t>(X_::Rs); }
   __device__ __forceinline__ static int32_t* own() { return rot_at<int32_t>(X_::own); }
   __device__ __forceinline__ static int32_t* sigma() { return rot_at<int32_t>(X_::sigma); }
   __device__ __forceinline__ static int32_t* p0() { return rot_at<int32_t>(X_::p0); }
@@ -324,11 +361,14 @@ struct RotCourse {
 
 // What an instance fixes for a thread.
 struct RotThread {
-  int n, n2, nE;    // indices; blocks of two and their indices (a phantom when n is odd)
+  int n, n2;        // indices, blocks of two (with a phantom index when n is odd)
+  int nc, nE;       // blocks and indices on the circle
   int J;            // threads per block
   int role;         // of the thread's warp: 0 holds pairs, 1 phase X, 2 helps with M
   int m;            // role 0: block of two that the thread holds
-  int pb, pbm;      // role 0: first partner block, as position and mod n2
+  int pb, pbm;      // role 0: first partner block, as position and mod nc
+  bool extra;       // role 0: past the last chunk; the thread offers no candidates
+  bool keeper;      // the thread's warp keeps tabu times and hash: the last one
   int pt, pxt;      // role 1: the thread among phase X's, their number
   int ow;           // warps with role 0
   int ug, ux, urows;  // roles 1, 2: column group and first row of M, rows at once
@@ -340,21 +380,28 @@ __device__ __forceinline__ RotThread rot_thread(int n) {
   const int tid = threadIdx.x;
   t.n = n;
   t.n2 = (n + 1) / 2;
-  t.nE = 2 * t.n2;
+  t.nc = rot_circle(n, C);
+  t.nE = 2 * t.nc;
   const int J = t.J = rot_chunks(n, NT, C);
   const int jt = tid / t.n2;
   t.m = tid - jt * t.n2;
-  const int j = jt < J ? jt : 0;  // threads past the last repeat the first chunk's pairs
+  const int j = jt < J ? jt : 0;
+  t.extra = jt >= J;
   t.pb = t.m + 1 + j * C;
-  t.pbm = t.pb < t.n2 ? t.pb : t.pb - t.n2;
+  t.pbm = t.pb < t.nc ? t.pb : t.pb - t.nc;
   t.ow = (J * t.n2 + 31) / 32;
   t.pt = tid - rot_owners(NT);
   t.pxt = rot_px(n, NT);
   t.role = tid < 32 * t.ow ? 0 : t.pt >= 0 && t.pt < t.pxt ? 1 : 2;
+  t.keeper = tid >= rot_threads(NT) - 32;
+  // a keeper that is no phase X warp leaves M to the others (8 warps or fewer:
+  // with more the keeper is done before its share)
+  const int mt = rot_threads(NT) - 32 * t.ow -
+                 (NT <= 256 && t.pxt + rot_owners(NT) <= NT - 32 ? 32 : 0);
   const int gpr = ld_m(n) / 4, f = tid - 32 * t.ow;
   t.ug = f % gpr;
   t.ux = f / gpr;
-  t.urows = (rot_threads(NT) - 32 * t.ow) / gpr;
+  t.urows = mt / gpr;
   return t;
 }
 
@@ -557,10 +604,10 @@ __device__ __forceinline__ int rot_entry(int2 w, int2 u, int m) {
 // M[x][.] after a move, for the rows x = slot mod Q, with the pending words:
 // a group of 4 columns of every urows-th such row per thread, 4 rows (large n:
 // 8) in flight.
-template <int NT, int Q, typename FE>
+template <int NT, typename FE>
 __device__ __forceinline__ void rot_update_m(const RotThread& T, char* gM, uint32_t aM,
                                              uint32_t aVw, uint32_t aVwu, int n, int ldm,
-                                             int slot) {
+                                             int Q, int slot) {
   using P = RotPending<NT, FE>;
   constexpr int B = rot_big(NT) ? 8 : 4;
   if (T.ux >= T.urows) return;
@@ -632,8 +679,30 @@ __device__ __forceinline__ int rot_pair(const RotSmem<NT, FE>& S, const InstArgs
   return ((M[u * ldm + v] + M[v * ldm + u]) << (I.symF && I.symD ? 1 : 0)) + f * p - 2 * I.g0;
 }
 
+// d's slots with the partner of residue and parity x (the same in every lane),
+// where the lane holds it: a branch tree.
+template <int LO, int HI, int NS>
+__device__ __forceinline__ void put_partner(int (&d)[NS], int x, bool hold, int w0, int w1) {
+  if constexpr (HI - LO > 4) {
+    constexpr int MID = (LO + HI) / 2;
+    if (x < MID) put_partner<LO, MID>(d, x, hold, w0, w1);
+    else put_partner<MID, HI>(d, x, hold, w0, w1);
+  } else {
+#pragma unroll
+    for (int y = LO; y < HI; ++y) {
+      const bool here = hold && x == y;
+      constexpr int STEP = 2;
+      const int q = 4 * (y >> 1) + (y & 1);
+      d[q] = here ? w0 : d[q];
+      d[q + STEP] = here ? w1 : d[q + STEP];
+    }
+  }
+}
+
 // The warps that hold pairs: the table, its update after each move, and the
-// scan for the next iteration.
+// scan for the next iteration.  Slot group i of a thread holds the partner
+// block of residue i mod C in its window: a block has the same group in every
+// thread, so that the two columns of a move are written by one uniform branch.
 template <int NT, int C, typename FE>
 __device__ __forceinline__ void rot_owner() {
   using S = RotSmem<NT, FE>;
@@ -641,10 +710,10 @@ __device__ __forceinline__ void rot_owner() {
   const InstArgs& I = W.I;
   const int aspiration = W.s.aspiration;
   const RotThread T = rot_thread<NT, C>(I.n);
-  const int n = T.n, n2 = T.n2, nE = T.nE, m = T.m;
+  const int n = T.n, nc = T.nc, nE = T.nE, m = T.m;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int v0 = 2 * m, v1 = v0 + 1;
-  const bool half = v1 >= n;  // the block's second index is the phantom of an odd n
+  const bool half = v1 >= n || T.extra;  // no candidates from the second row: a phantom
   constexpr bool RANK = rot_rank(NT);
   constexpr int SB = rot_key_bits(NT);
   constexpr uint32_t MUL = 1u << SB;
@@ -652,6 +721,16 @@ __device__ __forceinline__ void rot_owner() {
   static_assert(!RANK || 2 * C < TOP, "ranks fit below the top bit");
   constexpr int BIG = 1 << (31 - SB);  // on top of a tabu pair's d
   constexpr int NS = 4 * C + 1;        // slots; the last holds the pair inside the block
+
+  // position of slot group i's block, and its offset in arrays of two words
+  // per block
+  const int c0 = T.pb % C;
+  int o0 = 8 * (T.pb - c0), o1 = o0 + 8 * C;
+  auto off = [&](int i) { return (i < c0 ? o1 : o0) + 8 * i; };
+  // many slots leave no registers to hold the offsets from one use to the next
+  auto again = [&] {
+    if constexpr (C > 13) asm volatile("" : "+r"(o0), "+r"(o1));
+  };
 
   // the table: from where rot_start left it, or (large n) by the pairs
   int32_t* const mark = S(I, n, W.notr != 0).mark();
@@ -664,7 +743,7 @@ __device__ __forceinline__ void rot_owner() {
   };
 #pragma unroll
   for (int i = 0; i < C; ++i) {
-    const int b = T.pb + i < n2 ? T.pb + i : T.pb + i - n2;
+    const int b = off(i) / 8 < nc ? off(i) / 8 : off(i) / 8 - nc;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       d[4 * i + q] = d_init(v0 + (q >> 1), 2 * b + (q & 1));
@@ -676,22 +755,25 @@ __device__ __forceinline__ void rot_owner() {
   d[4 * C] = d_init(v0, v1);
   rot_barrier();  // the others now clear the marks
 
-  const int2* const X = reinterpret_cast<const int2*>(S::X());
-  const int2* const psi = reinterpret_cast<const int2*>(S::psi());
-  const int2* const X2 = reinterpret_cast<const int2*>(S::X2());  // int16 flows
-  const int4* const R = reinterpret_cast<const int4*>(S::R());
+  // arrays of two words per block, by byte offset
+  auto two = [](const int32_t* a, int at) {
+    return *reinterpret_cast<const int2*>(reinterpret_cast<const char*>(a) + at);
+  };
 
   // Scan of the table: the warp's candidate into red.  A tabu pair aspires
   // when its delta is below `lim` (at most 0, at least NOLIM).
   constexpr int NOLIM = -(INT_MAX >> SB);
   auto scan = [&](int lim) {
+    again();
     int m0 = INT_MAX, m1 = INT_MAX;
     uint32_t t0 = 0xffffffffu, t1 = 0xffffffffu;
 #pragma unroll
     for (int i = 0; i < C; ++i) {
-      const int2 y = psi[T.pb + i];
-      const uint32_t y0 = (uint32_t)y.x + (RANK ? 2 * i + 1 : 0);  // (the pair inside: rank 0)
-      const uint32_t y1 = (uint32_t)y.y + (RANK ? 2 * i + 2 : 0);
+      const int2 y = two(S::psi(), off(i));
+      // rank: twice the block's place in the window, from 1 (the pair inside: 0)
+      const uint32_t rk = RANK ? (uint32_t)((i < c0 ? 2 * C : 0) - 2 * c0) : 0u;
+      const uint32_t y0 = (uint32_t)y.x + rk + (RANK ? 2 * i + 1 : 0);
+      const uint32_t y1 = (uint32_t)y.y + rk + (RANK ? 2 * i + 2 : 0);
       const uint32_t e00 = (uint32_t)d[4 * i] * MUL + y0;
       const uint32_t e01 = (uint32_t)d[4 * i + 1] * MUL + y1;
       const uint32_t e10 = (uint32_t)d[4 * i + 2] * MUL + y0;
@@ -701,9 +783,11 @@ __device__ __forceinline__ void rot_owner() {
       t0 = min(t0, min(e00, e01));
       t1 = min(t1, min(e10, e11));
     }
-    const int2 o = psi[m];
+    const int2 o = two(S::psi(), 8 * m);
     {
-      const uint32_t e = (uint32_t)d[4 * C] * MUL + (uint32_t)o.y;
+      // the pair inside the block: its first thread offers it
+      uint32_t e = (uint32_t)d[4 * C] * MUL + (uint32_t)o.y;
+      e = warp * 32 + lane == m ? e : INT_MAX;
       m0 = min(m0, (int)e);
       t0 = min(t0, e);
     }
@@ -712,19 +796,20 @@ __device__ __forceinline__ void rot_owner() {
     const uint32_t q0 = (uint32_t)o.x - (RANK ? TOP : v0) + 0x80000000u;
     const uint32_t q1 = (uint32_t)o.y - (RANK ? TOP : v1) + 0x80000000u;
     const int ls = (int)((uint32_t)lim * MUL);
-    int c0 = m0 < 0 ? (int)((uint32_t)m0 + q0) : INT_MAX;
-    int c1 = m1 < 0 ? (int)((uint32_t)m1 + q1) : INT_MAX;
+    int b0 = m0 < 0 ? (int)((uint32_t)m0 + q0) : INT_MAX;
+    int b1 = m1 < 0 ? (int)((uint32_t)m1 + q1) : INT_MAX;
     const int x0 = (int)(t0 + q0 + 0x80000000u), x1 = (int)(t1 + q1 + 0x80000000u);
-    if ((int)t0 >= 0 && x0 < ls) c0 = min(c0, x0);
-    if ((int)t1 >= 0 && x1 < ls) c1 = min(c1, x1);
-    if (half) c1 = INT_MAX;  // the phantom's row
+    if ((int)t0 >= 0 && x0 < ls) b0 = min(b0, x0);
+    if ((int)t1 >= 0 && x1 < ls) b1 = min(b1, x1);
+    if (half) b1 = INT_MAX;
+    if (T.extra) b0 = INT_MAX;
     // the lower pair of the two rows
-    const int d0 = c0 >> SB, d1 = c1 >> SB;
-    int u0 = c0 & (int)(MUL - 1), u1 = c1 & (int)(MUL - 1);
+    const int d0 = b0 >> SB, d1 = b1 >> SB;
+    int u0 = b0 & (int)(MUL - 1), u1 = b1 & (int)(MUL - 1);
     if (RANK) {
       u0 = (u0 & (TOP - 1)) + 2 * T.pb - 1;
       u0 = u0 >= nE ? u0 - nE : u0;
-      u0 = (c0 & (TOP - 1)) == 0 ? v1 : u0;
+      u0 = (b0 & (TOP - 1)) == 0 ? v1 : u0;
       u1 = (u1 & (TOP - 1)) + 2 * T.pb - 1;
       u1 = u1 >= nE ? u1 - nE : u1;
     }
@@ -747,49 +832,39 @@ __device__ __forceinline__ void rot_owner() {
     c.best = c.tabu_phase ? min(c.best, c.cur) : c.cur;
     using Cost = typename RotCourse<FE>::Cost;
     const int lim = aspiration ? (int)max(c.best - c.cur, (Cost)NOLIM) : NOLIM;
-    // pairs whose tabu time ends with the next iteration (in the shadow of
-    // phase X)
+    // slots whose tabu time ends with the next iteration
     uint32_t w = S::ring()[(it + 1) & (rot_ring(NT) - 1)];
-    while (__builtin_expect(w != 0xffffffffu, 1)) {
-      const int u = (int)(w >> 8 & 0xffu), v = (int)(w & 0xffu);
-      const int bu = u >> 1, bv = v >> 1;
-      const bool own_u = m == bu;
-      int kx = (own_u ? bv : bu) - T.pbm;  // slot group of the other one
-      kx = kx < 0 ? kx + n2 : kx;
-      int q = 4 * kx + (own_u ? 2 * (u & 1) + (v & 1) : 2 * (v & 1) + (u & 1));
-      q = bu == bv ? 4 * C : q;
-      // (applied again since: its end is another)
-      const int at = v * (v - 1) / 2 + u;
-      const bool ends = rot_big(NT) ? reinterpret_cast<const uint16_t*>(mark)[at] ==
-                                          rot_mark16(it + 1)
-                                    : mark[at] == it + 1;
-      const bool hold = ends && (own_u || m == bv) && (kx < C || bu == bv);
-      for (unsigned b = __ballot_sync(kFull, hold); b; b &= b - 1) {
-        const int src = __ffs(b) - 1;
-        clear_tabu<0, NS>(d, __shfl_sync(kFull, q, src), lane == src ? BIG : 0);
-      }
+    while (w != 0xffffffffu) {
+      const int at = (int)(w & 0xffffu) >> rot_slot_bits(NT);
+      if (at >> 5 == warp)
+        clear_tabu<0, NS>(d, (int)w & ((1 << rot_slot_bits(NT)) - 1),
+                          (at & 31) == lane ? BIG : 0);
       w = w >> 16 == 0xffffu ? 0xffffffffu : S::node()[w >> 16];
     }
     const int br = r >> 1, bs = s >> 1;
-    int kr = br - T.pbm, ks = bs - T.pbm;  // slot groups of r and s as partners, if below C
-    kr = kr < 0 ? kr + n2 : kr;
-    ks = ks < 0 ? ks + n2 : ks;
+    // slot groups of r and s as partners, and whether the thread holds them
+    const int xr = 2 * (br % C) + (r & 1), xs = 2 * (bs % C) + (s & 1);
+    int kr = br - T.pbm, ks = bs - T.pbm;
+    kr = kr < 0 ? kr + nc : kr;
+    ks = ks < 0 ? ks + nc : ks;
+    const bool hold_r = kr < C, hold_s = ks < C;
     const bool row0 = v0 == r || v0 == s, row1 = v1 == r || v1 == s;
     rot_barrier();
 
     // the new table
-    const int4 Rm = R[m];  // the pairs (v0, r), (v0, s), (v1, r), (v1, s)
+    again();
+    const int2 wr = two(S::Rr(), 8 * m), ws = two(S::Rs(), 8 * m);  // v0, v1 with r, with s
     if constexpr (sizeof(FE) == 1) {
-      const int2 A = reinterpret_cast<const int2*>(S::own())[m];
+      const int2 A = two(S::own(), 8 * m);
 #pragma unroll
       for (int i = 0; i < C; ++i) {
-        const int2 x = X[T.pb + i];
+        const int2 x = two(S::X(), off(i));
         d[4 * i] = __dp4a(A.x, x.x, d[4 * i]);
         d[4 * i + 1] = __dp4a(A.x, x.y, d[4 * i + 1]);
         d[4 * i + 2] = __dp4a(A.y, x.x, d[4 * i + 2]);
         d[4 * i + 3] = __dp4a(A.y, x.y, d[4 * i + 3]);
       }
-      d[4 * C] = __dp4a(A.x, X[m].y, d[4 * C]);
+      d[4 * C] = __dp4a(A.x, S::X()[v1], d[4 * C]);
     } else {
       // (-a, -c) of a row with the partner's (b, e), its (-b, -e) with (a, c)
       const int4 A = reinterpret_cast<const int4*>(S::own())[m];
@@ -798,56 +873,188 @@ __device__ __forceinline__ void rot_owner() {
       };
 #pragma unroll
       for (int i = 0; i < C; ++i) {
-        const int2 x = X[T.pb + i], x2 = X2[T.pb + i];
+        const int2 x = two(S::X(), off(i)), x2 = two(S::X2(), off(i));
         d[4 * i] = upd(A.x, A.y, x.x, x2.x, d[4 * i]);
         d[4 * i + 1] = upd(A.x, A.y, x.y, x2.y, d[4 * i + 1]);
         d[4 * i + 2] = upd(A.z, A.w, x.x, x2.x, d[4 * i + 2]);
         d[4 * i + 3] = upd(A.z, A.w, x.y, x2.y, d[4 * i + 3]);
       }
-      d[4 * C] = upd(A.x, A.y, X[m].y, X2[m].y, d[4 * C]);
+      d[4 * C] = upd(A.x, A.y, S::X()[v1], S::X2()[v1], d[4 * C]);
     }
-    // partners r and s
-    auto partner = [&](int kk, bool odd, int w0, int w1) {
-      if (odd) {
-#pragma unroll
-        for (int i = 0; i < C; ++i) {
-          d[4 * i + 1] = kk == i ? w0 : d[4 * i + 1];
-          d[4 * i + 3] = kk == i ? w1 : d[4 * i + 3];
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < C; ++i) {
-          d[4 * i] = kk == i ? w0 : d[4 * i];
-          d[4 * i + 2] = kk == i ? w1 : d[4 * i + 2];
-        }
-      }
-    };
-    partner(kr, r & 1, Rm.x, Rm.z);
-    partner(ks, s & 1, Rm.y, Rm.w);
-    // the rows of r and s
+    // the columns of r and s
+    put_partner<0, 2 * C>(d, xr, hold_r, wr.x, wr.y);
+    put_partner<0, 2 * C>(d, xs, hold_s, ws.x, ws.y);
+    // their rows
     if (row0 || row1) {
-      const int* const x0 = reinterpret_cast<const int*>(R) + (v0 == r ? 0 : 1);
-      const int* const x1 = reinterpret_cast<const int*>(R) + (v1 == r ? 0 : 1);
+      again();
       if (row0) {
+        const int32_t* const x = v0 == r ? S::Rr() : S::Rs();
 #pragma unroll
         for (int i = 0; i < C; ++i) {
-          d[4 * i] = x0[4 * (T.pb + i)];
-          d[4 * i + 1] = x0[4 * (T.pb + i) + 2];
+          const int2 y = two(x, off(i));
+          d[4 * i] = y.x;
+          d[4 * i + 1] = y.y;
         }
-        d[4 * C] = x0[4 * m + 2];
+        d[4 * C] = x[v1];
       }
       if (row1) {
+        const int32_t* const x = v1 == r ? S::Rr() : S::Rs();
 #pragma unroll
         for (int i = 0; i < C; ++i) {
-          d[4 * i + 2] = x1[4 * (T.pb + i)];
-          d[4 * i + 3] = x1[4 * (T.pb + i) + 2];
+          const int2 y = two(x, off(i));
+          d[4 * i + 2] = y.x;
+          d[4 * i + 3] = y.y;
         }
-        d[4 * C] = x1[4 * m];
+        d[4 * C] = x[v0];
       }
     }
     scan(lim);
   }
 }
+
+// The tabu times and the hash of a walk, kept by one warp beside the scan.
+template <int NT, int C, typename FE>
+struct RotKeeper {
+  using S = RotSmem<NT, FE>;
+  static constexpr bool M16 = rot_big(NT);
+  static constexpr int RING = rot_ring(NT), SL = rot_slot_bits(NT);
+  static constexpr uint64_t kH0 = 14695981039346656037ull;
+  const int n2, nc, J, iters, p_stride;
+  int32_t* const mark;
+  int32_t* const fq;
+  uint64_t h, dh;
+  bool was_tabu;
+  int2 late;     // lane 0: the last move, while its slots are to be hung
+  int late_end;  // the end of its tabu time (0: none)
+
+  __device__ __forceinline__ RotKeeper(const RotWalkArgs& W, const RotThread& T, int32_t* marks)
+      : n2(T.n2), nc(T.nc), J(T.J), iters(W.s.iters), p_stride(W.s.p_stride), mark(marks),
+        fq(W.s.freq ? W.s.freq + (size_t)W.row * W.s.p_stride * W.s.p_stride : nullptr), h(kH0),
+        dh(kH0), was_tabu(!W.s.descend), late(make_int2(0, 0)), late_end(0) {}
+
+  // The tenure of an iteration, one of the 32 that the warp draws ahead.
+  __device__ __noinline__ static void tenures(int it) {
+    const RotWalkArgs& W = S::args();
+    S::ten()[(it - 1) & 63] = RotTenure(W.s, W.I.n).of(W.s.seed, W.wid, it);
+  }
+
+  // The slot that block u's threads hold pair (u, v) in, or -1 when v is not
+  // in their windows.
+  __device__ __forceinline__ int slot(int u, int v) const {
+    const int bu = u >> 1, bv = v >> 1;
+    int o = bv - bu;
+    o = (o < 0 ? o + nc : o) - 1;
+    const int j = o / C;
+    return j < J ? (j * n2 + bu) << SL | (4 * (bv % C) + 2 * (u & 1) + (v & 1)) : -1;
+  }
+  // The slots of a pair, one or two (the one inside a block is its first
+  // thread's).
+  __device__ __forceinline__ int2 slots(int r, int s) const {
+    if (r >> 1 == s >> 1) return make_int2((r >> 1) << SL | 4 * C, -1);
+    const int a = slot(r, s), b = slot(s, r);
+    return a >= 0 ? make_int2(a, b) : make_int2(b, -1);
+  }
+  // The pair of a slot, as its place in the triangle of marks.
+  __device__ __forceinline__ int pair_at(int w) const {
+    const int t = w >> SL, q = w & ((1 << SL) - 1), j = t / n2, m = t - j * n2;
+    int v = 2 * m, u = v + 1;
+    if (q < 4 * C) {
+      const int pb = m + 1 + j * C, c0 = pb % C, i = q >> 2;
+      const int b = pb - c0 + i + (i < c0 ? C : 0);
+      v += q >> 1 & 1;
+      u = 2 * (b < nc ? b : b - nc) + (q & 1);
+    }
+    const int hi = max(u, v);
+    return hi * (hi - 1) / 2 + min(u, v);
+  }
+  __device__ __forceinline__ void hang(uint32_t w, int end, uint32_t node) const {
+    uint32_t* const at = S::ring() + (end & (RING - 1));
+    const uint32_t old = *at;
+    if (old != 0xffffffffu) S::node()[node] = old;
+    *at = w | (old != 0xffffffffu ? node : 0xffffu) << 16;
+  }
+  // Take a slot off the ring word of iteration `end`.
+  __device__ __noinline__ static void unhang(uint32_t w, int end) {
+    uint32_t* at = S::ring() + (end & (RING - 1));
+    while (*at != 0xffffffffu) {
+      const uint32_t next = *at >> 16;
+      if ((*at & 0xffffu) == w) {
+        *at = next == 0xffffu ? 0xffffffffu : S::node()[next];
+      } else {
+        if (next == 0xffffu) break;
+        at = S::node() + next;
+      }
+    }
+  }
+
+  // Move (r, s) of iteration `it` (0 in the descent), by the whole warp.  With
+  // LATE the slots are hung by finish(), after the next barrier, unless the
+  // pairs' warps may read the ring word by then.
+  template <bool LATE>
+  __device__ __forceinline__ void move(int r, int s, int it) {
+    const int lane = threadIdx.x & 31;
+    if (it > 0) {
+      const int end = it + S::ten()[(it - 1) & 63];
+      __syncwarp();  // (its place takes the tenure of iteration it + 64)
+      if ((it & 31) == 0) tenures(it + 33 + lane);
+      if (lane == 0) {
+        const int at = s * (s - 1) / 2 + r;
+        // a pair applied while tabu: its old end no longer counts
+        int old = 0;
+        if constexpr (M16) {
+          uint16_t* const m = reinterpret_cast<uint16_t*>(mark);
+          // the marks that end with the next iteration
+          for (uint32_t x = S::ring()[(it + 1) & (RING - 1)]; x != 0xffffffffu;
+               x = x >> 16 == 0xffffu ? 0xffffffffu : S::node()[x >> 16])
+            m[pair_at((int)(x & 0xffffu))] = 0;
+          old = m[at] & 0x7fff;
+          m[at] = end > it + 1 ? (uint16_t)rot_mark16(end) : 0;
+        } else {
+          old = mark[at] > it + 1 ? mark[at] : 0;
+          mark[at] = end;
+        }
+        // the ring word of the iteration just served is free again
+        S::ring()[(it + 1) & (RING - 1)] = 0xffffffffu;
+        late = make_int2(r << 8 | s, it);
+        late_end = end;
+        if (old != 0) {
+          int2 w = slots(r, s);
+#pragma unroll 1
+          for (; w.x >= 0; w = make_int2(w.y, -1)) unhang((uint32_t)w.x, old);
+        }
+        if (!LATE || end <= it + 2) finish();
+        if (fq) atomicAdd(fq + s * p_stride + r, 1);
+      }
+      if (!was_tabu) {  // the first tabu move
+        was_tabu = true;
+        dh = h;
+        h = kH0;
+      }
+    }
+    h = fnv_step(h, r, s);
+  }
+  // The last move's slots on the ring, by lane 0.
+  __device__ __forceinline__ void finish() {
+    const int it = late.y;
+    if (late_end > it + 1 && late_end <= iters) {
+      int2 w = slots(late.x >> 8, late.x & 0xff);
+      uint32_t node = 2 * ((uint32_t)it & (RING - 1));
+#pragma unroll 1
+      for (; w.x >= 0; w = make_int2(w.y, -1)) hang((uint32_t)w.x, late_end, node++);
+    }
+    late_end = 0;
+  }
+
+  __device__ __forceinline__ void results(const SearchArgs& a, int row) {
+    if ((threadIdx.x & 31) != 0) return;
+    if (!was_tabu) {
+      dh = h;
+      h = kH0;
+    }
+    if (a.hash) a.hash[row] = h;
+    if (a.descent_hash) a.descent_hash[row] = dh;
+  }
+};
 
 // The phase X warps: one thread per index k (large n: two indices) computes what
 // move (r, s) changes (see phase_m_prep for the algebra), and keeps the labels, the pending words,
@@ -860,6 +1067,8 @@ __device__ __forceinline__ void rot_owner() {
 template <int NT, int C, bool SYM, typename FE>
 __device__ __forceinline__ void rot_phase_x() {
   constexpr int FB = sizeof(FE), KX = rot_kx(NT);
+  // the last warp may be one of these
+  constexpr bool KEEPS = rot_px(rot_max_n(NT), NT) + rot_owners(NT) > rot_threads(NT) - 32;
   constexpr bool PW2 = kRotWords<FE> == 2;
   using P = RotPending<NT, FE>;
   constexpr int RW = P::RW, LW = P::LW, Q = P::template Q<SYM>;
@@ -874,18 +1083,13 @@ __device__ __forceinline__ void rot_phase_x() {
   const RotSmem<NT, FE> S(I, T.n, W.notr != 0);
   const int n = T.n, ldF = I.ldF, ldP = I.ldP, ldm = ld_m(n), nE = T.nE;
   const int g0 = I.g0, g2 = 2 * g0;
-  const uint32_t wid = W.wid;
-  const uint64_t seed = W.s.seed;
-  int32_t* const fq = W.s.freq ? W.s.freq + (size_t)W.row * W.s.p_stride * W.s.p_stride : nullptr;
-  const int lane = threadIdx.x & 31;
-  const bool first = T.pt < 32;  // the first warp, that keeps the tabu times
   // addresses
   const uint32_t base = smem_addr(rot_smem);
   const uint32_t aF = base + S.L.F, aP = base + S.L.P, aM = rot_big(NT) ? 0 : base + S.L.M;
   const uint32_t aFt = base + S.ft, aPt = base + S.pt, aMark = base + S.L.mark;
   const uint32_t aVw = base + X_::vw, aVwu = base + X_::vwu, aSig = base + X_::sigma;
   const uint32_t aX = base + X_::X, aPsi = base + X_::psi, aOwn = base + X_::own;
-  const uint32_t aR = base + X_::R, aTen = base + X_::ten;
+  const uint32_t aRr = base + X_::Rr, aRs = base + X_::Rs, aTen = base + X_::ten;
   char* const gM = reinterpret_cast<char*>(W.M);
   // per index of the thread (past the last: a repeat of n - 1 that stores
   // nothing)
@@ -904,12 +1108,9 @@ __device__ __forceinline__ void rot_phase_x() {
     gk[j] = (S.M()[k[j] * ldm + k[j]] << (SYM ? 1 : 0)) - g0;
   }
   int best_iter = 0, mv = 0;
-  const RotTenure tenure(W.s, n);
-  const uint64_t h0 = 14695981039346656037ull;
-  uint64_t h = h0, dh = h0;
   rot_clear_marks<NT>(S.mark(), n, T.ow);
   RotCourse<FE> course(W, T.ow);
-  bool was_tabu = course.tabu_phase;
+  RotKeeper<NT, C, FE> keeper(W, T, S.mark());
 
   while (course.next(S.red())) {
     const int r = course.r, s = course.s, it = course.it;
@@ -1067,18 +1268,21 @@ __device__ __forceinline__ void rot_phase_x() {
         sts32(aPsi + 4 * nE + 4 * kj, rot_rank(NT) ? psi - TOP : psi);
         if constexpr (!PW2) sts32(aOwn + 4 * kj, (int)own);
         else sts64(aOwn + 8 * kj, (int)own, (int)own2);
-        sts64(aR + 8 * kj, Rr, Rs);
-        sts64(aR + 8 * nE + 8 * kj, Rr, Rs);
+        sts32(aRr + 4 * kj, Rr);
+        sts32(aRr + 4 * nE + 4 * kj, Rr);
+        sts32(aRs + 4 * kj, Rs);
+        sts32(aRs + 4 * nE + 4 * kj, Rs);
         if constexpr (RW == 1) sts32(aVw + wt + 4 * kj, wn.x);
         else sts64(aVw + 2 * wt + 8 * kj, wn.x, wn.y);
         if constexpr (LW == 1) sts32(aVwu + wt + 4 * uj, wuk.x);
         else sts64(aVwu + 2 * wt + 8 * uj, wuk.x, wuk.y);
       }
     }
+    if (T.pt == 0) S.red()[33] = make_int2(r << 8 | s, tabu_phase ? it : 0);  // for the keeper
     rot_barrier();
-    // while the other warps bring the table up to date: M, the labels, the
-    // best solution, the tabu times and the hash
-    rot_update_m<NT, Q, FE>(T, gM, aM, aVw + RW * wt, aVwu + LW * wt, n, ldm, slot);
+    // while the other warps bring the table up to date: M, the labels and the
+    // best solution
+    rot_update_m<NT, FE>(T, gM, aM, aVw + RW * wt, aVwu + LW * wt, n, ldm, Q, slot);
     ++mv;
     const bool better = !tabu_phase || course.cur < course.best;
 #pragma unroll
@@ -1091,53 +1295,7 @@ __device__ __forceinline__ void rot_phase_x() {
     }
     course.best = better ? course.cur : course.best;
     best_iter = better ? it : best_iter;  // 0 in the descent
-    if (first) {
-      if (tabu_phase && !was_tabu) {  // this was the first tabu move
-        was_tabu = true;
-        dh = h;
-        h = h0;
-      }
-      h = fnv_step(h, r, s);
-      if (tabu_phase) {
-        if ((it & 31) == 0)  // the tenures of iterations it + 33 .. it + 64
-          S.ten()[(it + 32 + lane) & 63] = tenure.of(seed, wid, it + 33 + lane);
-        if (T.pt == 0) {
-          const int end = it + ten;
-          uint32_t* const now = S.ring() + ((it + 1) & (rot_ring(NT) - 1));
-          if constexpr (M16) {
-            // the marks that end with the next iteration
-            uint16_t* const mark = reinterpret_cast<uint16_t*>(S.mark());
-            for (uint32_t w = *now; w != 0xffffffffu;
-                 w = w >> 16 == 0xffffu ? 0xffffffffu : S.node()[w >> 16]) {
-              const int u = (int)(w >> 8 & 0xffu), v = (int)(w & 0xffu);
-              uint16_t* const m = mark + v * (v - 1) / 2 + u;
-              if (*m == rot_mark16(it + 1)) *m = 0;
-            }
-            mark[stri + r] = end > it + 1 ? (uint16_t)rot_mark16(end) : 0;
-          } else {
-            S.mark()[stri + r] = end;
-          }
-          // the ring word of the iteration just served is free again
-          *now = 0xffffffffu;
-          if (end > it + 1 && end <= course.iters) {
-            uint32_t* const at = S.ring() + (end & (rot_ring(NT) - 1));
-            const uint32_t old = *at, key = (uint32_t)(r << 8 | s);
-            const uint32_t nd = (uint32_t)it & (rot_ring(NT) - 1);
-            // (there already when the pair, applied while tabu, ends when it
-            // once did: the owners would clear its bit twice)
-            bool there = false;
-            for (uint32_t w = old; w != 0xffffffffu;
-                 w = w >> 16 == 0xffffu ? 0xffffffffu : S.node()[w >> 16])
-              there |= (w & 0xffffu) == key;
-            if (!there) {
-              if (old != 0xffffffffu) S.node()[nd] = old;
-              *at = key | (old != 0xffffffffu ? nd : 0xffffu) << 16;
-            }
-          }
-          if (fq) atomicAdd(fq + s * W.s.p_stride + r, 1);
-        }
-      }
-    }
+    if (KEEPS && T.keeper) keeper.template move<false>(r, s, tabu_phase ? it : 0);
   }
 
   // ---- outputs
@@ -1147,47 +1305,47 @@ __device__ __forceinline__ void rot_phase_x() {
   for (int j = 0; j < KX; ++j)
     if (a.best_p && live[j]) a.best_p[(size_t)row * a.p_stride + k[j]] = S.p0()[best_uk[j]];
   if (T.pt == 0) {
-    if (!was_tabu) {
-      dh = h;
-      h = h0;
-    }
     a.best_cost[row] = (int64_t)course.best;
     if (a.final_cost) a.final_cost[row] = (int64_t)course.cur;
     if (a.best_iter) a.best_iter[row] = best_iter;
     if (a.iters_done) a.iters_done[row] = course.it;
     if (a.status) a.status[row] = course.stalled && course.it < course.iters ? 1 : 0;
     if (a.descent_moves) a.descent_moves[row] = course.dmoves;
-    if (a.hash) a.hash[row] = h;
-    if (a.descent_hash) a.descent_hash[row] = dh;
   }
+  if (KEEPS && T.keeper) keeper.results(a, row);
 }
 
 // The other warps: M's update, until the flag beside the candidates is set.
-template <int NT, int C, bool SYM, typename FE>
+template <int NT, int C, typename FE>
 __device__ __forceinline__ void rot_helper() {
   using P = RotPending<NT, FE>;
-  constexpr int Q = P::template Q<SYM>;
   using X_ = RotFixed<NT, FE>;
   const RotWalkArgs& W = RotSmem<NT, FE>::args();
   const RotThread T = rot_thread<NT, C>(W.I.n);
   const RotSmem<NT, FE> S(W.I, T.n, W.notr != 0);
   const int n = T.n, ldm = ld_m(n);
+  const int Q = W.I.symF && W.I.symD ? P::template Q<true> : P::template Q<false>;
   const uint32_t base = smem_addr(rot_smem);
   rot_clear_marks<NT>(S.mark(), n, T.ow);
+  RotKeeper<NT, C, FE> keeper(W, T, S.mark());
   for (int mv = 0;; ++mv) {
     rot_barrier();
+    if (T.keeper && (threadIdx.x & 31) == 0) keeper.finish();
     rot_barrier();
     if (lds32(base + X_::red + 8 * 32)) break;
+    const int2 move = lds64(base + X_::red + 8 * 33);
     const uint32_t wt = mv & 1 ? 0 : 4 * ldm;
-    rot_update_m<NT, Q, FE>(T, reinterpret_cast<char*>(W.M), rot_big(NT) ? 0 : base + S.L.M,
-                            base + X_::vw + P::RW * wt, base + X_::vwu + P::LW * wt, n, ldm,
-                            mv & (Q - 1));
+    if (T.keeper) keeper.template move<true>(move.x >> 8, move.x & 0xff, move.y);
+    rot_update_m<NT, FE>(T, reinterpret_cast<char*>(W.M), rot_big(NT) ? 0 : base + S.L.M,
+                         base + X_::vw + P::RW * wt, base + X_::vwu + P::LW * wt, n, ldm, Q,
+                         mv & (Q - 1));
   }
+  if (T.keeper) keeper.results(W.s, W.row);
 }
 
 // The start of a walk: permutation, P0, M, the scan addends and the cost.
 // Starts and ends with every thread of the CTA together.
-template <int NT, typename FE>
+template <int NT, int C, typename FE>
 __device__ __forceinline__ void rot_start() {
   constexpr int TH = rot_threads(NT);
   RotWalkArgs& W = RotSmem<NT, FE>::args();
@@ -1200,15 +1358,17 @@ __device__ __forceinline__ void rot_start() {
   const RotSmem<NT, FE> S(I, n, notr);
   const int lane = tid & 31, warp = tid >> 5;
   const bool sym = I.symF && I.symD;
-  const int ldm = ld_m(n), nE = (n + 1) / 2 * 2, g0 = I.g0;
+  const int ldm = ld_m(n), nE = 2 * rot_circle(n, C), g0 = I.g0;
   const int hsh = sym ? 1 : 0;  // M is stored halved
   constexpr int SB = rot_key_bits(NT);
 
   // ---- start permutation: given, or Fisher-Yates on stream 0 (the draws by
   // all threads, the exchanges by one)
   if (start) {
+#pragma unroll 1
     for (int x = tid; x < n; x += TH) S.p0()[x] = start[x];
   } else {
+#pragma unroll 1
     for (int i = tid; i < n; i += TH) {
       S.p0()[i] = i;
       if (i >= 1) S.vw()[i] = (int)below(walk_draw(a.seed, wid, 0u, (uint32_t)(n - 1 - i)),
@@ -1230,6 +1390,7 @@ __device__ __forceinline__ void rot_start() {
     const int8_t* Dg = static_cast<const int8_t*>(I.D);
     const bool tr = !I.symD && !notr;
     int8_t* Pt = S.Pt();
+#pragma unroll 1
     for (int i = warp; i < n; i += TH / 32) {
       const int8_t* Di = Dg + (size_t)S.p0()[i] * n;
       for (int j = lane; j < n; j += 32) {
@@ -1238,22 +1399,28 @@ __device__ __forceinline__ void rot_start() {
         if (tr) Pt[j * ldP + i] = v;
       }
     }
+#pragma unroll 1
     for (int x = tid; x < n; x += TH) S.sigma()[x] = x;
     // phantom indices: never candidates, never updated
+#pragma unroll 1
     for (int x = n + tid; x < nE; x += TH) {
       S.X()[x] = S.X()[x + nE] = 0;
       S.psi()[x] = S.psi()[x + nE] = INT_MAX - 128;
-      S.R()[x] = S.R()[x + nE] = make_int2(0, 0);
+      S.Rr()[x] = S.Rr()[x + nE] = S.Rs()[x] = S.Rs()[x + nE] = 0;
       for (int w = 0; w < kRotWords<FE>; ++w) S.own()[kRotWords<FE> * x + w] = 0;
       if (kRotWords<FE> == 2) S.X2()[x] = S.X2()[x + nE] = 0;
     }
     // no pending moves; M's padding columns take updates from these words only
     using Pd = RotPending<NT, FE>;
+#pragma unroll 1
     for (int x = tid; x < 2 * Pd::LW * ldm; x += TH) S.vwu()[x] = 0;
+#pragma unroll 1
     for (int x = tid; x < 2 * Pd::RW * ldm; x += TH) S.vw()[x] = 0;
+#pragma unroll 1
     for (int x = tid; x < rot_ring(NT); x += TH) S.ring()[x] = 0xffffffffu;
     if (a.iters > 0) {
       const RotTenure tenure(a, n);
+#pragma unroll 1
       for (int x = tid; x < 64; x += TH) S.ten()[x] = tenure.of(a.seed, wid, x + 1);
     }
     if (tid == 0) S.red()[32] = make_int2(0, 0);
@@ -1270,6 +1437,7 @@ __device__ __forceinline__ void rot_start() {
   // ---- scan addends of every index; the walk's cost (Eq. 1): M's diagonal
   // sums to twice the cost
   int64_t c0 = 0;
+#pragma unroll 1
   for (int x = tid; x < n; x += TH) {
     const int mxx = S.M()[x * ldm + x];
     c0 += mxx;
@@ -1290,15 +1458,14 @@ __device__ __forceinline__ void rot_start() {
 // and ends with every thread of the CTA together.
 template <int NT, int C, typename FE>
 __device__ __forceinline__ void rot_walk() {
-  rot_start<NT, FE>();
+  rot_start<NT, C, FE>();
   const RotWalkArgs& W = RotSmem<NT, FE>::args();
   const int role = rot_thread<NT, C>(W.I.n).role;
   const bool sym = W.I.symF && W.I.symD;
   if (role == 0) rot_owner<NT, C, FE>();
   else if (role == 1 && sym) rot_phase_x<NT, C, true, FE>();
   else if (role == 1) rot_phase_x<NT, C, false, FE>();
-  else if (sym) rot_helper<NT, C, true, FE>();
-  else rot_helper<NT, C, false, FE>();
+  else rot_helper<NT, C, FE>();
   __syncthreads();
 }
 
@@ -1325,17 +1492,6 @@ __device__ __forceinline__ void rot_load(const InstArgs& I, bool notr) {
     if (pt) rot_at<int4>(L.Pt)[i] = zero;
   }
   __syncthreads();
-}
-
-// The partner blocks per thread (C) compiled for a shape: below 16 (large n: 32)
-// for their ranks.
-constexpr int kRotMaxC = 22;
-__host__ __device__ constexpr bool rot_compiled(int nt, int c) {
-  return rot_big(nt)  ? c == 8 || c == 10 || c == 12 || c == 16 || c == 19 || c == 22
-         : nt == 128  ? c == 1 || c == 2 || c == 4 || c == 7
-         : nt == 256  ? c <= 4 || c == 6 || c == 7 || c == 11 || c == 13
-         : nt == 512  ? c <= 3 || c == 5 || c == 7 || c == 8 || c == 11 || c == 13
-                      : c == 2 || c == 4 || c == 5 || c == 6;
 }
 
 // CTAs per SM to compile for.

@@ -21,21 +21,28 @@ void fail(const char* what, int n, int nt, int c) {
 void check(int n, int nt, int c) {
   const int J = qapk::rot_chunks(n, nt, c);
   if (J == 0) return;
-  const int n2 = (n + 1) / 2, nE = 2 * n2;
-  if (n > qapk::rot_max_n(nt)) fail("fixed arrays too small", n, nt, c);
+  const int n2 = (n + 1) / 2, nc = qapk::rot_circle(n, c), nE = 2 * nc;
+  if (nc % c != 0 || nc < n2) fail("circle", n, nt, c);
+  if (n > qapk::rot_max_n(nt) || nE > qapk::rot_max_e(nt)) fail("fixed arrays too small", n, nt, c);
   if (qapk::ld_m(n) > qapk::rot_max_n(nt) + 4) fail("pending words too small", n, nt, c);
   if (J * n2 > qapk::rot_owners(nt)) fail("too many pair threads", n, nt, c);
-  if (n > qapk::rot_kx(nt) * (qapk::rot_threads(nt) - qapk::rot_owners(nt))) fail("no thread per index", n, nt, c);
+  if (n > qapk::rot_kx(nt) * (qapk::rot_threads(nt) - qapk::rot_owners(nt)))
+    fail("no thread per index", n, nt, c);
   if (qapk::rot_rank(nt) ? 2 * c >= 1 << (qapk::rot_key_bits(nt) - 1)
-                         : nE > 1 << qapk::rot_key_bits(nt))
+                         : n > 1 << qapk::rot_key_bits(nt))
     fail("partner does not fit the key bits", n, nt, c);
+  if (4 * c >= 1 << qapk::rot_slot_bits(nt) ||
+      (J * n2 - 1) << qapk::rot_slot_bits(nt) >= 0xffff - (1 << qapk::rot_slot_bits(nt)))
+    fail("a slot does not fit 16 bits", n, nt, c);
   std::vector<char> held((size_t)nE * nE, 0);
   for (int tid = 0; tid < J * n2; ++tid) {
-    const int j = tid / n2, m = tid - j * n2, pb = m + 1 + j * c;
-    held[(size_t)2 * m * nE + 2 * m + 1] = 1;
-    if (pb + c - 1 >= 2 * n2) fail("window beyond the doubled circle", n, nt, c);
+    const int j = tid / n2, m = tid - j * n2, pb = m + 1 + j * c, c0 = pb % c;
+    if (j == 0) held[(size_t)2 * m * nE + 2 * m + 1] = 1;
     for (int i = 0; i < c; ++i) {
-      const int b = (pb + i) % n2;
+      // the block of residue i in the window [pb, pb + c)
+      const int pos = pb - c0 + i + (i < c0 ? c : 0), b = pos % nc;
+      if (pos < pb || pos >= pb + c || b % c != i) fail("slot group off its window", n, nt, c);
+      if (pos >= 2 * nc) fail("window beyond the doubled circle", n, nt, c);
       if (b == m) fail("a block against itself", n, nt, c);
       for (int q = 0; q < 4; ++q) {
         const int v = 2 * m + (q >> 1), u = 2 * b + (q & 1);

@@ -38,8 +38,8 @@ def check(F, D, W, threads=0, flow_bytes=1, **kw):
 # the last n of a warp of phase X, of the fixed arrays, and of a plan; n = 40:
 # the triangle of marks ends on a 16-byte boundary
 @pytest.mark.parametrize("sym", [False, True])
-@pytest.mark.parametrize("n", [3, 4, 5, 6, 7, 9, 16, 31, 32, 33, 40, 49, 63, 64, 65, 99, 104, 127,
-                               128, 129, 138, 149, 151, 160])
+@pytest.mark.parametrize("n", [3, 4, 5, 6, 7, 9, 16, 31, 32, 33, 40, 49, 57, 63, 64, 65, 85, 99,
+                               104, 105, 127, 128, 129, 138, 145, 149, 151, 157, 160])
 def test_sizes(n, sym):
     F, D = instances.uniform_instance(n, 2000 + n, symmetric=sym)
     np.fill_diagonal(F, np.arange(n) % 7)  # diagonal terms count too
@@ -85,7 +85,7 @@ def test_thread_counts(n, threads):
 # M in the workspace: the sizes at the edges of its plans, of its warps and of
 # its marks, with the frequency memory, both tenure rules, 2opt first
 @pytest.mark.parametrize("sym", [False, True])
-@pytest.mark.parametrize("n", [182, 183, 191, 192, 193, 200, 217, 255, 256])
+@pytest.mark.parametrize("n", [182, 183, 191, 192, 193, 200, 205, 217, 229, 252, 253, 255, 256])
 def test_large_n(n, sym):
     F, D = instances.uniform_instance(n, 3000 + n, symmetric=sym)
     np.fill_diagonal(F, np.arange(n) % 7)
@@ -129,6 +129,15 @@ def test_large_n_in_batches_and_from_several_walks(gpu):
                          walk_ids=np.array([0, W // 2, W - 1]))
     for k in FIELDS:
         assert np.array_equal(g[k][[0, W // 2, W - 1]].astype(np.int64), o[k].astype(np.int64)), k
+
+
+# tabu times of one and two iterations: slots that are on the ring for none, or
+# read right after they were hung
+@pytest.mark.parametrize("n", [8, 23, 50, 70, 100, 139, 190])
+@pytest.mark.parametrize("tmax", [1, 2, 3])
+def test_shortest_tenures(n, tmax):
+    F, D = instances.uniform_instance(n, 2300 + n, symmetric=n % 2 == 0)
+    check(F, D, 3, seed=17, iters=200, tenure=(1, tmax, 0))
 
 
 # many ties (small values), short random tenures with aspiration: pairs are
