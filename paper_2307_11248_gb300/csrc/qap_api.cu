@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <numeric>
@@ -482,9 +483,6 @@ qap_status qap_cost(qap_ctx* ctx, int32_t count, const int32_t* p, int64_t* cost
   if (!ctx || count < 0 || (count > 0 && (!p || !cost))) return QAP_EINVAL;
   if (count == 0) return QAP_OK;
   const int n = ctx->di.n;
-  std::vector<char> seen;
-  for (int k = 0; k < count; ++k)
-    if (!is_permutation(p + (size_t)k * n, n, seen)) return QAP_EINVAL;
   DeviceGuard dg;
   QAP_TRY(dg.set(ctx->device));
   const size_t pbytes = (size_t)count * n * sizeof(int32_t);
@@ -495,22 +493,39 @@ qap_status qap_cost(qap_ctx* ctx, int32_t count, const int32_t* p, int64_t* cost
   int64_t* dc = reinterpret_cast<int64_t*>(base + off_cost);
   cudaStream_t s = ctx->stream;
   QAP_CUDA(cudaMemcpyAsync(dp, p, pbytes, cudaMemcpyHostToDevice, s));
-  const int grid = std::min(count, ctx->sms * 8);
-  if (ctx->fbytes == 1)
-    qapk::cost_kernel<int8_t, int8_t, 256><<<grid, 256, 0, s>>>(
-        static_cast<const int8_t*>(ctx->dF), ctx->di.ldF, static_cast<const int8_t*>(ctx->dD), n,
-        dp, count, dc);
-  else if (ctx->fbytes == 2)
-    qapk::cost_kernel<int16_t, int8_t, 256><<<grid, 256, 0, s>>>(
-        static_cast<const int16_t*>(ctx->dF), ctx->di.ldF, static_cast<const int8_t*>(ctx->dD),
-        n, dp, count, dc);
-  else
-    qapk::cost_kernel<int64_t, int64_t, 256><<<grid, 256, 0, s>>>(
+  const int smem = qapk::cost_smem(n, ctx->di.ldF, ctx->fbytes);
+  const int per_sm = std::min(2048 / qapk::kCostThreads, ctx->smem_optin / (smem + 1024));
+  const int per_cta = qapk::kCostThreads / 32;
+  const int grid = std::min((count - 1) / per_cta + 1, ctx->sms * std::max(per_sm, 1));
+  auto narrow = [&](auto* fn, const auto* F) -> qap_status {
+    QAP_TRY(prepare_kernel(reinterpret_cast<const void*>(fn), smem));
+    fn<<<grid, qapk::kCostThreads, smem, s>>>(F, ctx->di.ldF, static_cast<const int8_t*>(ctx->dD),
+                                              n, dp, count, dc);
+    return QAP_OK;
+  };
+  if (ctx->fbytes == 1) {
+    const int8_t* F = static_cast<const int8_t*>(ctx->dF);
+    QAP_TRY(n <= 128 ? narrow(qapk::cost_kernel<int8_t, 1>, F)
+                     : narrow(qapk::cost_kernel<int8_t, 2>, F));
+  } else if (ctx->fbytes == 2) {
+    const int16_t* F = static_cast<const int16_t*>(ctx->dF);
+    QAP_TRY(n <= 128 ? narrow(qapk::cost_kernel<int16_t, 1>, F)
+                     : narrow(qapk::cost_kernel<int16_t, 2>, F));
+  } else {
+    qapk::cost_kernel_wide<int64_t><<<grid, qapk::kCostThreads, 0, s>>>(
         static_cast<const int64_t*>(ctx->dF), ctx->di.ldF, static_cast<const int64_t*>(ctx->dD),
         n, dp, count, dc);
+  }
   QAP_CUDA(cudaGetLastError());
-  QAP_CUDA(cudaMemcpyAsync(cost, dc, (size_t)count * 8, cudaMemcpyDeviceToHost, s));
+  // the caller's costs are written only when every row is a permutation
+  const std::unique_ptr<int64_t[]> got(new (std::nothrow) int64_t[count]);
+  if (!got) return QAP_ENOMEM;
+  QAP_CUDA(cudaMemcpyAsync(got.get(), dc, (size_t)count * 8, cudaMemcpyDeviceToHost, s));
   QAP_CUDA(cudaStreamSynchronize(s));
+  bool bad = false;
+  for (int k = 0; k < count; ++k) bad |= got[k] == qapk::kNoCost;
+  if (bad) return QAP_EINVAL;
+  std::memcpy(cost, got.get(), (size_t)count * 8);
   return QAP_OK;
 }
 
