@@ -23,7 +23,9 @@ UNITS = ["qap_api.cu", "qap_walk_i32_f8.cu", "qap_walk_i32_f8m.cu", "qap_walk_i3
          "qap_batch_i32_f16.cu", "qap_batch_i64_f16.cu", "qap_walk_i64_f64.cu",
          "qap_walk_i64_f64p.cu", "qap_batch_i64_f64.cu", "qap_batch_i64_f64p.cu", "qap_server.cu",
          "qap_walk_i32_f16m.cu", "qap_walk_i64_f16m.cu", "qap_batch_i32_f16m.cu",
-         "qap_batch_i64_f16m.cu", "qap_rot.cu", "qap_rot_f8_big.cu"]
+         "qap_batch_i64_f16m.cu", "qap_rot.cu", "qap_rot_f8_big.cu",
+         "qap_walk_i64_f32.cu", "qap_walk_i64_f32p.cu", "qap_batch_i64_f32.cu",
+         "qap_batch_i64_f32p.cu"]
 UNITS += [f"qap_rot_{f}_{nt}.cu" for f in ("f8", "f16")
           for nt in ("128", "256", "256w", "512", "512w", "1024")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

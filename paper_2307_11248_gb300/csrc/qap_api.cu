@@ -344,7 +344,7 @@ qap_status qap_create(const int64_t* F, const int64_t* D, int32_t n, uint32_t fl
   };
   c->dbytes = ((flags & QAP_FORCE_INT64) || di.wide || di.bound > (int64_t)INT_MAX - 1) ? 8 : 4;
   c->force64 = (flags & QAP_FORCE_INT64) != 0;
-  c->fbytes = flow_bytes(di, c->dbytes);
+  c->fbytes = stored_bytes(di, c->dbytes);
   di.ldF = pad_ldF(n, c->fbytes);
   di.ldP = pad_ldP(n, pbytes_of(c->fbytes));
   c->di = di;
@@ -385,8 +385,8 @@ qap_status qap_info(const qap_ctx* ctx, qap_ctx_info* out) {
   out->sym_flow = ctx->di.symF;
   out->sym_dist = ctx->di.symD;
   out->bound = ctx->di.bound;
-  out->flow_bytes = ctx->fbytes;
-  out->dist_bytes = pbytes_of(ctx->fbytes);
+  out->flow_bytes = stated_bytes(ctx->fbytes);
+  out->dist_bytes = stated_bytes(pbytes_of(ctx->fbytes));
   return QAP_OK;
 }
 
@@ -511,6 +511,10 @@ qap_status qap_cost(qap_ctx* ctx, int32_t count, const int32_t* p, int64_t* cost
     const int16_t* F = static_cast<const int16_t*>(ctx->dF);
     QAP_TRY(n <= 128 ? narrow(qapk::cost_kernel<int16_t, 1>, F)
                      : narrow(qapk::cost_kernel<int16_t, 2>, F));
+  } else if (ctx->fbytes == 4) {
+    qapk::cost_kernel_wide<int32_t><<<grid, qapk::kCostThreads, 0, s>>>(
+        static_cast<const int32_t*>(ctx->dF), ctx->di.ldF, static_cast<const int32_t*>(ctx->dD),
+        n, dp, count, dc);
   } else {
     qapk::cost_kernel_wide<int64_t><<<grid, qapk::kCostThreads, 0, s>>>(
         static_cast<const int64_t*>(ctx->dF), ctx->di.ldF, static_cast<const int64_t*>(ctx->dD),
@@ -596,12 +600,13 @@ qap_status qap_batch_create(int32_t count, const int64_t* const* F, const int64_
   b->count = count;
   b->di.resize(count);
   int64_t maxB = 0;
-  int bytevec = 1, wide = 0;
+  int bytevec = 1, wide = 0, mid = 1;
   for (int i = 0; i < count; ++i) {
     qap_status st = inspect_instance(F[i], D[i], n[i], &b->di[i]);
     if (st != QAP_OK) return fail(st);
     bytevec &= b->di[i].bytevec;
     wide |= b->di[i].wide;
+    mid &= b->di[i].mid;
     maxB = std::max(maxB, b->di[i].bound);
     b->nmax = std::max(b->nmax, n[i]);
   }
@@ -611,7 +616,8 @@ qap_status qap_batch_create(int32_t count, const int64_t* const* F, const int64_
   DevInstance all;
   all.bytevec = bytevec;
   all.wide = wide;
-  b->fbytes = flow_bytes(all, b->dbytes);
+  all.mid = mid;
+  b->fbytes = stored_bytes(all, b->dbytes);
   qap_status st = device_attrs(&b->device, &b->sms, &b->smem_optin);
   if (st != QAP_OK) return fail(st);
   std::vector<unsigned char> blob;
@@ -728,8 +734,8 @@ qap_status qap_batch_classes(qap_batch* b, const qap_search_params* params,
     o.ctas_per_sm = sh.ctas_per_sm;
     o.smem_bytes = sh.smem;
     o.delta_bytes = b->dbytes;
-    o.flow_bytes = b->fbytes;
-    o.dist_bytes = pbytes_of(b->fbytes);
+    o.flow_bytes = stated_bytes(b->fbytes);
+    o.dist_bytes = stated_bytes(pbytes_of(b->fbytes));
     o.last_ms = -1.f;
     if (c.timed) {
       QAP_CUDA(cudaEventSynchronize(c.t1));
@@ -814,7 +820,7 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
     }
     if (qapk::row_segments(nmax, kLargePlan.maxpt) <= kLargePlan.nt) {
       Plan p = kLargePlan;
-      if (b->fbytes == 8)
+      if (b->fbytes >= 4)
         p = wide_store(p, dm.data(), (int)dm.size(), b->fbytes, b->dbytes, b->smem_optin, 16);
       else if (!fits(p))
         p.store |= qapk::kGlobalFlow;
@@ -1058,7 +1064,22 @@ extern "C" qap_status qap_batch_search_noalloc(qap_batch* b, const qap_search_pa
   QAP_TRY(noalloc_scratch(b->device, &base));
   Launch L;
   QAP_TRY(plan_batch(b, params, &L));
-  if (ws_layout(L.plan, b->dbytes, b->fbytes, b->nmax, params).stride != 0) {
+  size_t need = ws_layout(L.plan, b->dbytes, b->fbytes, b->nmax, params).stride;
+  if (b->fbytes == 4) {
+    // the call takes the sizes that it takes with int64 elements
+    std::vector<DevInstance> d8 = b->di;
+    for (DevInstance& d : d8) {
+      d.ldF = pad_ldF(d.n, 8);
+      d.ldP = pad_ldP(d.n, 8);
+    }
+    Plan p8;
+    if (!search_plan(b->nmax, (int64_t)b->count * params->starts >= 2 * (int64_t)b->sms, d8.data(),
+                     b->count, 8, b->dbytes, b->force64, b->smem_optin, 16, b->nmax > 181, params,
+                     &p8))
+      return QAP_EUNSUPPORTED;
+    need += ws_layout(p8, b->dbytes, 8, b->nmax, params).stride;
+  }
+  if (need != 0) {
     snprintf(g_last_error, sizeof(g_last_error),
              "qap_batch_search_noalloc: n = %d needs a plan with a per-CTA workspace, which is "
              "allocated (the large-n plan, or int64 elements beyond shared memory)", b->nmax);

@@ -24,11 +24,13 @@ WalkKernelFn walk_kernel_i32_f8m(int nt, int maxpt, int store);
 WalkKernelFn walk_kernel_i32_f16(int nt, int maxpt, int store);
 WalkKernelFn walk_kernel_i64_f16(int nt, int maxpt, int store);
 WalkKernelFn walk_kernel_i64_f64(int nt, int maxpt, int store);
+WalkKernelFn walk_kernel_i64_f32(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i32_f8(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i32_f8m(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i32_f16(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i64_f16(int nt, int maxpt, int store);
 BatchKernelFn batch_kernel_i64_f64(int nt, int maxpt, int store);
+BatchKernelFn batch_kernel_i64_f32(int nt, int maxpt, int store);
 BatchKernelFn rot_kernel_of(int fbytes, int nt, int c);
 }  // namespace qapk
 
@@ -136,7 +138,8 @@ struct DevInstance {
   int64_t maxF = 0;
   int bytevec = 0;  // every difference of two F entries, and of two D entries, fits int8
   int diff16 = 0;   // every difference of two F entries fits int16, of two D entries int8
-  int wide = 0;     // outside the narrow paths: int64 elements and arithmetic
+  int wide = 0;     // outside the narrow paths: int64 arithmetic, int32 or int64 elements
+  int mid = 0;      // values of F and D fit int32, their differences 30 bits
   // narrow paths, for the rotation layout: the mid-range of g[u] = sum_j
   // F[u][j] P[u][j] + F[j][u] P[j][u] over all u and P, and a bound on |delta|
   // plus g's half range (see rot_bounds)
@@ -202,8 +205,17 @@ inline int flow_bytes(const DevInstance& di, int dbytes) {
   return (di.bytevec && dbytes == 4) ? 1 : 2;
 }
 
-// P and D are int8 beside int8 or int16 flows and int64 beside int64 flows.
-inline int pbytes_of(int fbytes) { return fbytes == 8 ? 8 : 1; }
+// The width that elements are stored in: int32 on the wide path where they fit.
+inline int stored_bytes(const DevInstance& di, int dbytes) {
+  const int b = flow_bytes(di, dbytes);
+  return b == 8 && di.mid ? 4 : b;
+}
+// The width that the interface states for it.
+inline int stated_bytes(int bytes) { return bytes == 4 ? 8 : bytes; }
+
+// P and D are int8 beside int8 or int16 flows and as wide as the flows beside
+// int32 or int64 ones.
+inline int pbytes_of(int fbytes) { return fbytes >= 4 ? fbytes : 1; }
 
 inline int pad_ldF(int n, int fbytes) { return (16 / fbytes) * (((n * fbytes + 15) / 16) | 1); }
 inline int pad_ldP(int n, int pbytes) { return (16 / pbytes) * (((n * pbytes + 15) / 16) | 1); }
@@ -212,7 +224,7 @@ inline int pad_ldP(int n, int pbytes) { return (16 / pbytes) * (((n * pbytes + 1
 //  - narrow (int8 or int16 flows, int8 distances, 32-bit element sums) when
 //    F fits int16, D fits int8 and every dot product of two length-n rows
 //    pairs, 2 n max|F| max|D|, stays below 2^31;
-//  - wide (int64 elements and arithmetic) otherwise;
+//  - wide (int64 arithmetic; elements int32 where they fit, else int64) otherwise;
 //  - QAP_EOVERFLOW when B = (n^2 + 8n + 32) max|F| max|D| reaches 2^62.
 inline qap_status inspect_instance(const int64_t* F, const int64_t* D, int n, DevInstance* di) {
   if (!F || !D || n < 2) return QAP_EINVAL;
@@ -244,6 +256,7 @@ inline qap_status inspect_instance(const int64_t* F, const int64_t* D, int n, De
   di->bound = (int64_t)B;
   di->maxF = (int64_t)mF;
   di->wide = !(in16 && dots <= (unsigned __int128)INT32_MAX);
+  di->mid = mF <= INT32_MAX && mD <= INT32_MAX && hiF - loF < (1 << 30) && hiD - loD < (1 << 30);
   // differences of two F entries and of two D entries fit a byte (no
   // overflow here: on this branch the ranges fit int16 and int8)
   di->bytevec = !di->wide && mF <= 127 && hiF - loF <= 127 && hiD - loD <= 127;
@@ -270,6 +283,9 @@ inline void build_images(const int64_t* F, const int64_t* D, const DevInstance& 
       } else if (fbytes == 2) {
         reinterpret_cast<int16_t*>(img_F.data())[(size_t)i * ld + j] = (int16_t)f;
         reinterpret_cast<int16_t*>(img_Ft.data())[(size_t)j * ld + i] = (int16_t)f;
+      } else if (fbytes == 4) {
+        reinterpret_cast<int32_t*>(img_F.data())[(size_t)i * ld + j] = (int32_t)f;
+        reinterpret_cast<int32_t*>(img_Ft.data())[(size_t)j * ld + i] = (int32_t)f;
       } else {
         reinterpret_cast<int64_t*>(img_F.data())[(size_t)i * ld + j] = f;
         reinterpret_cast<int64_t*>(img_Ft.data())[(size_t)j * ld + i] = f;
@@ -277,6 +293,8 @@ inline void build_images(const int64_t* F, const int64_t* D, const DevInstance& 
       const int64_t d = D[(size_t)i * n + j];
       if (pbytes == 1)
         img_D[(size_t)i * n + j] = (unsigned char)(int8_t)d;
+      else if (pbytes == 4)
+        reinterpret_cast<int32_t*>(img_D.data())[(size_t)i * n + j] = (int32_t)d;
       else
         reinterpret_cast<int64_t*>(img_D.data())[(size_t)i * n + j] = d;
     }
@@ -292,6 +310,7 @@ inline qap_status device_attrs(int* device, int* sms, int* smem_optin) {
 inline const void* pick_walk_kernel(int dbytes, int fbytes, const Plan& p) {
   auto row = [&]() -> qapk::WalkKernelFn {
     if (fbytes == 8) return qapk::walk_kernel_i64_f64(p.nt, p.maxpt, p.store);
+    if (fbytes == 4) return qapk::walk_kernel_i64_f32(p.nt, p.maxpt, p.store);
     if (dbytes == 8) return qapk::walk_kernel_i64_f16(p.nt, p.maxpt, p.store);
     if (fbytes == 1) return qapk::walk_kernel_i32_f8(p.nt, p.maxpt, p.store);
     return qapk::walk_kernel_i32_f16(p.nt, p.maxpt, p.store);
@@ -303,6 +322,7 @@ inline const void* pick_walk_kernel(int dbytes, int fbytes, const Plan& p) {
 inline const void* pick_batch_kernel(int dbytes, int fbytes, const Plan& p) {
   auto row = [&]() -> qapk::BatchKernelFn {
     if (fbytes == 8) return qapk::batch_kernel_i64_f64(p.nt, p.maxpt, p.store);
+    if (fbytes == 4) return qapk::batch_kernel_i64_f32(p.nt, p.maxpt, p.store);
     if (dbytes == 8) return qapk::batch_kernel_i64_f16(p.nt, p.maxpt, p.store);
     if (fbytes == 1) return qapk::batch_kernel_i32_f8(p.nt, p.maxpt, p.store);
     return qapk::batch_kernel_i32_f16(p.nt, p.maxpt, p.store);
@@ -387,7 +407,7 @@ inline int products_form(const Plan& p) {
 // without the copies.  `fits` says whether a plan fits.
 template <typename Fits>
 inline Plan with_products(Plan p, int fbytes, int form, Fits fits) {
-  if (form == QAP_PHASE_X_DOTS || fbytes == 8 || !has_product_form(p, fbytes)) return p;
+  if (form == QAP_PHASE_X_DOTS || fbytes >= 4 || !has_product_form(p, fbytes)) return p;
   Plan m = p;
   m.store |= qapk::kProductM;
   if (fits(m)) return m;
@@ -464,12 +484,12 @@ inline bool rot_holds_tenures(const Plan& p, const qap_search_params* sp, int nm
   return qapk::rot_ring_holds(p.shape(), tmax);
 }
 
-// The int64 element path reads F and F^T from global memory (L1-cached,
+// The wide element path reads F and F^T from global memory (L1-cached,
 // read-only), and keeps P and P^T in the CTA's workspace too when they do
 // not fit shared memory.
 inline Plan wide_store(Plan p, const DevInstance* d, int count, int fbytes, int dbytes,
                        int smem_optin, int reserve) {
-  if (fbytes != 8) return p;
+  if (fbytes < 4) return p;
   p.store |= qapk::kGlobalFlow;
   if (plan_smem(p, d, count, fbytes, dbytes) + reserve > smem_optin) p.store |= qapk::kGlobalP;
   return p;
@@ -507,7 +527,7 @@ inline bool choose_plan_fit(int nmax, int threads, bool many, const DevInstance*
   if (threads != 0 && threads != kLargePlan.nt) return false;
   if (qapk::row_segments(nmax, kLargePlan.maxpt) > kLargePlan.nt) return false;
   p = kLargePlan;
-  if (fbytes == 8)
+  if (fbytes >= 4)
     p = wide_store(p, d, count, fbytes, dbytes, smem_optin, reserve);
   else if (plan_smem(p, d, count, fbytes, dbytes) + reserve > smem_optin)
     p.store |= qapk::kGlobalFlow;

@@ -137,7 +137,7 @@ constexpr int kGlobalFlow = 2;
 // update them after each move (see phase_m_update), so that phase X reads
 // the dot products it needs instead of computing them.
 constexpr int kProductM = 4;
-// Plans with bit kGlobalP (int64 elements only) keep P and P^T in the CTA's
+// Plans with bit kGlobalP (wide elements only) keep P and P^T in the CTA's
 // workspace (at SearchArgs::p_off) instead of shared memory; they read F and
 // F^T from global memory too.
 constexpr int kGlobalP = 8;
@@ -167,8 +167,8 @@ struct SmemLayout {
 
 __host__ __device__ inline int align16(int x) { return (x + 15) & ~15; }
 
-// fbytes: bytes per F element (1, 2, or 8 for the int64 element path, whose
-// P and update vectors are int64 too)
+// fbytes: bytes per F element (1, 2, or 4 and 8 for the wide element path,
+// whose P and update vectors are as wide)
 __host__ __device__ inline SmemLayout smem_layout(int n, int ldF, int fbytes, int ldP, int symF,
                                                   int symD, int dbytes, int slots,
                                                   int store = 0) {
@@ -176,7 +176,7 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int ldF, int fbytes, in
   int o = 0;
   const bool fg = store & kGlobalFlow;
   const bool pg = store & kGlobalP;
-  const int pbytes = fbytes == 8 ? 8 : 1;   // P element
+  const int pbytes = fbytes >= 4 ? fbytes : 1;  // P element
   const int vbytes = fbytes == 8 ? 32 : 16; // update vector (a, b, c, e) of one index
   if (store & kGlobalDelta) slots = 0;
   L.offF = o;    o = fg ? o : align16(o + n * ldF * fbytes);
@@ -219,6 +219,11 @@ template <typename FE> struct Elem;
 template <> struct Elem<int8_t> { using P = int8_t; using S = int; };
 template <> struct Elem<int16_t> { using P = int8_t; using S = int; };
 template <> struct Elem<int64_t> { using P = int64_t; using S = int64_t; };
+// Wide instances whose values and differences fit 32 bits: half the bytes of
+// every row, and a product is one 32 x 32 -> 64 bit multiply-add in place of a
+// 64 x 64 bit multiplication (n = 61 asymmetric, 160 walks x 1000 8.23 -> 5.10
+// ms).  Sums and deltas are int64 as before.
+template <> struct Elem<int32_t> { using P = int32_t; using S = int64_t; };
 
 // ---------------------------------------------------------------------------
 // row chunks: F rows as int8 (16 per chunk, dp4a) or int16 (8, dp2a)
@@ -246,6 +251,19 @@ template <> struct Chunk<int16_t> {
     acc = __dp2a_hi(f.y, q.x, acc);
     acc = __dp2a_lo(f.z, q.y, acc);
     return __dp2a_hi(f.w, q.y, acc);
+  }
+};
+
+// int32 flows and distances: four elements per chunk
+template <> struct Chunk<int32_t> {
+  static constexpr int W = 4;
+  using FV = int4;
+  using QV = int4;
+  __device__ __forceinline__ static int64_t dot(const FV f, const QV q, int64_t acc) {
+    acc += (int64_t)f.x * q.x;
+    acc += (int64_t)f.y * q.y;
+    acc += (int64_t)f.z * q.z;
+    return acc + (int64_t)f.w * q.w;
   }
 };
 
@@ -325,6 +343,27 @@ template <> struct VecOps<int16_t> {
   template <typename DT>
   __device__ __forceinline__ static DT update(const U& u, const V v, DT d) {
     return d + (DT)((u.x - v.x) * (u.y - v.y) + (u.z - v.z) * (u.w - v.w));
+  }
+  __device__ __forceinline__ static void put(void* vec, int, int k, V v) {
+    reinterpret_cast<V*>(vec)[k] = v;
+  }
+  __device__ __forceinline__ static V get(const void* vec, int, int k) {
+    return reinterpret_cast<const V*>(vec)[k];
+  }
+};
+
+// int32 elements: differences below 2^30, so that theirs fit 32 bits
+template <> struct VecOps<int32_t> {
+  using V = int4;                  // (a, b, c, e)
+  using U = int4;
+  __device__ __forceinline__ static V pack(int64_t a, int64_t b, int64_t c, int64_t e) {
+    return make_int4((int)a, (int)b, (int)c, (int)e);
+  }
+  __device__ __forceinline__ static U prep(const V u) { return u; }
+  template <typename DT>
+  __device__ __forceinline__ static DT update(const U& u, const V v, DT d) {
+    d += (DT)(u.x - v.x) * (u.y - v.y);
+    return d + (DT)(u.z - v.z) * (u.w - v.w);
   }
   __device__ __forceinline__ static void put(void* vec, int, int k, V v) {
     reinterpret_cast<V*>(vec)[k] = v;
@@ -1589,7 +1628,7 @@ constexpr int64_t kNoCost = INT64_MIN;  // |costs| stay below 2^62
 
 // Shared memory of cost_kernel: F's image, then D.
 __host__ __device__ inline int cost_smem(int n, int ldF, int fbytes) {
-  return fbytes == 8 ? 0 : n * ldF * fbytes + (n * n + 3) / 4 * 4;
+  return fbytes >= 4 ? 0 : n * ldF * fbytes + (n * n + 3) / 4 * 4;
 }
 
 // The lane's columns of a permutation (those from n on read 0), in range; the
@@ -1715,7 +1754,7 @@ __global__ void __launch_bounds__(kCostThreads) cost_kernel_wide(
       const E* const d = D + (size_t)pb[i] * n;
 #pragma unroll
       for (int t = 0; t < 8; ++t)
-        if (column(t) < n) c += F[(size_t)i * ldF + column(t)] * d[q[t]];
+        if (column(t) < n) c += (int64_t)F[(size_t)i * ldF + column(t)] * d[q[t]];
     }
     for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (lane == 0) out[b] = c;

@@ -402,7 +402,7 @@ qap_status qap_server_submit(qap_server* sv, const int64_t* F, const int64_t* D,
   r->force64 = (flags & QAP_FORCE_INT64) != 0;
   r->dbytes = ((flags & QAP_FORCE_INT64) || r->di.wide || r->di.bound > (int64_t)INT_MAX - 1 ||
                check_penalty(params, 4, r->di.bound) != QAP_OK) ? 8 : 4;
-  r->fbytes = flow_bytes(r->di, r->dbytes);
+  r->fbytes = stored_bytes(r->di, r->dbytes);
   r->di.ldF = pad_ldF(n, r->fbytes);
   r->di.ldP = pad_ldP(n, pbytes_of(r->fbytes));
   r->params = *params;
