@@ -132,7 +132,7 @@ def gpu_uuid_of(dev):
 # the sources of the kernels' code and of the rules that pick a launch's
 # plan (the qap_walk_* / qap_batch_* units only list which template
 # instances exist)
-KERNEL_SOURCES = ("qap_kernels.cuh", "qap_philox.cuh", "qap_host.cuh")
+KERNEL_SOURCES = ("qap_kernels.cuh", "qap_rotation.cuh", "qap_philox.cuh", "qap_host.cuh")
 
 
 def kernel_source_hash():
@@ -374,7 +374,8 @@ def measure_asym50(args, q, stream, flush, dev, world, rank, khash, baselines=Tr
     sm_mhz = clk["sm_max_mhz"] or 2070.0
     roof, issue = rooflines(bpu * iters_done, iters_done, float(np.mean(ms)) / 1e3, plan["sms"],
                             sm_mhz, profile_figures("walk_kernel_asym50", khash),
-                            f"walk_kernel (int32 deltas, int{8 * info['flow_bytes']} flows, "
+                            f"{'rot' if args.phase_x == 'auto' else 'walk'}_kernel (int32 deltas, "
+                            f"int{8 * info['flow_bytes']} flows, "
                             f"{plan['threads_per_walk']} x {plan['pairs_per_thread']}, "
                             f"products {plan['products']})")
     roof["bytes_per_unit"] = bpu
@@ -480,7 +481,8 @@ def measure_grid100(args, q, stream, flush, dev, world, rank, khash, baselines=T
     sm_mhz = clk["sm_max_mhz"] or 2070.0
     roof, issue = rooflines(bpu * moves, moves, float(np.mean(ms)) / 1e3, plan["sms"], sm_mhz,
                             profile_figures("walk_kernel_grid100", khash),
-                            f"walk_kernel (int32 deltas, int{8 * info['flow_bytes']} flows, "
+                            f"{'rot' if args.phase_x == 'auto' else 'walk'}_kernel (int32 deltas, "
+                            f"int{8 * info['flow_bytes']} flows, "
                             f"{plan['threads_per_walk']} x {plan['pairs_per_thread']})")
     roof["bytes_per_unit"] = bpu
     roof["unit_def"] = "one 2opt move or tabu iteration of one walk"
