@@ -1411,7 +1411,7 @@ __device__ __forceinline__ void run_walk(const WalkSmem<DT, FE>& S, const InstAr
     for (int c = tid; c < 2 * n * n + n; c += NT) t[c] = 0;
   }
   if (fq || rules) __syncthreads();
-  // locations of the move's units before it: S.sum's first two words (the
+  // locations of the move's units before it, and its tenure: S.sum's first words (the
   // block sum is done by now); written after the arg-min, read after the
   // next barrier, before swap_rs can have moved them
   int32_t* moved_from = reinterpret_cast<int32_t*>(S.sum);
@@ -1462,6 +1462,14 @@ __device__ __forceinline__ void run_walk(const WalkSmem<DT, FE>& S, const InstAr
           moved_from[0] = S.perm[r];
           moved_from[1] = S.perm[s];
         }
+        // the paper's rule: a fresh tenure per move, drawn beside phase X by the
+        // last warp (that has no part in it, or the shortest), where every thread
+        // drew it after the barrier (the same case 12.6 -> 12.0 ms; n = 47, 160
+        // walks x 2000 5.95 -> 5.59 ms)
+        if (period == 0 && tid == NT - 32) {
+          const uint32_t x = walk_draw(a.seed, wid, 1u, (uint32_t)(it - 1));
+          moved_from[2] = tmin + (int)below(x, (uint32_t)(tmax - tmin + 1));
+        }
       }
       cur += bd;
       done = it;
@@ -1481,9 +1489,9 @@ __device__ __forceinline__ void run_walk(const WalkSmem<DT, FE>& S, const InstAr
       int stamp = it + tenure;
       const bool owner =
           su == r && (kInterleave ? slot_of(s) >= 0 : s >= sv && s < sv + slen);
-      if (period == 0 && (owner || (EXT && a.crit != 0))) {
-        // the paper's rule: a fresh tenure per move, drawn by the owner only
-        // (by every thread when the other criteria restamp touching pairs)
+      if (EXT && period == 0) {
+        stamp = it + moved_from[2];
+      } else if (period == 0 && owner) {  // a fresh tenure per move, drawn by the owner
         const uint32_t x = walk_draw(a.seed, wid, 1u, (uint32_t)(it - 1));
         stamp = it + tmin + (int)below(x, (uint32_t)(tmax - tmin + 1));
       }
@@ -1505,7 +1513,17 @@ __device__ __forceinline__ void run_walk(const WalkSmem<DT, FE>& S, const InstAr
                                : max(unit_mark(u), unit_mark(v));
           };
           if (su == r || su == s) {
-            for (int i = 0; i < slen; ++i) S.tabu[i * NT + tid] = mark(su, sv + i * sk);
+            // four marks' loads in flight at once (each a chain of two, that no
+            // store separates from the next: n = 100, unit-location criterion and
+            // penalty, 304 walks x 1000 14.3 -> 12.6 ms)
+            for (int i0 = 0; i0 < slen; i0 += 4) {
+              int t[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) t[i] = mark(su, sv + min(i0 + i, slen - 1) * sk);
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                if (i0 + i < slen) S.tabu[(i0 + i) * NT + tid] = t[i];
+            }
           } else if constexpr (kInterleave) {
             const int ir = slot_of(r), is = slot_of(s);
             if (ir >= 0) S.tabu[ir * NT + tid] = mark(su, r);
