@@ -48,9 +48,11 @@
  *                     entries fits a byte, and the deltas are int32;
  *   int16 F, int8 D   F fits int16, D fits int8, and 2 n max|F| max|D| is
  *                     below 2^31 (the dot products of phase X sum in 32 bits);
- *   int64 F, int64 D  every other instance: int64 storage and arithmetic, F
- *                     read from global memory, P in shared memory while it
- *                     fits and in a per-CTA device workspace otherwise.
+ *   int64 F, int64 D  every other instance: int64 arithmetic, F read from
+ *                     global memory, P in shared memory while it fits and in a
+ *                     per-CTA device workspace otherwise; stored as int32 where
+ *                     every value fits and differences fit 30 bits (flow_bytes
+ *                     and dist_bytes say 8 for both).
  *
  * Errors: every entry point returns a qap_status; on error nothing has been
  * written to the outputs unless stated otherwise.  A CUDA error is returned

@@ -52,10 +52,10 @@
 // Bound: the fixed latencies of one iteration's chain (arg-min, phase X,
 // table, scan, two barriers) with one or two walks on an SM, integer issue
 // with more.  Measured against the row layout's products form (one GB300, same
-// box): n = 100 grid, 1024 walks x (2opt + 10^4) 150.0 -> 47.5 ms; n = 50
+// box): n = 100 grid, 1024 walks x (2opt + 10^4) 150.0 -> 48.0 ms; n = 50
 // asymmetric, 256 walks x 5000 7.85 -> 4.24 ms; n = 139 asymmetric, 150 walks
 // x 2000 8.74 -> 2.89 ms; n = 23, 100 walks x 1000 in one blocking call 1.21 ->
-// 0.65 ms; 2opt from 32 starts at n = 12 16.4 -> 12.3 us.  Warp instructions per
+// 0.60 ms; 2opt from 32 starts at n = 12 16.4 -> 12.3 us.  Warp instructions per
 // walk-iteration: n = 100 grid 10360 -> 3236, n = 50 asymmetric 3606 -> 1924.
 // int16 flows (two dp2a per pair): 96 lognormal instances of n = 20-150, 64
 // walks x 1000 each, 103.4 -> 39.4 ms; their costs need 64 bits, their deltas
