@@ -466,7 +466,11 @@ __device__ __forceinline__ int lds16u(uint32_t at) {
   return v;
 }
 // A tabu time's end in 16 bits: 0 for a pair that is not tabu.
-__device__ __forceinline__ int rot_mark16(int end) { return (end & 0x7fff) | 0x8000; }
+__host__ __device__ __forceinline__ int rot_mark16(int end) { return (end & 0x7fff) | 0x8000; }
+// Whether a pair with that mark is tabu after iteration `it`.
+__host__ __device__ __forceinline__ bool rot_tabu16(int mark, int it) {
+  return mark != 0 && mark != rot_mark16(it + 1);
+}
 // Entries of M at byte offset `at`: in shared memory, or (large n) in the
 // workspace, past L1.
 template <int NT>
@@ -912,35 +916,27 @@ __device__ __forceinline__ void rot_owner() {
   }
 }
 
-// The tabu times and the hash of a walk, kept by one warp beside the scan.
-template <int NT, int C, typename FE>
-struct RotKeeper {
-  using S = RotSmem<NT, FE>;
+// The ends of a walk's tabu times: each pair's mark, and the ring that the slots
+// whose time ends hang on.  Kept by one thread.  Mem says where the ring and its
+// nodes lie: shared memory, or (to check the bookkeeping on the host) an array.
+template <int NT, int C, typename Mem>
+struct RotEnds {
   static constexpr bool M16 = rot_big(NT);
   static constexpr int RING = rot_ring(NT), SL = rot_slot_bits(NT);
-  static constexpr uint64_t kH0 = 14695981039346656037ull;
-  const int n2, nc, J, iters, p_stride;
+  static_assert(0x8000 % RING == 0, "a 16-bit mark gives its end modulo the ring's length");
+  const int n2, nc, J, iters;
   int32_t* const mark;
-  int32_t* const fq;
-  uint64_t h, dh;
-  bool was_tabu;
-  int2 late;     // lane 0: the last move, while its slots are to be hung
+  int2 late;     // the last move, while its slots are to be hung
   int late_end;  // the end of its tabu time (0: none)
 
-  __device__ __forceinline__ RotKeeper(const RotWalkArgs& W, const RotThread& T, int32_t* marks)
-      : n2(T.n2), nc(T.nc), J(T.J), iters(W.s.iters), p_stride(W.s.p_stride), mark(marks),
-        fq(W.s.freq ? W.s.freq + (size_t)W.row * W.s.p_stride * W.s.p_stride : nullptr), h(kH0),
-        dh(kH0), was_tabu(!W.s.descend), late(make_int2(0, 0)), late_end(0) {}
-
-  // The tenure of an iteration, one of the 32 that the warp draws ahead.
-  __device__ __noinline__ static void tenures(int it) {
-    const RotWalkArgs& W = S::args();
-    S::ten()[(it - 1) & 63] = RotTenure(W.s, W.I.n).of(W.s.seed, W.wid, it);
-  }
+  __host__ __device__ __forceinline__ RotEnds(int blocks, int circle, int chunks, int its,
+                                              int32_t* marks)
+      : n2(blocks), nc(circle), J(chunks), iters(its), mark(marks), late(make_int2(0, 0)),
+        late_end(0) {}
 
   // The slot that block u's threads hold pair (u, v) in, or -1 when v is not
   // in their windows.
-  __device__ __forceinline__ int slot(int u, int v) const {
+  __host__ __device__ __forceinline__ int slot(int u, int v) const {
     const int bu = u >> 1, bv = v >> 1;
     int o = bv - bu;
     o = (o < 0 ? o + nc : o) - 1;
@@ -949,13 +945,13 @@ struct RotKeeper {
   }
   // The slots of a pair, one or two (the one inside a block is its first
   // thread's).
-  __device__ __forceinline__ int2 slots(int r, int s) const {
+  __host__ __device__ __forceinline__ int2 slots(int r, int s) const {
     if (r >> 1 == s >> 1) return make_int2((r >> 1) << SL | 4 * C, -1);
     const int a = slot(r, s), b = slot(s, r);
     return a >= 0 ? make_int2(a, b) : make_int2(b, -1);
   }
   // The pair of a slot, as its place in the triangle of marks.
-  __device__ __forceinline__ int pair_at(int w) const {
+  __host__ __device__ __forceinline__ int pair_at(int w) const {
     const int t = w >> SL, q = w & ((1 << SL) - 1), j = t / n2, m = t - j * n2;
     int v = 2 * m, u = v + 1;
     if (q < 4 * C) {
@@ -964,32 +960,98 @@ struct RotKeeper {
       v += q >> 1 & 1;
       u = 2 * (b < nc ? b : b - nc) + (q & 1);
     }
-    const int hi = max(u, v);
-    return hi * (hi - 1) / 2 + min(u, v);
+    const int hi = u > v ? u : v, lo = u > v ? v : u;
+    return hi * (hi - 1) / 2 + lo;
   }
-  __device__ __forceinline__ void hang(uint32_t w, int end, uint32_t node) const {
-    uint32_t* const at = S::ring() + (end & (RING - 1));
+#pragma nv_exec_check_disable
+  __host__ __device__ __forceinline__ void hang(uint32_t w, int end, uint32_t node) const {
+    uint32_t* const at = Mem::ring() + (end & (RING - 1));
     const uint32_t old = *at;
-    if (old != 0xffffffffu) S::node()[node] = old;
+    if (old != 0xffffffffu) Mem::node()[node] = old;
     *at = w | (old != 0xffffffffu ? node : 0xffffu) << 16;
   }
   // Take a slot off the ring word of iteration `end`.
-  __device__ __noinline__ static void unhang(uint32_t w, int end) {
-    uint32_t* at = S::ring() + (end & (RING - 1));
+#pragma nv_exec_check_disable
+  __host__ __device__ __noinline__ static void unhang(uint32_t w, int end) {
+    uint32_t* at = Mem::ring() + (end & (RING - 1));
     while (*at != 0xffffffffu) {
       const uint32_t next = *at >> 16;
       if ((*at & 0xffffu) == w) {
-        *at = next == 0xffffu ? 0xffffffffu : S::node()[next];
+        *at = next == 0xffffu ? 0xffffffffu : Mem::node()[next];
       } else {
         if (next == 0xffffu) break;
-        at = S::node() + next;
+        at = Mem::node() + next;
       }
     }
   }
 
-  // Move (r, s) of iteration `it` (0 in the descent), by the whole warp.  With
-  // LATE the slots are hung by finish(), after the next barrier, unless the
-  // pairs' warps may read the ring word by then.
+  // Move (r, s) of iteration `it`, tabu up to `end`.  With LATE the slots are
+  // hung by finish(), after the next barrier, unless the pairs' warps may read
+  // the ring word by then.
+#pragma nv_exec_check_disable
+  template <bool LATE>
+  __host__ __device__ __forceinline__ void apply(int r, int s, int it, int end) {
+    const int at = s * (s - 1) / 2 + r;
+    // a pair applied while tabu: its old end no longer counts
+    int old = 0;
+    if constexpr (M16) {
+      uint16_t* const m = reinterpret_cast<uint16_t*>(mark);
+      // the marks that end with the next iteration
+      for (uint32_t x = Mem::ring()[(it + 1) & (RING - 1)]; x != 0xffffffffu;
+           x = x >> 16 == 0xffffu ? 0xffffffffu : Mem::node()[x >> 16])
+        m[pair_at((int)(x & 0xffffu))] = 0;
+      old = m[at];  // with its top bit: the other 15 are 0 at multiples of 2^15
+      m[at] = end > it + 1 ? (uint16_t)rot_mark16(end) : 0;
+    } else {
+      old = mark[at] > it + 1 ? mark[at] : 0;
+      mark[at] = end;
+    }
+    // the ring word of the iteration just served is free again
+    Mem::ring()[(it + 1) & (RING - 1)] = 0xffffffffu;
+    late = make_int2(r << 8 | s, it);
+    late_end = end;
+    if (old != 0) {
+      int2 w = slots(r, s);
+#pragma unroll 1
+      for (; w.x >= 0; w = make_int2(w.y, -1)) unhang((uint32_t)w.x, old);
+    }
+    if (!LATE || end <= it + 2) finish();
+  }
+  // The last move's slots on the ring.
+  __host__ __device__ __forceinline__ void finish() {
+    const int it = late.y;
+    if (late_end > it + 1 && late_end <= iters) {
+      int2 w = slots(late.x >> 8, late.x & 0xff);
+      uint32_t node = 2 * ((uint32_t)it & (RING - 1));
+#pragma unroll 1
+      for (; w.x >= 0; w = make_int2(w.y, -1)) hang((uint32_t)w.x, late_end, node++);
+    }
+    late_end = 0;
+  }
+};
+
+// The tabu times and the hash of a walk, kept by one warp beside the scan.
+template <int NT, int C, typename FE>
+struct RotKeeper : RotEnds<NT, C, RotSmem<NT, FE>> {
+  using S = RotSmem<NT, FE>;
+  static constexpr uint64_t kH0 = 14695981039346656037ull;
+  const int p_stride;
+  int32_t* const fq;
+  uint64_t h, dh;
+  bool was_tabu;
+
+  __device__ __forceinline__ RotKeeper(const RotWalkArgs& W, const RotThread& T, int32_t* marks)
+      : RotEnds<NT, C, S>(T.n2, T.nc, T.J, W.s.iters, marks), p_stride(W.s.p_stride),
+        fq(W.s.freq ? W.s.freq + (size_t)W.row * W.s.p_stride * W.s.p_stride : nullptr), h(kH0),
+        dh(kH0), was_tabu(!W.s.descend) {}
+
+  // The tenure of an iteration, one of the 32 that the warp draws ahead.
+  __device__ __noinline__ static void tenures(int it) {
+    const RotWalkArgs& W = S::args();
+    S::ten()[(it - 1) & 63] = RotTenure(W.s, W.I.n).of(W.s.seed, W.wid, it);
+  }
+
+  // Move (r, s) of iteration `it` (0 in the descent), by the whole warp.
   template <bool LATE>
   __device__ __forceinline__ void move(int r, int s, int it) {
     const int lane = threadIdx.x & 31;
@@ -998,31 +1060,7 @@ struct RotKeeper {
       __syncwarp();  // (its place takes the tenure of iteration it + 64)
       if ((it & 31) == 0) tenures(it + 33 + lane);
       if (lane == 0) {
-        const int at = s * (s - 1) / 2 + r;
-        // a pair applied while tabu: its old end no longer counts
-        int old = 0;
-        if constexpr (M16) {
-          uint16_t* const m = reinterpret_cast<uint16_t*>(mark);
-          // the marks that end with the next iteration
-          for (uint32_t x = S::ring()[(it + 1) & (RING - 1)]; x != 0xffffffffu;
-               x = x >> 16 == 0xffffu ? 0xffffffffu : S::node()[x >> 16])
-            m[pair_at((int)(x & 0xffffu))] = 0;
-          old = m[at] & 0x7fff;
-          m[at] = end > it + 1 ? (uint16_t)rot_mark16(end) : 0;
-        } else {
-          old = mark[at] > it + 1 ? mark[at] : 0;
-          mark[at] = end;
-        }
-        // the ring word of the iteration just served is free again
-        S::ring()[(it + 1) & (RING - 1)] = 0xffffffffu;
-        late = make_int2(r << 8 | s, it);
-        late_end = end;
-        if (old != 0) {
-          int2 w = slots(r, s);
-#pragma unroll 1
-          for (; w.x >= 0; w = make_int2(w.y, -1)) unhang((uint32_t)w.x, old);
-        }
-        if (!LATE || end <= it + 2) finish();
+        this->template apply<LATE>(r, s, it, end);
         if (fq) atomicAdd(fq + s * p_stride + r, 1);
       }
       if (!was_tabu) {  // the first tabu move
@@ -1032,17 +1070,6 @@ struct RotKeeper {
       }
     }
     h = fnv_step(h, r, s);
-  }
-  // The last move's slots on the ring, by lane 0.
-  __device__ __forceinline__ void finish() {
-    const int it = late.y;
-    if (late_end > it + 1 && late_end <= iters) {
-      int2 w = slots(late.x >> 8, late.x & 0xff);
-      uint32_t node = 2 * ((uint32_t)it & (RING - 1));
-#pragma unroll 1
-      for (; w.x >= 0; w = make_int2(w.y, -1)) hang((uint32_t)w.x, late_end, node++);
-    }
-    late_end = 0;
   }
 
   __device__ __forceinline__ void results(const SearchArgs& a, int row) {
@@ -1180,9 +1207,8 @@ __device__ __forceinline__ void rot_phase_x() {
       const int ar = kj < r ? rtri + kj : ktri + r, as = kj < s ? stri + kj : ktri + s;
       bool tabu_r, tabu_s;
       if constexpr (M16) {
-        const int er = lds16u(aMark + 2 * ar), es = lds16u(aMark + 2 * as);
-        tabu_r = er != 0 && er != rot_mark16(it + 1);
-        tabu_s = es != 0 && es != rot_mark16(it + 1);
+        tabu_r = rot_tabu16(lds16u(aMark + 2 * ar), it);
+        tabu_s = rot_tabu16(lds16u(aMark + 2 * as), it);
       } else {
         tabu_r = lds32(aMark + 4 * ar) > it + 1;
         tabu_s = lds32(aMark + 4 * as) > it + 1;
