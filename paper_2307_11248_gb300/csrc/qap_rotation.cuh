@@ -160,8 +160,14 @@ struct RotPending {
   static constexpr int Q = (rot_big(NT) ? 4 : 2) * (SYM ? 2 : 1);
 };
 
-// Barrier of the CTA; the warps of each role reach it from their own code.
-__device__ __forceinline__ void rot_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
+// Barrier of the CTA; the warps of each role reach it from their own code.  bar.sync
+// is the aligned form: all lanes of a warp must come to it together, also where
+// one lane alone had work before it.  (The form for diverged warps, barrier.sync,
+// takes 3 to 7 registers more, 40 to 140 bytes of spill at large n.)
+__device__ __forceinline__ void rot_barrier() {
+  __syncwarp();
+  asm volatile("bar.sync 0;" ::: "memory");
+}
 
 // What a walk is, for the functions of its roles: in shared memory, so that
 // no register holds it through the iterations.
