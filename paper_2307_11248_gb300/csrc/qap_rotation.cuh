@@ -161,13 +161,12 @@ struct RotPending {
 };
 
 // Barrier of the CTA; the warps of each role reach it from their own code.  bar.sync
-// is the aligned form: all lanes of a warp must come to it together, also where
-// one lane alone had work before it.  (The form for diverged warps, barrier.sync,
-// takes 3 to 7 registers more, 40 to 140 bytes of spill at large n.)
-__device__ __forceinline__ void rot_barrier() {
-  __syncwarp();
-  asm volatile("bar.sync 0;" ::: "memory");
-}
+// is the aligned form: all lanes of a warp come to it together, so a __syncwarp()
+// stands where lanes part before one.  (Measured, one box: with it there, n = 139
+// 2.83 ms, n = 203 3.24, n = 50 4.15, n = 100 grid 47.3; in this function 2.95, 3.66,
+// 4.30, 49.2.  The form for diverged warps, barrier.sync, takes 3 to 7 registers
+// more, 40 to 140 bytes of spill at large n.)
+__device__ __forceinline__ void rot_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
 
 // What a walk is, for the functions of its roles: in shared memory, so that
 // no register holds it through the iterations.
@@ -353,6 +352,7 @@ struct RotCourse {
     if (tabu_phase) {
       if (__builtin_expect(it == iters || stalled, 0)) {
         if (lane == 0) red[32].x = 1;  // for the helpers
+        __syncwarp();
         rot_barrier();
         return false;
       }
@@ -582,6 +582,7 @@ __device__ __forceinline__ void rot_clear_marks(int32_t* mark, int n, int ow) {
   rot_barrier();
   const int words = rot_big(NT) ? (n * (n - 1) / 2 + 1) / 2 : n * (n - 1) / 2;
   for (int x = (int)threadIdx.x - 32 * ow; x < words; x += rot_threads(NT) - 32 * ow) mark[x] = 0;
+  __syncwarp();
 }
 
 // Tenure of iteration it (from 1).
@@ -763,6 +764,7 @@ __device__ __forceinline__ void rot_owner() {
     }
   }
   d[4 * C] = d_init(v0, v1);
+  __syncwarp();
   rot_barrier();  // the others now clear the marks
 
   // arrays of two words per block, by byte offset
@@ -831,7 +833,8 @@ __device__ __forceinline__ void rot_owner() {
     const int wd = __reduce_min_sync(kFull, dd);
     const uint32_t wk = __reduce_min_sync(kFull, dd == wd ? kk : kNoMove);
     const bool none = wd == INT_MAX >> SB;
-    if (lane == 0) S::red()[warp] = make_int2(none ? INT_MAX : wd, (int)(none ? kNoMove : wk));
+    // (by every lane: lanes that part cost more)
+    S::red()[warp] = make_int2(none ? INT_MAX : wd, (int)(none ? kNoMove : wk));
   };
 
   scan(NOLIM);
@@ -1311,6 +1314,7 @@ __device__ __forceinline__ void rot_phase_x() {
       }
     }
     if (T.pt == 0) S.red()[33] = make_int2(r << 8 | s, tabu_phase ? it : 0);  // for the keeper
+    __syncwarp();
     rot_barrier();
     // while the other warps bring the table up to date: M, the labels and the
     // best solution
@@ -1328,6 +1332,7 @@ __device__ __forceinline__ void rot_phase_x() {
     course.best = better ? course.cur : course.best;
     best_iter = better ? it : best_iter;  // 0 in the descent
     if (KEEPS && T.keeper) keeper.template move<false>(r, s, tabu_phase ? it : 0);
+    __syncwarp();
   }
 
   // ---- outputs
@@ -1362,7 +1367,10 @@ __device__ __forceinline__ void rot_helper() {
   RotKeeper<NT, C, FE> keeper(W, T, S.mark());
   for (int mv = 0;; ++mv) {
     rot_barrier();
-    if (T.keeper && (threadIdx.x & 31) == 0) keeper.finish();
+    if (T.keeper) {
+      if ((threadIdx.x & 31) == 0) keeper.finish();
+      __syncwarp();
+    }
     rot_barrier();
     if (lds32(base + X_::red + 8 * 32)) break;
     const int2 move = lds64(base + X_::red + 8 * 33);
@@ -1371,6 +1379,7 @@ __device__ __forceinline__ void rot_helper() {
     rot_update_m<NT, FE>(T, reinterpret_cast<char*>(W.M), rot_big(NT) ? 0 : base + S.L.M,
                          base + X_::vw + P::RW * wt, base + X_::vwu + P::LW * wt, n, ldm, Q,
                          mv & (Q - 1));
+    __syncwarp();
   }
   if (T.keeper) keeper.results(W.s, W.row);
 }
