@@ -1064,22 +1064,13 @@ extern "C" qap_status qap_batch_search_noalloc(qap_batch* b, const qap_search_pa
   QAP_TRY(noalloc_scratch(b->device, &base));
   Launch L;
   QAP_TRY(plan_batch(b, params, &L));
-  size_t need = ws_layout(L.plan, b->dbytes, b->fbytes, b->nmax, params).stride;
-  if (b->fbytes == 4) {
-    // the call takes the sizes that it takes with int64 elements
-    std::vector<DevInstance> d8 = b->di;
-    for (DevInstance& d : d8) {
-      d.ldF = pad_ldF(d.n, 8);
-      d.ldP = pad_ldP(d.n, 8);
-    }
-    Plan p8;
-    if (!search_plan(b->nmax, (int64_t)b->count * params->starts >= 2 * (int64_t)b->sms, d8.data(),
-                     b->count, 8, b->dbytes, b->force64, b->smem_optin, 16, b->nmax > 181, params,
-                     &p8))
-      return QAP_EUNSUPPORTED;
-    need += ws_layout(p8, b->dbytes, 8, b->nmax, params).stride;
-  }
-  if (need != 0) {
+  bool bad = false;
+  const bool many = (int64_t)b->count * params->starts >= 2 * (int64_t)b->sms;
+  const bool takes = batch_takes_workspace(L.plan, b->nmax, many, b->di.data(), b->count,
+                                           b->fbytes, b->dbytes, b->force64, b->smem_optin,
+                                           params, &bad);
+  if (bad) return QAP_EUNSUPPORTED;
+  if (takes) {
     snprintf(g_last_error, sizeof(g_last_error),
              "qap_batch_search_noalloc: n = %d needs a plan with a per-CTA workspace, which is "
              "allocated (the large-n plan, or int64 elements beyond shared memory)", b->nmax);

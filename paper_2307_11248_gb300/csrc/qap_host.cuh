@@ -350,22 +350,22 @@ inline void launch_walks(const void* fn, const Plan& p, int grid, int smem, cuda
   reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(fn))<<<grid, p.nt, smem, stream>>>(b);
 }
 
-// Shared memory of a plan for the instance shapes `d` (the largest over them).
+// Shared memory of a plan for the instance shapes `d` (the largest over them),
+// with elements of fbytes (whatever width d's own images have).
 inline int plan_smem(const Plan& p, const DevInstance* d, int count, int fbytes, int dbytes) {
   int smem = 0;
-  if (p.rot) {
-    for (int i = 0; i < count; ++i)
-      smem = std::max(smem, qapk::rot_layout(d[i].n, d[i].ldF, fbytes, d[i].ldP, d[i].symF,
-                                             d[i].symD, p.store & qapk::kNoTransposed,
-                                             p.store & qapk::kGlobalM,
-                                             qapk::rot_fixed_bytes(p.shape(), fbytes))
-                                .bytes);
-    return smem;
+  for (int i = 0; i < count; ++i) {
+    const int ldF = pad_ldF(d[i].n, fbytes), ldP = pad_ldP(d[i].n, pbytes_of(fbytes));
+    const int bytes =
+        p.rot ? qapk::rot_layout(d[i].n, ldF, fbytes, ldP, d[i].symF, d[i].symD,
+                                 p.store & qapk::kNoTransposed, p.store & qapk::kGlobalM,
+                                 qapk::rot_fixed_bytes(p.shape(), fbytes))
+                    .bytes
+              : qapk::smem_layout(d[i].n, ldF, fbytes, ldP, d[i].symF, d[i].symD, dbytes,
+                                  p.nt * p.maxpt, p.store)
+                    .bytes;
+    smem = std::max(smem, bytes);
   }
-  for (int i = 0; i < count; ++i)
-    smem = std::max(smem, qapk::smem_layout(d[i].n, d[i].ldF, fbytes, d[i].ldP, d[i].symF,
-                                            d[i].symD, dbytes, p.nt * p.maxpt, p.store)
-                              .bytes);
   return smem;
 }
 
@@ -596,6 +596,21 @@ inline WsLayout ws_layout(const Plan& p, int dbytes, int fbytes, int nmax,
   w.stride = w.rws_off;
   if (uses_rule_tables(sp)) w.stride += ((size_t)(2 * nmax * nmax + nmax) * 4 + 255) / 256 * 256;
   return w;
+}
+
+// Whether a batch search in plan p takes a workspace, or would with int64
+// elements where its instances are stored as int32: the call that may not
+// allocate one takes the same sizes for both.  No plan with int64 elements counts
+// as one that takes it (bad: QAP_EUNSUPPORTED).  Allocates nothing itself.
+inline bool batch_takes_workspace(const Plan& p, int nmax, bool many, const DevInstance* d,
+                                  int count, int fbytes, int dbytes, bool force64, int smem_optin,
+                                  const qap_search_params* sp, bool* bad) {
+  *bad = false;
+  if (ws_layout(p, dbytes, fbytes, nmax, sp).stride != 0) return true;
+  if (fbytes != 4) return false;
+  Plan p8;
+  *bad = !search_plan(nmax, many, d, count, 8, dbytes, force64, smem_optin, 16, nmax > 181, sp, &p8);
+  return *bad || ws_layout(p8, dbytes, 8, nmax, sp).stride != 0;
 }
 
 // With the frequency penalty a non-improving move's rank is delta + lambda *
