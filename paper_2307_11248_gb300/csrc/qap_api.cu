@@ -88,9 +88,10 @@ struct qap_batch {
   size_t scratch_bytes = 0;
   void* ws = nullptr;  // workspace of large-n plans and rule tables
   size_t ws_bytes = 0;
-  // size classes of the last search shape (threads_per_walk, starts)
+  // size classes of the last search shape (threads_per_walk, starts, rule
+  // tables, form of phase X)
   std::vector<BatchClass> classes;
-  int classes_threads = -1, classes_walks = 0, classes_rules = -1;
+  int classes_threads = -1, classes_walks = 0, classes_rules = -1, classes_phase_x = -1;
   int32_t* d_class_items = nullptr;  // per class item_inst | item_walk, then row_base
   cudaEvent_t fork = nullptr;
   std::vector<Plan> tuned;  // per instance: the autotuner's plan (nt == 0: none)
@@ -211,12 +212,16 @@ qap_status class_shape(qap_batch* b, BatchClass& c, int W, const qap_search_para
 // launch.  Classes run on side streams, largest n first, so the longest
 // walks start first and the other classes fill the SMs as those finish.
 // The instance tables (one per thread count) and the item lists are written
-// synchronously and cached for the same (threads, starts, rule tables).
-qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
+// synchronously and cached for the same (threads, starts, rule tables, form of
+// phase X).  `captured`: the search is being captured, where nothing can be
+// written; the form of phase X changes no walk, so classes made for the other
+// form serve it.
+qap_status plan_classes(qap_batch* b, const qap_search_params* p, bool captured = false) {
   const int rules = uses_rule_tables(p) ? 1 : 0;
   const int W = p->starts;
   if (!b->classes.empty() && b->classes_threads == p->threads_per_walk &&
-      b->classes_walks == W && b->classes_rules == rules)
+      b->classes_walks == W && b->classes_rules == rules &&
+      (b->classes_phase_x == p->phase_x || captured))
     return QAP_OK;
   if ((size_t)b->count * W > (size_t)INT_MAX / 2) return QAP_EINVAL;
   b->classes_threads = -1;
@@ -225,7 +230,8 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
     if (p->threads_per_walk == 0 && !b->tuned.empty() && b->tuned[i].nt != 0) {
       plan_of[i] = b->tuned[i];
       if (p->phase_x == QAP_PHASE_X_DOTS || rules) plan_of[i] = plan_of[i].rows();
-      if (p->phase_x == QAP_PHASE_X_DOTS) plan_of[i].store &= ~qapk::kProductM;
+      if (p->phase_x == QAP_PHASE_X_DOTS)  // (only the products go without the copies)
+        plan_of[i].store &= ~(qapk::kProductM | qapk::kNoTransposed);
       continue;
     }
     // the batch kernel also holds one static int
@@ -303,6 +309,7 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p) {
   b->classes_threads = p->threads_per_walk;
   b->classes_walks = W;
   b->classes_rules = rules;
+  b->classes_phase_x = p->phase_x;
   return QAP_OK;
 }
 
@@ -916,8 +923,10 @@ qap_status qap_batch_search_async(qap_batch* b, const qap_search_params* params,
   for (const DevInstance& d : b->di) QAP_TRY(check_penalty(params, b->dbytes, d.bound));
   DeviceGuard dg;
   QAP_TRY(dg.set(b->device));
-  QAP_TRY(plan_classes(b, params));
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (b->classes_phase_x != params->phase_x) QAP_CUDA(cudaStreamIsCapturing(s, &capturing));
+  QAP_TRY(plan_classes(b, params, capturing != cudaStreamCaptureStatusNone));
   const size_t total = (size_t)b->count * params->starts;
   const bool fork = b->classes.size() > 1;
   if (fork) QAP_CUDA(cudaEventRecord(b->fork, s));
