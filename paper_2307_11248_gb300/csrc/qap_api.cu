@@ -52,8 +52,9 @@ struct BatchClass {
   // is in the rotation layout): both made with the class, so that a search
   // whose tenures need the rows finds them ready
   struct Shape {
+    Plan plan{};
     const void* fn = nullptr;
-    int nt = 0, smem = 0, grid = 0, ctas_per_sm = 0, notr = 0;
+    int smem = 0, grid = 0, ctas_per_sm = 0;
     size_t ws_stride = 0, p_off = 0, rws_off = 0;  // workspace: bytes per CTA, offsets in them
   } own, rows;
   int nmax = 0;
@@ -181,8 +182,7 @@ qap_status class_shape(qap_batch* b, BatchClass& c, int W, const qap_search_para
     if (occ < 1) return QAP_EUNSUPPORTED;
     o->ctas_per_sm = occ;
     o->grid = std::min(c.items, occ * b->sms);
-    o->notr = (plan.store & qapk::kNoTransposed) != 0;
-    o->nt = plan.nt;
+    o->plan = plan;
     const WsLayout wl = ws_layout(plan, b->dbytes, b->fbytes, nmax, p);
     o->ws_stride = wl.stride;
     o->p_off = wl.p_off;
@@ -412,7 +412,7 @@ qap_status qap_plan(qap_ctx* ctx, const qap_search_params* params, qap_plan_info
   out->sms = ctx->sms;
   out->classes = 1;
   out->products = products_form(L.plan);
-  out->workspace = (L.plan.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
+  out->workspace = has_workspace(L.plan);
   return QAP_OK;
 }
 
@@ -690,16 +690,16 @@ qap_status qap_batch_plan(qap_batch* b, const qap_search_params* params, qap_pla
   QAP_TRY(dg.set(b->device));
   QAP_TRY(plan_classes(b, params));
   const BatchClass& c = b->classes.front();  // the class of the largest n
-  out->pairs_per_thread = c.plan.maxpt;
   const BatchClass::Shape& sh = c.shape(params);
-  out->threads_per_walk = sh.nt;
+  out->threads_per_walk = sh.plan.nt;
+  out->pairs_per_thread = sh.plan.maxpt;
   out->smem_bytes = sh.smem;
   out->grid = sh.grid;
   out->ctas_per_sm = sh.ctas_per_sm;
   out->sms = b->sms;
   out->classes = (int32_t)b->classes.size();
-  out->products = products_form(c.plan);
-  out->workspace = (c.plan.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
+  out->products = products_form(sh.plan);
+  out->workspace = has_workspace(sh.plan);
   return QAP_OK;
 }
 
@@ -732,11 +732,11 @@ qap_status qap_batch_classes(qap_batch* b, const qap_search_params* params,
     }
     o.instances = (int32_t)c.members.size();
     o.walks = c.items;
-    o.pairs_per_thread = c.plan.maxpt;
-    o.products = products_form(c.plan);
     const BatchClass::Shape& sh = c.shape(params);
-    o.threads_per_walk = sh.nt;
-    o.workspace = (c.plan.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
+    o.threads_per_walk = sh.plan.nt;
+    o.pairs_per_thread = sh.plan.maxpt;
+    o.products = products_form(sh.plan);
+    o.workspace = has_workspace(sh.plan);
     o.grid = sh.grid;
     o.ctas_per_sm = sh.ctas_per_sm;
     o.smem_bytes = sh.smem;
@@ -862,13 +862,13 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       const BatchClass::Shape& sh = c.shape(&tp);
       if ((st = grow(&b->ws, &b->ws_bytes, c.workspace())) != QAP_OK) return fail(st);
       qapk::BatchArgs a{};
-      a.insts = b->d_insts + (size_t)nt_index(sh.nt) * b->count;
+      a.insts = b->d_insts + (size_t)nt_index(sh.plan.nt) * b->count;
       a.item_inst = d_items;
       a.item_walk = d_items + items;
       a.row_base = d_items + 2 * items;
       a.items = c.items;
       a.counter = counter;
-      a.notr = sh.notr;
+      a.notr = (sh.plan.store & qapk::kNoTransposed) != 0;
       a.s = make_search_args(&tp, &dout, b->nmax);
       a.s.rws_off = sh.rws_off;
       a.s.p_off = sh.p_off;
@@ -879,7 +879,7 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       for (int rep = 0; rep < 2; ++rep) {  // a warm-up run, then the timed one
         cudaMemsetAsync(counter, 0, sizeof(int), b->stream);
         if (rep) cudaEventRecord(t0, b->stream);
-        fn<<<sh.grid, sh.nt, sh.smem, b->stream>>>(a);
+        fn<<<sh.grid, sh.plan.nt, sh.smem, b->stream>>>(a);
         if (rep) cudaEventRecord(t1, b->stream);
       }
       // a trial that did not launch would time as the fastest
@@ -899,10 +899,11 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       r.nmax = nmax;
       r.instances = (int32_t)rc.members.size();
       r.candidates = (int32_t)cands.size();
-      r.threads_per_walk = best.nt;
-      r.pairs_per_thread = best.maxpt;
-      r.workspace = (best.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
-      r.products = products_form(best);
+      const Plan ran = rot_holds_tenures(best, &tp, nmax) ? best : best.rows();
+      r.threads_per_walk = ran.nt;
+      r.pairs_per_thread = ran.maxpt;
+      r.workspace = has_workspace(ran);
+      r.products = products_form(ran);
       r.trial_ms = best_ms;
       r.rule_ms = rule_ms;
     }
@@ -938,13 +939,13 @@ qap_status qap_batch_search_async(qap_batch* b, const qap_search_params* params,
     if (fork) QAP_CUDA(cudaStreamWaitEvent(cs, b->fork, 0));
     const BatchClass::Shape& sh = c.shape(params);
     qapk::BatchArgs a{};
-    a.insts = b->d_insts + (size_t)nt_index(sh.nt) * b->count;
+    a.insts = b->d_insts + (size_t)nt_index(sh.plan.nt) * b->count;
     a.item_inst = b->d_class_items + c.item_off;
     a.item_walk = b->d_class_items + total + c.item_off;
     a.row_base = b->d_class_items + 2 * total;
     a.items = c.items;
     a.counter = b->d_counter + k * kCounterStride;
-    a.notr = sh.notr;
+    a.notr = (sh.plan.store & qapk::kNoTransposed) != 0;
     a.s = make_search_args(params, out, p_stride);
     a.s.rws_off = sh.rws_off;
     a.s.p_off = sh.p_off;
@@ -953,7 +954,7 @@ qap_status qap_batch_search_async(qap_batch* b, const qap_search_params* params,
     QAP_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(int), cs));
     const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(sh.fn));
     if (b->timing) QAP_CUDA(cudaEventRecord(c.t0, cs));
-    fn<<<sh.grid, sh.nt, sh.smem, cs>>>(a);
+    fn<<<sh.grid, sh.plan.nt, sh.smem, cs>>>(a);
     QAP_CUDA(cudaGetLastError());
     if (b->timing) QAP_CUDA(cudaEventRecord(c.t1, cs));
     c.timed = b->timing != 0;

@@ -395,6 +395,11 @@ inline int products_form(const Plan& p) {
   return !(p.store & qapk::kProductM) ? 0 : (p.store & qapk::kNoTransposed) ? 2 : 1;
 }
 
+// Whether M, or deltas and marks, lie in the CTA's workspace.
+inline int has_workspace(const Plan& p) {
+  return (p.store & (qapk::kGlobalDelta | qapk::kGlobalM)) != 0;
+}
+
 // The products form of a register plan when the flows are stored as int8 or
 // int16 and M fits shared memory too (phase X then reads M instead of
 // computing dot products), unless the caller asks for the dot products.
