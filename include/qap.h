@@ -381,7 +381,7 @@ typedef struct {
  * flows also in its products form, which keeps the n x n dot products of
  * phase X in shared memory and updates them per move), and the workspace
  * plan that keeps the deltas and tabu marks in L2/HBM instead of registers
- * and shared memory.  The trial runs params->starts walks of
+ * and shared memory; the rule's own plan is among them.  The trial runs params->starts walks of
  * `trial_iters` iterations; the fastest plan is kept for the class, and
  * later searches with threads_per_walk = 0 use the kept plans (classes are
  * regrouped by them).  Results are unchanged: every plan computes the same

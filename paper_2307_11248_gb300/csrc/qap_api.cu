@@ -754,7 +754,7 @@ qap_status qap_batch_classes(qap_batch* b, const qap_search_params* params,
 
 // The autotuner: for every size class of the rule, time each compiled plan
 // that holds the class's largest n (each thread count with its fewest slots,
-// and the workspace plan) on the class's own instances with the search's
+// the workspace plan, and the rule's own) on the class's own instances with the search's
 // walk count and `trial_iters` iterations, and keep the fastest.  Every plan
 // computes the same walks, so the choice changes only the speed.
 qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
@@ -839,6 +839,9 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
         if (big.rot) cands.push_back(big);
       }
     }
+    // the rule's own plan, which may leave out what these keep (the transposed
+    // copies, so that two walks share an SM)
+    if (std::find(cands.begin(), cands.end(), rc.plan) == cands.end()) cands.push_back(rc.plan);
     // items of this class, longest instances first; row bases for all
     const size_t items = rc.members.size() * (size_t)W;
     std::vector<int32_t> h(items * 2 + b->count);
