@@ -562,6 +562,10 @@ inline bool uses_rule_tables(const qap_search_params* sp) {
   return sp->iters > 0 && (sp->criterion != QAP_TABU_PAIR || sp->freq_penalty != 0);
 }
 
+// Static shared memory of the rotation kernels (an item's number), that searches
+// of one instance, whose other kernels have none, must leave room for too.
+constexpr int kRotStatic = 16;
+
 // The plan a search takes: choose_plan_fit's, in the rotation layout where
 // that applies and still lets two CTAs share an SM where the row layout does.
 // (Its tenures are another condition: rot_holds_tenures.)  `workspace`: a plan
@@ -573,7 +577,8 @@ inline bool search_plan(int nmax, bool many, const DevInstance* d, int count, in
                        reserve, sp->phase_x, out))
     return false;
   auto ctas = [&](const Plan& x) {  // by shared memory (1 KB reserved for each), 2 at most
-    const int smem = plan_smem(x, d, count, fbytes, dbytes) + reserve;
+    const int fixed = x.rot ? std::max(reserve, kRotStatic) : reserve;
+    const int smem = plan_smem(x, d, count, fbytes, dbytes) + fixed;
     return smem > smem_optin ? 0 : 2 * (smem + 1024) <= smem_optin + 1024 ? 2 : 1;
   };
   const int want = out->nt <= 256 ? ctas(*out) : 1;  // (above, registers hold one)
