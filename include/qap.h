@@ -271,7 +271,8 @@ qap_status qap_search(qap_ctx* ctx, const qap_search_params* params, const int32
  *            call's work.
  *   stream   a cudaStream_t (NULL = legacy default stream).
  * Kernel launches only; capturable into a CUDA graph once a search with the
- * same n, starts, threads_per_walk and delta width has run outside capture.
+ * same n, starts, threads_per_walk, delta width and rule tables (criterion !=
+ * PAIR or a penalty: on or off) has run outside capture.
  * Errors: QAP_EINVAL, QAP_EUNSUPPORTED, QAP_ECUDA (launch errors only). */
 qap_status qap_search_async(qap_ctx* ctx, const qap_search_params* params,
                             const int32_t* d_starts, const qap_walk_outputs* out,

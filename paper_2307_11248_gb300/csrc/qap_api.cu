@@ -43,6 +43,7 @@ struct qap_ctx {
   // workspace of large-n plans (one slice per CTA of the persistent grid)
   void* ws = nullptr;
   size_t ws_bytes = 0;
+  int rows_per_sm = 0;  // CTAs per SM of the row layout beside a workspace plan (0: not asked yet)
 };
 
 // Instances of a batch that share one launch plan (a size class).
@@ -131,6 +132,30 @@ qap_status plan_ctx(qap_ctx* ctx, const qap_search_params* p, Launch* L) {
   L->smem = plan_smem(L->plan, &ctx->di, 1, ctx->fbytes, ctx->dbytes);
   QAP_TRY(prepare_kernel(L->fn, L->smem));
   return occupancy(L, ctx->sms, p->starts);
+}
+
+// Workspace of a search by plan L, and of one with the same walks by its row
+// layout (longer tenures, dot products), whichever is larger: so that once a
+// search has run, another of its size can be captured whatever its layout.
+qap_status ctx_workspace(qap_ctx* ctx, const qap_search_params* p, const Launch& L, size_t stride,
+                         size_t* bytes) {
+  const bool plain = p->launch == QAP_LAUNCH_PLAIN;  // one CTA per launch
+  *bytes = stride * (plain ? 1 : L.grid);
+  if (!L.plan.rot) return QAP_OK;
+  const Plan rows = L.plan.rows();
+  if (ctx->rows_per_sm == 0) {  // (the same row plan for every search of the context)
+    Launch R{};
+    R.plan = rows;
+    R.fn = pick_walk_kernel(ctx->dbytes, ctx->fbytes, rows);
+    if (!R.fn) return QAP_EUNSUPPORTED;
+    R.smem = plan_smem(rows, &ctx->di, 1, ctx->fbytes, ctx->dbytes);
+    QAP_TRY(prepare_kernel(R.fn, R.smem));
+    QAP_TRY(occupancy(&R, ctx->sms, 1));
+    ctx->rows_per_sm = R.ctas_per_sm;
+  }
+  const int ctas = plain ? 1 : std::min(p->starts, ctx->rows_per_sm * ctx->sms);
+  *bytes = std::max(*bytes, ws_layout(rows, ctx->dbytes, ctx->fbytes, ctx->di.n, p).stride * ctas);
+  return QAP_OK;
 }
 
 qap_status plan_batch(qap_batch* b, const qap_search_params* p, Launch* L) {
@@ -439,9 +464,9 @@ qap_status qap_search_async(qap_ctx* ctx, const qap_search_params* params,
   a.s.rws_off = wl.rws_off;
   a.s.p_off = wl.p_off;
   if (a.ws_stride) {
-    // the plain form runs one CTA per launch; launches on one stream share it
-    const int ctas = params->launch == QAP_LAUNCH_PLAIN ? 1 : L.grid;
-    QAP_TRY(grow(&ctx->ws, &ctx->ws_bytes, a.ws_stride * ctas));
+    size_t bytes = 0;  // (the plain form's launches, on one stream, share it)
+    QAP_TRY(ctx_workspace(ctx, params, L, a.ws_stride, &bytes));
+    QAP_TRY(grow(&ctx->ws, &ctx->ws_bytes, bytes));
     a.ws = static_cast<unsigned char*>(ctx->ws);
   }
   if (params->launch == QAP_LAUNCH_PLAIN) {
