@@ -443,8 +443,8 @@ qap_status qap_batch_classes(qap_batch* b, const qap_search_params* params,
  *   `stream` by an event and joined back into it).  The first call for a
  *   given (starts, thread count, rule tables on or off) writes device
  *   tables synchronously and must not be captured in a CUDA graph; later
- *   calls can be.  A call for another form of phase X writes them again,
- *   but not under capture: there it runs the form of the call before.
+ *   calls can be (also for the other form of phase X, which then runs only
+ *   if it has run before: both give the same walks).
  * Errors: QAP_EINVAL, QAP_EUNSUPPORTED, QAP_ENOMEM, QAP_ECUDA. */
 qap_status qap_batch_search(qap_batch* b, const qap_search_params* params,
                             const qap_walk_outputs* out, int32_t p_stride);

@@ -74,6 +74,17 @@ struct BatchClass {
   bool timed = false;                      // t0, t1 bracket the class's last launch
 };
 
+// The size classes of a search shape, and their device tables.
+struct ClassSet {
+  std::vector<BatchClass> classes;
+  int threads = -1, walks = 0, rules = -1;  // the shape (threads -1: none)
+  int32_t* items = nullptr;  // on the device: per class item_inst | item_walk, then row_base
+  bool serves(const qap_search_params* p) const {
+    return !classes.empty() && threads == p->threads_per_walk && walks == p->starts &&
+           rules == (uses_rule_tables(p) ? 1 : 0);
+  }
+};
+
 struct qap_batch {
   int device = 0, sms = 0, smem_optin = 0;
   int count = 0, nmax = 0;
@@ -90,11 +101,9 @@ struct qap_batch {
   size_t scratch_bytes = 0;
   void* ws = nullptr;  // workspace of large-n plans and rule tables
   size_t ws_bytes = 0;
-  // size classes of the last search shape (threads_per_walk, starts, rule
-  // tables, form of phase X)
-  std::vector<BatchClass> classes;
-  int classes_threads = -1, classes_walks = 0, classes_rules = -1, classes_phase_x = -1;
-  int32_t* d_class_items = nullptr;  // per class item_inst | item_walk, then row_base
+  // of the last search shape of each form of phase X (a search of one form
+  // leaves the tables that captured searches of the other read)
+  ClassSet sets[2];
   cudaEvent_t fork = nullptr;
   std::vector<Plan> tuned;  // per instance: the autotuner's plan (nt == 0: none)
   int timing = 0;           // record timing events around each class's launch
@@ -232,24 +241,31 @@ qap_status class_shape(qap_batch* b, BatchClass& c, int W, const qap_search_para
   return QAP_OK;
 }
 
+int form_of(const qap_search_params* p) { return p->phase_x == QAP_PHASE_X_DOTS ? 1 : 0; }
+
 // Size classes of a batch search: every instance takes the plan its own n
 // would get alone, and instances with the same plan share one persistent
 // launch.  Classes run on side streams, largest n first, so the longest
 // walks start first and the other classes fill the SMs as those finish.
 // The instance tables (one per thread count) and the item lists are written
-// synchronously and cached for the same (threads, starts, rule tables, form of
-// phase X).  `captured`: the search is being captured, where nothing can be
-// written; the form of phase X changes no walk, so classes made for the other
-// form serve it.
-qap_status plan_classes(qap_batch* b, const qap_search_params* p, bool captured = false) {
+// synchronously and cached for the same (threads, starts, rule tables), one set
+// for each form of phase X.  `captured`: the search is being captured, where
+// nothing can be written; the form of phase X changes no walk, so classes made for
+// the other form serve it.
+qap_status plan_classes(qap_batch* b, const qap_search_params* p, ClassSet** out,
+                        bool captured = false) {
   const int rules = uses_rule_tables(p) ? 1 : 0;
   const int W = p->starts;
-  if (!b->classes.empty() && b->classes_threads == p->threads_per_walk &&
-      b->classes_walks == W && b->classes_rules == rules &&
-      (b->classes_phase_x == p->phase_x || captured))
+  ClassSet& set = b->sets[form_of(p)];
+  ClassSet& other = b->sets[1 - form_of(p)];
+  *out = &set;
+  if (set.serves(p)) return QAP_OK;
+  if (captured && other.serves(p)) {
+    *out = &other;
     return QAP_OK;
+  }
   if ((size_t)b->count * W > (size_t)INT_MAX / 2) return QAP_EINVAL;
-  b->classes_threads = -1;
+  set.threads = -1;
   std::vector<Plan> plan_of(b->count);
   for (int i = 0; i < b->count; ++i) {
     if (p->threads_per_walk == 0 && !b->tuned.empty() && b->tuned[i].nt != 0) {
@@ -272,24 +288,24 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p, bool captured 
                    [&](int x, int y) { return b->di[x].n > b->di[y].n; });
   // keep the old classes' streams and events for reuse
   std::vector<BatchClass> old;
-  old.swap(b->classes);
+  old.swap(set.classes);
   for (int i : order) {  // classes appear in order of their largest n
     BatchClass* c = nullptr;
-    for (BatchClass& k : b->classes)
+    for (BatchClass& k : set.classes)
       if (k.plan == plan_of[i]) c = &k;
     if (!c) {
-      b->classes.emplace_back();
-      c = &b->classes.back();
+      set.classes.emplace_back();
+      c = &set.classes.back();
       c->plan = plan_of[i];
     }
     c->members.push_back(i);
   }
-  for (size_t k = 0; k < b->classes.size(); ++k) {
+  for (size_t k = 0; k < set.classes.size(); ++k) {
     if (k < old.size()) {
-      b->classes[k].side = old[k].side;
-      b->classes[k].done = old[k].done;
-      b->classes[k].t0 = old[k].t0;
-      b->classes[k].t1 = old[k].t1;
+      set.classes[k].side = old[k].side;
+      set.classes[k].done = old[k].done;
+      set.classes[k].t0 = old[k].t0;
+      set.classes[k].t1 = old[k].t1;
       old[k].side = nullptr;
       old[k].done = nullptr;
       old[k].t0 = old[k].t1 = nullptr;
@@ -298,24 +314,24 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p, bool captured 
   for (BatchClass& c : old) destroy_class_handles(c);
   int item_off = 0;
   size_t ws_off = 0;
-  for (BatchClass& c : b->classes) {
+  for (BatchClass& c : set.classes) {
     QAP_TRY(class_shape(b, c, W, p));
     c.item_off = item_off;
     item_off += c.items;
     c.ws_off = ws_off;
     ws_off += (c.workspace() + 255) / 256 * 256;
-    if (b->classes.size() > 1) {
+    if (set.classes.size() > 1) {
       if (!c.side) QAP_CUDA(cudaStreamCreateWithFlags(&c.side, cudaStreamNonBlocking));
       if (!c.done) QAP_CUDA(cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming));
     }
     c.timed = false;
   }
-  if (b->classes.size() > 1 && !b->fork)
+  if (set.classes.size() > 1 && !b->fork)
     QAP_CUDA(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
   // item lists: class after class, each longest instances first; row bases
   const size_t total = (size_t)item_off;
   std::vector<int32_t> h(total * 2 + b->count);
-  for (const BatchClass& c : b->classes) {
+  for (const BatchClass& c : set.classes) {
     size_t k = c.item_off;
     for (int inst : c.members)
       for (int w = 0; w < W; ++w, ++k) {
@@ -324,17 +340,16 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p, bool captured 
       }
   }
   for (int i = 0; i < b->count; ++i) h[2 * total + i] = i * W;
-  if (b->d_class_items) cudaFree(b->d_class_items);
-  b->d_class_items = nullptr;
-  if (cudaMalloc(&b->d_class_items, h.size() * sizeof(int32_t)) != cudaSuccess)
+  if (set.items) cudaFree(set.items);
+  set.items = nullptr;
+  if (cudaMalloc(&set.items, h.size() * sizeof(int32_t)) != cudaSuccess)
     return QAP_ENOMEM;
-  QAP_CUDA(cudaMemcpy(b->d_class_items, h.data(), h.size() * sizeof(int32_t),
+  QAP_CUDA(cudaMemcpy(set.items, h.data(), h.size() * sizeof(int32_t),
                       cudaMemcpyHostToDevice));
   QAP_TRY(grow(&b->ws, &b->ws_bytes, ws_off));
-  b->classes_threads = p->threads_per_walk;
-  b->classes_walks = W;
-  b->classes_rules = rules;
-  b->classes_phase_x = p->phase_x;
+  set.threads = p->threads_per_walk;
+  set.walks = W;
+  set.rules = rules;
   return QAP_OK;
 }
 
@@ -692,8 +707,10 @@ void qap_batch_destroy(qap_batch* b) {
   if (b->d_counter) cudaFree(b->d_counter);
   if (b->scratch) cudaFree(b->scratch);
   if (b->ws) cudaFree(b->ws);
-  if (b->d_class_items) cudaFree(b->d_class_items);
-  for (BatchClass& c : b->classes) destroy_class_handles(c);
+  for (ClassSet& set : b->sets) {
+    if (set.items) cudaFree(set.items);
+    for (BatchClass& c : set.classes) destroy_class_handles(c);
+  }
   if (b->fork) cudaEventDestroy(b->fork);
   if (b->stream) cudaStreamDestroy(b->stream);
   delete b;
@@ -713,8 +730,9 @@ qap_status qap_batch_plan(qap_batch* b, const qap_search_params* params, qap_pla
   QAP_TRY(validate_params(params));
   DeviceGuard dg;
   QAP_TRY(dg.set(b->device));
-  QAP_TRY(plan_classes(b, params));
-  const BatchClass& c = b->classes.front();  // the class of the largest n
+  ClassSet* set = nullptr;
+  QAP_TRY(plan_classes(b, params, &set));
+  const BatchClass& c = set->classes.front();  // the class of the largest n
   const BatchClass::Shape& sh = c.shape(params);
   out->threads_per_walk = sh.plan.nt;
   out->pairs_per_thread = sh.plan.maxpt;
@@ -722,7 +740,7 @@ qap_status qap_batch_plan(qap_batch* b, const qap_search_params* params, qap_pla
   out->grid = sh.grid;
   out->ctas_per_sm = sh.ctas_per_sm;
   out->sms = b->sms;
-  out->classes = (int32_t)b->classes.size();
+  out->classes = (int32_t)set->classes.size();
   out->products = products_form(sh.plan);
   out->workspace = has_workspace(sh.plan);
   return QAP_OK;
@@ -741,10 +759,11 @@ qap_status qap_batch_classes(qap_batch* b, const qap_search_params* params,
   QAP_TRY(validate_params(params));
   DeviceGuard dg;
   QAP_TRY(dg.set(b->device));
-  QAP_TRY(plan_classes(b, params));
-  if (count) *count = (int32_t)b->classes.size();
-  for (size_t k = 0; k < b->classes.size(); ++k) {
-    BatchClass& c = b->classes[k];
+  ClassSet* set = nullptr;
+  QAP_TRY(plan_classes(b, params, &set));
+  if (count) *count = (int32_t)set->classes.size();
+  for (size_t k = 0; k < set->classes.size(); ++k) {
+    BatchClass& c = set->classes[k];
     if (inst_class)
       for (int i : c.members) inst_class[i] = (int32_t)k;
     if ((int32_t)k >= max_out) continue;
@@ -797,11 +816,12 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
   DeviceGuard dg;
   QAP_TRY(dg.set(b->device));
   b->tuned.clear();
-  b->classes_threads = -1;
-  QAP_TRY(plan_classes(b, &tp));
+  for (ClassSet& s : b->sets) s.threads = -1;
+  ClassSet* set = nullptr;
+  QAP_TRY(plan_classes(b, &tp, &set));
   struct RuleClass { Plan plan; std::vector<int> members; };
   std::vector<RuleClass> rule;
-  for (const BatchClass& c : b->classes) rule.push_back({c.plan, c.members});
+  for (const BatchClass& c : set->classes) rule.push_back({c.plan, c.members});
   const int W = params->starts;
   const size_t rows = (size_t)b->count * W;
   QAP_TRY(grow(&b->scratch, &b->scratch_bytes, rows * 8));
@@ -939,7 +959,7 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
   }
   if (nresults) *nresults = found;
   b->tuned = tuned;
-  b->classes_threads = -1;  // the next search regroups by the tuned plans
+  for (ClassSet& s : b->sets) s.threads = -1;  // the next search regroups by the tuned plans
   return fail(QAP_OK);
 }
 
@@ -954,13 +974,14 @@ qap_status qap_batch_search_async(qap_batch* b, const qap_search_params* params,
   QAP_TRY(dg.set(b->device));
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (b->classes_phase_x != params->phase_x) QAP_CUDA(cudaStreamIsCapturing(s, &capturing));
-  QAP_TRY(plan_classes(b, params, capturing != cudaStreamCaptureStatusNone));
+  if (!b->sets[form_of(params)].serves(params)) QAP_CUDA(cudaStreamIsCapturing(s, &capturing));
+  ClassSet* set = nullptr;
+  QAP_TRY(plan_classes(b, params, &set, capturing != cudaStreamCaptureStatusNone));
   const size_t total = (size_t)b->count * params->starts;
-  const bool fork = b->classes.size() > 1;
+  const bool fork = set->classes.size() > 1;
   if (fork) QAP_CUDA(cudaEventRecord(b->fork, s));
-  for (size_t k = 0; k < b->classes.size(); ++k) {
-    BatchClass& c = b->classes[k];
+  for (size_t k = 0; k < set->classes.size(); ++k) {
+    BatchClass& c = set->classes[k];
     cudaStream_t cs = fork ? c.side : s;
     if (b->timing && !c.t0) QAP_CUDA(cudaEventCreate(&c.t0));
     if (b->timing && !c.t1) QAP_CUDA(cudaEventCreate(&c.t1));
@@ -968,9 +989,9 @@ qap_status qap_batch_search_async(qap_batch* b, const qap_search_params* params,
     const BatchClass::Shape& sh = c.shape(params);
     qapk::BatchArgs a{};
     a.insts = b->d_insts + (size_t)nt_index(sh.plan.nt) * b->count;
-    a.item_inst = b->d_class_items + c.item_off;
-    a.item_walk = b->d_class_items + total + c.item_off;
-    a.row_base = b->d_class_items + 2 * total;
+    a.item_inst = set->items + c.item_off;
+    a.item_walk = set->items + total + c.item_off;
+    a.row_base = set->items + 2 * total;
     a.items = c.items;
     a.counter = b->d_counter + k * kCounterStride;
     a.notr = (sh.plan.store & qapk::kNoTransposed) != 0;
