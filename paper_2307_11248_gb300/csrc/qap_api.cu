@@ -95,7 +95,7 @@ struct qap_batch {
   void* data = nullptr;  // every instance's F, F^T and D
   qapk::InstArgs* d_insts = nullptr;  // one table per thread count (128..1024)
   int insts_written = 0;              // bit t: the table for 128 << t is written
-  int* d_counter = nullptr;           // one work counter per class
+  int* d_counter = nullptr;           // one work counter per class (count at most), the autotuner's
   cudaStream_t stream = nullptr;
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
@@ -692,7 +692,8 @@ qap_status qap_batch_create(int32_t count, const int64_t* const* F, const int64_
   if (e != cudaSuccess) return fail(cuda_fail(e, "cudaMemcpy"));
   if (cudaMalloc(&b->d_insts, sizeof(qapk::InstArgs) * count * 4) != cudaSuccess)
     return fail(QAP_ENOMEM);
-  if (cudaMalloc(&b->d_counter, kCounterStride * 4 * 64) != cudaSuccess) return fail(QAP_ENOMEM);
+  if (cudaMalloc(&b->d_counter, sizeof(int) * kCounterStride * ((size_t)count + 1)) != cudaSuccess)
+    return fail(QAP_ENOMEM);
   e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) return fail(cuda_fail(e, "cudaStreamCreateWithFlags"));
   *out = b;
@@ -842,7 +843,7 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
     return fail(QAP_ENOMEM);
   if (cudaEventCreate(&t0) != cudaSuccess || cudaEventCreate(&t1) != cudaSuccess)
     return fail(cuda_fail(cudaGetLastError(), "cudaEventCreate"));
-  int* counter = b->d_counter + 63 * kCounterStride;
+  int* counter = b->d_counter + (size_t)b->count * kCounterStride;
   auto chk = [](cudaError_t e, const char* where) {
     return e == cudaSuccess ? QAP_OK : cuda_fail(e, where);
   };
