@@ -7,8 +7,6 @@ BatchKernelFn rot_f16_1024(int c) {
   switch (c) {
     case 2: return rot_kernel<1024, 2, int16_t>;
     case 4: return rot_kernel<1024, 4, int16_t>;
-    case 5: return rot_kernel<1024, 5, int16_t>;
-    case 6: return rot_kernel<1024, 6, int16_t>;
     default: return nullptr;
   }
 }

@@ -9,7 +9,6 @@ BatchKernelFn rot_f16_256w(int c) {
     case 7: return rot_kernel<256, 7, int16_t>;
     case 12: return rot_kernel<256, 12, int16_t>;
     case 13: return rot_kernel<256, 13, int16_t>;
-    case 14: return rot_kernel<256, 14, int16_t>;
     default: return nullptr;
   }
 }

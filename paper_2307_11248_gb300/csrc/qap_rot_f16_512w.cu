@@ -10,7 +10,6 @@ BatchKernelFn rot_f16_512w(int c) {
     case 8: return rot_kernel<512, 8, int16_t>;
     case 12: return rot_kernel<512, 12, int16_t>;
     case 13: return rot_kernel<512, 13, int16_t>;
-    case 14: return rot_kernel<512, 14, int16_t>;
     default: return nullptr;
   }
 }

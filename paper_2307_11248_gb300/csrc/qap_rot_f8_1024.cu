@@ -7,8 +7,6 @@ BatchKernelFn rot_f8_1024(int c) {
   switch (c) {
     case 2: return rot_kernel<1024, 2, int8_t>;
     case 4: return rot_kernel<1024, 4, int8_t>;
-    case 5: return rot_kernel<1024, 5, int8_t>;
-    case 6: return rot_kernel<1024, 6, int8_t>;
     default: return nullptr;
   }
 }

@@ -9,7 +9,6 @@ BatchKernelFn rot_f8_128(int c) {
     case 2: return rot_kernel<128, 2, int8_t>;
     case 4: return rot_kernel<128, 4, int8_t>;
     case 7: return rot_kernel<128, 7, int8_t>;
-    case 8: return rot_kernel<128, 8, int8_t>;
     default: return nullptr;
   }
 }

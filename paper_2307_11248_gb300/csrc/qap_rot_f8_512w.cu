@@ -10,7 +10,6 @@ BatchKernelFn rot_f8_512w(int c) {
     case 8: return rot_kernel<512, 8, int8_t>;
     case 12: return rot_kernel<512, 12, int8_t>;
     case 13: return rot_kernel<512, 13, int8_t>;
-    case 14: return rot_kernel<512, 14, int8_t>;
     default: return nullptr;
   }
 }

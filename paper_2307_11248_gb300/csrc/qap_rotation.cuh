@@ -105,10 +105,10 @@ __host__ __device__ constexpr int rot_max_n(int nt) {
 constexpr int kRotMaxC = 22;
 __host__ __device__ constexpr bool rot_compiled(int nt, int c) {
   return rot_big(nt)  ? c == 10 || c == 12 || c == 17 || c == 19 || c == 21 || c == 22
-         : nt == 128  ? c == 1 || c == 2 || c == 4 || c == 7 || c == 8
-         : nt == 256  ? c <= 4 || c == 6 || c == 7 || (c >= 12 && c <= 14)
-         : nt == 512  ? c <= 3 || c == 5 || c == 7 || c == 8 || (c >= 12 && c <= 14)
-                      : c == 2 || c == 4 || c == 5 || c == 6;
+         : nt == 128  ? c == 1 || c == 2 || c == 4 || c == 7
+         : nt == 256  ? c <= 4 || c == 6 || c == 7 || c == 12 || c == 13
+         : nt == 512  ? c <= 3 || c == 5 || c == 7 || c == 8 || c == 12 || c == 13
+                      : c == 2 || c == 4;
 }
 
 // Blocks on the circle: a multiple of c, with phantom blocks at the end.

@@ -1,7 +1,8 @@
 // Host-only checks of which layout a search takes (search_plan in qap_host.cuh; no
 // GPU, no CUDA calls): for every n, flow width, symmetry and number of walks the
 // ranges that the documents state, and a rotation plan whose shared memory, with
-// the kernel's static part, would pass the limit is not taken.  Built and run by
+// the kernel's static part, would pass the limit is not taken; every compiled number
+// of partner blocks is the fewest for some n.  Built and run by
 // tests/test_host_layouts.py; prints "ok" and exits 0, or the first violations.
 #include <cstdio>
 #include <string>
@@ -76,6 +77,21 @@ int main() {
               std::printf("FAIL beyond shared memory: n=%d fb=%d sym=%d many=%d batch=%d\n", n, fb,
                           sym, many, batch);
           }
+  for (int nt : {128, 256, 512, 1024, qapk::kRotBig})
+    for (int c = 1; c <= qapk::kRotMaxC; ++c) {
+      if (!qapk::rot_compiled(nt, c)) continue;
+      bool fewest = false;
+      for (int n = 3; n <= 256 && !fewest; ++n) {
+        qaph::Plan p;
+        const bool products = nt == qapk::kRotBig
+                                  ? n >= 152
+                                  : n <= 181 && qaph::plan_for(n, nt, &p) && qaph::has_product_form(p, 2);
+        int k = 1;
+        while (k < c && !(qapk::rot_compiled(nt, k) && qapk::rot_chunks(n, nt, k) > 0)) ++k;
+        fewest = products && k == c && qapk::rot_chunks(n, nt, c) > 0;
+      }
+      if (!fewest && fails++ < 10) std::printf("FAIL shape (%d, %d) is never taken\n", nt, c);
+    }
   if (fails) return 1;
   std::printf("ok\n");
   return 0;
