@@ -134,7 +134,8 @@ typedef struct {
 
 typedef struct {
   int32_t n;
-  int32_t delta_bytes;     /* 4 (int32 path) or 8 (int64 path)              */
+  int32_t delta_bytes;     /* 4 (int32 path) or 8 (int64 path: costs, and the
+                              row layout's deltas)                        */
   int32_t sym_flow;        /* F == F^T                                      */
   int32_t sym_dist;        /* D == D^T                                      */
   int64_t bound;           /* B above                                       */
@@ -148,10 +149,11 @@ typedef struct {
  *          the caller may free them when the call returns.  The element path
  *          and the delta width follow from the values (see above).
  *   n      2 <= n <= 256.  Up to n = 181 a walk keeps its deltas in
- *          registers; beyond, a workspace in device memory (allocated by the
- *          library on first use) holds its products M (int8 flows; batches and
- *          the serving loop use it from n = 152 on) or its deltas and marks,
- *          with F in shared or global memory.
+ *          registers (asymmetric int8 flows up to 176, int16 up to 156); beyond,
+ *          a workspace in device memory (allocated by the library on first use)
+ *          holds its products M (int8 flows from n = 182 on; in batches and the
+ *          serving loop from n = 152 on) or its deltas and marks, with F in
+ *          shared or global memory.
  *   flags  0 or QAP_FORCE_INT64.
  *   out    receives the context (NULL on error).
  * Uses the CUDA device current at the call for all later calls.
@@ -282,10 +284,12 @@ qap_status qap_search_async(qap_ctx* ctx, const qap_search_params* params,
 typedef struct {
   int32_t threads_per_walk;
   int32_t pairs_per_thread;  /* register slots per thread of the plan's row
-                                layout; int8 and int16 flows under
-                                QAP_TABU_PAIR without a penalty run a layout
-                                of the same threads in which fewer of them
-                                hold more pairs                              */
+                                layout; under QAP_TABU_PAIR without a penalty,
+                                int8 flows of n = 3-146 and int16 flows of n =
+                                3-149 run a layout of the same threads in
+                                which fewer of them hold more pairs, and int8
+                                flows with their products in the workspace one
+                                of 512 threads                               */
   int32_t smem_bytes;        /* dynamic shared memory per CTA             */
   int32_t grid;              /* CTAs of the persistent launch             */
   int32_t ctas_per_sm;

@@ -1515,7 +1515,7 @@ __device__ __forceinline__ void run_walk(const WalkSmem<DT, FE>& S, const InstAr
           if (su == r || su == s) {
             // four marks' loads in flight at once (each a chain of two, that no
             // store separates from the next: n = 100, unit-location criterion and
-            // penalty, 304 walks x 1000 14.3 -> 12.6 ms)
+            // penalty, 304 walks x 1000 14.3 -> 12.6 ms; n = 47, 160 walks, no change)
             for (int i0 = 0; i0 < slen; i0 += 4) {
               int t[4];
 #pragma unroll
@@ -1638,7 +1638,7 @@ using BatchKernelFn = void (*)(const BatchArgs);
 // Wide elements: both from global memory (L1, L2).
 // Host to host, with the check on the host and a CTA per permutation before
 // (the check alone 1030 us of the first) and now: n = 100, 20000 permutations
-// 1490 -> 145 us (60 us of it their copy to the GPU), 100 permutations 36 -> 31
+// 1490 -> 156 us (60 us of it their copy to the GPU), 100 permutations 36 -> 31
 // us; n = 256, 20000 permutations 4730 -> 510 us; n = 8 207 -> 62 us.
 // ---------------------------------------------------------------------------
 constexpr int kCostThreads = 512;

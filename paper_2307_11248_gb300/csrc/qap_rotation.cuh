@@ -19,7 +19,7 @@
 // mod C: the same slot in every thread, so that a move's columns, and a slot
 // whose tabu time ends, are found by one branch for the whole warp (against
 // slots in the window's order, where each thread compares each slot, n = 100
-// takes 3230 for 3385 warp instructions per walk-iteration).
+// went from 3385 to 3230 warp instructions per walk-iteration).
 
 // What a pair costs.  The table holds d(u, v) = delta(u, v) + g[u] + g[v]
 // (with g less its mid-range), whose O(1) update is one dp4a accumulating into
@@ -52,18 +52,18 @@
 // Bound: the fixed latencies of one iteration's chain (arg-min, phase X,
 // table, scan, two barriers) with one or two walks on an SM, integer issue
 // with more.  Measured against the row layout's products form (one GB300, same
-// box): n = 100 grid, 1024 walks x (2opt + 10^4) 150.0 -> 48.0 ms; n = 50
-// asymmetric, 256 walks x 5000 7.85 -> 4.24 ms; n = 139 asymmetric, 150 walks
-// x 2000 8.74 -> 2.89 ms; n = 23, 100 walks x 1000 in one blocking call 1.21 ->
-// 0.60 ms; 2opt from 32 starts at n = 12 16.4 -> 12.3 us.  Warp instructions per
-// walk-iteration: n = 100 grid 10360 -> 3236, n = 50 asymmetric 3606 -> 1924.
+// box): n = 100 grid, 1024 walks x (2opt + 10^4) 150.0 -> 47.4 ms; n = 50
+// asymmetric, 256 walks x 5000 7.85 -> 4.16 ms; n = 139 asymmetric, 150 walks
+// x 2000 8.74 -> 2.83 ms; n = 23, 100 walks x 1000 in one blocking call 1.21 ->
+// 0.58 ms; 2opt from 32 starts at n = 12 16.4 -> 10.9 us.  Warp instructions per
+// walk-iteration: n = 100 grid 10360 -> 3196, n = 50 asymmetric 3606 -> 1924.
 // int16 flows (two dp2a per pair): 96 lognormal instances of n = 20-150, 64
-// walks x 1000 each, 103.4 -> 39.4 ms; their costs need 64 bits, their deltas
+// walks x 1000 each, 103.4 -> 38.9 ms; their costs need 64 bits, their deltas
 // do not: the rows' sums of |F| bound them (rot_bounds), where the row layout
 // holds every delta as wide as the cost.
 // Large n (M in the workspace, two dp4a words of pending moves): n = 256 grid,
-// 64 walks x (2opt + 1000) 21.4 -> 6.6 ms, n = 203 asymmetric, 48 walks x 1000
-// 15.9 -> 3.6 ms against the workspace plan, that keeps deltas and marks in L2
+// 64 walks x (2opt + 1000) 21.4 -> 6.25 ms, n = 203 asymmetric, 48 walks x 1000
+// 15.9 -> 3.27 ms against the workspace plan, that keeps deltas and marks in L2
 // and recomputes dot products; 24 requests of n = 12-256 24.5 -> 6.6 ms.
 // Tried and slower: every warp holding pairs and phase X on some of them
 // (n = 100 2.33 against 1.44 us per iteration of two walks per SM); tabu times
