@@ -79,6 +79,8 @@ struct ClassSet {
   std::vector<BatchClass> classes;
   int threads = -1, walks = 0, rules = -1;  // the shape (threads -1: none)
   int32_t* items = nullptr;  // on the device: per class item_inst | item_walk, then row_base
+  void* ws = nullptr;        // workspace of large-n plans and rule tables
+  size_t ws_bytes = 0;
   bool serves(const qap_search_params* p) const {
     return !classes.empty() && threads == p->threads_per_walk && walks == p->starts &&
            rules == (uses_rule_tables(p) ? 1 : 0);
@@ -99,10 +101,8 @@ struct qap_batch {
   cudaStream_t stream = nullptr;
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
-  void* ws = nullptr;  // workspace of large-n plans and rule tables
-  size_t ws_bytes = 0;
   // of the last search shape of each form of phase X (a search of one form
-  // leaves the tables that captured searches of the other read)
+  // leaves what captured searches of the other read)
   ClassSet sets[2];
   cudaEvent_t fork = nullptr;
   std::vector<Plan> tuned;  // per instance: the autotuner's plan (nt == 0: none)
@@ -346,7 +346,7 @@ qap_status plan_classes(qap_batch* b, const qap_search_params* p, ClassSet** out
     return QAP_ENOMEM;
   QAP_CUDA(cudaMemcpy(set.items, h.data(), h.size() * sizeof(int32_t),
                       cudaMemcpyHostToDevice));
-  QAP_TRY(grow(&b->ws, &b->ws_bytes, ws_off));
+  QAP_TRY(grow(&set.ws, &set.ws_bytes, ws_off));
   set.threads = p->threads_per_walk;
   set.walks = W;
   set.rules = rules;
@@ -707,9 +707,9 @@ void qap_batch_destroy(qap_batch* b) {
   if (b->d_insts) cudaFree(b->d_insts);
   if (b->d_counter) cudaFree(b->d_counter);
   if (b->scratch) cudaFree(b->scratch);
-  if (b->ws) cudaFree(b->ws);
   for (ClassSet& set : b->sets) {
     if (set.items) cudaFree(set.items);
+    if (set.ws) cudaFree(set.ws);
     for (BatchClass& c : set.classes) destroy_class_handles(c);
   }
   if (b->fork) cudaEventDestroy(b->fork);
@@ -909,7 +909,7 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       c.members = rc.members;
       if ((st = class_shape(b, c, W, &tp)) != QAP_OK) return fail(st);
       const BatchClass::Shape& sh = c.shape(&tp);
-      if ((st = grow(&b->ws, &b->ws_bytes, c.workspace())) != QAP_OK) return fail(st);
+      if ((st = grow(&set->ws, &set->ws_bytes, c.workspace())) != QAP_OK) return fail(st);
       qapk::BatchArgs a{};
       a.insts = b->d_insts + (size_t)nt_index(sh.plan.nt) * b->count;
       a.item_inst = d_items;
@@ -922,7 +922,7 @@ qap_status qap_batch_autotune(qap_batch* b, const qap_search_params* params,
       a.s.rws_off = sh.rws_off;
       a.s.p_off = sh.p_off;
       a.ws_stride = sh.ws_stride;
-      a.ws = sh.ws_stride ? static_cast<unsigned char*>(b->ws) : nullptr;
+      a.ws = sh.ws_stride ? static_cast<unsigned char*>(set->ws) : nullptr;
       const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(sh.fn));
       float ms = 0.f;
       for (int rep = 0; rep < 2; ++rep) {  // a warm-up run, then the timed one
@@ -1000,7 +1000,7 @@ qap_status qap_batch_search_async(qap_batch* b, const qap_search_params* params,
     a.s.rws_off = sh.rws_off;
     a.s.p_off = sh.p_off;
     a.ws_stride = sh.ws_stride;
-    a.ws = sh.ws_stride ? static_cast<unsigned char*>(b->ws) + c.ws_off : nullptr;
+    a.ws = sh.ws_stride ? static_cast<unsigned char*>(set->ws) + c.ws_off : nullptr;
     QAP_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(int), cs));
     const auto fn = reinterpret_cast<qapk::BatchKernelFn>(const_cast<void*>(sh.fn));
     if (b->timing) QAP_CUDA(cudaEventRecord(c.t0, cs));

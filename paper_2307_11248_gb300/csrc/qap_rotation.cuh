@@ -55,7 +55,7 @@
 // box): n = 100 grid, 1024 walks x (2opt + 10^4) 150.0 -> 47.4 ms; n = 50
 // asymmetric, 256 walks x 5000 7.85 -> 4.16 ms; n = 139 asymmetric, 150 walks
 // x 2000 8.74 -> 2.83 ms; n = 23, 100 walks x 1000 in one blocking call 1.21 ->
-// 0.58 ms; 2opt from 32 starts at n = 12 16.4 -> 10.9 us.  Warp instructions per
+// 0.58 ms; 2opt from 32 starts at n = 12 16.4 -> 11-12 us.  Warp instructions per
 // walk-iteration: n = 100 grid 10360 -> 3196, n = 50 asymmetric 3606 -> 1924.
 // int16 flows (two dp2a per pair): 96 lognormal instances of n = 20-150, 64
 // walks x 1000 each, 103.4 -> 38.9 ms; their costs need 64 bits, their deltas

@@ -80,21 +80,23 @@ def test_a_captured_call_may_ask_for_the_other_form(gpu, first, captured):
             assert gpu.equal(outs[k], ref[k]), k
 
 
-def test_a_graph_outlives_searches_of_the_other_form(gpu):
-    """A captured search's tables stay while searches of the other form run."""
-    with _batch([20, 50, 145]) as b:
+@pytest.mark.parametrize("captured", [AUTO, DOTS])
+def test_a_graph_outlives_searches_of_the_other_form(gpu, captured):
+    """A captured search's tables and workspace stay while searches of the other
+    form run (n = 160 needs a workspace in one form only)."""
+    with _batch([20, 50, 145, 160, 200]) as b:
         outs = b.device_outputs(3)
         stream = gpu.cuda.Stream()
         with gpu.cuda.stream(stream):
-            b.search_async(_params(AUTO), outs, stream=stream)
+            b.search_async(_params(captured), outs, stream=stream)
         stream.synchronize()
         ref = {k: outs[k].clone() for k in FIELDS}
         g = gpu.cuda.CUDAGraph()
         with gpu.cuda.graph(g, stream=stream):
-            b.search_async(_params(AUTO), outs, stream=stream)
-        items = b.search(_params(DOTS))  # its own tables
+            b.search_async(_params(captured), outs, stream=stream)
+        other = b.search(_params(1 - captured))  # its own tables
         fill = gpu.full((1 << 20,), 7, dtype=gpu.int32, device="cuda")  # memory freed would be in use
-        for form in (AUTO, DOTS):
+        for form in (captured, 1 - captured):
             b.search(_params(form))
         for k in FIELDS:
             outs[k].zero_()
@@ -103,5 +105,5 @@ def test_a_graph_outlives_searches_of_the_other_form(gpu):
         gpu.cuda.synchronize()
         for k in FIELDS:
             assert gpu.equal(outs[k], ref[k]), k
-            assert np.array_equal(items[k].astype(np.int64), ref[k].cpu().numpy().astype(np.int64)), k
+            assert np.array_equal(other[k].astype(np.int64), ref[k].cpu().numpy().astype(np.int64)), k
         assert int(fill.sum()) == 7 << 20
